@@ -487,6 +487,37 @@ def test_dispatch_alg1_workloads(M, ws, oracle, name, S):
     check_dispatch(M, ws, oracle, 3, w["D"], w["H"], None, cap, Q, w["cand_prompt"], cb, S, res)
 
 
+@pytest.mark.parametrize("D,J,S,spread", [
+    # decoders at the edges of the registers-per-lane variants; a last chunk of
+    # candidates that is not full, and one candidate
+    (1, 33, 1, 2000), (31, 65, 16, 3000), (32, 1, 16, 3000), (33, 700, 1, 3000),
+    (64, 1000, 16, 5000), (65, 500, 32, 5000), (200, 500, 16, 5000), (257, 300, 1, 4000),
+    (600, 400, 16, 4000), (1024, 300, 16, 4000),
+    # budgets further apart than a 32-bit key holds (the wide comparison), from
+    # the start and after some reservations
+    (5, 400, 1, 2**30), (1000, 300, 1, 2**24), (2, 3000, 1, 2**29)])
+def test_dispatch_alg1_sequential_edges(M, ws, oracle, D, J, S, spread):
+    rng = np.random.default_rng(D * 31 + J)
+    per = 3
+    off = np.arange(D + 1, dtype=np.int64) * per
+    p = rng.integers(0, 400, D * per).astype(np.int32)
+    g = rng.integers(0, 300, D * per).astype(np.int32)
+    U = rng.integers(0, 600, D * per).astype(np.int32)
+    cap = rng.integers(0, spread, D).astype(np.int32)
+    Q = rng.integers(0, 4, D).astype(np.int32)
+    big = 600 if spread < 2**20 else 500000
+    cp = rng.integers(0, big, J).astype(np.int32)
+    cb = rng.integers(0, big, J).astype(np.int32)
+    check_dispatch(M, ws, oracle, 3, D, 1, None, cap, Q, cp, cb, S, (off, p, g, U))
+    # invalid candidates are skipped and reported; a queue length that passes
+    # int32 is reported
+    cp[J // 2] = -1
+    check_dispatch(M, ws, oracle, 3, D, 1, None, cap, Q, cp, cb, S, (off, p, g, U))
+    cp[J // 2] = 1
+    full = np.full(D, I32_MAX, np.int32)
+    check_dispatch(M, ws, oracle, 3, D, 1, None, cap, full, cp, cb, S, (off, p, g, U))
+
+
 def test_dispatch_errors(M, ws, oracle):
     K = np.zeros((2, 8), np.int32)
     st, ch, _, _, _ = gpu_dispatch(M, ws, 0, 2, 8, 1, K, [5, 5], [0, 0], [1, -1], [2, 2])
