@@ -820,156 +820,443 @@ dispatch_snapshot_kernel(const __grid_constant__ CUtensorMap tmap, SnapArgs a) {
 }
 
 // ---------------------------------------------------------------------------
-// Selection order shared by the sequential kernels: feasible before
-// infeasible; feasible by queue length, infeasible by largest headroom; then
-// the lowest decoder index.
+// SEQUENTIAL horizon dispatch: one block walks the candidates in order.
+// With F_k(t) = K[k][t] + t, scoring decoder k needs M_k(u) = max_{t<u} F_k(t);
+// reserving the footprint adds p + t + 1 to F_k*(t) for t < u.
+//
+// The walk is one chain of dependent decisions, so its cost is a decision's
+// latency: the instructions and barriers on the chain, at five to six cycles
+// an instruction for a warp.  A decision takes one barrier.  In phase j
+//   * each row warp picks candidate j's decoder (all the same one) from the
+//     scores of the phase before, adds the footprint to its chunk (128 steps)
+//     of that row and takes the maximum of F below the next candidate's u over
+//     it: together the chosen decoder's score for candidate j + 1.  A booking
+//     warp picks too, and writes the outputs;
+//   * the column warps, four lanes a decoder, meanwhile score every decoder for
+//     candidate j + 1.  Only the row being written may be read half updated,
+//     and its entry is the one that the row warps' maximum replaces.
+// A score is the maximum of the chunk maxima below u, at most 7 maxima of 16
+// steps, 3 of 4 and 3 cells: one kind to each of the four lanes.  The first P0
+// steps of each row with these maxima live in shared memory, the steps past
+// them in L2 (with maxima of 16 steps), where a candidate costs some L2 round
+// trips.
+//
+// The 32-bit pick keys, the smallest wins: a feasible decoder is
+// min(Q - q0, lim) << kb | k, an infeasible one 1 << 31 |
+// min(M - cap - x0, lim) << kb | k, q0 and x0 lower bounds for the whole call
+// (Q and K only grow, and M >= K[k][0]).  If even the smallest key is at lim
+// the pick is made on 64-bit keys.
+//
+// Measured, occupancy and walk: 16 decoders, H 16,384, 1,024 candidates 3.51 ->
+// 0.64 ms; 64 decoders, H 32,763, 2,003 candidates 8.1 -> 1.31 ms.  Before, one
+// block scored every decoder from global memory with four barriers a decision
+// (3.4 and 4.0 us each).  Forms in between: two warps a decoder, each scoring
+// and reserving in lockstep, 1.58 and 4.44 ms (issue bound: every warp ran the
+// whole pick); one chain warp reserving alone, 1.34 and 1.86 ms; a lane a
+// decoder in the columns and the pick and its bookkeeping in every row warp,
+// 0.93 and 1.68 ms.
 // ---------------------------------------------------------------------------
-struct Pick {
-  int inf;      // 0 feasible, 1 infeasible, 2 none yet
-  long long v;  // Q (feasible) or -headroom (infeasible)
-  int k;
-  long long h;  // headroom
+constexpr int kSeqChunk = 128;
+constexpr int kRowWarps = 8;
+constexpr int kColWarps = 16;  // at most
+constexpr int kSeqD = 32 * ((kMaxD + 31) / 32);
+
+struct SeqArgs {
+  int D, H;
+  int P0;              // resident steps of a row (whole chunks)
+  int P2;              // chunks whose maxima are resident
+  int ncol;            // column warps
+  int kb, mc;
+  int32_t *K;
+  uint32_t *km;        // [D][ceil(H/16)]  max of F per 16 steps
+  uint32_t *cm;        // [D][ceil(H/128)]  max of F per chunk, from chunk P2 on
+  const int32_t *cap;
+  int32_t *Q;
+  int64_t J;
+  const int32_t *cp, *cb;
+  int32_t *choice;
+  int64_t *headroom;
+  int32_t *status;
 };
-__device__ __forceinline__ bool better(const Pick &x, const Pick &y) {
-  if (x.inf != y.inf) return x.inf < y.inf;
-  if (x.v != y.v) return x.v < y.v;
-  return x.k < y.k;
-}
-// mc: rank every decoder by headroom alone (the memory-only ablation): all
-// picks take the infeasible class, whose order is the largest headroom first.
-__device__ __forceinline__ Pick make_pick(long long h, int32_t q, int k, bool mc = false) {
-  Pick p;
-  const bool feas = h >= 0 && !mc;
-  p.inf = feas ? 0 : 1;
-  p.v = feas ? static_cast<long long>(q) : -h;
-  p.k = k;
-  p.h = h;
-  return p;
-}
-__device__ __forceinline__ Pick shfl_pick(const Pick &x, int off) {
-  Pick y;
-  y.inf = __shfl_xor_sync(0xffffffffu, x.inf, off);
-  y.v = __shfl_xor_sync(0xffffffffu, x.v, off);
-  y.k = __shfl_xor_sync(0xffffffffu, x.k, off);
-  y.h = __shfl_xor_sync(0xffffffffu, x.h, off);
-  return y;
-}
-// Block-wide best; every thread gets the result.
-__device__ Pick block_best(Pick mine, Pick *s_w) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    const Pick y = shfl_pick(mine, off);
-    if (better(y, mine)) mine = y;
-  }
-  if (lane == 0) s_w[warp] = mine;
-  __syncthreads();
-  Pick b = s_w[0];
-  for (int w = 1; w < nw; ++w)
-    if (better(s_w[w], b)) b = s_w[w];
-  __syncthreads();
-  return b;
-}
-__device__ __forceinline__ Pick no_pick() {
-  Pick p;
-  p.inf = 2;
-  p.v = 0;
-  p.k = 0x7fffffff;
-  p.h = 0;
-  return p;
+
+// Shared memory of a row: F, the maxima of 4, of 16 and of 128 steps, each with
+// four words of padding (16-byte reads of eight rows then spread over the
+// banks).  A score reads up to 8 words from any place of a row's part, hence
+// the padding at the end of all of them.
+constexpr int kSeqPad = 16;
+__host__ __device__ constexpr int seq_ldc(int P2) { return (P2 + 3) / 4 * 4 + 4; }
+__host__ __device__ constexpr int64_t seq_row_words(int64_t P0, int P2) {
+  return P0 + P0 / 4 + P0 / 16 + 12 + seq_ldc(P2);
 }
 
-// ---------------------------------------------------------------------------
-// SEQUENTIAL horizon dispatch: one block walks the candidates in order.
-// Scoring decoder k needs M_k(u) = max_{t<u} (K[k][t] + t); it is read from
-// the 16-step summary kmax (built from K just before) for the whole blocks
-// below u plus at most 15 cells of K.  Reserving the footprint adds
-// p + t + 1 to K[k*][t] for t < u and rebuilds the summary entries of the
-// blocks it touched, so the summary always matches K.
-// ---------------------------------------------------------------------------
+// The packed 64-bit decision key, the smallest wins: inf << 63 | v << 10 | k.
+// mc (rank by headroom alone) puts every decoder in the infeasible class, by
+// 2^33 - h (positive: h <= cap < 2^31).
+__device__ __forceinline__ unsigned long long seq_key64(long long h, int32_t q, int k, int mc) {
+  const bool feas = h >= 0 && !mc;
+  const unsigned long long v = feas ? static_cast<unsigned long long>(q)
+                               : mc ? static_cast<unsigned long long>((1ll << 33) - h)
+                                    : static_cast<unsigned long long>(-h);
+  return (feas ? 0ull : 1ull << 63) | (v << 10) | static_cast<unsigned>(k);
+}
+
+__device__ __forceinline__ void seq_bar(int warps) {
+  asm volatile("bar.sync 1, %0;" ::"r"(32 * warps) : "memory");
+}
+
+__device__ __forceinline__ uint32_t max4(uint4 v) { return max(max(v.x, v.y), max(v.z, v.w)); }
+// the larger of m and the first n of v (n may be below 0 or above 4)
+__device__ __forceinline__ uint32_t max4_below(uint4 v, int n, uint32_t m) {
+  m = max(m, n > 0 ? v.x : 0u);
+  m = max(m, n > 1 ? v.y : 0u);
+  m = max(m, n > 2 ? v.z : 0u);
+  return max(m, n > 3 ? v.w : 0u);
+}
+
+// RD: decoders per lane of a pick, 0 for any number.
+template <int RD>
 __global__ void __launch_bounds__(1024, 1)
-dispatch_sequential_kernel(int D, int H, int32_t *K, uint32_t *kmax, const int32_t *cap,
-                           int32_t *Q, int64_t J, const int32_t *cp, const int32_t *cb,
-                           int32_t *choice, int64_t *headroom, int mc, int32_t *status) {
+dispatch_sequential_kernel(const __grid_constant__ SeqArgs a) {
+  constexpr unsigned kAll = 0xffffffffu;
+  extern __shared__ __align__(16) uint32_t seq_smem[];
+  __shared__ int32_t s_cap[kMaxD], s_q[kMaxD];
+  __shared__ int32_t s_off[kMaxD];      // M + off is the infeasible key term
+  __shared__ uint2 s_col[2][kSeqD];     // (key, M) of each decoder for a candidate, by its parity
+  __shared__ int32_t s_colq[2][kMaxD];  // the queue length behind that key
+  __shared__ int2 s_cand[64];           // (p, u) of candidate i at i mod 64; u = 0: none or invalid
+  __shared__ __align__(16) uint32_t s_part[2][kRowWarps];  // the chosen row's maxima, per row warp
+  __shared__ int4 s_crit[2];            // its (cap, Q, off)
+  __shared__ int s_q0, s_umax, s_wide;
+  __shared__ long long s_x0;
   pdl_prologue();
-  __shared__ uint32_t s_M[kMaxD];
-  __shared__ Pick s_w[32];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarp = blockDim.x >> 5;
+  const int D = a.D, H = a.H, P0 = a.P0, P2 = a.P2, mc = a.mc, kb = a.kb;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int nwarp = 32;
   const int64_t nb = (static_cast<int64_t>(H) + kSumBlock - 1) / kSumBlock;
-  bool bad = false;
-  for (int k = tid; k < D; k += blockDim.x)
-    if ((cap[k] | Q[k]) < 0) bad = true;
-  if (bad) flag_error(status, MAPS_E_RANGE);  // K < 0 is reported by the summary pass
+  const int64_t nch = (static_cast<int64_t>(H) + kSeqChunk - 1) / kSeqChunk;
+  // offsets into shared memory, in words
+  const int ldF = P0 + 4, ld4 = P0 / 4 + 4, ld16 = P0 / 16 + 4, ldc = seq_ldc(P2);
+  const int o4 = D * ldF, o16 = o4 + D * ld4, oc = o16 + D * ld16;
+  uint32_t *const F = seq_smem;
+  // --- capacities, the first candidates ---------------------------------------
+  if (tid == 0) {
+    s_q0 = 0x7fffffff;
+    s_x0 = LLONG_MAX;
+    s_umax = s_wide = 0;
+  }
+  for (int k = D + tid; k < kSeqD; k += blockDim.x) s_col[0][k] = s_col[1][k] = make_uint2(~0u, 0u);
   __syncthreads();
-  for (int64_t j = 0; j < J; ++j) {
-    const int32_t p = cp[j], U = cb[j];
-    if ((p | U) < 0) {
-      if (tid == 0) {
-        flag_error(status, MAPS_E_RANGE);
-        choice[j] = -1;
-        if (headroom) headroom[j] = 0;
-      }
-      continue;
+  bool bad = false;
+  for (int k = tid; k < D; k += blockDim.x) {
+    const int32_t ck = a.cap[k], qk = a.Q[k];
+    if ((ck | qk) < 0) bad = true;  // K < 0 is reported by the summary pass
+    s_cap[k] = ck;
+    s_q[k] = qk;
+    atomicMin(&s_q0, qk);
+    atomicMin(&s_x0, static_cast<long long>(a.K[static_cast<int64_t>(k) * H]) - ck);
+  }
+  auto load_cand = [&](int64_t j) {
+    const int32_t p = j < a.J ? __ldg(a.cp + j) : -1, U = j < a.J ? __ldg(a.cb + j) : -1;
+    return (p | U) < 0 ? make_int2(0, 0) : make_int2(p, candidate_steps(U, H));
+  };
+  int umax = 0;
+  for (int64_t j = tid; j < a.J; j += blockDim.x) {
+    const int2 c = load_cand(j);
+    umax = max(umax, c.y);
+    if (c.y == 0) {
+      bad = true;
+      a.choice[j] = -1;
+      if (a.headroom) a.headroom[j] = 0;
     }
-    const int u = candidate_steps(U, H);
-    const int nfull = u / kSumBlock, rem = u - nfull * kSumBlock;
-    for (int k = warp; k < D; k += nwarp) {
-      const uint32_t *km = kmax + static_cast<int64_t>(k) * nb;
-      const int32_t *row = K + static_cast<int64_t>(k) * H;
-      uint32_t m = 0;
-      for (int b = lane; b < nfull; b += 32) m = max(m, km[b]);
-      if (lane < rem) {
-        const int t = nfull * kSumBlock + lane;
-        m = max(m, static_cast<uint32_t>(row[t]) + static_cast<uint32_t>(t));
-      }
+  }
+  umax = __reduce_max_sync(kAll, umax);
+  if (lane == 0) atomicMax(&s_umax, umax);
+  if (tid < 64) s_cand[tid] = load_cand(tid);
+  // --- the resident rows --------------------------------------------------------
+  const int rch = P0 / kSeqChunk;  // resident chunks of a row
+  for (int e = warp; e < D * rch; e += nwarp) {
+    const int k = e / rch, t0 = (e - k * rch) * kSeqChunk;
+    const int32_t *row = a.K + static_cast<int64_t>(k) * H + t0;
+    uint32_t *const f = F + k * ldF + t0;
+    uint32_t x[4];
 #pragma unroll
-      for (int off = 16; off > 0; off >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, off));
-      if (lane == 0) s_M[k] = m;
+    for (int i = 0; i < 4; ++i) {
+      const int t = 32 * i + lane;
+      x[i] = t0 + t < H ? static_cast<uint32_t>(row[t]) + static_cast<uint32_t>(t0 + t) : 0u;
     }
-    __syncthreads();
-    Pick mine = no_pick();
-    for (int k = tid; k < D; k += blockDim.x) {
-      const long long h = static_cast<long long>(cap[k]) - (static_cast<long long>(p) + 1 + s_M[k]);
-      const Pick c = make_pick(h, Q[k], k, mc != 0);
-      if (better(c, mine)) mine = c;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) f[32 * i + lane] = x[i];
+    __syncwarp();
+    uint32_t m = max4(reinterpret_cast<const uint4 *>(f)[lane]);
+    F[o4 + k * ld4 + t0 / 4 + lane] = m;
+    m = max(m, __shfl_xor_sync(kAll, m, 1));
+    m = max(m, __shfl_xor_sync(kAll, m, 2));
+    if ((lane & 3) == 0) F[o16 + k * ld16 + t0 / 16 + (lane >> 2)] = m;
+  }
+  __syncthreads();
+  const int cmax = s_umax >> 7;  // scores read the chunk maxima below this one
+  for (int e = tid; e < cmax * D; e += blockDim.x) {
+    const int k = e / cmax, c = e - k * cmax;
+    uint32_t m = 0;
+    for (int i = 0; i < 8; ++i)
+      if ((c * 8 + i) * kSumBlock < H) m = max(m, __ldcg(a.km + k * nb + c * 8 + i));
+    if (c < P2)
+      F[oc + k * ldc + c] = m;
+    else
+      a.cm[k * nch + c] = m;
+  }
+  const long long x0 = s_x0;
+  for (int k = tid; k < D; k += blockDim.x) {
+    const long long off = -(x0 + s_cap[k]);
+    s_off[k] = static_cast<int32_t>(off);
+    // M < 2^31 + 2^28 while K is within int32: M + off cannot wrap
+    if (off > (1ll << 30) || off < INT_MIN) s_wide = 1;
+  }
+  __syncthreads();
+  const int32_t q0 = s_q0;
+  const uint32_t kmask = (1u << kb) - 1u;
+  // key terms stop at lim (no key is ~0); 0 where the terms need more bits
+  const uint32_t lim = s_wide ? 0u : (1u << (31 - kb)) - 2u;
+  const uint32_t lim_key = lim << kb;
+  auto key32 = [&](uint32_t M, int32_t p, int32_t cap, int32_t q, int32_t off, int k) {
+    const int32_t room = mc ? 0 : max(cap - p, 0);  // p + 1 + M <= cap: M < cap - p
+    const bool feas = M < static_cast<uint32_t>(room);
+    const uint32_t term = feas ? static_cast<uint32_t>(q - q0) : M + static_cast<uint32_t>(off);
+    return (feas ? 0u : 0x80000000u) + (min(term, lim) << kb) + static_cast<uint32_t>(k);
+  };
+  // a column's lane: which maxima of its decoder it reads, as the first n words
+  // from a place of the row's part: w = u >> sh, n = w & low, place w & ~low
+  const int part = lane & 3;
+  const int sh = part == 0 ? 7 : part == 1 ? 4 : part == 2 ? 2 : 0;
+  const int low = part == 0 ? -1 : part == 1 ? 7 : 3;
+  const int ldp = part == 0 ? ldc : part == 1 ? ld16 : part == 2 ? ld4 : ldF;
+  const int op = part == 0 ? oc : part == 1 ? o16 : part == 2 ? o4 : 0;
+  auto score_col = [&](int64_t j, int k) {  // four lanes, decoder k
+    const int2 cd = s_cand[j & 63];
+    const int u = cd.y, kc = min(k, D - 1);
+    const bool in = u < P0;  // its chunk is resident (P0 is whole chunks)
+    const int w = u >> sh;
+    const int n = part == 0 ? min(w, P2) : in ? w & low : 0;
+    const uint32_t *b = F + op + kc * ldp + (in ? w & ~low : 0);
+    const uint4 v0 = *reinterpret_cast<const uint4 *>(b), v1 = *reinterpret_cast<const uint4 *>(b + 4);
+    uint32_t m = max(max4_below(v0, n, 0u), max4_below(v1, n - 4, 0u));
+    if (n > 8)
+      for (int i = 8; i < n; i += 4) m = max4_below(*reinterpret_cast<const uint4 *>(b + i), n - i, m);
+    if (!in && (u & (kSeqChunk - 1)) != 0) {  // the last chunk in global memory
+      const int c = u >> 7, n16 = (u >> 4) & 7, t0 = u & ~15;
+      const uint32_t *bg = a.km + kc * nb + c * 8;
+      const int32_t *row = a.K + static_cast<int64_t>(kc) * H + t0;
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+        if (part + 4 * i < n16) m = max(m, bg[part + 4 * i]);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int t = part + 4 * i;
+        if (t < (u & 15)) m = max(m, static_cast<uint32_t>(row[t]) + static_cast<uint32_t>(t0 + t));
+      }
     }
-    const Pick b = block_best(mine, s_w);
-    if (tid == 0) {
-      choice[j] = b.k;
-      if (headroom) headroom[j] = b.h;
-      if (Q[b.k] == 0x7fffffff)
-        flag_error(status, MAPS_E_RANGE);
-      else
-        Q[b.k] += 1;
+    if ((u >> 7) > P2)
+      for (int c = P2 + part; c < (u >> 7); c += 4) m = max(m, a.cm[kc * nch + c]);
+    m = max(m, __shfl_xor_sync(kAll, m, 1));
+    m = max(m, __shfl_xor_sync(kAll, m, 2));
+    const int32_t q = s_q[kc];
+    const uint32_t key = key32(m, cd.x, s_cap[kc], q, s_off[kc], k);
+    if (part == 0 && k < D) {
+      s_col[j & 1][k] = make_uint2(key, m);
+      s_colq[j & 1][k] = q;
     }
-    // reserve the candidate's footprint at the chosen decoder; the blocks it
-    // touches are whole 16-lane groups of the loop, so a group's shuffle
-    // maximum is that block's new summary entry
-    int32_t *row = K + static_cast<int64_t>(b.k) * H;
-    uint32_t *km = kmax + static_cast<int64_t>(b.k) * nb;
-    const int end = min(((u + kSumBlock - 1) / kSumBlock) * kSumBlock, H);
-    bool over = false;
-    for (int t0 = 0; t0 < end; t0 += blockDim.x) {
-      const int t = t0 + tid;
-      uint32_t x = 0;
-      if (t < end) {
-        long long v = row[t];
-        if (t < u) {
-          v += static_cast<long long>(p) + t + 1;
-          if (v > 0x7fffffffLL) {
-            over = true;
-            v = 0x7fffffffLL;
-          }
-          row[t] = static_cast<int32_t>(v);
+  };
+  for (int k0 = warp * 8; k0 < D; k0 += nwarp * 8) score_col(0, k0 + (lane >> 2));
+  __syncthreads();
+
+  // The pick of candidate j (with p) at phase parity par: the decoder, and this
+  // lane's best key and its M; `best` is that key in the winner's lane alone.
+  // The entry of decoder kprev, chosen before, comes from the row warps.
+  auto pick = [&](int p, int par, int kprev, uint32_t &best, uint32_t &key, uint32_t &M) {
+    const uint4 pa = *reinterpret_cast<const uint4 *>(&s_part[par ^ 1][0]);
+    const uint4 pb = *reinterpret_cast<const uint4 *>(&s_part[par ^ 1][4]);
+    const int4 cr = s_crit[par ^ 1];
+    const uint32_t cM = max(max4(pa), max4(pb));
+    const uint32_t ckey = key32(cM, p, cr.x, cr.y, cr.z, kprev);
+    key = ~0u;
+    M = 0;
+    auto take = [&](int k) {
+      uint2 e = s_col[par][k];
+      if (k == kprev) e = make_uint2(ckey, cM);
+      M = e.x < key ? e.y : M;
+      key = min(key, e.x);
+    };
+    if (RD > 0) {
+#pragma unroll
+      for (int i = 0; i < (RD > 0 ? RD : 1); ++i) take(32 * i + lane);
+    } else {
+#pragma unroll 4
+      for (int k = lane; k < D; k += 32) take(k);
+    }
+    best = __reduce_min_sync(kAll, key);
+    if ((best & 0x7fffffffu) < lim_key) return static_cast<int>(best & kmask);
+    unsigned long long k64 = ~0ull;  // the wide keys
+    for (int k = lane; k < D; k += 32) {
+      const uint32_t Mk = k == kprev ? cM : s_col[par][k].y;
+      const int32_t qk = k == kprev ? cr.y : s_colq[par][k];
+      const unsigned long long y =
+          seq_key64(static_cast<long long>(s_cap[k]) - (static_cast<long long>(p) + 1 + Mk), qk, k, mc);
+      if (y < k64) {
+        k64 = y;
+        M = Mk;
+        key = static_cast<uint32_t>(k);  // this lane's best decoder
+      }
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      const unsigned long long y = __shfl_xor_sync(kAll, k64, off);
+      k64 = y < k64 ? y : k64;
+    }
+    best = static_cast<uint32_t>(k64 & 1023u);
+    return static_cast<int>(best);
+  };
+
+  const int walkers = kRowWarps + 1 + a.ncol;  // warps of the per-decision barrier
+  if (warp < kRowWarps) {
+    int kprev = -1;  // the decoder chosen before
+    int2 c1 = s_cand[0];
+    const bool res0 = warp < rch;           // this warp's first chunk is resident
+    const int tb = warp * kSeqChunk, tl = tb + 4 * lane;
+    for (int64_t j = 0; j < a.J; ++j) {
+      const int2 cd = c1;
+      c1 = s_cand[(j + 1) & 63];
+      const int p = cd.x, u = cd.y, u1 = c1.y, ue = max(u, u1);
+      const int par = static_cast<int>(j & 1);
+      int kk = -1;
+      if (u > 0) {
+        uint32_t best, key, M;
+        kk = pick(p, par, kprev, best, key, M);
+        uint32_t m1 = 0, bm0 = 0;
+        uint32_t *const fr = F + kk * ldF + 4 * lane;
+        auto add_to = [&](uint4 &v, int t) {  // the footprint on steps t.. t + 3 below u
+          const uint32_t x = static_cast<uint32_t>(p) + 1u + static_cast<uint32_t>(t);
+          const int n = u - t;
+          v.x += n > 0 ? x : 0u;
+          v.y += n > 1 ? x + 1u : 0u;
+          v.z += n > 2 ? x + 2u : 0u;
+          v.w += n > 3 ? x + 3u : 0u;
+        };
+        auto set_cm = [&](int c, uint32_t m) {
+          if (c < P2)
+            F[oc + kk * ldc + c] = m;
+          else
+            a.cm[kk * nch + c] = m;
+        };
+        auto fold = [&](int c, uint32_t bm) {  // the chunk's maxima, from its 4-step ones
+          F[o4 + kk * ld4 + c * 32 + lane] = bm;
+          bm = max(bm, __shfl_xor_sync(kAll, bm, 1));
+          bm = max(bm, __shfl_xor_sync(kAll, bm, 2));
+          if ((lane & 3) == 0) F[o16 + kk * ld16 + c * 8 + (lane >> 2)] = bm;
+          bm = __reduce_max_sync(kAll, bm);
+          if (lane == 0) set_cm(c, bm);
+        };
+        if (res0 && tb < ue) {
+          uint4 v = *reinterpret_cast<const uint4 *>(fr + tb);
+          add_to(v, tl);
+          m1 = max4_below(v, u1 - tl, 0u);
+          bm0 = max4(v);  // folded once the score is published
+          if (tb < u) *reinterpret_cast<uint4 *>(fr + tb) = v;
         }
-        x = static_cast<uint32_t>(v) + static_cast<uint32_t>(t);
-      }
+        // the later chunks of a long horizon
+        for (int c = res0 ? warp + kRowWarps : warp; c * kSeqChunk < ue; c += kRowWarps) {
+          const int t0 = c * kSeqChunk;
+          if (c < rch) {
+            uint4 v = *reinterpret_cast<const uint4 *>(fr + t0);
+            add_to(v, t0 + 4 * lane);
+            m1 = max4_below(v, u1 - (t0 + 4 * lane), m1);
+            if (t0 < u) {
+              *reinterpret_cast<uint4 *>(fr + t0) = v;
+              fold(c, max4(v));
+            }
+            continue;
+          }
+          int32_t *const row = a.K + static_cast<int64_t>(kk) * H;
+          uint32_t x[4], cx = 0;
 #pragma unroll
-      for (int off = 8; off > 0; off >>= 1) x = max(x, __shfl_xor_sync(0xffffffffu, x, off));
-      if ((lane & (kSumBlock - 1)) == 0 && t < end) km[t / kSumBlock] = x;
+          for (int i = 0; i < 4; ++i) {
+            const int t = t0 + 32 * i + lane;
+            x[i] = t < H ? static_cast<uint32_t>(row[t]) : 0u;
+          }
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int t = t0 + 32 * i + lane;
+            const uint32_t te = static_cast<uint32_t>(t);
+            if (t < u) {
+              x[i] += static_cast<uint32_t>(p) + 1u + te;
+              row[t] = static_cast<int32_t>(x[i]);
+            }
+            uint32_t f = t < H ? x[i] + te : 0u;
+            if (t < u1) m1 = max(m1, f);
+            if (t0 < u) {
+              cx = max(cx, f);
+#pragma unroll
+              for (int off = 8; off > 0; off >>= 1) f = max(f, __shfl_xor_sync(kAll, f, off));
+              const int b = (t0 >> 4) + 2 * i + (lane >> 4);
+              if ((lane & 15) == 0 && b * kSumBlock < H) a.km[kk * nb + b] = f;
+            }
+          }
+          if (t0 < u) {
+            cx = __reduce_max_sync(kAll, cx);
+            if (lane == 0) set_cm(c, cx);
+          }
+        }
+        m1 = __reduce_max_sync(kAll, m1);
+        if (lane == 0) s_part[par][warp] = m1;
+        if (res0 && tb < u) fold(warp, bm0);
+      }
+      kprev = kk;
+      seq_bar(walkers);
     }
-    if (over) flag_error(status, MAPS_E_RANGE);
-    __syncthreads();
+  } else if (warp == kRowWarps) {
+    int kprev = -1;
+    for (int64_t j = 0; j < a.J; ++j) {
+      const int2 cd = s_cand[j & 63];
+      const int p = cd.x, par = static_cast<int>(j & 1);
+      int kk = -1;
+      if (cd.y > 0) {
+        uint32_t best, key, M;
+        kk = pick(p, par, kprev, best, key, M);
+        if (key == best) {  // the chosen decoder's lane books the decision
+          const int32_t cap = s_cap[kk], q = s_q[kk];
+          const int32_t qn = q == 0x7fffffff ? q : q + 1;
+          s_q[kk] = qn;
+          s_crit[par] = make_int4(cap, qn, s_off[kk], 0);
+          a.choice[j] = kk;
+          if (a.headroom)
+            a.headroom[j] = static_cast<long long>(cap) - (static_cast<long long>(p) + 1 + M);
+          // the largest new cell, K + p + t + 1, is M + p + 1
+          if (q == 0x7fffffff || static_cast<long long>(p) + 1 + M > 0x7fffffffLL) bad = true;
+        }
+      }
+      kprev = kk;
+      seq_bar(walkers);
+    }
+  } else if (warp < walkers) {
+    const int cw = warp - kRowWarps - 1;
+    int2 cn = make_int2(0, 0);  // column warp 0: the 32 candidates of the next ring refill
+    if (cw == 0) cn = load_cand(64 + lane);
+    for (int64_t j = 0; j < a.J; ++j) {
+      if (cw == 0 && (j & 31) == 0 && j > 0) {
+        s_cand[(j + 32 + lane) & 63] = cn;
+        cn = load_cand(j + 64 + lane);
+      }
+      for (int k0 = cw * 8; k0 < D; k0 += 8 * a.ncol) score_col(j + 1, k0 + (lane >> 2));
+      seq_bar(walkers);
+    }
+  }
+  __syncthreads();
+  if (bad) flag_error(a.status, MAPS_E_RANGE);
+  for (int k = tid; k < D; k += blockDim.x) a.Q[k] = s_q[k];
+  for (int k = warp; k < D; k += nwarp) {
+    int32_t *row = a.K + static_cast<int64_t>(k) * H;
+#pragma unroll 8
+    for (int t = lane; t < P0 && t < H; t += 32)
+      row[t] = static_cast<int32_t>(F[k * ldF + t] - static_cast<uint32_t>(t));
   }
 }
 
@@ -1511,19 +1798,64 @@ int launch_snapshot(int D, int H, const int32_t *K, const uint32_t *kmax, const 
 }  // namespace maps
 
 namespace maps {
+namespace {
+struct SeqWs {
+  uint32_t *km;  // [D][ceil(H/16)]
+  uint32_t *cm;  // [D][ceil(H/128)]
+};
+SeqWs carve_seq(Carve &c, int D, int H) {
+  SeqWs w;
+  w.km = c.take<uint32_t>(static_cast<size_t>(D) * ((static_cast<size_t>(H) + kSumBlock - 1) / kSumBlock));
+  w.cm = c.take<uint32_t>(static_cast<size_t>(D) * ((static_cast<size_t>(H) + kSeqChunk - 1) / kSeqChunk));
+  return w;
+}
+}  // namespace
+
 int dispatch_sequential(int D, int H, int32_t *K, const int32_t *cap, int32_t *Q, int64_t J,
                         const int32_t *cp, const int32_t *cb, int32_t *choice, int64_t *headroom,
                         bool mc, void *ws, cudaStream_t s) {
   // a private summary of K (also validating K >= 0); updated in place
   int32_t *status = status_word(ws);
   Carve cv(ws);
+  const SeqWs w = carve_seq(cv, D, H);
   const int64_t nb = (static_cast<int64_t>(H) + kSumBlock - 1) / kSumBlock;
-  uint32_t *km = cv.take<uint32_t>(static_cast<size_t>(D) * nb);
   const int gk = static_cast<int>(std::min<int64_t>((nb * D + 255) / 256, 8LL * sm_count()));
-  launch_pdl(kmax_from_K_kernel, gk, 256, 0, s, D, H, K, km, status);
-  launch_pdl(dispatch_sequential_kernel, 1, 1024, 0, s, D, H, K, km, cap, Q, J, cp, cb, choice,
-             headroom, mc ? 1 : 0, status);
-  return launch_ok();
+  launch_pdl(kmax_from_K_kernel, gk, 256, 0, s, D, H, K, w.km, status);
+  SeqArgs a;
+  a.D = D;
+  a.H = H;
+  a.mc = mc ? 1 : 0;
+  a.K = K;
+  a.km = w.km;
+  a.cm = w.cm;
+  a.cap = cap;
+  a.Q = Q;
+  a.J = J;
+  a.cp = cp;
+  a.cb = cb;
+  a.choice = choice;
+  a.headroom = headroom;
+  a.status = status;
+  a.kb = 0;
+  while ((1 << a.kb) < D) ++a.kb;
+  a.ncol = std::min((D + 7) / 8, kColWarps);
+  // shared memory per row: a sixteenth for chunk maxima, the rest resident
+  // steps (1 + 1/4 + 1/16 words each); 44 KB are left to the static arrays
+  const int64_t words = ((max_smem_optin() - 45056) / 4 - kSeqPad) / D;
+  const int64_t chunks = (static_cast<int64_t>(H) + kSeqChunk - 1) / kSeqChunk;
+  a.P2 = static_cast<int>(std::min<int64_t>(chunks, words / 16));
+  a.P0 = 0;
+  while (a.P0 < chunks * kSeqChunk && seq_row_words(a.P0 + kSeqChunk, a.P2) <= words) a.P0 += kSeqChunk;
+  const size_t smem = 4 * (static_cast<size_t>(D) * seq_row_words(a.P0, a.P2) + kSeqPad);
+  auto launch = [&](void (*kern)(SeqArgs)) {
+    MAPS_TRY(cuda_ok(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          static_cast<int>(smem))));
+    launch_pdl(kern, 1, 1024, smem, s, a);
+    return launch_ok();
+  };
+  return D <= 32   ? launch(dispatch_sequential_kernel<1>)
+         : D <= 64 ? launch(dispatch_sequential_kernel<2>)
+                   : launch(dispatch_sequential_kernel<0>);
 }
 }  // namespace maps
 
@@ -1542,7 +1874,7 @@ size_t maps_dispatch_workspace_size(int32_t mode, int32_t D, int32_t H, int64_t 
     const SnapGeom g = snap_geom(D, H);
     carve_snap(c, D, H, g.T2, J);
   } else if (mode == MAPS_MODE_SEQUENTIAL && D >= 1 && H >= 1 && H <= kMaxH) {
-    c.take<uint32_t>(static_cast<size_t>(D) * ((static_cast<size_t>(H) + kSumBlock - 1) / kSumBlock));
+    carve_seq(c, D, H);
   } else if ((mode == MAPS_MODE_ALG1_SNAPSHOT || mode == MAPS_MODE_ALG1_SEQUENTIAL) && D >= 1) {
     c.take<long long>(static_cast<size_t>(D));
   }

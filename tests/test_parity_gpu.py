@@ -471,6 +471,42 @@ def test_dispatch_sequential_workloads(M, ws, oracle, name):
     check_dispatch(M, ws, oracle, 1, w["D"], w["H"], K, w["cap"], w["Q"], w["cand_prompt"], cb)
 
 
+@pytest.mark.parametrize("D,H,J,spread", [
+    # four, two and one warps a decoder, and several decoders a warp, at the
+    # edges; horizons around a 128-cell chunk and a 16-step block; rows past
+    # what shared memory holds; a last chunk of candidates that is not full
+    (1, 127, 33, 3000), (8, 129, 65, 3000), (9, 1000, 64, 3000), (16, 16384, 200, 6000),
+    (17, 2049, 100, 3000), (32, 4111, 150, 3000), (33, 4096, 100, 3000), (64, 9001, 130, 6000),
+    (100, 5000, 60, 3000), (300, 700, 50, 3000), (1, 300000, 40, 100000),
+    # headrooms further apart than the 32-bit keys hold
+    (5, 600, 60, 2**30), (40, 600, 60, 2**30)])
+def test_dispatch_sequential_edges(M, ws, oracle, D, H, J, spread):
+    rng = np.random.default_rng(D * 131 + H)
+    off, p, g, U = random_residents(rng, D, H, 20)
+    _, K = oracle.occupancy(D, H, off, p, g, U)
+    cap = diverse_caps(rng, K, spread)
+    Q = rng.integers(0, 3, D).astype(np.int32)
+    cp = rng.integers(0, 500, J).astype(np.int32)
+    cb = np.where(rng.random(J) < 0.5, rng.integers(0, H + 5, J), rng.integers(0, 40, J)).astype(np.int32)
+    cb[: min(J, 4)] = [0, 16, 128, H][: min(J, 4)]
+    check_dispatch(M, ws, oracle, 1, D, H, K, cap, Q, cp, cb)
+    cp[J // 2] = -1  # skipped and reported
+    check_dispatch(M, ws, oracle, 1, D, H, K, cap, Q, cp, cb)
+
+
+def test_dispatch_sequential_ranges(M, ws, oracle):
+    """Queue lengths far apart (past the 32-bit keys), one that passes int32,
+    and a reservation that takes K past int32."""
+    K = np.zeros((40, 50), np.int32)
+    cap = np.full(40, 10**6, np.int32)
+    cp, cb = np.full(30, 7, np.int32), np.full(30, 20, np.int32)
+    Q = (np.arange(40)[::-1] * 50_000_000).astype(np.int32)
+    check_dispatch(M, ws, oracle, 1, 40, 50, K, cap, Q, cp, cb)
+    check_dispatch(M, ws, oracle, 1, 40, 50, K, cap, np.full(40, I32_MAX, np.int32), cp, cb)
+    check_dispatch(M, ws, oracle, 1, 3, 50, np.full((3, 50), I32_MAX - 60, np.int32), cap[:3],
+                   Q[:3], cp, cb)
+
+
 @pytest.mark.parametrize("S", [1, 16])
 @pytest.mark.parametrize("name", ["tiny", "d16", "d64", "large"])
 def test_dispatch_alg1_workloads(M, ws, oracle, name, S):
