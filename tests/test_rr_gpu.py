@@ -74,6 +74,23 @@ def test_rr_random(M, oracle, N, C, n, theta, tie):
     check(M, oracle, N, C, 1000, theta, arr, prompt, out)
 
 
+@pytest.mark.parametrize("most", [31, 32, 33, 63, 64, 65, 255, 256, 257, 400])
+def test_rr_running_set_sizes(M, oracle, most):
+    """At most `most` requests run at once on a decoder (equal footprints):
+    the edges of a lane's register slots and of each variant's, and past them
+    the loop whose running set is in shared memory."""
+    rng = np.random.default_rng(most)
+    n = 3 * most + 50
+    out = rng.integers(1, 90, (2, n))
+    prompt = 100 - out
+    arr = np.cumsum(rng.integers(0, 40, (2, n)), axis=1)
+    check(M, oracle, 1, 100 * most, 1000, 850000, arr, prompt, out)
+    # the running set grows past what its average footprint suggests
+    prompt[:, : n // 2] = 0
+    out[:, : n // 2] = rng.integers(1, 9, (2, n // 2))
+    check(M, oracle, 1, 100 * most, 1000, 850000, arr, prompt, out)
+
+
 def test_rr_errors(M, oracle):
     # a footprint above C could never be admitted
     st, *_ = gpu_rr(M, 2, 100, 1000, 850000, [[0, 1, 2]], [[10, 95, 10]], [[5, 10, 5]])
