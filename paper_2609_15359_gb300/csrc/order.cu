@@ -16,12 +16,14 @@
 // Otherwise the kernels are a prep pass (validation, largest bound, entries
 // per decoder, arrival order check; its last block chooses the form), a key
 // pass, the segment sort, and a cooperative finishing kernel.
-// Segmented form (arrival non-decreasing along the index): the key pass
-// scatters each entry's index to its decoder's segment; one block sorts a
-// segment of at most kSegMax entries in shared memory on (not promoted,
-// primary, index), a unique key, and a longer segment is sorted as chunks of
-// kSegMax whose runs the finishing kernel ranks pairwise (up to kPairRuns
-// chunks) or merges pairwise level by level.
+// Segmented form (arrival non-decreasing along the index, or up to 1,024
+// decoders and (not promoted, primary, arrival, index) within 63 bits): the
+// entries are bucketed or scattered by decoder; one block sorts a segment of
+// at most kSegMax entries in shared memory on (not promoted, primary, index),
+// or with the arrival before the index where it is out of index order: a
+// unique key.  A longer segment is sorted as chunks of kSegMax whose runs the
+// finishing kernel ranks pairwise (up to kPairRuns chunks) or merges pairwise
+// level by level.
 // Otherwise the finishing kernel plans and runs one global sweep per digit:
 // tiles of 4096 keys are ranked stably in shared memory, each tile learns its
 // offsets from earlier tiles by decoupled look-back (one thread per digit
@@ -64,6 +66,7 @@ struct OrderCounts {
   uint32_t h[kPasses][kRadix];
   uint32_t unsorted;   // arrival decreases somewhere along the index
   uint32_t max_bound;  // largest bound of a non-promoted entry
+  uint32_t max_arrival;  // largest arrival (bucketed form)
   uint32_t segmented;  // decoder segments are sorted in shared memory
   uint32_t nitems;     // segments and chunks to sort
   uint32_t nmtiles;    // merge tiles of the long queues
@@ -112,6 +115,13 @@ constexpr int kSegMax = kSegThreads * kSegIPT;  // entries one block sorts
 // (kMergeTile divides kSegMax, so no tile straddles two runs).
 constexpr int kMergeTile = 512;
 constexpr int kMergeThreads = 512;  // the finishing kernel's block
+// With arrival out of index order, the most merge tiles times levels of the
+// segmented form.  Measured, whole call, segmented against global form: 200,003
+// entries on 64 decoders (no merges) 44 against 149 us; 1,000,000 on 200 (none)
+// 184 against 248; 1,000,000 on 32 (about 2,200 tile levels) 171 against 239;
+// 300,000 on one (4,100) 142 against 152; 1,000,000 on 4 (11,700) 240 against
+// 228; 1,000,000 on one (15,600) 318 against 227.
+constexpr uint32_t kMergesUnsorted = 4200;
 static_assert(kSegMax % kMergeTile == 0, "merge tiles align with runs");
 
 // A long queue of at most kPairRuns chunks is ranked pairwise instead: for
@@ -184,7 +194,7 @@ __device__ __forceinline__ int bit_width(uint32_t x) { return x ? 32 - __clz(x) 
 // marked by a negative count, whose sort writes keys for the merges) and the
 // merge tiles of the long queues; the form applies when arrival is already
 // in index order.
-__device__ void seg_plan_block(int D, OrderCounts *counts, const uint32_t *dec_count,
+__device__ void seg_plan_block(int64_t N, bool bucketed, int D, OrderCounts *counts, const uint32_t *dec_count,
                                int64_t *seg_off, int64_t *item_off, int32_t *item_n,
                                int32_t *item_dec, int64_t *mt_off, int32_t *mt_n, int32_t *mt_t,
                                PairQueues pq) {
@@ -273,7 +283,14 @@ __device__ void seg_plan_block(int D, OrderCounts *counts, const uint32_t *dec_c
     }
     __syncthreads();
   }
-  const bool segmented = __ldcg(&counts->unsorted) == 0;
+  // arrival out of index order: the bucketed form's keys then hold the arrival
+  // too, when (not promoted, primary, arrival, index) fits 63 bits
+  const int key_bits = 1 + bit_width(__ldcg(&counts->max_bound)) + bit_width(__ldcg(&counts->max_arrival)) +
+                       index_bits(N);
+  // and little is left to merge levels (in tiles times levels)
+  const bool segmented = __ldcg(&counts->unsorted) == 0 ||
+                         (bucketed && key_bits <= 63 &&
+                          __ldcg(&counts->nmtiles) * __ldcg(&counts->max_levels) <= kMergesUnsorted);
   const bool stable = segmented && D <= kStableD;
   if (t == 0) {
     counts->segmented = segmented ? 1u : 0u;
@@ -366,7 +383,8 @@ order_prep_kernel(int64_t N, int D, int64_t chunk, const int32_t *__restrict__ d
   __syncthreads();
   if (s_last) {
     __threadfence();
-    seg_plan_block(D, counts, dec_count, seg_off, item_off, item_n, item_dec, mt_off, mt_n, mt_t, pq);
+    seg_plan_block(N, false, D, counts, dec_count, seg_off, item_off, item_n, item_dec, mt_off, mt_n, mt_t,
+                   pq);
   }
 }
 
@@ -398,6 +416,7 @@ order_bucket_kernel(int64_t N, int D, int64_t chunk, int Dp, const int32_t *__re
   uint32_t *run = bsm + kPassWarps * Dp;  // [Dp] counts, then the next slot of each bucket
   __shared__ uint32_t s_w[kPassWarps];
   __shared__ bool s_last;
+  __shared__ uint32_t s_umax, s_amax;  // largest non-promoted bound, largest arrival
   constexpr int kU = kBucketU;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t r_begin = static_cast<int64_t>(blockIdx.x) * chunk;
@@ -410,7 +429,6 @@ order_bucket_kernel(int64_t N, int D, int64_t chunk, int Dp, const int32_t *__re
   int32_t d[kU];
   uint32_t kp[kU];  // not promoted << 31 | primary (the index follows from the position)
   bool bad = false, unsorted = false;
-  uint32_t umax = 0;
   auto load = [&](int64_t i0, bool all) {
     int32_t u[kU], w[kU], ar[kU], an[kU], dr[kU];
 #pragma unroll
@@ -429,6 +447,7 @@ order_bucket_kernel(int64_t N, int D, int64_t chunk, int Dp, const int32_t *__re
       }
     }
     if (!all) return;
+    uint32_t umax = 0, amax = 0;
 #pragma unroll
     for (int q = 0; q < kU; ++q) {
       const int64_t i = i0 + warp * (32 * kU) + q * 32 + lane;
@@ -436,28 +455,83 @@ order_bucket_kernel(int64_t N, int D, int64_t chunk, int Dp, const int32_t *__re
         if (dr[q] < 0 || dr[q] >= D || u[q] < 0 || ar[q] < 0) bad = true;
         if (w[q] <= max_wait && u[q] > 0) umax = max(umax, static_cast<uint32_t>(u[q]));
         if (an[q] < ar[q]) unsorted = true;
+        if (ar[q] > 0) amax = max(amax, static_cast<uint32_t>(ar[q]));
       }
       const uint32_t np = w[q] > max_wait ? 0u : 1u;
       kp[q] = np ? (1u << 31) | static_cast<uint32_t>(u[q] < 0 ? 0 : u[q]) : 0u;
     }
+    umax = __reduce_max_sync(0xffffffffu, umax);
+    amax = __reduce_max_sync(0xffffffffu, amax);
+    if (lane == 0) {
+      atomicMax(&s_umax, umax);
+      atomicMax(&s_amax, amax);
+    }
   };
-  for (int k = tid; k < Dp; k += blockDim.x) run[k] = 0;
-  __syncthreads();
-  // 1. counts
-  for (int64_t i0 = r_begin; i0 < r_end; i0 += kBucketRound) {
-    load(i0, one);
+  if (tid == 0) s_umax = s_amax = 0;
+  // base << 16 | leader lane << 8 | rank in the group, the base in the leader's
+  // lane alone: this warp's matches and per-warp counts, in item order, so ranks
+  // follow the index; the base is the entries of the decoder before the group
+  uint32_t rk[kU];
+  auto rank_round = [&] {
 #pragma unroll
     for (int q = 0; q < kU; ++q) {
       const unsigned pe = __match_any_sync(0xffffffffu, d[q]);
-      if (d[q] >= 0 && lane == __ffs(pe) - 1) atomicAdd(&run[d[q]], static_cast<uint32_t>(__popc(pe)));
+      const int leader = __ffs(pe) - 1;
+      rk[q] = (static_cast<uint32_t>(leader) << 8) | static_cast<uint32_t>(__popc(pe & lanemask_lt()));
+      if (lane == leader) rk[q] |= static_cast<uint32_t>(__popc(pe)) << 16;
     }
+#pragma unroll
+    for (int q = 0; q < kU; ++q)
+      if (d[q] >= 0 && (rk[q] >> 16) != 0)
+        rk[q] = (atomicAdd(&hw[warp * Dp + d[q]], rk[q] >> 16) << 16) | (rk[q] & 0xffffu);
+  };
+  auto base_of = [&](int q) {  // the group's base, from its leader
+    return __shfl_sync(0xffffffffu, rk[q], static_cast<int>((rk[q] >> 8) & 31u)) >> 16;
+  };
+  // 1. counts.  A range of one round ranks its entries once, and the counts are
+  // the sums over the warps (hw then holds each warp's start in the bucket);
+  // two matches and two shared atomics an entry: 30 against 21 us cold at
+  // 1,000,000 entries.
+  uint32_t v0 = 0, v1 = 0;
+  const int k0 = 2 * tid;
+  if (one) {
+    load(r_begin, true);
+    for (int k = tid; k < kPassWarps * Dp; k += blockDim.x) hw[k] = 0;
+    __syncthreads();
+    rank_round();
+    __syncthreads();
+    if (k0 < Dp) {  // Dp is a multiple of four
+#pragma unroll
+      for (int h = 0; h < kPassWarps; h += 4) {
+        uint2 c[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) c[i] = *reinterpret_cast<const uint2 *>(&hw[(h + i) * Dp + k0]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          *reinterpret_cast<uint2 *>(&hw[(h + i) * Dp + k0]) = make_uint2(v0, v1);
+          v0 += c[i].x;
+          v1 += c[i].y;
+        }
+      }
+    }
+  } else {
+    for (int k = tid; k < Dp; k += blockDim.x) run[k] = 0;
+    __syncthreads();
+    for (int64_t i0 = r_begin; i0 < r_end; i0 += kBucketRound) {
+      load(i0, false);
+#pragma unroll
+      for (int q = 0; q < kU; ++q) {
+        const unsigned pe = __match_any_sync(0xffffffffu, d[q]);
+        if (d[q] >= 0 && lane == __ffs(pe) - 1) atomicAdd(&run[d[q]], static_cast<uint32_t>(__popc(pe)));
+      }
+    }
+    __syncthreads();
+    v0 = k0 < Dp ? run[k0] : 0u;
+    v1 = k0 + 1 < Dp ? run[k0 + 1] : 0u;
   }
-  __syncthreads();
   {
     // block exclusive scan of the counts over the decoders (two per thread;
     // Dp <= 2 * blockDim.x), published with the counts
-    const int k0 = 2 * tid;
-    const uint32_t v0 = k0 < Dp ? run[k0] : 0u, v1 = k0 + 1 < Dp ? run[k0 + 1] : 0u;
     uint32_t incl = v0 + v1;
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
@@ -487,21 +561,21 @@ order_bucket_kernel(int64_t N, int D, int64_t chunk, int Dp, const int32_t *__re
   __syncthreads();
   // 2. and 3., round by round in index order
   unsigned long long *out = raw + r_begin;
-  for (int64_t i0 = r_begin; i0 < r_end; i0 += kBucketRound) {
-    for (int k = tid; k < kPassWarps * Dp; k += blockDim.x) hw[k] = 0;
-    if (!one) load(i0, true);
-    __syncthreads();  // counts zeroed
-    uint32_t rk[kU], base[kU];  // leader lane << 8 | rank in the group; group size, then base
+  if (one) {
 #pragma unroll
     for (int q = 0; q < kU; ++q) {
-      const unsigned pe = __match_any_sync(0xffffffffu, d[q]);
-      const int leader = __ffs(pe) - 1;
-      rk[q] = (static_cast<uint32_t>(leader) << 8) | static_cast<uint32_t>(__popc(pe & lanemask_lt()));
-      base[q] = lane == leader ? static_cast<uint32_t>(__popc(pe)) : 0u;
+      const uint32_t b = base_of(q);
+      const int64_t i = r_begin + warp * (32 * kU) + q * 32 + lane;
+      if (d[q] >= 0)
+        out[run[d[q]] + hw[warp * Dp + d[q]] + b + (rk[q] & 255u)] =
+            (static_cast<unsigned long long>(kp[q]) << 32) | static_cast<unsigned long long>(i & 0xffffffff);
     }
-#pragma unroll
-    for (int q = 0; q < kU; ++q)  // in item order, so ranks follow the index
-      if (d[q] >= 0 && base[q] != 0) base[q] = atomicAdd(&hw[warp * Dp + d[q]], base[q]);
+  }
+  for (int64_t i0 = one ? r_end : r_begin; i0 < r_end; i0 += kBucketRound) {
+    for (int k = tid; k < kPassWarps * Dp; k += blockDim.x) hw[k] = 0;
+    load(i0, true);
+    __syncthreads();  // counts zeroed
+    rank_round();
     __syncthreads();
     for (int k = tid; k < D; k += blockDim.x) {  // exclusive over the warps
       uint32_t r = run[k];
@@ -515,7 +589,7 @@ order_bucket_kernel(int64_t N, int D, int64_t chunk, int Dp, const int32_t *__re
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < kU; ++q) {
-      const uint32_t b = __shfl_sync(0xffffffffu, base[q], static_cast<int>(rk[q] >> 8));
+      const uint32_t b = base_of(q);
       const int64_t i = i0 + warp * (32 * kU) + q * 32 + lane;
       if (d[q] >= 0)
         out[hw[warp * Dp + d[q]] + b + (rk[q] & 255u)] =
@@ -524,10 +598,11 @@ order_bucket_kernel(int64_t N, int D, int64_t chunk, int Dp, const int32_t *__re
     __syncthreads();  // the counts are zeroed again for the next round
   }
   if (bad) flag_error(status, MAPS_E_RANGE);
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) umax = max(umax, __shfl_xor_sync(0xffffffffu, umax, off));
-  if (lane == 0 && umax) atomicMax(&counts->max_bound, umax);
   if (__syncthreads_or(unsorted) && tid == 0) atomicOr(&counts->unsorted, 1u);
+  if (tid == 0) {
+    atomicMax(&counts->max_bound, s_umax);
+    atomicMax(&counts->max_arrival, s_amax);
+  }
   // the last block to finish plans the segmented form (one thread publishes
   // the block's results: the barrier orders every thread's atomics before
   // its fence, as a grid barrier does)
@@ -539,7 +614,8 @@ order_bucket_kernel(int64_t N, int D, int64_t chunk, int Dp, const int32_t *__re
   __syncthreads();
   if (s_last) {
     __threadfence();
-    seg_plan_block(D, counts, dec_count, seg_off, item_off, item_n, item_dec, mt_off, mt_n, mt_t, pq);
+    seg_plan_block(N, true, D, counts, dec_count, seg_off, item_off, item_n, item_dec, mt_off, mt_n, mt_t,
+                   pq);
   }
 }
 
@@ -1209,7 +1285,10 @@ order_segsort_kernel(int64_t N, OrderCounts *counts, const int64_t *item_off,
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int ub = counts->max_bound ? 32 - __clz(counts->max_bound) : 0;
   const int ib = index_bits(N);
-  const int nbits = 1 + ub + ib;  // <= 1 + 31 + 31
+  // arrival out of index order: the key holds it between primary and index
+  const bool by_arrival = counts->unsorted != 0;
+  const int ab = by_arrival ? bit_width(counts->max_arrival) : 0;
+  const int nbits = 1 + ub + ab + ib;  // <= 63
   const int lo_bit = counts->stable ? ib : 0;  // first digit that needs sorting
   const int nitems = static_cast<int>(counts->nitems);
   for (int item = blockIdx.x; item < nitems; item += gridDim.x) {
@@ -1251,9 +1330,11 @@ order_segsort_kernel(int64_t N, OrderCounts *counts, const int64_t *item_off,
         s_src[r] = static_cast<long long>(tid) * bv.chunk + st0;
       }
       __syncthreads();
+      unsigned long long raw[kSegIPT];
 #pragma unroll
       for (int it = 0; it < kSegIPT; ++it) {
         const int x = it * kSegThreads + tid;
+        raw[it] = 0;
         if (x < n) {
           const uint32_t pos = o0 + static_cast<uint32_t>(x);
           int lo = 0, hi = static_cast<int>(nruns) - 1;  // the last run with P <= pos
@@ -1264,10 +1345,22 @@ order_segsort_kernel(int64_t N, OrderCounts *counts, const int64_t *item_off,
             else
               hi = mid - 1;
           }
-          const unsigned long long r = seg_keys[s_src[lo] + (pos - s_P[lo])];
-          // r = not promoted << 63 | primary << 32 | index
-          const unsigned long long key = ((r >> 63) << (ub + ib)) | (((r >> 32) & 0x7fffffffull) << ib) |
-                                         (r & 0xffffffffull);
+          // not promoted << 63 | primary << 32 | index
+          raw[it] = seg_keys[s_src[lo] + (pos - s_P[lo])];
+        }
+      }
+      int32_t arr[kSegIPT];
+#pragma unroll
+      for (int it = 0; it < kSegIPT; ++it)
+        arr[it] = by_arrival && it * kSegThreads + tid < n ? __ldg(bv.arrival + (raw[it] & 0xffffffffull)) : 0;
+#pragma unroll
+      for (int it = 0; it < kSegIPT; ++it) {
+        const int x = it * kSegThreads + tid;
+        if (x < n) {
+          const unsigned long long r = raw[it];
+          const unsigned long long key =
+              ((r >> 63) << (ub + ab + ib)) | (((r >> 32) & 0x7fffffffull) << (ab + ib)) |
+              (static_cast<unsigned long long>(arr[it] < 0 ? 0 : arr[it]) << ib) | (r & 0xffffffffull);
           sm.key[0][x] = key;
           orv |= key;
           andv &= key;
@@ -1415,52 +1508,86 @@ __device__ void merge_level(int level, int ntiles, const int64_t *mt_off, const 
 
 // The pairwise-ranked long queues: pair counts, a grid barrier, then every
 // key to its place.  Runs are the segment sort's sorted chunks in keys.
+// There may be hundreds of such queues (ragged queues just past kSegMax), so
+// their records are read into shared memory once, a pair finds its queue with
+// one look by every thread, and a queue's keys are placed by blocks that start
+// at its own place in the order (walking the records from global memory, all
+// queues placed from block 0 on, made up most of the kernel's time there).  A
+// thread's keys are searched side by side.  1,000,000 entries on 200 decoders
+// (400 pairs), whole call: 294 -> 113 us.
+constexpr int kPairQueues = 1024 / 2 + 1;
 __device__ void pair_rank_all(int64_t N, const OrderCounts *counts, const PairQueues &pq,
                               const unsigned long long *keys, int32_t *perm,
                               unsigned long long *sB, GridBar *bar, int32_t *status) {
+  __shared__ int64_t s_off[kPairQueues];
+  __shared__ int32_t s_n[kPairQueues], s_pair0[kPairQueues];
+  __shared__ uint16_t s_first[kPairQueues];  // the block that places the queue's first keys
+  __shared__ int s_q;
   const int nq = static_cast<int>(counts->npairq);
   const int64_t npairs = min(static_cast<int64_t>(counts->npairs), pq.budget);
+  for (int i = threadIdx.x; i < nq; i += blockDim.x) {
+    s_off[i] = pq.off[i];
+    s_n[i] = pq.n[i];
+    s_pair0[i] = pq.pair0[i];
+    s_first[i] = static_cast<uint16_t>(s_off[i] / blockDim.x % gridDim.x);
+  }
   // (1) pair p = (queue q, runs A != B): for each key of A, the keys of B below it
   for (int64_t p = blockIdx.x; p < npairs; p += gridDim.x) {
-    int q = -1;
-    for (int i = 0; i < nq; ++i) {  // the queue holding pair p (few queues)
-      const int C = static_cast<int>((pq.n[i] + kSegMax - 1) / kSegMax);
-      if (p >= pq.pair0[i] && p < pq.pair0[i] + static_cast<int64_t>(C) * (C - 1)) q = i;
-    }
-    if (q < 0) continue;  // a reservation no queue kept (uniform per block)
-    const int64_t off = pq.off[q];
-    const int n = pq.n[q], C = (n + kSegMax - 1) / kSegMax;
-    const int l = static_cast<int>(p - pq.pair0[q]);
-    const int A = l / (C - 1), b = l % (C - 1), B = b < A ? b : b + 1;
-    const int nA = min(kSegMax, n - A * kSegMax), nB = min(kSegMax, n - B * kSegMax);
-    const unsigned long long *rA = keys + off + static_cast<int64_t>(A) * kSegMax;
-    const unsigned long long *rB = keys + off + static_cast<int64_t>(B) * kSegMax;
-    for (int x = threadIdx.x; x < nB; x += blockDim.x) sB[x] = rB[x];
+    if (threadIdx.x == 0) s_q = -1;
     __syncthreads();
-    uint16_t *out = pq.cnt + p * kSegMax;
-    for (int x = threadIdx.x; x < nA; x += blockDim.x) {
-      const unsigned long long key = rA[x];
-      int lo = 0, hi = nB;  // keys of B below key
-      while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (sB[mid] < key)
-          lo = mid + 1;
-        else
-          hi = mid;
-      }
-      out[x] = static_cast<uint16_t>(lo);
+    for (int i = threadIdx.x; i < nq; i += blockDim.x) {  // the queue holding pair p
+      const int C = (s_n[i] + kSegMax - 1) / kSegMax;
+      if (p >= s_pair0[i] && p < s_pair0[i] + static_cast<int64_t>(C) * (C - 1)) s_q = i;
     }
-    __syncthreads();  // sB serves the next pair
+    __syncthreads();
+    const int q = s_q;
+    if (q >= 0) {  // else a reservation no queue kept (uniform per block)
+      const int64_t off = s_off[q];
+      const int n = s_n[q], C = (n + kSegMax - 1) / kSegMax;
+      const int l = static_cast<int>(p - s_pair0[q]);
+      const int A = l / (C - 1), b = l % (C - 1), B = b < A ? b : b + 1;
+      const int nA = min(kSegMax, n - A * kSegMax), nB = min(kSegMax, n - B * kSegMax);
+      const unsigned long long *rA = keys + off + static_cast<int64_t>(A) * kSegMax;
+      const unsigned long long *rB = keys + off + static_cast<int64_t>(B) * kSegMax;
+      // a thread's keys are searched side by side (loads in flight together,
+      // the halving the same for all); ~0 past the run's end, never stored
+      unsigned long long key[kSegIPT];
+      int lo[kSegIPT];
+#pragma unroll
+      for (int i = 0; i < kSegIPT; ++i) {
+        const int x = i * kSegThreads + static_cast<int>(threadIdx.x);
+        if (x < nB) sB[x] = rB[x];
+        key[i] = x < nA ? rA[x] : ~0ull;
+        lo[i] = 0;
+      }
+      __syncthreads();
+      for (int len = nB; len > 1; len -= len / 2) {  // keys of B below each key
+#pragma unroll
+        for (int i = 0; i < kSegIPT; ++i)
+          if (sB[lo[i] + len / 2 - 1] < key[i]) lo[i] += len / 2;
+      }
+      uint16_t *out = pq.cnt + p * kSegMax;
+#pragma unroll
+      for (int i = 0; i < kSegIPT; ++i) {
+        const int x = i * kSegThreads + static_cast<int>(threadIdx.x);
+        if (x < nA) out[x] = static_cast<uint16_t>(lo[i] + (sB[lo[i]] < key[i] ? 1 : 0));
+      }
+    }
+    __syncthreads();  // sB and s_q serve the next pair
   }
   if (!grid_barrier(bar, status, g_lookback_spins)) return;
   // (2) each key's place: its place in its run plus its counts in the others
   const unsigned long long imask = (1ull << index_bits(N)) - 1;
   const int64_t gstride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int q = 0; q < nq; ++q) {
-    const int64_t off = pq.off[q];
-    const int n = pq.n[q], C = (n + kSegMax - 1) / kSegMax;
-    const int64_t pair0 = pq.pair0[q];
-    for (int64_t e = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; e < n; e += gstride) {
+    const int n = s_n[q];
+    const unsigned first = s_first[q];
+    const unsigned vb = blockIdx.x >= first ? blockIdx.x - first : blockIdx.x + gridDim.x - first;
+    if (static_cast<int64_t>(vb) * blockDim.x >= n) continue;
+    const int64_t off = s_off[q];
+    const int C = (n + kSegMax - 1) / kSegMax;
+    const int64_t pair0 = s_pair0[q];
+    for (int64_t e = static_cast<int64_t>(vb) * blockDim.x + threadIdx.x; e < n; e += gstride) {
       const int A = static_cast<int>(e / kSegMax), x = static_cast<int>(e - static_cast<int64_t>(A) * kSegMax);
       int64_t pos = x;
       for (int B = 0; B < C; ++B) {
@@ -1734,6 +1861,7 @@ order_finish_kernel(int n_hi, int64_t N, int D, int dbits, const OrderCounts *co
     for (int64_t i = first; i < N; i += stride) perm[i] = static_cast<int32_t>(i);
 }
 
+static_assert(kPassThreads == kSegThreads, "a pair's keys are kSegIPT a thread");
 static_assert(sizeof(PassSmem) >= kSegMax * sizeof(unsigned long long),
               "one sorted run fits the finishing kernel's shared memory");
 

@@ -694,6 +694,35 @@ def test_order_long_queues(M, ws, oracle, N, D, blo, bhi, skew):
     assert np.array_equal(seg, so)
 
 
+@pytest.mark.parametrize("N,D,ubits,abits,skew", [
+    # arrival out of index order past one block: (not promoted, bound, arrival,
+    # index) in exactly 63 bits, sorted per decoder, and in 64, sorted globally
+    (16384, 5, 17, 31, 0.0), (16384, 5, 18, 31, 0.0),
+    # one decoder; ragged last chunks ranked pairwise; a queue past the pairwise
+    # ranks merged level by level; many queues of two runs; the most decoders
+    (4609, 1, 14, 20, 0.0), (60001, 3, 14, 20, 0.5), (90000, 2, 14, 24, 0.9),
+    (300000, 60, 14, 22, 0.0), (50000, 1024, 14, 20, 0.0),
+    # one entry past a bucketing round, and ranges of several rounds
+    (4097, 9, 10, 10, 0.0), (1300000, 300, 14, 25, 0.0),
+    # too many merges: sorted globally
+    (400000, 1, 14, 22, 0.0)])
+def test_order_shuffled_arrival_forms(M, ws, oracle, N, D, ubits, abits, skew):
+    rng = np.random.default_rng(N + D + ubits)
+    dec = rng.integers(0, D, N).astype(np.int32)
+    dec[rng.random(N) < skew] = D // 2
+    U = rng.integers(0, 2**ubits, N, dtype=np.int64).astype(np.int32)
+    wait = rng.integers(-10, 3000, N).astype(np.int32)
+    U[7], wait[7] = 2**ubits - 1, 0  # the full widths
+    arr = rng.integers(0, 2**abits, N, dtype=np.int64).astype(np.int32)
+    arr[N // 2] = 2**abits - 1
+    arr[: N // 4] = arr[N // 4]  # ties on arrival: by index
+    sto, po, so = oracle.order_local(D, dec, U, wait, arr, 1000)
+    st, perm, seg = gpu_order(M, ws, D, dec, U, wait, arr, 1000)
+    assert st == sto == 0
+    assert np.array_equal(perm, po)
+    assert np.array_equal(seg, so)
+
+
 def test_order_degenerate_keys(M, ws, oracle):
     # every key identical: all digit passes trivial -> identity order
     N = 9000
