@@ -597,7 +597,8 @@ stream_csr_kernel(int nact, int D, int rr, const int32_t *q_dev, int32_t *q_out_
 // smallest Q, else the largest headroom, ties to the lowest index), inserts
 // (u, p + 1) into the chosen decoder's list and rebuilds its tables.  The
 // decisions and range errors are those of the dense projection followed by
-// maps_dispatch SEQUENTIAL.
+// maps_dispatch SEQUENTIAL.  (At most 32 decoders take walk_registers below
+// while their lists fit it.)
 // Shared memory: the pool of pairs (the residents of decoder k plus room for
 // nb reservations at base_k = res_off[k] + k nb), the unsorted pairs, and the
 // per-decoder tables.
@@ -669,6 +670,191 @@ __device__ bool rebuild_tables(const int32_t *E, const int32_t *Bv, uint32_t *SS
   }
   __syncwarp();
   return __any_sync(0xffffffffu, over);
+}
+
+// The walk with a warp a decoder (at most 32): warp k keeps decoder k's pairs
+// in registers, kS a lane in any order, each with V = K(t) + t at its last live
+// step t = e - 1.  Reserving (u, p + 1) adds p + e to V where e <= u, and the
+// new pair's own V is P + p + u with P = K(u - 1) + u - 1, known from scoring
+// the candidate, so a reservation moves nothing.  M(u) is the larger of the V
+// with e < u and P: two warp reductions and a ballot.  A decision takes one
+// barrier: every warp picks from the keys published before it, the winner's
+// reserves, and all score the next candidate.  Keys as for maps_dispatch
+// SEQUENTIAL: a feasible decoder is min(Q - q0, lim) << 5 | k, an infeasible one
+// 1 << 31 | min(M - cap - x0, lim) << 5 | k; at lim the 64-bit keys decide.
+// Returns false when a list outgrows 32 kS pairs (nothing is kept then).
+// 32 warps issue every decision's instructions, so those are counted: 32
+// decoders at 16,000 tokens, 256 candidates: the dispatch kernel 160 -> 101 us
+// (0.33 us a candidate); before, two warps shared the walk on sorted lists in
+// shared memory.  (140 us with M and Q published beside every key and the
+// candidates clamped in every warp.)
+struct WalkShared {
+  uint32_t key[2][32];  // of each decoder for a candidate, by its parity
+  uint32_t M[32];       // where the 64-bit keys decide: M and the queue length
+  int32_t q[32];
+  long long x0;
+  int q0, wide, over;
+};
+template <int kS>
+__device__ bool walk_registers(int D, int nb, int mc, const int32_t *uE, const int32_t *uB,
+                               const int32_t *s_base, const int32_t *s_n, int32_t *s_q,
+                               const int32_t *s_cap, const int2 *cand, int32_t *choice,
+                               int64_t *headroom, WalkShared &w, bool &bad) {
+  constexpr unsigned kAll = 0xffffffffu;
+  const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
+  const bool has = k < D;
+  int n = has ? s_n[k] : 0;
+  const int lo = has ? s_base[k] - k * nb : 0;  // the decoder's pairs in uE, uB
+  const int32_t cap = has ? s_cap[k] : 0;
+  int32_t q = has ? s_q[k] : 0;
+  uint32_t e[kS], b[kS], V[kS];
+  if (threadIdx.x == 0) {
+    w.x0 = LLONG_MAX;
+    w.q0 = 0x7fffffff;
+    w.wide = w.over = 0;
+  }
+  __syncthreads();
+  long long sb = 0;
+  if (has) {
+    const bool fit = n <= 32 * kS;
+    if (!fit && lane == 0) w.over = 1;
+#pragma unroll
+    for (int s = 0; s < kS; ++s) {
+      const int i = 32 * s + lane;
+      e[s] = fit && i < n ? static_cast<uint32_t>(uE[lo + i]) : 0u;
+      b[s] = fit && i < n ? static_cast<uint32_t>(uB[lo + i]) : 0u;
+      sb += b[s];
+    }
+    // b-sum and count of the pairs live at e - 1
+    unsigned long long S[kS];
+    uint32_t C[kS];
+#pragma unroll
+    for (int s = 0; s < kS; ++s) S[s] = C[s] = 0;
+    for (int m = 0; fit && m < n; ++m) {
+      const uint32_t em = static_cast<uint32_t>(uE[lo + m]), bm = static_cast<uint32_t>(uB[lo + m]);
+#pragma unroll
+      for (int s = 0; s < kS; ++s)
+        if (em >= e[s]) {
+          S[s] += bm;
+          C[s] += 1;
+        }
+    }
+#pragma unroll
+    for (int s = 0; s < kS; ++s) {
+      V[s] = 0;
+      if (e[s] > 0) {
+        const unsigned long long Kt = S[s] + static_cast<unsigned long long>(e[s] - 1) * C[s];
+        if (Kt > 0x7fffffffull) bad = true;  // K at e - 1: the projection's range error
+        V[s] = static_cast<uint32_t>(Kt) + e[s] - 1;
+      }
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) sb += __shfl_xor_sync(kAll, sb, off);
+    if (sb > 0x7fffffffLL) bad = true;  // K at step 0
+    if (lane == 0) {
+      atomicMin(&w.x0, sb - cap);
+      atomicMin(&w.q0, q);
+    }
+  }
+  __syncthreads();
+  if (w.over) return false;
+  const long long off64 = -(w.x0 + cap);
+  const uint32_t off = static_cast<uint32_t>(off64);
+  // M < 2^31 + 2^28 while K is within int32: M + off cannot wrap
+  if (has && lane == 0 && (off64 > (1ll << 30) || off64 < INT_MIN)) w.wide = 1;
+  __syncthreads();
+  const int32_t q0 = w.q0;
+  const uint32_t lim = w.wide ? 0u : (1u << 26) - 2u;
+  const uint32_t lim_key = lim << 5;
+  if (k >= D) {
+    __syncthreads();  // the one after the walk
+    return w.over == 0;
+  }
+  if (lane >= D) w.key[0][lane] = w.key[1][lane] = ~0u;
+  uint32_t P = 0, M = 0;
+  // candidate (p, u) scored into column `par`
+  const uint32_t kbit = static_cast<uint32_t>(k), kinf = kbit + 0x80000000u;
+  const int32_t capf = mc ? 0 : cap;  // mc: no decoder is feasible
+  auto score = [&](int2 c, int par) {
+    const uint32_t u = static_cast<uint32_t>(c.y);
+    uint32_t sum = 0, cnt = 1, vm = 0;
+#pragma unroll
+    for (int s = 0; s < kS; ++s) {
+      const bool live = e[s] >= u;  // at step u - 1
+      sum += live ? b[s] : 0u;
+      cnt += __popc(__ballot_sync(kAll, live));
+      vm = max(vm, live ? 0u : V[s]);
+    }
+    sum = __reduce_add_sync(kAll, sum);
+    vm = __reduce_max_sync(kAll, vm);
+    P = sum + (u - 1) * cnt;
+    M = max(vm, P);
+    // p + 1 + M <= cap: M < cap - p
+    const bool feas = M < static_cast<uint32_t>(max(capf - c.x, 0));
+    const uint32_t term = min(feas ? static_cast<uint32_t>(q - q0) : M + off, lim);
+    if (lane == 0) w.key[par][k] = (term << 5) + (feas ? kbit : kinf);
+  };
+  int2 c = cand[0];
+  score(c, 0);
+  named_bar(1, 32 * D);
+  for (int j = 0; j < nb; ++j) {
+    const int2 c1 = cand[j + 1];  // there is one past the end
+    if (c.y > 0) {
+      const uint32_t best = __reduce_min_sync(kAll, w.key[j & 1][lane]);
+      int kk = static_cast<int>(best & 31u);
+      if ((best & 0x7fffffffu) >= lim_key) {  // in every warp alike
+        if (lane == 0) {
+          w.M[k] = M;
+          w.q[k] = q;
+        }
+        named_bar(1, 32 * D);
+        unsigned long long k64 = ~0ull;
+        if (lane < D)
+          k64 = dispatch_key(static_cast<long long>(s_cap[lane]) -
+                                 (static_cast<long long>(c.x) + 1 + w.M[lane]),
+                             w.q[lane], lane, mc);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          const unsigned long long y = __shfl_xor_sync(kAll, k64, o);
+          k64 = y < k64 ? y : k64;
+        }
+        kk = static_cast<int>(k64 & 1023u);
+        named_bar(1, 32 * D);  // M and q have been read
+      }
+      if (kk == k) {
+        const uint32_t p = static_cast<uint32_t>(c.x), u = static_cast<uint32_t>(c.y);
+        if (lane == 0) {
+          choice[j] = kk;
+          if (headroom) headroom[j] = static_cast<long long>(cap) - (static_cast<long long>(p) + 1 + M);
+          if (n == 32 * kS) w.over = 1;
+        }
+#pragma unroll
+        for (int s = 0; s < kS; ++s) {
+          if (e[s] - 1u < u) V[s] += p + e[s];
+          if (n == 32 * s + lane) {
+            e[s] = u;
+            b[s] = p + 1u;
+            V[s] = P + p + u;
+          }
+        }
+        n += 1;
+        // the largest new cell, K + p + t + 1, is M + p + 1
+        bad |= q == 0x7fffffff || static_cast<long long>(p) + 1 + M > 0x7fffffffLL;
+        q += q == 0x7fffffff ? 0 : 1;
+      }
+    } else if (threadIdx.x == 0) {
+      bad = true;
+      choice[j] = -1;
+      if (headroom) headroom[j] = 0;
+    }
+    score(c1, (j + 1) & 1);
+    c = c1;
+    named_bar(1, 32 * D);
+  }
+  __syncthreads();
+  const bool ok = w.over == 0;
+  if (ok && lane == 0) s_q[k] = q;
+  return ok;
 }
 
 __global__ void __launch_bounds__(kSt, 1)
@@ -854,7 +1040,35 @@ stream_dispatch_kernel(int D, int H, int nb, int mc, const int64_t *res_off, con
   }
   __syncthreads();
 
-  if (!s_fast) {
+  // At most 32 decoders: a warp each, with the lists in registers; a list that
+  // outgrows a variant moves on to the next, the last one below.
+  __shared__ WalkShared walk;
+  bool walked = s_fast != 0;
+  if (!walked && D <= 32) {
+    int nmax = 0;
+    for (int k = 0; k < D; ++k) nmax = max(nmax, s_n[k]);
+    const int about = nmax + 2 * nb / D;
+    // (p, u) of the batch, u = 0 marking an invalid candidate and the end, over
+    // the space of the sorted lists
+    int2 *cand = reinterpret_cast<int2 *>(E);
+    for (int j = tid; j <= nb; j += kSt) {
+      const int32_t p = j < nb ? s_cp[j] : -1, U = j < nb ? s_cu[j] : -1;
+      cand[j] = (p | U) < 0 ? make_int2(0, 0) : make_int2(p, U < 1 ? 1 : (U > H ? H : U));
+    }
+    bool wbad = false;
+    auto go = [&](auto walk_fn) {
+      wbad = false;
+      walked = walk_fn(D, nb, mc, uE, uB, s_base, s_n, s_q, s_cap, cand, choice, headroom, walk, wbad);
+      __syncthreads();
+    };
+    if (about <= 32) go(walk_registers<1>);
+    if (!walked && about <= 64) go(walk_registers<2>);
+    if (!walked && about <= 128) go(walk_registers<4>);
+    if (walked && wbad) s_bad = 1;
+    __syncthreads();
+  }
+
+  if (!walked) {
     // sort each decoder's pairs by e (rank among the decoder's pairs, ties by
     // position), and check sum b <= INT32_MAX (K at step 0)
     for (int k = warp; k < D; k += kSt / 32) {
@@ -886,232 +1100,7 @@ stream_dispatch_kernel(int D, int H, int nb, int mc, const int64_t *res_off, con
   // e <= u), then M = max(PM[c - 1], SS[c] + (u - 1)(n - c + 1)); a packed key
   // picks (feasible first, then Q or the largest headroom, then the lowest
   // index); the warp inserts the footprint and rebuilds that decoder's tables.
-  if (s_fast) {
-    // decided by the fast path
-  } else if (D <= 32) {
-    // Two warps, one decoder per lane.  Warp 0 holds each decoder's list
-    // length, base, Q and capacity in registers, scores the candidates, picks
-    // and books each decision and hands it to warp 1 through shared memory
-    // (named barrier 1); warp 1 inserts the reservation into the chosen
-    // decoder's list and scores that decoder again for the next candidate
-    // (named barrier 2).  Meanwhile warp 0 scores the next candidate on the
-    // lists as they stand: a reservation only raises the chosen decoder's Q
-    // and occupancy, so every other decoder's key is already final and the
-    // chosen one's is replaced by warp 1's.  Keys: inf << 63 | v << 10 | k,
-    // the smallest wins.
-    __shared__ int h_bk, h_pos, h_n, h_base, h_q, h_cap, h_c;
-    __shared__ long long h_M;
-    __shared__ unsigned long long h_key;
-    auto clampu = [&](int32_t U) { return U < 1 ? 1 : (U > H ? H : U); };
-    // c = the pairs with e <= u of a sorted list (8-ary search: eight
-    // independent probes per level, one level for up to 8 pairs)
-    auto count_le = [&](const int32_t *Ek, int n, int u) {
-      int lo = 0, hi = n;
-      while (lo < hi) {
-        const int len = hi - lo;
-        int nlo = lo, nhi = hi;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {  // probes cover every position when len <= 8
-          const int pi = lo + (len * i) / 8;
-          if (Ek[pi] <= u)
-            nlo = max(nlo, pi + 1);
-          else
-            nhi = min(nhi, pi);
-        }
-        lo = nlo;
-        hi = nhi;
-      }
-      return lo;
-    };
-    auto key_of = [mc](int k, int q, int cap, int32_t p, long long M) {
-      const long long h = static_cast<long long>(cap) - (static_cast<long long>(p) + 1 + M);
-      return dispatch_key(h, q, k, mc);
-    };
-    if (warp == 0) {
-      const int k = lane;
-      const bool has = k < D;
-      int n_r = has ? s_n[k] : 0, q_r = has ? s_q[k] : 0;
-      const int base_r = has ? s_base[k] : 0, cap_r = has ? s_cap[k] : 0;
-      bool bad = false, have = false;  // have: key, c and M are the current candidate's
-      unsigned long long key = ~0ull;
-      long long M = 0;
-      int c = 0;
-      auto score = [&](int32_t pp, int uu) {
-        key = ~0ull;
-        if (!has) return;
-        if (quick && n_r > 0) {
-          const long long mub = max(static_cast<long long>(PM[base_r + n_r - 1]),
-                                    static_cast<long long>(SS[base_r]) +
-                                        static_cast<long long>(uu - 1) * (n_r + 1));
-          if (static_cast<long long>(pp) + 1 + mub <= cap_r) {
-            key = (static_cast<unsigned long long>(q_r) << 10) | static_cast<unsigned>(k);
-            c = -1;   // found at insertion
-            M = mub;  // bounds every new cell: no range error (cap <= INT32_MAX)
-            return;
-          }
-        }
-        c = count_le(E + base_r, n_r, uu);
-        const long long full = c > 0 ? static_cast<long long>(PM[base_r + c - 1]) : LLONG_MIN;
-        const long long part = static_cast<long long>(c < n_r ? SS[base_r + c] : 0u) +
-                               static_cast<long long>(uu - 1) * (n_r - c + 1);
-        M = max(full, part);
-        key = key_of(k, q_r, cap_r, pp, M);
-      };
-      for (int j = 0; j < nb; ++j) {
-        const int32_t p = s_cp[j], U = s_cu[j];
-        int bk = -1;
-        if ((p | U) >= 0) {
-          if (!have) score(p, clampu(U));
-          // the warp's smallest key: one 32-bit reduction when every value
-          // fits 21 bits (inf << 31 | v << 10 | k, the same order), else a ladder
-          const unsigned long long kv = (key >> 10) & ((1ull << 53) - 1);
-          const bool none = key == ~0ull;
-          if (__all_sync(0xffffffffu, none || kv < (1ull << 21))) {
-            const uint32_t k32 = none ? 0xffffffffu
-                                      : (static_cast<uint32_t>(key >> 63) << 31) |
-                                            (static_cast<uint32_t>(kv) << 10) | static_cast<uint32_t>(key & 1023u);
-            bk = static_cast<int>(__reduce_min_sync(0xffffffffu, k32) & 1023u);
-          } else {
-            unsigned long long kk = key;
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-              const unsigned long long o = __shfl_xor_sync(0xffffffffu, kk, off);
-              kk = o < kk ? o : kk;
-            }
-            bk = static_cast<int>(kk & 1023u);
-          }
-          if (lane == bk) {  // the chosen decoder's lane books the decision
-            choice[j] = bk;
-            if (headroom) headroom[j] = static_cast<long long>(cap_r) - (static_cast<long long>(p) + 1 + M);
-            bad |= q_r == 0x7fffffff;
-            q_r += q_r == 0x7fffffff ? 0 : 1;
-            // every new cell K + p + t + 1 (t < u) is at most M + p + 1
-            bad |= static_cast<long long>(p) + 1 + M > 0x7fffffffLL;
-            h_bk = bk;
-            h_pos = c;
-            h_n = n_r;
-            h_base = base_r;
-            h_q = q_r;
-            h_cap = cap_r;
-            n_r += 1;
-          }
-        } else if (lane == 0) {
-          bad = true;
-          choice[j] = -1;
-          if (headroom) headroom[j] = 0;
-          h_bk = -1;
-        }
-        named_bar(1, 64);  // the decision goes to warp 1
-        const bool nxt = j + 1 < nb;
-        const int32_t p1 = nxt ? s_cp[j + 1] : 0, U1 = nxt ? s_cu[j + 1] : 0;
-        const bool ok1 = nxt && (p1 | U1) >= 0;
-        if (ok1) score(p1, clampu(U1));  // the chosen decoder's key is replaced below
-        named_bar(2, 64);  // warp 1 has updated the list and scored it again
-        if (ok1 && lane == bk) {
-          key = h_key;
-          c = h_c;
-          M = h_M;
-        }
-        have = ok1;
-      }
-      if (__any_sync(0xffffffffu, bad) && lane == 0) flag_error(status, MAPS_E_RANGE);
-      if (has) {
-        s_n[k] = n_r;
-        s_q[k] = q_r;
-      }
-    } else if (warp == 1) {
-      for (int j = 0; j < nb; ++j) {
-        named_bar(1, 64);
-        const int bk = h_bk;
-        if (bk >= 0) {
-          const int n = h_n, base = h_base, m = n + 1;
-          const int32_t p = s_cp[j];
-          const int u = clampu(s_cu[j]);
-          int pos = h_pos;  // -1: the scoring took the bound, count the pairs with e <= u here
-          if (pos < 0) {
-            if (n < 32)
-              pos = __popc(__ballot_sync(0xffffffffu, lane < n && E[base + lane] <= u));
-            else
-              pos = count_le(E + base, n, u);
-          }
-          const bool nxt = j + 1 < nb;
-          const int32_t p1 = nxt ? s_cp[j + 1] : 0, U1 = nxt ? s_cu[j + 1] : 0;
-          const bool ok1 = nxt && (p1 | U1) >= 0;
-          const int u1 = clampu(U1);
-          int c1 = 0;
-          long long M1 = 0;
-          if (m <= 32) {
-            // one round: lane i takes pair i of the new list; the suffix sums
-            // follow from the old ones (b more before the new pair, the same
-            // after it) and one shuffle scan gives the prefix maxima of V, in
-            // 32 bits (the booking's check keeps every K + t within INT32_MAX)
-            const int src = lane <= pos ? lane : lane - 1;
-            const bool old_ok = src < n;
-            const int eo = old_ok ? E[base + src] : 0, bo = old_ok ? Bv[base + src] : 0;
-            const uint32_t so = old_ok ? SS[base + src] : 0u;
-            const uint32_t bnew = static_cast<uint32_t>(p) + 1u;
-            const int e2 = lane == pos ? u : eo;
-            const int b2 = lane == pos ? static_cast<int>(bnew) : bo;
-            const uint32_t suf = lane <= pos ? so + bnew : so;
-            uint32_t V = lane < m ? suf + static_cast<uint32_t>(e2 - 1) * static_cast<uint32_t>(m - lane + 1) : 0u;
-#pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-              const uint32_t y = __shfl_up_sync(0xffffffffu, V, off);
-              if (lane >= off) V = max(V, y);
-            }
-            __syncwarp();  // every lane has read the old list
-            if (lane < m) {
-              E[base + lane] = e2;
-              Bv[base + lane] = b2;
-              SS[base + lane] = suf;
-              PM[base + lane] = V;
-            }
-            // the new list's count and table values at the next candidate's u
-            c1 = __popc(__ballot_sync(0xffffffffu, lane < m && e2 <= u1));
-            const uint32_t pmb = __shfl_sync(0xffffffffu, V, c1 > 0 ? c1 - 1 : 0);
-            const uint32_t ssb = __shfl_sync(0xffffffffu, suf, c1 < m ? c1 : 0);
-            const long long full = c1 > 0 ? static_cast<long long>(pmb) : LLONG_MIN;
-            const long long part = static_cast<long long>(c1 < m ? ssb : 0u) +
-                                   static_cast<long long>(u1 - 1) * (m - c1 + 1);
-            M1 = max(full, part);
-          } else {
-            // a list past 32 pairs: shift [pos, n) up by one (last round
-            // first), place the new pair, rebuild the tables
-            for (int r = (n - 1) >> 5; r >= 0; --r) {
-              const int i = r * 32 + lane;
-              const bool mv = i < n && i >= pos;
-              const int e = mv ? E[base + i] : 0, b = mv ? Bv[base + i] : 0;
-              __syncwarp();
-              if (mv) {
-                E[base + i + 1] = e;
-                Bv[base + i + 1] = b;
-              }
-              __syncwarp();
-            }
-            if (lane == 0) {
-              E[base + pos] = u;
-              Bv[base + pos] = p + 1;
-            }
-            __syncwarp();
-            rebuild_tables(E + base, Bv + base, SS + base, PM + base, m);
-            if (ok1) {
-              c1 = count_le(E + base, m, u1);
-              const long long full = c1 > 0 ? static_cast<long long>(PM[base + c1 - 1]) : LLONG_MIN;
-              const long long part = static_cast<long long>(c1 < m ? SS[base + c1] : 0u) +
-                                     static_cast<long long>(u1 - 1) * (m - c1 + 1);
-              M1 = max(full, part);
-            }
-          }
-          if (ok1 && lane == 0) {
-            h_key = key_of(bk, h_q, h_cap, p1, M1);
-            h_c = c1;
-            h_M = M1;
-          }
-        }
-        named_bar(2, 64);
-      }
-    }
-  } else if (warp == 0) {
+  if (!walked && warp == 0) {
     for (int j = 0; j < nb; ++j) {
       const int32_t p = s_cp[j], U = s_cu[j];
       if ((p | U) < 0) {

@@ -970,6 +970,16 @@ def test_stream_prefix(M, ws, oracle, N, D, H, cap, B, Wn, a, mw):
     assert (qo >= 0).any() or N < 1000
 
 
+@pytest.mark.parametrize("N,D,cap,B", [
+    # lists around 32, 64 and 128 pairs a decoder, some outgrowing the variant
+    # they start on within a batch; one decoder, and as many as a warp's lanes
+    (1500, 1, 30000, 16), (2000, 1, 9000, 40), (2000, 2, 50000, 90), (3000, 3, 40000, 200),
+    (4000, 31, 9000, 256), (4000, 32, 14000, 300), (4000, 32, 60, 100)])
+def test_stream_walk_list_sizes(M, ws, oracle, N, D, cap, B):
+    w = W.make_stream(n_requests=N)
+    check_stream(M, ws, oracle, N, D, 16384, cap, B, 300, 100000, 1000, w)
+
+
 def test_stream_full_workload(M, ws, oracle):
     """All 1,000,000 requests of the streaming workload, bit for bit."""
     w = W.make_stream()
