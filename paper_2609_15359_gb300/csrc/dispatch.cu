@@ -124,6 +124,23 @@ kmax_from_K_kernel(int D, int H, const int32_t *__restrict__ K, uint32_t *__rest
   if (neg) flag_error(status, MAPS_E_RANGE);
 }
 
+// A caller's summary is compared with K at four blocks of every row (the
+// first, the last, the middle and one that varies with the decoder); a
+// mismatch there is reported, any other gives unspecified results.
+__device__ __forceinline__ bool summary_matches(const int32_t *__restrict__ K,
+                                                const uint32_t *__restrict__ kmax, int H, int64_t nb,
+                                                int k, int which) {
+  const int64_t b = which == 0 ? 0 : which == 1 ? nb - 1 : which == 2 ? nb / 2 : (k * 7919LL) % nb;
+  const int32_t *kr = K + static_cast<int64_t>(k) * H;
+  const int64_t t_end = (b + 1) * kSumBlock < H ? (b + 1) * kSumBlock : static_cast<int64_t>(H);
+  long long mx = -1;
+  for (int64_t t = b * kSumBlock; t < t_end; ++t) {
+    const long long v = static_cast<long long>(__ldg(kr + t)) + t;
+    mx = v > mx ? v : mx;
+  }
+  return mx >= 0 && static_cast<uint32_t>(mx) == __ldg(kmax + k * nb + b);
+}
+
 // carry[k][i] = max of K[k][t] + t over t < i*W2 (0 for i = 0): the prefix
 // maximum that horizon tile i inherits from the tiles before it.  One block
 // per decoder; each thread reads 16 consecutive summary entries at once
@@ -213,21 +230,8 @@ __device__ void carry_scan_block(int kk, int D, int H, int W2, int T2, const int
     run = all > run ? all : run;
     __syncthreads();
   }
-  if (check_kmax && threadIdx.x < 4) {
-    // a caller's summary is compared with K at four blocks of this row (the
-    // first, the last, the middle and one that varies with the decoder); a
-    // mismatch there is reported, any other gives unspecified results
-    const int64_t b = threadIdx.x == 0 ? 0 : threadIdx.x == 1 ? nb - 1 : threadIdx.x == 2 ? nb / 2
-                                                                     : (k * 7919LL) % nb;
-    const int32_t *kr = K + static_cast<int64_t>(k) * H;
-    const int64_t t_end = (b + 1) * kSumBlock < H ? (b + 1) * kSumBlock : static_cast<int64_t>(H);
-    long long mx = -1;
-    for (int64_t t = b * kSumBlock; t < t_end; ++t) {
-      const long long v = static_cast<long long>(__ldg(kr + t)) + t;
-      mx = v > mx ? v : mx;
-    }
-    if (mx < 0 || static_cast<uint32_t>(mx) != __ldg(row + b)) flag_error(status, MAPS_E_INVALID);
-  }
+  if (check_kmax && threadIdx.x < 4 && !summary_matches(K, kmax, H, nb, k, threadIdx.x))
+    flag_error(status, MAPS_E_INVALID);
 }
 
 __device__ __forceinline__ unsigned lanemask_lt() {
@@ -817,6 +821,168 @@ dispatch_snapshot_kernel(const __grid_constant__ CUtensorMap tmap, SnapArgs a) {
       if (a.headroom) a.headroom[jj[i]] = static_cast<long long>(pm[l]) - p;
     }
   }
+}
+
+// ---------------------------------------------------------------------------
+// SNAPSHOT of few candidates (direct_fits): one launch instead of a memset and
+// three.  One to eight warps take a candidate and score its decoders, a slice
+// each: per decoder M, the maximum of the 16-step summary below u by all the
+// lanes, and of at most 15 cells.  Nothing is bucketed and nothing carried, at the
+// price of reading each row's summary once a candidate, from L2.
+//
+// The grid also reads K once for negative values, and compares a caller's
+// summary with K at four blocks of every row, as the bucketed form does.
+// ---------------------------------------------------------------------------
+constexpr int kDirectWarps = 8;
+constexpr int kDirectRows = 8;
+
+// At most this many (candidate, decoder) scores, half as many of them times the
+// 2,048-step spans of the horizon, and cells of K, and a horizon that a warp
+// reads in time even if every candidate lives through all of it.  Measured,
+// one launch against four (candidates of a few hundred steps; all through the
+// horizon): 4 decoders, H 4,096, 32 candidates 4.7 against 13.1 us (5.2; 12.9);
+// 16, 16,381, 1,021: 7.2 against 20.6 (11.2; 18.6); 100, 8,192, 600: 12.1
+// against 16.4 (19.2; 16.5); 64, 4,096, 2,048: 16.2 against 18.6; past the
+// line 16, 2,048, 16,384: 25.9 against 20.7; 256, 2,048, 1,024: 22.6 against
+// 18.4; 12, 50,000, 100: 7.8 against 16.4, but 63 against 14.5.
+constexpr int64_t kDirectScores = 1 << 17;
+constexpr int64_t kDirectCells = 1 << 20;
+constexpr int kDirectH = 32768;
+bool direct_fits(int D, int H, int64_t J) {
+  return J * D <= kDirectScores && J * D * std::max(1, H / 2048) <= 2 * kDirectScores &&
+         H <= kDirectH && static_cast<int64_t>(D) * H <= kDirectCells;
+}
+
+template <bool VEC>
+__global__ void __launch_bounds__(32 * kDirectWarps)
+dispatch_direct_kernel(int D, int H, const int32_t *__restrict__ K, const uint32_t *__restrict__ kmax,
+                       int check_kmax, const int32_t *__restrict__ cap, const int32_t *__restrict__ Q,
+                       int64_t J, const int32_t *__restrict__ cp, const int32_t *__restrict__ cb,
+                       int32_t *__restrict__ choice, int64_t *__restrict__ headroom, int32_t *status,
+                       int share) {
+  constexpr unsigned kAll = 0xffffffffu;
+  __shared__ unsigned long long s_key[kDirectWarps];
+  __shared__ long long s_h[kDirectWarps];
+  pdl_prologue();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t nb = (static_cast<int64_t>(H) + kSumBlock - 1) / kSumBlock;
+  // this warp's candidate of the block's, and its decoders [d0, d1)
+  const int per = kDirectWarps / share, mine = warp / share, part = warp % share;
+  const int slice = ((D + share - 1) / share + kDirectRows - 1) / kDirectRows * kDirectRows;
+  const int d0 = min(D, part * slice), d1 = min(D, d0 + slice);
+  for (int64_t j0 = static_cast<int64_t>(blockIdx.x) * per; j0 < J; j0 += static_cast<int64_t>(gridDim.x) * per) {
+    const int64_t j = j0 + mine;
+    const int32_t p = j < J ? __ldg(cp + j) : -1, U = j < J ? __ldg(cb + j) : -1;
+    unsigned long long best = ~0ull;  // infeasible << 63 | Q or deficit << 10 | decoder
+    long long best_h = 0;
+    if ((p | U) >= 0) {
+      const int u = candidate_steps(U, H);
+      const int nfull = u / kSumBlock, rem = u - nfull * kSumBlock;
+      // kDirectRows rows at a time, their loads in flight together; lane i
+      // keeps the M of the i-th of 32 rows
+      for (int k0 = d0; k0 < d1; k0 += 32) {
+        uint32_t M = 0;
+        for (int i0 = 0; i0 < 32 && k0 + i0 < d1; i0 += kDirectRows) {
+          uint32_t m[kDirectRows];
+#pragma unroll
+          for (int i = 0; i < kDirectRows; ++i) {
+            const int k = min(k0 + i0 + i, D - 1), t = nfull * kSumBlock + lane;
+            m[i] = lane < rem ? static_cast<uint32_t>(__ldg(K + static_cast<int64_t>(k) * H + t)) +
+                                    static_cast<uint32_t>(t)
+                              : 0u;
+          }
+          const uint32_t *km = kmax + static_cast<int64_t>(k0 + i0) * nb;
+          const int64_t rows = D - 1 - (k0 + i0);  // the last row's distance
+          if (VEC) {  // rows are whole 16-byte words
+            for (int b = 4 * lane; b < nfull; b += 128) {
+              uint4 v[kDirectRows];
+#pragma unroll
+              for (int i = 0; i < kDirectRows; ++i)
+                v[i] = __ldg(reinterpret_cast<const uint4 *>(km + (i < rows ? i : rows) * nb + b));
+#pragma unroll
+              for (int i = 0; i < kDirectRows; ++i) {
+                m[i] = max(m[i], v[i].x);
+                if (b + 1 < nfull) m[i] = max(m[i], v[i].y);
+                if (b + 2 < nfull) m[i] = max(m[i], v[i].z);
+                if (b + 3 < nfull) m[i] = max(m[i], v[i].w);
+              }
+            }
+          } else {
+            for (int b = lane; b < nfull; b += 32) {
+              uint32_t v[kDirectRows];
+#pragma unroll
+              for (int i = 0; i < kDirectRows; ++i) v[i] = __ldg(km + (i < rows ? i : rows) * nb + b);
+#pragma unroll
+              for (int i = 0; i < kDirectRows; ++i) m[i] = max(m[i], v[i]);
+            }
+          }
+#pragma unroll
+          for (int i = 0; i < kDirectRows; ++i) {
+            const uint32_t r = __reduce_max_sync(kAll, m[i]);
+            if (lane == i0 + i) M = r;
+          }
+        }
+        if (k0 + lane < d1) {
+          const int k = k0 + lane;
+          const long long h = static_cast<long long>(__ldg(cap + k)) - (static_cast<long long>(p) + 1 + M);
+          const unsigned long long v =
+              h >= 0 ? static_cast<unsigned long long>(__ldg(Q + k)) & 0xffffffffull
+                     : (1ull << 53) | static_cast<unsigned long long>(-h);
+          const unsigned long long key = (v << 10) | static_cast<unsigned>(k);
+          if (key < best) {
+            best = key;
+            best_h = h;
+          }
+        }
+      }
+    }
+    unsigned long long all = best;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      const unsigned long long y = __shfl_xor_sync(kAll, all, off);
+      all = y < all ? y : all;
+    }
+    if (best == all && (best != ~0ull || lane == 0)) {  // the best decoder's lane (keys are unique)
+      s_key[warp] = best;
+      s_h[warp] = best_h;
+    }
+    __syncthreads();
+    if (part == 0 && lane == 0 && j < J) {
+      int w = warp;
+      for (int i = 1; i < share; ++i)
+        if (s_key[warp + i] < s_key[w]) w = warp + i;
+      const bool ok = (p | U) >= 0;
+      if (!ok) flag_error(status, MAPS_E_RANGE);
+      choice[j] = ok ? static_cast<int32_t>(s_key[w] & 1023u) : -1;
+      if (headroom) headroom[j] = ok ? s_h[w] : 0;
+    }
+    __syncthreads();  // the keys serve the block's next candidates
+  }
+  bool bad = false;
+  const int64_t gt = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  const int64_t nt = static_cast<int64_t>(gridDim.x) * blockDim.x;
+  for (int64_t k = gt; k < D; k += nt)
+    if ((__ldg(cap + k) | __ldg(Q + k)) < 0) bad = true;
+  if (check_kmax) {  // the summary pass of a call without one reports these
+    const int64_t cells = static_cast<int64_t>(D) * H;
+    int32_t any = 0;
+    if ((reinterpret_cast<uintptr_t>(K) & 15) == 0) {
+#pragma unroll 4
+      for (int64_t i = gt; i < cells / 4; i += nt) {
+        const int4 v = __ldg(reinterpret_cast<const int4 *>(K) + i);
+        any |= v.x | v.y | v.z | v.w;
+      }
+      if (gt < cells % 4) any |= __ldg(K + cells - 1 - gt);
+    } else {
+      for (int64_t i = gt; i < cells; i += nt) any |= __ldg(K + i);
+    }
+    if (any < 0) bad = true;
+    for (int64_t e = gt; e < 4ll * D; e += nt) {
+      const int k = static_cast<int>(e >> 2);
+      if (!summary_matches(K, kmax, H, nb, k, static_cast<int>(e & 3))) flag_error(status, MAPS_E_INVALID);
+    }
+  }
+  if (bad) flag_error(status, MAPS_E_RANGE);
 }
 
 // ---------------------------------------------------------------------------
@@ -1722,13 +1888,36 @@ int launch_snapshot(int D, int H, const int32_t *K, const uint32_t *kmax, const 
   uint32_t *nunits = w.zero + 2 * static_cast<size_t>(g.T2);
   uint32_t *ticket = nunits + 1;  // bin_count blocks finished
   const int sms = sm_count();
-  MAPS_TRY(cuda_ok(cudaMemsetAsync(w.zero, 0, w.zero_words * 4, s)));
   const bool check_kmax = kmax != nullptr;
+  const int64_t nb = (static_cast<int64_t>(H) + kSumBlock - 1) / kSumBlock;
+  const bool direct = direct_fits(D, H, J);
+  if (!direct) MAPS_TRY(cuda_ok(cudaMemsetAsync(w.zero, 0, w.zero_words * 4, s)));
   if (kmax == nullptr) {
-    const int64_t nb = (static_cast<int64_t>(H) + kSumBlock - 1) / kSumBlock;
     const int gk = static_cast<int>(std::min<int64_t>((nb * D + 255) / 256, 8LL * sms));
     launch_pdl(kmax_from_K_kernel, gk, 256, 0, s, D, H, K, w.kmax, status);
     kmax = w.kmax;
+  }
+  if (direct) {
+    // warps to a candidate: as many as have kDirectRows rows each
+    int share = 1;
+    while (share < kDirectWarps && share * kDirectRows < D) share *= 2;
+    const int64_t blocks = (J * share + kDirectWarps - 1) / kDirectWarps;
+    // the reading of K takes blocks of its own where the candidates have few
+    const int64_t reading = static_cast<int64_t>(D) * H / (32 * kDirectWarps * 16);
+    const int grid = static_cast<int>(
+        std::min<int64_t>(std::max(blocks, std::min<int64_t>(reading, 2LL * sms)), 8LL * sms));
+    if (g_score_ev[0]) MAPS_TRY(cuda_ok(cudaEventRecord(g_score_ev[0], s)));
+    auto launch = [&](auto kern) {
+      launch_pdl(kern, grid, 32 * kDirectWarps, 0, s, D, H, K, kmax, check_kmax ? 1 : 0, cap, Q, J, cp, cb,
+                 choice, headroom, status, share);
+    };
+    if (nb % 4 == 0 && aligned(kmax, 16))
+      launch(dispatch_direct_kernel<true>);
+    else
+      launch(dispatch_direct_kernel<false>);
+    MAPS_TRY(launch_ok());
+    if (g_score_ev[1]) MAPS_TRY(cuda_ok(cudaEventRecord(g_score_ev[1], s)));
+    return MAPS_OK;
   }
   // carries of D decoders, and candidate counts in blocks of 256 candidates
   const int gc = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>((J + 255) / 256, 4LL * sms)));

@@ -42,6 +42,13 @@ constexpr int kPerThread = 4;  // entries a thread loads per round
 constexpr int kRound = kPerThread * kOccThreads;
 constexpr int kBucketRound = kPerThread * kBucketThreads;
 constexpr int kMaxTiles = 128;  // tiles per decoder of the bucketed form
+// Residents read over all tiles up to which every tile CTA streams its
+// decoder's residents itself: one launch instead of two.  Measured, one launch
+// against two: 4 decoders of 64 residents, H 4,096 2.7 against 5.3 us; 16 of
+// 509, 16,381 4.6 against 7.9; 8 of 9,000, 4,096 7.2 against 17.8; 64 of 2,048,
+// 32,768 (1,048,576 reads) 7.0 against 8.9; 256 of 4,096, 65,536 (16 times as
+// many) 29 for the two.
+constexpr int64_t kDirectReads = 1 << 20;
 constexpr int kBHold = 8;       // residents a bucket thread keeps in registers
 // A tile holding at most this many end steps skips the histogram: its pairs
 // are kept as a list that every thread scans for its own cells.
@@ -644,7 +651,7 @@ OccPlan plan_occ(int32_t H, int64_t R) {
   p.cpt = H <= 1024 ? 4 : (H <= 2048 ? 8 : 16);
   p.log2W = 8 + (p.cpt == 4 ? 2 : (p.cpt == 8 ? 3 : 4));  // W = 256 threads x CPT
   p.T = static_cast<int>((static_cast<int64_t>(H) + (1 << p.log2W) - 1) >> p.log2W);
-  p.bucketed = p.T <= kMaxTiles && R <= 0x7fffffffLL;
+  p.bucketed = p.T <= kMaxTiles && R <= 0x7fffffffLL && R * p.T > kDirectReads;
   return p;
 }
 

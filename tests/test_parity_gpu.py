@@ -313,7 +313,11 @@ def test_occupancy_workloads(M, ws, oracle, name):
     assert np.array_equal(km, kmax_of(Ko))
 
 
-@pytest.mark.parametrize("D,H,per", [(2, 20000, 9000), (3, 3000, 4097)])
+@pytest.mark.parametrize("D,H,per", [(2, 20000, 9000), (3, 3000, 4097),
+                                     # 1,048,576 reads over all tiles exactly, and past
+                                     # them, bucketed
+                                     (16, 65536, 4096), (16, 65536, 4097), (2, 60001, 40000),
+                                     (3, 400000, 4097)])
 def test_occupancy_many_residents_per_decoder(M, ws, oracle, D, H, per):
     """More residents on one decoder than a block stages at once."""
     rng = np.random.default_rng(H + per)
@@ -397,6 +401,50 @@ def test_dispatch_snapshot_random(M, ws, oracle, D, H, J):
         assert (ho >= 0).any() and (ho < 0).any()  # both branches exercised
         if D >= 8:
             assert len(set(co.tolist())) > 1
+
+
+@pytest.mark.parametrize("D,H,J,unaligned", [
+    # the one-launch form at its limits and the bucketed form just past them:
+    # scores, scores times spans of the horizon, cells of K
+    (16, 2048, 8192, False), (16, 2048, 8193, False), (32, 9001, 2048, False),
+    (32, 9001, 2049, False), (1000, 1048, 60, False), (1000, 1049, 60, False),
+    (7, 32768, 300, False), (7, 32769, 300, False),
+    # summary rows of whole 16-byte words and not, at an aligned address and
+    # not; 32-decoder groups at their edges; one candidate
+    (31, 640, 100, True), (33, 1000, 1, False), (64, 64, 65, False), (1024, 100, 9, True),
+    # wide tiles of the bucketed form (few decoders, many candidates)
+    (5, 4099, 60000, False), (40, 4096, 9000, True)])
+def test_dispatch_snapshot_forms(M, ws, oracle, D, H, J, unaligned):
+    rng = np.random.default_rng(D * 37 + H + J)
+    off, p, g, U = random_residents(rng, D, H, 12)
+    _, K = oracle.p_occupancy(D, H, off, p, g, U)
+    cap = diverse_caps(rng, K, 4000)
+    Q = rng.integers(0, 4, D).astype(np.int32)
+    cp = rng.integers(0, 3000, J).astype(np.int32)
+    cb = rng.integers(0, H + 2, J).astype(np.int32)
+    cb[: min(J, 5)] = [0, 15, 16, 17, H][: min(J, 5)]
+    _, co, ho = oracle.p_dispatch_snapshot(D, H, K, cap, Q, cp, cb)
+    km = kmax_of(K)
+    shift = 1 if unaligned else 0
+    kd = torch.empty(km.size + shift, dtype=torch.int32, device="cuda")[shift:].view(*km.shape)
+    kd.copy_(torch.from_numpy(km.view(np.int32)))
+    Kd = torch.empty(K.size + shift, dtype=torch.int32, device="cuda")[shift:].view(*K.shape)
+    Kd.copy_(torch.from_numpy(K))
+    ch = torch.empty(J, dtype=torch.int32, device="cuda")
+    hr = torch.empty(J, dtype=torch.int64, device="cuda")
+    for summary in (kd, None):
+        assert M.maps_dispatch(0, D, H, 1, Kd, dev(cap), dev(Q), dev(cp), dev(cb), ch, hr,
+                               kmax=summary, ws=ws) == 0
+        assert M.maps_check(ws) == 0
+        assert np.array_equal(host(ch), co) and np.array_equal(host(hr), ho)
+    # a negative cell is reported: without a summary, and with one too in the
+    # one-launch form (the bucketed form reads only the candidates' tiles then)
+    one_launch = (J * D <= 2**17 and J * D * max(1, H // 2048) <= 2**18 and H <= 32768
+                  and D * H <= 2**20)
+    Kd[D - 1, H // 2] = -5
+    for summary in (kd, None) if one_launch else (None,):
+        M.maps_dispatch(0, D, H, 1, Kd, dev(cap), dev(Q), dev(cp), dev(cb), ch, hr, kmax=summary, ws=ws)
+        assert M.maps_check(ws) in (M.MAPS_E_RANGE, M.MAPS_E_INVALID)
 
 
 @pytest.mark.parametrize("name", ["tiny", "d16", "d64"])
