@@ -9,6 +9,7 @@ loads the library and fails loudly when it is missing.
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 
 import torch
@@ -113,21 +114,39 @@ EXPORTS = ("maps_version", "maps_last_cuda_error", "maps_check", "maps_set_dispa
            "maps_rr_pressure_workspace_size", "maps_rr_pressure")
 
 
-def _stream(stream) -> ctypes.c_void_p:
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+# A call's marshalling is on the path of every small call (a launch costs 2 to
+# 3 us, a step of four calls took 72 us on the host): addresses go to ctypes as
+# plain ints, the current stream comes from the one-word query, and a workspace
+# size, a pure function of the sizes asked for, is asked of the library once.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
-def _ptr(t, dtype=None) -> ctypes.c_void_p:
+def _stream(stream):
+    """Address of the cudaStream_t: the current stream's when None."""
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(torch.cuda.current_device())
+
+
+def _ptr(t, dtype=None):
+    """Device address of a contiguous CUDA tensor (None: a null pointer)."""
     if t is None:
-        return ctypes.c_void_p(0)
+        return None
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError("expected a CUDA tensor")
     if dtype is not None and t.dtype != dtype:
         raise TypeError(f"expected {dtype}, got {t.dtype}")
     if not t.is_contiguous():
         raise TypeError("expected a contiguous tensor")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
+
+
+_calibrate_ws = functools.lru_cache(256)(lib.maps_calibrate_workspace_size)
+_occupancy_ws = functools.lru_cache(256)(lib.maps_project_occupancy_workspace_size)
+_dispatch_ws = functools.lru_cache(256)(lib.maps_dispatch_workspace_size)
+_order_ws = functools.lru_cache(256)(lib.maps_order_local_workspace_size)
 
 
 class Workspace:
@@ -152,7 +171,7 @@ class Workspace:
 
 
 def maps_check(ws: Workspace, stream=None) -> int:
-    return lib.maps_check(ws.ptr, _stream(stream))
+    return lib.maps_check(ws.buf.data_ptr(), _stream(stream))
 
 
 def maps_set_dispatch_events(before=None, after=None) -> int:
@@ -171,12 +190,12 @@ def maps_calibrate(true_len, pred_len, alpha_ppm: int, query_pred=None, bound_ou
     n = true_len.numel()
     m = 0 if query_pred is None else query_pred.numel()
     ws = ws or Workspace()
-    ws.ensure(lib.maps_calibrate_workspace_size(n, m))
+    ws.ensure(_calibrate_ws(n, m))
     qh = ctypes.c_int32(0)
     st = lib.maps_calibrate(_ptr(true_len, torch.int32), _ptr(pred_len, torch.int32), n,
                             int(alpha_ppm), _ptr(query_pred, torch.int32), m,
                             _ptr(bound_out, torch.int32), _ptr(q_dev_out, torch.int32),
-                            ctypes.byref(qh) if q_host else None, ws.ptr, ws.nbytes,
+                            ctypes.byref(qh) if q_host else None, ws.buf.data_ptr(), ws.buf.numel(),
                             _stream(stream))
     return st, (int(qh.value) if q_host else None)
 
@@ -190,11 +209,11 @@ def maps_project_occupancy(D: int, H: int, res_off, prompt, gen, bound, K_out, k
                            ws: Workspace | None = None, stream=None) -> int:
     R = prompt.numel()
     ws = ws or Workspace()
-    ws.ensure(lib.maps_project_occupancy_workspace_size(D, H, R))
+    ws.ensure(_occupancy_ws(D, H, R))
     return lib.maps_project_occupancy(D, H, _ptr(res_off, torch.int64), R,
                                       _ptr(prompt, torch.int32), _ptr(gen, torch.int32),
                                       _ptr(bound, torch.int32), _ptr(K_out, torch.int32),
-                                      _ptr(kmax_out, torch.int32), ws.ptr, ws.nbytes,
+                                      _ptr(kmax_out, torch.int32), ws.buf.data_ptr(), ws.buf.numel(),
                                       _stream(stream))
 
 
@@ -204,14 +223,14 @@ def maps_dispatch(mode: int, D: int, H: int, S: int, K, cap, Q, cand_prompt, can
     J = cand_prompt.numel()
     R = 0 if prompt is None else prompt.numel()
     ws = ws or Workspace()
-    ws.ensure(lib.maps_dispatch_workspace_size(mode, D, H, J))
+    ws.ensure(_dispatch_ws(mode, D, H, J))
     return lib.maps_dispatch(mode, D, H, S, _ptr(K, torch.int32), _ptr(kmax, torch.int32),
                              _ptr(cap, torch.int32),
                              _ptr(Q, torch.int32), _ptr(res_off, torch.int64), R,
                              _ptr(prompt, torch.int32), _ptr(gen, torch.int32),
                              _ptr(bound, torch.int32), J, _ptr(cand_prompt, torch.int32),
                              _ptr(cand_bound, torch.int32), _ptr(choice_out, torch.int32),
-                             _ptr(headroom_out, torch.int64), ws.ptr, ws.nbytes,
+                             _ptr(headroom_out, torch.int64), ws.buf.data_ptr(), ws.buf.numel(),
                              _stream(stream))
 
 
@@ -219,11 +238,11 @@ def maps_order_local(D: int, dec, bound, wait, arrival, max_wait: int, perm_out,
                      ws: Workspace | None = None, stream=None) -> int:
     N = dec.numel()
     ws = ws or Workspace()
-    ws.ensure(lib.maps_order_local_workspace_size(N, D))
+    ws.ensure(_order_ws(N, D))
     return lib.maps_order_local(N, D, _ptr(dec, torch.int32), _ptr(bound, torch.int32),
                                 _ptr(wait, torch.int32), _ptr(arrival, torch.int32),
                                 int(max_wait), _ptr(perm_out, torch.int32),
-                                _ptr(seg_off_out, torch.int64), ws.ptr, ws.nbytes,
+                                _ptr(seg_off_out, torch.int64), ws.buf.data_ptr(), ws.buf.numel(),
                                 _stream(stream))
 
 
@@ -263,7 +282,7 @@ def maps_stream_run(cfg: StreamCfg, arrival_ms, prompt, true_len, pred, choice_o
                                _ptr(pred, torch.int32), _ptr(pred_delay, torch.int32),
                                _ptr(choice_out, torch.int32),
                                _ptr(q_out, torch.int32), _ptr(stats_out, torch.int64),
-                               _ptr(dec_stats_out, torch.int64), ws.ptr, ws.nbytes,
+                               _ptr(dec_stats_out, torch.int64), ws.buf.data_ptr(), ws.buf.numel(),
                                _stream(stream))
 
 
@@ -282,4 +301,4 @@ def maps_rr_pressure(N: int, C: int, t_tok_us: int, theta_ppm: int, arrival_us, 
                                 _ptr(prompt, torch.int32), _ptr(out_len, torch.int32),
                                 _ptr(admit_out, torch.int64), _ptr(done_out, torch.int64),
                                 _ptr(stats_out, torch.int64), _ptr(t_sim_out, torch.int64),
-                                ws.ptr, ws.nbytes, _stream(stream))
+                                ws.buf.data_ptr(), ws.buf.numel(), _stream(stream))
