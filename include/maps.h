@@ -21,7 +21,7 @@
  *           on it and return without waiting, except where a `_host` output
  *           is non-NULL: then the call synchronises the stream and returns
  *           the full status, data-dependent errors included.
- * Grids.    maps_calibrate with more than 8,192 residuals and
+ * Grids.    maps_calibrate with more than 16,384 residuals and
  *           maps_order_local past one block each launch one cooperative
  *           kernel (every block resident at once, with bounded grid
  *           barriers): such a launch starts when the multiprocessors it

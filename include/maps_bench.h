@@ -47,7 +47,7 @@ int maps_test_withhold_lookback(int32_t tile, uint32_t spin_limit);
 int maps_test_absent_block(int32_t block);
 
 /* Exercises the bounded grid barrier of maps_calibrate's cooperative kernel
- * (calibration sets above 8,192 residuals): on the current device, later
+ * (calibration sets above 16,384 residuals): on the current device, later
  * calls make block `block` of that kernel return at once, so the other
  * blocks' barrier gives up after `spin_limit` polls (0: the library default),
  * records MAPS_E_TIMEOUT (read with maps_check) and ends each block without

@@ -12,7 +12,7 @@
 //     scores inside the range.
 // A range of one value is q, so a quantile below 1,024 takes one pass and any
 // quantile at most three.
-// Calibration sets above 8,192 scores take one cooperative kernel: one block
+// Calibration sets above 16,384 scores take one cooperative kernel: one block
 // of 1,024 threads per multiprocessor, each thread holding up to eight scores
 // and eight of the queries' predictions in registers.  A pass adds the
 // blocks' shared histograms into a global one and waits at a bounded grid
@@ -59,6 +59,19 @@ __device__ __forceinline__ int first_bin(uint32_t s) {
   const int e = 31 - __clz(s);  // leading bit, 10..31
   return static_cast<int>(kExactBins) + ((e - 10) << kMantBits) +
          static_cast<int>((s >> (e - kMantBits)) & ((1u << kMantBits) - 1u));
+}
+
+// The range of scores that first-pass bin d covers: [lo, lo + 2^w).
+__device__ __forceinline__ void first_range(int d, uint32_t &lo, int &w) {
+  if (d < static_cast<int>(kExactBins)) {
+    lo = static_cast<uint32_t>(d);
+    w = 0;
+    return;
+  }
+  const int x = d - static_cast<int>(kExactBins), e = 10 + (x >> kMantBits);
+  const uint32_t top = (1u << kMantBits) | static_cast<uint32_t>(x & ((1 << kMantBits) - 1));
+  lo = top << (e - kMantBits);
+  w = e - kMantBits;
 }
 
 // Item u * 4 + c of thread t (of T in the grid) is element 4 (t + u T) + c:
@@ -206,24 +219,9 @@ calibrate_fused_kernel(const int32_t *__restrict__ L, const int32_t *__restrict_
         cum += c[j];
       }
       // the new range: the bin's values
-      uint32_t nlo;
-      int nw;
-      if (pass == 0) {
-        if (d < static_cast<int>(kExactBins)) {
-          nlo = static_cast<uint32_t>(d);
-          nw = 0;
-        } else {
-          const int e = 10 + ((d - static_cast<int>(kExactBins)) >> kMantBits);
-          const uint32_t top = (1u << kMantBits) |
-                               static_cast<uint32_t>((d - static_cast<int>(kExactBins)) &
-                                                     ((1 << kMantBits) - 1));
-          nlo = top << (e - kMantBits);
-          nw = e - kMantBits;
-        }
-      } else {
-        nlo = lo + (static_cast<uint32_t>(d) << shift);
-        nw = shift;
-      }
+      uint32_t nlo = lo + (static_cast<uint32_t>(d) << shift);
+      int nw = shift;
+      if (pass == 0) first_range(d, nlo, nw);
       s_lo = nlo;
       s_w = nw;
       s_k = k - cum;
@@ -322,104 +320,119 @@ bound_kernel(const int32_t *__restrict__ pred, int64_t m, const SelectState *st,
   if (bad) flag_error(status, MAPS_E_RANGE);
 }
 
-// Small calibration sets (n <= kSmallN): a three-digit (11, 11, 10 bits) radix select,
-// run by one block over the scores held in shared memory, then the bounds of
-// up to kSmallM queries by the same block: one launch instead of a memset and
-// four.
-constexpr int kSmallN = 8192;
-constexpr int kSmallM = 8192;
+// Small calibration sets (n <= kSmallN): the same select in one block, scores
+// in registers, then the bounds of up to kSmallM queries: one
+// launch without a memset or a grid barrier.  A chain of latencies: loads, the
+// block's histogram, its scan (the bins' totals by warp shuffles, the warps' by
+// one reduction), the bounds.  Replayed calls: 1,000 scores and 288 bounds 4.7 us
+// (sorted by a bitonic network: 10.1), 2,000 and 1,000 5.0 (17.2), 8,000 and
+// 8,000 6.5 (three fixed digits: 6.8); 10,007 and 9,165 6.9 (the cooperative
+// kernel: 10.0), 16,384 and 16,384 8.3 (9.6).
+constexpr int kSmallItems = 16;  // scores a thread keeps
+constexpr int kSmallHold = 8;    // predictions loaded before the select
 constexpr int kSmallThreads = 1024;
-constexpr int kBitonicN = 2048;  // up to this many scores are sorted outright
-constexpr int kSmallBins = 2 * kSmallThreads;  // 11-bit digits, two bins per thread
+constexpr int kSmallN = kSmallItems * kSmallThreads;
+constexpr int kSmallM = kSmallItems * kSmallThreads;
+static_assert(kBins == 4 * kSmallThreads, "four bins a thread");
 
 __global__ void __launch_bounds__(kSmallThreads)
 select_small_kernel(const int32_t *__restrict__ L, const int32_t *__restrict__ P, int n,
-                    unsigned long long k, const int32_t *__restrict__ pred, int m_inblock,
+                    uint32_t k, const int32_t *__restrict__ pred, int m_inblock,
                     int32_t *__restrict__ out, SelectState *st, int32_t *q_dev_out,
                     int32_t *status) {
   pdl_prologue();
-  extern __shared__ uint32_t s[];  // the scores (kBitonicN or kSmallN words, as launched)
-  __shared__ uint32_t hist[kSmallBins];
+  __shared__ __align__(16) uint32_t hist[kBins];
   __shared__ uint32_t s_warp[kSmallThreads / 32];
-  __shared__ uint32_t s_pick[2];  // the chosen bin, the rank left inside it
+  __shared__ uint32_t s_lo, s_k;
+  __shared__ int s_w;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int i = tid; i < n; i += kSmallThreads) s[i] = score(__ldg(L + i), __ldg(P + i));
-  uint32_t prefix = 0;
-  if (n <= kBitonicN) {
-    // few scores: sort them (bitonic network, padded to a power of two with
-    // the largest value) and take the k-th smallest
-    int Pn = 1;
-    while (Pn < n) Pn <<= 1;
-    for (int i = n + tid; i < Pn; i += kSmallThreads) s[i] = 0xffffffffu;
-    __syncthreads();
-    for (int kk = 2; kk <= Pn; kk <<= 1)
-      for (int j = kk >> 1; j > 0; j >>= 1) {
-        for (int i = tid; i < Pn; i += kSmallThreads) {
-          const int l = i ^ j;
-          if (l > i) {
-            const uint32_t x = s[i], y = s[l];
-            if ((x > y) == ((i & kk) == 0)) {
-              s[i] = y;
-              s[l] = x;
-            }
-          }
-        }
-        __syncthreads();
-      }
-    prefix = s[k - 1];
-  } else {
-    unsigned long long kr = k;  // rank still to find among the scores matching prefix
-    for (int pass = 0; pass < kPasses; ++pass) {
-      const int shift = pass == 0 ? 21 : (pass == 1 ? 10 : 0);
-      const int bits = pass == 2 ? 10 : 11;
-      const int prev = pass == 0 ? 32 : (pass == 1 ? 21 : 10);  // bits above this digit
-      for (int b = tid; b < kSmallBins; b += kSmallThreads) hist[b] = 0;
-      __syncthreads();
-      for (int i = tid; i < n; i += kSmallThreads) {
-        const uint32_t v = s[i];
-        if (prev == 32 || (v >> prev) == prefix) atomicAdd(&hist[(v >> shift) & ((1u << bits) - 1)], 1u);
-      }
-      __syncthreads();
-      // exclusive scan of the bins (two per thread), then the bin holding rank kr
-      const uint32_t c0 = hist[2 * tid], c1 = hist[2 * tid + 1];
-      const uint32_t tot = c0 + c1;
-      uint32_t incl = tot;
-  #pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, off);
-        if (lane >= off) incl += y;
-      }
-      if (lane == 31) s_warp[warp] = incl;
-      __syncthreads();
-      uint32_t excl = incl - tot;
-      for (int w = 0; w < warp; ++w) excl += s_warp[w];
-      if (excl < kr && kr <= static_cast<unsigned long long>(excl) + tot) {
-        const bool first = kr <= static_cast<unsigned long long>(excl) + c0;
-        s_pick[0] = 2 * tid + (first ? 0 : 1);
-        s_pick[1] = static_cast<uint32_t>(kr - excl - (first ? 0 : c0));
-      }
-      __syncthreads();
-      prefix = (prefix << bits) | s_pick[0];
-      kr = s_pick[1];
-      __syncthreads();  // hist and s_pick are reused by the next pass
-    }
+  uint32_t sv[kSmallItems];
+  int32_t pv[kSmallHold];
+#pragma unroll
+  for (int i = 0; i < kSmallItems; ++i) {
+    const int x = i * kSmallThreads + tid;
+    sv[i] = x < n ? score(__ldg(L + x), __ldg(P + x)) : 0u;
   }
-  if (prefix > 0x7fffffffu) {
+#pragma unroll
+  for (int i = 0; i < kSmallHold; ++i) {
+    const int x = i * kSmallThreads + tid;
+    pv[i] = x < m_inblock ? __ldg(pred + x) : 0;
+  }
+  uint32_t lo = 0;
+  int w = 32;
+  for (int pass = 0; pass < kPasses && w > 0; ++pass) {
+    const int shift = w > kStepBits ? w - kStepBits : 0;
+    reinterpret_cast<uint4 *>(hist)[tid] = make_uint4(0, 0, 0, 0);
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kSmallItems; ++i) {
+      if (i * kSmallThreads >= n) break;
+      const bool valid = i * kSmallThreads + tid < n;
+      if (pass == 0) {  // zero scores by one ballot a warp, the others alone
+        const int d = first_bin(sv[i]);
+        const unsigned zeros = __ballot_sync(0xffffffffu, valid && d == 0);
+        if (zeros && lane == __ffs(zeros) - 1) atomicAdd(&hist[0], static_cast<uint32_t>(__popc(zeros)));
+        if (valid && d > 0) atomicAdd(&hist[d], 1u);
+      } else {  // the scores inside the range, w <= 24 here; equal bins together
+        const uint32_t r = sv[i] - lo;
+        const int d = valid && sv[i] >= lo && r < (1u << w) ? static_cast<int>(r >> shift) : -1;
+        const unsigned peers = __match_any_sync(0xffffffffu, d);
+        if (d >= 0 && lane == __ffs(peers) - 1) atomicAdd(&hist[d], static_cast<uint32_t>(__popc(peers)));
+      }
+    }
+    __syncthreads();
+    const uint4 c = reinterpret_cast<const uint4 *>(hist)[tid];
+    const uint32_t tot = c.x + c.y + c.z + c.w;
+    uint32_t incl = tot;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, incl, off);
+      if (lane >= off) incl += y;
+    }
+    if (lane == 31) s_warp[warp] = incl;
+    __syncthreads();
+    uint32_t cum = __reduce_add_sync(0xffffffffu, lane < warp ? s_warp[lane] : 0u) + incl - tot;
+    if (cum < k && k <= cum + tot) {  // the bin holding rank k is one of this thread's
+      int d = 4 * tid;
+      if (k > cum + c.x) {
+        cum += c.x, ++d;
+        if (k > cum + c.y) {
+          cum += c.y, ++d;
+          if (k > cum + c.z) cum += c.z, ++d;
+        }
+      }
+      uint32_t nlo = lo + (static_cast<uint32_t>(d) << shift);
+      int nw = shift;
+      if (pass == 0) first_range(d, nlo, nw);
+      s_lo = nlo;
+      s_w = nw;
+      s_k = k - cum;
+    }
+    __syncthreads();
+    lo = s_lo;
+    w = s_w;
+    k = s_k;
+  }
+  if (lo > 0x7fffffffu) {
     if (tid == 0) flag_error(status, MAPS_E_RANGE);
     return;
   }
-  const int32_t q = static_cast<int32_t>(prefix);
+  const int32_t q = static_cast<int32_t>(lo);
   if (tid == 0) {
     st->q = q;
     if (q_dev_out) *q_dev_out = q;
   }
   bool bad = false;
-  for (int i = tid; i < m_inblock; i += kSmallThreads) {
-    const long long u = static_cast<long long>(__ldg(pred + i)) + q;  // Eq. (conformal_upper)
-    bad |= u > 0x7fffffffLL;
-    out[i] = static_cast<int32_t>(u > 0x7fffffffLL ? 0x7fffffffLL : u);
+#pragma unroll
+  for (int i = 0; i < kSmallItems; ++i) {
+    const int x = i * kSmallThreads + tid;
+    if (x < m_inblock) {
+      const long long u = static_cast<long long>(i < kSmallHold ? pv[i % kSmallHold] : __ldg(pred + x)) + q;
+      bad |= u > 0x7fffffffLL;  // Eq. (conformal_upper)
+      out[x] = static_cast<int32_t>(u > 0x7fffffffLL ? 0x7fffffffLL : u);
+    }
   }
-  if (__syncthreads_or(bad) && tid == 0) flag_error(status, MAPS_E_RANGE);
+  if (bad) flag_error(status, MAPS_E_RANGE);
 }
 
 // Blocks of the fused kernel that can be resident at once (its grid limit as
@@ -471,10 +484,8 @@ int maps_calibrate(const int32_t *true_len, const int32_t *pred_len, int64_t n,
   const unsigned long long kk = static_cast<unsigned long long>(k);
   if (n <= kSmallN) {
     const int mi = m <= kSmallM ? static_cast<int>(m) : 0;  // bounds in the same block
-    launch_pdl(select_small_kernel, 1, kSmallThreads,
-               (n <= kBitonicN ? kBitonicN : kSmallN) * sizeof(uint32_t), s, true_len, pred_len,
-               static_cast<int>(n),
-               kk, query_pred, mi, bound_out, st, q_dev_out, status);
+    launch_pdl(select_small_kernel, 1, kSmallThreads, 0, s, true_len, pred_len, static_cast<int>(n),
+               static_cast<uint32_t>(k), query_pred, mi, bound_out, st, q_dev_out, status);
     MAPS_TRY(launch_ok());
     if (m <= kSmallM) m = 0;
   } else {

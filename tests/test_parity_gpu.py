@@ -228,7 +228,11 @@ def test_calibrate_grid_bucket_edges(M, ws, oracle, seed):
     # more predictions than the grid keeps in registers, at an unaligned address
     (20011, 1300003, 1),
     # just past the one-block limit, no queries; then a ragged, unaligned few
-    (8193, 0, 0), (10001, 777, 1)])
+    (8193, 0, 0), (10001, 777, 1),
+    # the one-block form at 16,384 residuals and queries, and past each limit;
+    # a thread's last items, and queries past those loaded before the select
+    (16384, 16384, 0), (16384, 16385, 1), (16385, 0, 0), (16385, 777, 1), (1024, 8193, 1),
+    (1025, 1, 0), (15361, 9000, 0)])
 def test_calibrate_fused_register_limits(M, ws, oracle, n, m, shift):
     """Calibration sets above the one-block limit take one cooperative kernel;
     its scores and predictions live in registers up to eight per thread, else
@@ -1011,6 +1015,8 @@ def test_stream_golden(M, ws, stream_golden):
     # a window of 10,000 completions: once it holds more than 8,192 the quantile is
     # taken by the cooperative calibration kernel inside the loop
     (30000, 8, 16384, 262144, 512, 10000, 100000, 1000),
+    # and one of 17,000, past the one-block calibration
+    (40000, 8, 16384, 262144, 512, 17000, 100000, 1000),
 ])
 def test_stream_prefix(M, ws, oracle, N, D, H, cap, B, Wn, a, mw):
     w = W.make_stream(n_requests=N)
