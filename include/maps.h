@@ -358,9 +358,10 @@ int maps_order_local_static(int64_t N, int32_t D, const int32_t *dec,
  *                       admission happens at dispatch steps only), the
  *                       batches after whose advance its running requests
  *                       exceed capacity, its admissions, its preemptions.
- * The call runs the whole loop: it synchronises the stream once per batch
- * (to read the request counts that size the next launches) and at the end,
- * and returns the full status.  A negative length or decreasing arrival is
+ * The call runs the whole loop: it synchronises the stream once per batch, or
+ * once per 256 batches while the system fits one block (to read the request
+ * counts that size the next launches), and at the end, and returns the full
+ * status.  A negative length or decreasing arrival is
  * MAPS_E_RANGE before any batch runs.
  * ---------------------------------------------------------------------- */
 typedef struct {

@@ -117,6 +117,42 @@ __device__ __forceinline__ void pdl_prologue() {
 }
 
 // ---------------------------------------------------------------------------
+// Calibration scores and the bins of the select's passes (Sec. 3.2): shared by
+// maps_calibrate and the streaming loop's own quantile.
+// ---------------------------------------------------------------------------
+constexpr int kBins = 4096;
+constexpr uint32_t kExactBins = 1024;  // scores below this have a bin each
+constexpr int kMantBits = 7;           // bits after the leading one, first pass
+constexpr int kStepBits = 12;          // bits per later pass
+
+// One-sided score max(0, L - P): fits 32 bits unsigned.
+__device__ __forceinline__ uint32_t score(int32_t L, int32_t P) {
+  long long d = static_cast<long long>(L) - static_cast<long long>(P);
+  return d > 0 ? static_cast<uint32_t>(d) : 0u;
+}
+
+// First-pass bin: non-decreasing in s, at most 1024 + 22 * 128 = 3,840 bins.
+__device__ __forceinline__ int first_bin(uint32_t s) {
+  if (s < kExactBins) return static_cast<int>(s);
+  const int e = 31 - __clz(s);  // leading bit, 10..31
+  return static_cast<int>(kExactBins) + ((e - 10) << kMantBits) +
+         static_cast<int>((s >> (e - kMantBits)) & ((1u << kMantBits) - 1u));
+}
+
+// The range of scores that first-pass bin d covers: [lo, lo + 2^w).
+__device__ __forceinline__ void first_range(int d, uint32_t &lo, int &w) {
+  if (d < static_cast<int>(kExactBins)) {
+    lo = static_cast<uint32_t>(d);
+    w = 0;
+    return;
+  }
+  const int x = d - static_cast<int>(kExactBins), e = 10 + (x >> kMantBits);
+  const uint32_t top = (1u << kMantBits) | static_cast<uint32_t>(x & ((1 << kMantBits) - 1));
+  lo = top << (e - kMantBits);
+  w = e - kMantBits;
+}
+
+// ---------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------
 void set_last_cuda_error(cudaError_t e);

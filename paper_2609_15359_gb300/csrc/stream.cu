@@ -53,6 +53,8 @@ struct StreamState {
   int32_t nto;       // deferral: requests timed out to round robin at this step
   int32_t adm_i;     // per-step mode: admissions between the dispatch steps
   int32_t pad;
+  long long next_b;      // the one-block loop: the batch it stopped before
+  long long total_done;  // completions by then
 };
 
 // Exclusive position of a 0/1 flag across the block (kSt threads) and the
@@ -100,6 +102,8 @@ __global__ void stream_init_kernel(int64_t first_hi, int D, int32_t cap, const i
     S->nc = 0;
     S->nto = 0;
     S->adm_i = 0;
+    S->next_b = 0;
+    S->total_done = 0;
   }
 }
 
@@ -107,13 +111,12 @@ __global__ void stream_init_kernel(int64_t first_hi, int D, int32_t cap, const i
 //    occupancy = p + g of the running requests (the over-capacity count);
 //    used = what admission counts for them: p + g, p + max(U*, g) (staged)
 //    or 2p + max(U*, g) (held), U* the bound reserved at admission.
-__global__ void __launch_bounds__(kSt, 1)
-stream_advance_kernel(int64_t hi, int D, int32_t cap, int acct, int per_step, const int64_t *arrival,
-                      const int32_t *prompt, const int32_t *true_len, const int32_t *res_u,
-                      uint8_t *st, int32_t *g, const int32_t *dec, const int32_t *act_in,
-                      int32_t *act_out, int32_t *done_id, int32_t *done_rem, long long *used,
-                      StreamState *S, int64_t *stats_b, int64_t *dst) {
-  pdl_prologue();
+__device__ void
+advance_block(int64_t hi, int D, int32_t cap, int acct, int per_step, const int64_t *arrival,
+              const int32_t *prompt, const int32_t *true_len, const int32_t *res_u,
+              uint8_t *st, int32_t *g, const int32_t *dec, const int32_t *act_in,
+              int32_t *act_out, int32_t *done_id, int32_t *done_rem, long long *used,
+              StreamState *S, int64_t *stats_b, int64_t *dst) {
   __shared__ unsigned long long s_occ[kStreamMaxD], s_used[kStreamMaxD];
   __shared__ int s_w[kStWarps];
   __shared__ int s_nwait;
@@ -182,6 +185,16 @@ stream_advance_kernel(int64_t hi, int D, int32_t cap, int acct, int per_step, co
     stats_b[3] = over;
   }
 }
+__global__ void __launch_bounds__(kSt, 1)
+stream_advance_kernel(int64_t hi, int D, int32_t cap, int acct, int per_step, const int64_t *arrival,
+                      const int32_t *prompt, const int32_t *true_len, const int32_t *res_u,
+                      uint8_t *st, int32_t *g, const int32_t *dec, const int32_t *act_in,
+                      int32_t *act_out, int32_t *done_id, int32_t *done_rem, long long *used,
+                      StreamState *S, int64_t *stats_b, int64_t *dst) {
+  pdl_prologue();
+  advance_block(hi, D, cap, acct, per_step, arrival, prompt, true_len, res_u, st, g, dec, act_in,
+                act_out, done_id, done_rem, used, S, stats_b, dst);
+}
 
 // 1'. Per-step mode: the steps prev_s + 1 .. s, one warp per decoder
 //     (decoders do not interact between dispatch steps).  Each decoder holds
@@ -198,16 +211,15 @@ stream_advance_kernel(int64_t hi, int D, int32_t cap, int acct, int per_step, co
 //     grows and nothing is freed since the head last failed), so the warp
 //     jumps to the next step with a completion or a preemption, or to s.
 //     Every iteration advances the step, so the loop ends.
-__global__ void __launch_bounds__(kSt, 1)
-stream_interval_kernel(int64_t hi, int D, int32_t cap, int acct, const int64_t *arrival,
-                       const int32_t *prompt, const int32_t *true_len, const int32_t *U,
-                       int32_t *res_u, uint8_t *st, int32_t *g, const int32_t *dec,
-                       const int32_t *act, const int32_t *wid, const int32_t *wperm,
-                       const int64_t *wseg, const int64_t *qhead, long long *aseq,
-                       long long *dseq, int32_t *rbuf, int32_t *sbuf, int32_t *done_id,
-                       int32_t *done_rem, StreamState *S, int64_t *dst) {
-  pdl_prologue();
-  __shared__ int s_cnt[kStreamMaxD], s_run[kStreamMaxD], s_cur[kStreamMaxD];
+__device__ void
+interval_block(int32_t *scratch, int64_t hi, int D, int32_t cap, int acct, const int64_t *arrival,
+               const int32_t *prompt, const int32_t *true_len, const int32_t *U,
+               int32_t *res_u, uint8_t *st, int32_t *g, const int32_t *dec,
+               const int32_t *act, const int32_t *wid, const int32_t *wperm,
+               const int64_t *wseg, const int64_t *qhead, long long *aseq,
+               long long *dseq, int32_t *rbuf, int32_t *sbuf, int32_t *done_id,
+               int32_t *done_rem, StreamState *S, int64_t *dst) {
+  int32_t *s_cnt = scratch, *s_run = scratch + kStreamMaxD, *s_cur = scratch + 2 * kStreamMaxD;
   __shared__ int s_w[kStWarps];
   __shared__ int s_done, s_adm;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -402,17 +414,29 @@ stream_interval_kernel(int64_t hi, int D, int32_t cap, int acct, const int64_t *
     S->prev_s = s;  // the advance that follows moves nobody
   }
 }
+__global__ void __launch_bounds__(kSt, 1)
+stream_interval_kernel(int64_t hi, int D, int32_t cap, int acct, const int64_t *arrival,
+                       const int32_t *prompt, const int32_t *true_len, const int32_t *U,
+                       int32_t *res_u, uint8_t *st, int32_t *g, const int32_t *dec,
+                       const int32_t *act, const int32_t *wid, const int32_t *wperm,
+                       const int64_t *wseg, const int64_t *qhead, long long *aseq,
+                       long long *dseq, int32_t *rbuf, int32_t *sbuf, int32_t *done_id,
+                       int32_t *done_rem, StreamState *S, int64_t *dst) {
+  pdl_prologue();
+  __shared__ int32_t scratch[3 * kStreamMaxD];
+  interval_block(scratch, hi, D, cap, acct, arrival, prompt, true_len, U, res_u, st, g, dec, act, wid,
+                 wperm, wseg, qhead, aseq, dseq, rbuf, sbuf, done_id, done_rem, S, dst);
+}
 
 // Deferral: the requests arrived but not dispatched, then the batch, in index
 // order, split three ways (stable): a bound available by s (the arrival plus
 // the prediction delay) -> the dispatch policy; waited beta steps past
 // arrival without one, or the last dispatch step -> round robin; otherwise
 // they keep waiting for the next dispatch step.
-__global__ void __launch_bounds__(kSt, 1)
-stream_select_kernel(int64_t lo, int nb, int64_t hi, int32_t beta, int last, const int64_t *arrival,
-                     const int32_t *pred_delay, const int32_t *pend_in, int32_t *pend_out,
-                     int32_t *cid, int32_t *tout, StreamState *S) {
-  pdl_prologue();
+__device__ void
+select_block(int64_t lo, int nb, int64_t hi, int32_t beta, int last, const int64_t *arrival,
+             const int32_t *pred_delay, const int32_t *pend_in, int32_t *pend_out,
+             int32_t *cid, int32_t *tout, StreamState *S) {
   __shared__ int s_w[kStWarps];
   const long long s = arrival[hi - 1];
   const int np = S->npend, n = np + nb;
@@ -443,6 +467,13 @@ stream_select_kernel(int64_t lo, int nb, int64_t hi, int32_t beta, int last, con
     S->nto = nt;
     S->npend = nk;
   }
+}
+__global__ void __launch_bounds__(kSt, 1)
+stream_select_kernel(int64_t lo, int nb, int64_t hi, int32_t beta, int last, const int64_t *arrival,
+                     const int32_t *pred_delay, const int32_t *pend_in, int32_t *pend_out,
+                     int32_t *cid, int32_t *tout, StreamState *S) {
+  pdl_prologue();
+  select_block(lo, nb, hi, beta, last, arrival, pred_delay, pend_in, pend_out, cid, tout, S);
 }
 
 // 2. Completions, sorted by (step, id), enter the ring of the last Wn; the
@@ -497,9 +528,7 @@ __global__ void stream_rr_kernel(int n, int nb, int64_t lo, int D, int set_u, co
 //     ties to the lowest index.  Lane l keeps the counts of decoders l, l + 32,
 //     ... in shared memory; per candidate two warp minima give the smallest
 //     count and then the lowest decoder holding it.
-__global__ void stream_lr_kernel(int D, int nb, const int64_t *res_off, int32_t *choice) {
-  pdl_prologue();
-  __shared__ uint32_t s_c[kStreamMaxD];
+__device__ void lr_warp(uint32_t *s_c, int D, int nb, const int64_t *res_off, int32_t *choice) {
   const int lane = threadIdx.x;
   for (int k = lane; k < D; k += 32) s_c[k] = static_cast<uint32_t>(res_off[k + 1] - res_off[k]);
   __syncwarp();
@@ -519,18 +548,22 @@ __global__ void stream_lr_kernel(int D, int nb, const int64_t *res_off, int32_t 
     __syncwarp();
   }
 }
+__global__ void stream_lr_kernel(int D, int nb, const int64_t *res_off, int32_t *choice) {
+  pdl_prologue();
+  __shared__ uint32_t s_c[kStreamMaxD];
+  lr_warp(s_c, D, nb, res_off, choice);
+}
 
 // 4. Residents by decoder (running with g, waiting with g = 0) and the
 //    waiting count per decoder; new bounds of the requests in the system.
-__global__ void __launch_bounds__(kSt, 1)
 //    Under deferral a request whose prediction is not in by s (arrival +
 //    delay > s) is bounded by the horizon H.
-stream_csr_kernel(int nact, int D, int rr, const int32_t *q_dev, int32_t *q_out_b,
-                  const int32_t *act, const uint8_t *st, const int32_t *g, const int32_t *dec,
-                  const int32_t *prompt, int32_t *Uq, int32_t *U, int64_t *res_off,
-                  int32_t *rp, int32_t *rg, int32_t *rU, int32_t *Q, const int64_t *arrival,
-                  const int32_t *pred_delay, int64_t hi, int32_t H) {
-  pdl_prologue();
+__device__ void
+csr_block(int32_t *scratch, int nact, int D, int rr, const int32_t *q_dev, int32_t *q_out_b,
+          const int32_t *act, const uint8_t *st, const int32_t *g, const int32_t *dec,
+          const int32_t *prompt, int32_t *Uq, int32_t *U, int64_t *res_off,
+          int32_t *rp, int32_t *rg, int32_t *rU, int32_t *Q, const int64_t *arrival,
+          const int32_t *pred_delay, int64_t hi, int32_t H) {
   if (pred_delay != nullptr) {  // before anything reads Uq
     const long long s = arrival[hi - 1];
     for (int x = threadIdx.x; x < nact; x += kSt) {
@@ -539,7 +572,7 @@ stream_csr_kernel(int nact, int D, int rr, const int32_t *q_dev, int32_t *q_out_
     }
     __syncthreads();
   }
-  __shared__ int s_cnt[kStreamMaxD], s_q[kStreamMaxD], s_cur[kStreamMaxD];
+  int32_t *s_cnt = scratch, *s_q = scratch + kStreamMaxD, *s_cur = scratch + 2 * kStreamMaxD;
   __shared__ int s_w[kStWarps];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int k = tid; k < D; k += kSt) s_cnt[k] = s_q[k] = 0;
@@ -579,6 +612,17 @@ stream_csr_kernel(int nact, int D, int rr, const int32_t *q_dev, int32_t *q_out_
   }
   if (tid == 0) *q_out_b = rr ? -1 : q_dev[0];
 }
+__global__ void __launch_bounds__(kSt, 1)
+stream_csr_kernel(int nact, int D, int rr, const int32_t *q_dev, int32_t *q_out_b,
+                  const int32_t *act, const uint8_t *st, const int32_t *g, const int32_t *dec,
+                  const int32_t *prompt, int32_t *Uq, int32_t *U, int64_t *res_off,
+                  int32_t *rp, int32_t *rg, int32_t *rU, int32_t *Q, const int64_t *arrival,
+                  const int32_t *pred_delay, int64_t hi, int32_t H) {
+  pdl_prologue();
+  __shared__ int32_t scratch[3 * kStreamMaxD];
+  csr_block(scratch, nact, D, rr, q_dev, q_out_b, act, st, g, dec, prompt, Uq, U, res_off, rp, rg, rU, Q,
+            arrival, pred_delay, hi, H);
+}
 
 // 5. (shared-memory form) SEQUENTIAL dispatch of the batch without a dense K.
 // Decoder k's occupancy is held as its residents' pairs (e, b), sorted by e:
@@ -616,7 +660,7 @@ __device__ __forceinline__ unsigned long long dispatch_key(long long h, int q, i
   return (feas ? 0ull : 1ull << 63) | (v << 10) | static_cast<unsigned>(k);
 }
 
-size_t stream_dispatch_smem(int D, int nact, int nb) {
+__host__ __device__ size_t stream_dispatch_smem(int D, int nact, int nb) {
   const size_t pool = static_cast<size_t>(nact) + static_cast<size_t>(D) * nb;
   return 16 * pool + 8 * static_cast<size_t>(nact) + 16 * static_cast<size_t>(D) +
          12 * static_cast<size_t>(nb) + 64;
@@ -857,13 +901,11 @@ __device__ bool walk_registers(int D, int nb, int mc, const int32_t *uE, const i
   return ok;
 }
 
-__global__ void __launch_bounds__(kSt, 1)
-stream_dispatch_kernel(int D, int H, int nb, int mc, const int64_t *res_off, const int32_t *rp,
-                       const int32_t *rg, const int32_t *rU, const int32_t *capv, int32_t *Q,
-                       const int32_t *cp, const int32_t *cU, int32_t *choice, int64_t *headroom,
-                       int32_t *status) {
-  pdl_prologue();
-  extern __shared__ __align__(16) unsigned char sdm[];
+__device__ void
+dispatch_block(unsigned char *sdm, int D, int H, int nb, int mc, const int64_t *res_off,
+               const int32_t *rp, const int32_t *rg, const int32_t *rU, const int32_t *capv,
+               int32_t *Q, const int32_t *cp, const int32_t *cU, int32_t *choice,
+               int64_t *headroom, int32_t *status) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nact = static_cast<int>(res_off[D]);
   const int pool = nact + D * nb;
@@ -1253,17 +1295,23 @@ stream_dispatch_kernel(int D, int H, int nb, int mc, const int64_t *res_off, con
   __syncthreads();
   for (int k = tid; k < D; k += kSt) Q[k] = s_q[k];
 }
+__global__ void __launch_bounds__(kSt, 1)
+stream_dispatch_kernel(int D, int H, int nb, int mc, const int64_t *res_off, const int32_t *rp,
+                       const int32_t *rg, const int32_t *rU, const int32_t *capv, int32_t *Q,
+                       const int32_t *cp, const int32_t *cU, int32_t *choice, int64_t *headroom,
+                       int32_t *status) {
+  pdl_prologue();
+  extern __shared__ __align__(16) unsigned char sdm[];
+  dispatch_block(sdm, D, H, nb, mc, res_off, rp, rg, rU, capv, Q, cp, cU, choice, headroom, status);
+}
 
 // 5''. Deferral: the listed requests join the waiting queues at act[nact..]:
 //      with choices cch (and bounds Uq[nact + i]), or, with cch null, round
 //      robin with the horizon as their bound (timed out without one).
-__global__ void stream_enqueue_list_kernel(int n, int nact, int D, int32_t H, int64_t hi,
-                                           const int64_t *arrival, const int32_t *ids,
-                                           const int32_t *cch, const int32_t *Uq,
-                                           int32_t *choice_out, uint8_t *st, int32_t *dec,
-                                           long long *disp, int32_t *g, int32_t *U, int32_t *act,
-                                           StreamState *S, int32_t *status) {
-  pdl_prologue();
+__device__ void enqueue_list(int n, int nact, int D, int32_t H, int64_t hi, const int64_t *arrival,
+                             const int32_t *ids, const int32_t *cch, const int32_t *Uq,
+                             int32_t *choice_out, uint8_t *st, int32_t *dec, long long *disp,
+                             int32_t *g, int32_t *U, int32_t *act, StreamState *S, int32_t *status) {
   const long long s = arrival[hi - 1];
   const int stride = gridDim.x * blockDim.x;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
@@ -1283,14 +1331,21 @@ __global__ void stream_enqueue_list_kernel(int n, int nact, int D, int32_t H, in
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) S->nact = nact + n;
 }
+__global__ void stream_enqueue_list_kernel(int n, int nact, int D, int32_t H, int64_t hi,
+                                           const int64_t *arrival, const int32_t *ids,
+                                           const int32_t *cch, const int32_t *Uq,
+                                           int32_t *choice_out, uint8_t *st, int32_t *dec,
+                                           long long *disp, int32_t *g, int32_t *U, int32_t *act,
+                                           StreamState *S, int32_t *status) {
+  pdl_prologue();
+  enqueue_list(n, nact, D, H, hi, arrival, ids, cch, Uq, choice_out, st, dec, disp, g, U, act, S, status);
+}
 
 // 6. The batch joins the waiting queues of its decoders.
-__global__ void stream_enqueue_kernel(int64_t lo, int nb, int nact, int64_t hi, int D,
-                                      const int64_t *arrival, const int32_t *choice,
-                                      const int32_t *Uq, uint8_t *st, int32_t *dec,
-                                      long long *disp, int32_t *g, int32_t *U, int32_t *act,
-                                      StreamState *S, int32_t *status) {
-  pdl_prologue();
+__device__ void enqueue_batch(int64_t lo, int nb, int nact, int64_t hi, int D, const int64_t *arrival,
+                              const int32_t *choice, const int32_t *Uq, uint8_t *st, int32_t *dec,
+                              long long *disp, int32_t *g, int32_t *U, int32_t *act,
+                              StreamState *S, int32_t *status) {
   const long long s = arrival[hi - 1];
   const int stride = gridDim.x * blockDim.x;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nb; i += stride) {
@@ -1308,6 +1363,14 @@ __global__ void stream_enqueue_kernel(int64_t lo, int nb, int nact, int64_t hi, 
     act[nact + i] = static_cast<int32_t>(id);
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) S->nact = nact + nb;
+}
+__global__ void stream_enqueue_kernel(int64_t lo, int nb, int nact, int64_t hi, int D,
+                                      const int64_t *arrival, const int32_t *choice,
+                                      const int32_t *Uq, uint8_t *st, int32_t *dec,
+                                      long long *disp, int32_t *g, int32_t *U, int32_t *act,
+                                      StreamState *S, int32_t *status) {
+  pdl_prologue();
+  enqueue_batch(lo, nb, nact, hi, D, arrival, choice, Uq, st, dec, disp, g, U, act, S, status);
 }
 
 // 7. The waiting requests with their order keys.
@@ -1344,17 +1407,15 @@ stream_waitlist_kernel(int n, int64_t hi, const int64_t *arrival, const int32_t 
 //    entries admitted before) + p + U <= cap, the increment being p, p + U
 //    (staged) or 2p + U (held).  Each decoder's statistics gain its queue
 //    left waiting times the steps to the next batch, and its admissions.
-__global__ void __launch_bounds__(kSt, 1)
 //    Per-step mode: each admission's sequence number (aseq), the queue's
 //    first entry left (qhead), and the waiting requests count for the
 //    dispatch step alone (the steps after it are the next interval's).
-stream_admit_kernel(int D, int32_t cap, int acct, int per_step, int nw, int64_t hi, int64_t hi_next,
-                    const int64_t *arrival, const int64_t *wseg, const int32_t *wperm,
-                    const int32_t *wid, const int32_t *prompt, const int32_t *U,
-                    const long long *used, uint8_t *st, int32_t *g, int32_t *res_u,
-                    long long *aseq, long long *dseq, int64_t *qhead, const StreamState *S,
-                    int64_t *stats_b, int64_t *dst) {
-  pdl_prologue();
+__device__ void
+admit_block(int D, int32_t cap, int acct, int per_step, int nw, int64_t hi, int64_t hi_next,
+            const int64_t *arrival, const int64_t *wseg, const int32_t *wperm, const int32_t *wid,
+            const int32_t *prompt, const int32_t *U, const long long *used, uint8_t *st, int32_t *g,
+            int32_t *res_u, long long *aseq, long long *dseq, int64_t *qhead, const StreamState *S,
+            int64_t *stats_b, int64_t *dst) {
   __shared__ int s_adm;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const long long span = per_step ? (hi_next != hi ? 1 : 0) : arrival[hi_next - 1] - arrival[hi - 1];
@@ -1411,6 +1472,17 @@ stream_admit_kernel(int D, int32_t cap, int acct, int per_step, int nw, int64_t 
     stats_b[2] = nw - s_adm;
   }
 }
+__global__ void __launch_bounds__(kSt, 1)
+stream_admit_kernel(int D, int32_t cap, int acct, int per_step, int nw, int64_t hi, int64_t hi_next,
+                    const int64_t *arrival, const int64_t *wseg, const int32_t *wperm,
+                    const int32_t *wid, const int32_t *prompt, const int32_t *U,
+                    const long long *used, uint8_t *st, int32_t *g, int32_t *res_u,
+                    long long *aseq, long long *dseq, int64_t *qhead, const StreamState *S,
+                    int64_t *stats_b, int64_t *dst) {
+  pdl_prologue();
+  admit_block(D, cap, acct, per_step, nw, hi, hi_next, arrival, wseg, wperm, wid, prompt, U, used, st, g,
+              res_u, aseq, dseq, qhead, S, stats_b, dst);
+}
 
 struct StreamWs {
   size_t sub_bytes;  // [0, sub_bytes): workspace of the calls the loop makes
@@ -1437,6 +1509,348 @@ struct StreamWs {
   int32_t *rbuf, *sbuf;
   int64_t *qhead;
 };
+
+// ---------------------------------------------------------------------------
+// The loop in one block.  A batch's steps are chains of dependent small passes
+// over a few hundred requests, so launched one by one they cost their launches
+// (eleven, and the host's read of the counts that size them).  This kernel runs
+// batches one after another on one block, steps apart by block barriers, with
+// the two sorts and the quantile done in place.  32 decoders, batches of 256: 68
+// -> 32 us a batch where no queue forms (30,000 requests 8.1 -> 3.8 ms), 155 ->
+// 130 at 16,000 tokens, 207 -> 185 with per-step admission and deferral.
+//   * the completions and each decoder's waiting requests are sorted by rank
+//     (a key's place is the number of smaller keys of its group, each thread
+//     counting for one key), groups past kLoopRank by a bitonic network;
+//   * the quantile comes from a histogram of the window's scores, as in
+//     maps_calibrate's one-block form.
+// It stops before a batch that does not fit (the requests in the system, the
+// window, the dispatch's shared memory); the host then runs that batch by the
+// launches below and comes back when the system is smaller.
+// ---------------------------------------------------------------------------
+constexpr int kLoopActive = 2048;  // requests in the system and the batch, at most
+constexpr int kLoopWindow = 4096;
+constexpr int kLoopRank = 512;     // keys of a group ranked by counting
+constexpr int kLoopBatches = 256;  // batches of one launch
+
+struct LoopArgs {
+  maps_stream_cfg c;
+  StreamWs w;
+  const int64_t *arrival;
+  const int32_t *prompt, *true_len, *pred, *pred_delay;
+  int32_t *choice, *q_out;
+  int64_t *stats, *dst;
+  int32_t *status;
+  size_t smem;       // dynamic shared memory
+  int64_t nbatch;
+  int64_t b0;             // the first batch to run
+  long long total_done0;  // completions before it
+};
+
+// Sorts groups of unique keys: group i is key[seg[i], seg[i + 1]), with which[x]
+// the group of key x; out[x's place] gets the key.  Every thread of the block.
+__device__ void sort_groups(const unsigned long long *key, const int32_t *seg, const int16_t *which,
+                            int n, int groups, unsigned long long *out) {
+  for (int x = threadIdx.x; x < n; x += kSt) {
+    const int a = seg[which[x]], b = seg[which[x] + 1];
+    if (b - a > kLoopRank) {
+      out[x] = key[x];
+      continue;
+    }
+    const unsigned long long k = key[x];
+    int r = 0;
+#pragma unroll 4
+    for (int y = a; y < b; ++y) r += key[y] < k;
+    out[a + r] = k;
+  }
+  __syncthreads();
+  for (int i = 0; i < groups; ++i) {  // the long groups, one after another
+    const int a = seg[i], m = seg[i + 1] - a;
+    if (m <= kLoopRank) continue;
+    unsigned long long *v = out + a;
+    int P = 1;
+    while (P < m) P <<= 1;
+    // a network over P places, those past m holding the largest value: the
+    // compare-exchanges with them never move anything (ascending runs only)
+    for (int k = 2; k <= P; k <<= 1) {
+      for (int x = threadIdx.x; x < P; x += kSt) {  // mirror step: both runs ascending
+        const int base = x & ~(k - 1), o = x & (k - 1);
+        const int y = base + (k - 1 - o);
+        if (o < k / 2 && y < m && v[x] > v[y]) {
+          const unsigned long long t = v[x];
+          v[x] = v[y];
+          v[y] = t;
+        }
+      }
+      __syncthreads();
+      for (int j = k >> 2; j > 0; j >>= 1) {
+        for (int x = threadIdx.x; x < P; x += kSt) {
+          const int y = x + j;
+          if ((x & j) == 0 && y < m && v[x] > v[y]) {
+            const unsigned long long t = v[x];
+            v[x] = v[y];
+            v[y] = t;
+          }
+        }
+        __syncthreads();
+      }
+    }
+  }
+}
+
+// The k-th smallest score of the window (n <= kLoopWindow), by the passes of
+// maps_calibrate: hist has 4,096 words of shared memory.
+__device__ uint32_t window_quantile(const int32_t *win_true, const int32_t *win_pred, int n, uint32_t k,
+                                    uint32_t *hist) {
+  __shared__ uint32_t s_warp[kStWarps], s_lo, s_k;
+  __shared__ int s_wl;
+  constexpr int kItems = kLoopWindow / kSt;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  uint32_t sv[kItems];
+#pragma unroll
+  for (int i = 0; i < kItems; ++i) {
+    const int x = i * kSt + tid;
+    sv[i] = x < n ? score(win_true[x], win_pred[x]) : 0u;
+  }
+  uint32_t lo = 0;
+  int w = 32;
+  for (int pass = 0; pass < 3 && w > 0; ++pass) {  // three passes always close the range
+    const bool first = pass == 0;
+    const int shift = w > kStepBits ? w - kStepBits : 0;
+    reinterpret_cast<uint4 *>(hist)[tid] = make_uint4(0, 0, 0, 0);
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kItems; ++i) {
+      if (i * kSt >= n) break;
+      int d = -1;
+      if (i * kSt + tid < n && (first || (sv[i] >= lo && sv[i] - lo < (1u << w))))
+        d = first ? first_bin(sv[i]) : static_cast<int>((sv[i] - lo) >> shift);
+      const unsigned peers = __match_any_sync(0xffffffffu, d);
+      if (d >= 0 && lane == __ffs(peers) - 1) atomicAdd(&hist[d], static_cast<uint32_t>(__popc(peers)));
+    }
+    __syncthreads();
+    const uint4 c = reinterpret_cast<const uint4 *>(hist)[tid];
+    const uint32_t tot = c.x + c.y + c.z + c.w;
+    uint32_t incl = tot;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, incl, off);
+      if (lane >= off) incl += y;
+    }
+    if (lane == 31) s_warp[warp] = incl;
+    __syncthreads();
+    uint32_t cum = __reduce_add_sync(0xffffffffu, lane < warp ? s_warp[lane] : 0u) + incl - tot;
+    if (cum < k && k <= cum + tot) {
+      int d = 4 * tid;
+      if (k > cum + c.x) {
+        cum += c.x, ++d;
+        if (k > cum + c.y) {
+          cum += c.y, ++d;
+          if (k > cum + c.z) cum += c.z, ++d;
+        }
+      }
+      uint32_t nlo = lo + (static_cast<uint32_t>(d) << shift);
+      int nw = shift;
+      if (first) first_range(d, nlo, nw);
+      s_lo = nlo;
+      s_wl = nw;
+      s_k = k - cum;
+    }
+    __syncthreads();
+    lo = s_lo;
+    w = s_wl;
+    k = s_k;
+    __syncthreads();  // s_lo and the histogram are written again
+  }
+  return lo;
+}
+
+__global__ void __launch_bounds__(kSt, 1)
+stream_loop_kernel(const __grid_constant__ LoopArgs a) {
+  pdl_prologue();
+  extern __shared__ __align__(16) unsigned char ldm[];
+  __shared__ int32_t scratch[3 * kStreamMaxD];
+  __shared__ int s_w[kStWarps];
+  const maps_stream_cfg &c = a.c;
+  const StreamWs &w = a.w;
+  StreamState *const S = w.S;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int D = c.D;
+  const int64_t N = c.N, B = c.batch;
+  const bool defer = c.beta >= 0;
+  const int mc = c.dispatch_policy == MAPS_STREAM_MC ? 1 : 0;
+  // groups of the sorts over the dispatch's shared memory: keys, sorted keys, ids
+  unsigned long long *const key = reinterpret_cast<unsigned long long *>(ldm);
+  unsigned long long *const sorted = key + kLoopActive;
+  int16_t *const which = reinterpret_cast<int16_t *>(sorted + kLoopActive);
+  int32_t *const seg = scratch;                    // [D + 1] group starts
+  int32_t *const cur = scratch + kStreamMaxD + 8;  // [D] cursors
+  int64_t b = a.b0;
+  long long total_done = a.total_done0;
+  for (int run = 0; run < kLoopBatches && b < a.nbatch; ++run, ++b) {
+    const int64_t lo = b * B, hi = min(lo + B, N);
+    const int nb = static_cast<int>(hi - lo);
+    int32_t *const act_in = w.act[b & 1], *const act = w.act[(b & 1) ^ 1];
+    int64_t *const stats_b = a.stats + 4 * b;
+    const int npend = S->npend;
+    if (defer) {
+      __syncthreads();
+      select_block(lo, nb, hi, c.beta, b + 1 == a.nbatch ? 1 : 0, a.arrival, a.pred_delay, w.pend[b & 1],
+                   w.pend[(b & 1) ^ 1], w.cid, w.tout, S);
+      __syncthreads();
+    }
+    const int nc = defer ? S->nc : nb, nto = defer ? S->nto : 0;
+    const int most = S->nact + nto;  // requests in the system before this batch's, at most
+    if (most + nc > kLoopActive || stream_dispatch_smem(D, most, nc) > a.smem) {
+      __syncthreads();
+      if (tid == 0) S->npend = npend;  // the batch is not started
+      break;
+    }
+    __syncthreads();
+    if (c.per_step) {  // 1'.
+      interval_block(scratch, hi, D, c.cap, c.accounting, a.arrival, a.prompt, a.true_len, w.U, w.res_u, w.st,
+                     w.g, w.dec, act_in, w.wid, w.wperm, w.wseg, w.qhead, w.aseq, w.dseq, w.rbuf, w.sbuf,
+                     w.done_id, w.done_rem, S, a.dst);
+      __syncthreads();
+    }
+    advance_block(hi, D, c.cap, c.accounting, c.per_step, a.arrival, a.prompt, a.true_len, w.res_u, w.st, w.g,
+                  w.dec, act_in, act, w.done_id, w.done_rem, w.used, S, stats_b, a.dst);
+    __syncthreads();
+    int nact = S->nact;
+    const int ndone = S->ndone, nwait = S->nwait;
+    if (ndone > 0) {  // 2. by (step, id) into the ring
+      for (int x = tid; x < ndone; x += kSt) {
+        key[x] = (static_cast<unsigned long long>(w.done_rem[x]) << 32) | static_cast<uint32_t>(w.done_id[x]);
+        which[x] = 0;
+      }
+      if (tid == 0) {
+        seg[0] = 0;
+        seg[1] = ndone;
+      }
+      __syncthreads();
+      sort_groups(key, seg, which, ndone, 1, sorted);
+      for (int x = max(0, ndone - c.window) + tid; x < ndone; x += kSt) {
+        const int id = static_cast<int>(sorted[x] & 0xffffffffull);
+        const int slot = static_cast<int>((total_done + x) % c.window);
+        w.win_true[slot] = a.true_len[id];
+        w.win_pred[slot] = a.pred[id];
+      }
+      total_done += ndone;
+      __syncthreads();
+    }
+    // 3. the quantile; U = pred + q of the requests in the system and the candidates
+    const int win = static_cast<int>(min(total_done, static_cast<long long>(c.window)));
+    const long long rank = (static_cast<long long>(1000000u - c.alpha_ppm) * (win + 1) + 999999) / 1000000;
+    const bool rr = rank > win;
+    int32_t q = 0;
+    if (!rr) {
+      const uint32_t qq = window_quantile(w.win_true, w.win_pred, win, static_cast<uint32_t>(rank),
+                                          reinterpret_cast<uint32_t *>(ldm));
+      if (qq > 0x7fffffffu) {
+        if (tid == 0) flag_error(a.status, MAPS_E_RANGE);
+      } else {
+        q = static_cast<int32_t>(qq);
+      }
+    }
+    if (tid == 0) *w.q_dev = q;
+    if (nto > 0) {  // timed out: round robin with the horizon as bound
+      enqueue_list(nto, nact, D, c.H, hi, a.arrival, w.tout, nullptr, w.Uq, a.choice, w.st, w.dec, w.disp, w.g,
+                   w.U, act, S, a.status);
+      nact += nto;
+      __syncthreads();
+    }
+    const int32_t *const cids = defer ? w.cid : nullptr;
+    int32_t *const cch = defer ? w.cch : a.choice + lo;
+    const int32_t *const cpr = defer ? w.cp : a.prompt + lo;
+    for (int x = tid; x < nact + nc; x += kSt) {
+      const int id = x < nact ? act[x] : cids ? cids[x - nact] : static_cast<int>(lo + (x - nact));
+      const long long u = static_cast<long long>(a.pred[id]) + q;  // Eq. (conformal_upper)
+      if (u > 0x7fffffffLL) flag_error(a.status, MAPS_E_RANGE);
+      w.Uq[x] = static_cast<int32_t>(u > 0x7fffffffLL ? 0x7fffffffLL : u);
+      if (x >= nact && cids) w.cp[x - nact] = a.prompt[id];
+    }
+    if (rr || c.dispatch_policy == MAPS_STREAM_RR)  // 3'., 5'.
+      for (int x = tid; x < nc; x += kSt)
+        cch[x] = static_cast<int32_t>((cids ? static_cast<int64_t>(cids[x]) : lo + x) % D);
+    __syncthreads();
+    csr_block(scratch, nact, D, rr ? 1 : 0, w.q_dev, a.q_out + b, act, w.st, w.g, w.dec, a.prompt, w.Uq, w.U,
+              w.res_off, w.rp, w.rg, w.rU, w.Q, a.arrival, defer ? a.pred_delay : nullptr, hi, c.H);  // 4.
+    __syncthreads();
+    if (nc > 0 && !rr && c.dispatch_policy == MAPS_STREAM_LR) {
+      if (warp == 0) lr_warp(reinterpret_cast<uint32_t *>(scratch), D, nc, w.res_off, cch);
+      __syncthreads();
+    } else if (nc > 0 && !rr && c.dispatch_policy != MAPS_STREAM_RR) {  // 5.
+      dispatch_block(ldm, D, c.H, nc, mc, w.res_off, w.rp, w.rg, w.rU, w.capv, w.Q, cpr, w.Uq + nact, cch,
+                     nullptr, a.status);
+      __syncthreads();
+    }
+    if (!defer)  // 6.
+      enqueue_batch(lo, nb, nact, hi, D, a.arrival, a.choice, w.Uq, w.st, w.dec, w.disp, w.g, w.U, act, S,
+                    a.status);
+    else if (nc > 0)
+      enqueue_list(nc, nact, D, c.H, hi, a.arrival, w.cid, w.cch, w.Uq, a.choice, w.st, w.dec, w.disp, w.g, w.U,
+                   act, S, a.status);
+    // 7. each decoder's waiting requests in local order
+    const int n_all = nact + nc, nw = nwait + nto + nc;
+    for (int k = tid; k <= D; k += kSt) seg[k] = 0;
+    __syncthreads();
+    const long long s_b = a.arrival[hi - 1];
+    for (int x = tid; x < n_all; x += kSt) {
+      const int id = act[x];
+      if (w.st[id] == kWaiting) atomicAdd(&seg[w.dec[id] + 1], 1);
+    }
+    __syncthreads();
+    {  // inclusive scan of the counts: seg[k] becomes decoder k's start (D <= kSt)
+      int v = tid < D ? seg[tid + 1] : 0;
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, v, off);
+        if (lane >= off) v += y;
+      }
+      if (lane == 31) s_w[warp] = v;
+      __syncthreads();
+      v += static_cast<int>(__reduce_add_sync(0xffffffffu, lane < warp ? static_cast<unsigned>(s_w[lane]) : 0u));
+      if (tid < D) {
+        seg[tid + 1] = v;
+        w.wseg[tid + 1] = v;
+        if (tid + 1 < D) cur[tid + 1] = v;
+      }
+      if (tid == 0) {
+        w.wseg[0] = 0;
+        cur[0] = 0;
+      }
+      __syncthreads();
+    }
+    for (int x = tid; x < n_all; x += kSt) {
+      const int id = act[x];
+      if (w.st[id] == kWaiting) {
+        const int k = w.dec[id];
+        // promoted (waited past max_wait, or FCFS) before the rest, then the
+        // bound of the others, then the index, which is the arrival order
+        const bool promoted = c.local_order == MAPS_STREAM_FCFS || min(s_b - w.disp[id], 0x7fffffffLL) > c.max_wait;
+        const int o = atomicAdd(&cur[k], 1);
+        key[o] = (promoted ? 0ull : (1ull << 62) | (static_cast<unsigned long long>(w.U[id]) << 31)) |
+                 static_cast<uint32_t>(id);
+        which[o] = static_cast<int16_t>(k);
+      }
+    }
+    __syncthreads();
+    sort_groups(key, seg, which, nw, D, sorted);
+    for (int x = tid; x < nw; x += kSt) {
+      w.wid[x] = static_cast<int32_t>(sorted[x] & 0x7fffffffull);
+      w.wperm[x] = x;
+    }
+    __syncthreads();
+    const int64_t hi_next = b + 1 < a.nbatch ? min(hi + B, N) : hi;
+    admit_block(D, c.cap, c.accounting, c.per_step, nw, hi, hi_next, a.arrival, w.wseg, w.wperm, w.wid, a.prompt,
+                w.U, w.used, w.st, w.g, w.res_u, w.aseq, w.dseq, w.qhead, S, stats_b, a.dst);  // 8.
+    __syncthreads();
+  }
+  __syncthreads();
+  if (tid == 0) {
+    S->next_b = b;
+    S->total_done = total_done;
+  }
+}
 
 size_t stream_sub_bytes(const maps_stream_cfg &c) {
   size_t b = maps_calibrate_workspace_size(c.window, c.N);
@@ -1571,7 +1985,49 @@ int maps_stream_run(const maps_stream_cfg *cfg, const int64_t *arrival_ms, const
 
   long long total_done = 0;
   StreamState hs;
+  // the one-block loop, where a batch fits it
+  cudaFuncAttributes fa;
+  MAPS_TRY(cuda_ok(cudaFuncGetAttributes(&fa, stream_loop_kernel)));
+  const size_t loop_smem = static_cast<size_t>(max_smem_optin()) - fa.sharedSizeBytes;
+  MAPS_TRY(cuda_ok(cudaFuncSetAttribute(stream_loop_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        static_cast<int>(loop_smem))));
+  auto loop_fits = [&](int64_t system, int64_t cands) {  // requests in the system, candidates
+    return c.window <= kLoopWindow && system + cands <= kLoopActive &&
+           stream_dispatch_smem(D, static_cast<int>(system), static_cast<int>(cands)) <= loop_smem;
+  };
+  bool in_loop = loop_fits(0, std::min(N, B));
   for (int64_t b = 0; b < nbatch; ++b) {
+    if (in_loop) {
+      LoopArgs la;
+      la.c = c;
+      la.w = w;
+      la.arrival = arrival_ms;
+      la.prompt = prompt;
+      la.true_len = true_len;
+      la.pred = pred;
+      la.pred_delay = pred_delay;
+      la.choice = choice_out;
+      la.q_out = q_out;
+      la.stats = stats_out;
+      la.dst = dec_stats_out;
+      la.status = status;
+      la.smem = loop_smem;
+      la.nbatch = nbatch;
+      la.b0 = b;
+      la.total_done0 = total_done;
+      launch_pdl(stream_loop_kernel, 1, kSt, loop_smem, s, la);
+      MAPS_TRY(launch_ok());
+      MAPS_TRY(cuda_ok(cudaMemcpyAsync(&hs, w.S, sizeof(hs), cudaMemcpyDeviceToHost, s)));
+      MAPS_TRY(cuda_ok(cudaStreamSynchronize(s)));
+      const bool stopped = hs.next_b < nbatch && hs.next_b < b + kLoopBatches;
+      b = hs.next_b;
+      total_done = hs.total_done;
+      if (!stopped) {
+        --b;  // all done, or a launch's worth
+        continue;
+      }
+      in_loop = false;  // batch b does not fit: it runs here
+    }
     const int64_t lo = b * B, hi = std::min(lo + B, N);
     const int nb = static_cast<int>(hi - lo);
     int32_t *act_in = w.act[b & 1], *act = w.act[(b & 1) ^ 1];
@@ -1674,6 +2130,8 @@ int maps_stream_run(const maps_stream_cfg *cfg, const int64_t *arrival_ms, const
                arrival_ms, w.wseg, w.wperm, w.wid, prompt, w.U, w.used, w.st, w.g, w.res_u, w.aseq,
                w.dseq, w.qhead, w.S, stats_b, dec_stats_out);  // 8.
     MAPS_TRY(launch_ok());
+    // back to the one block once the next batch is sure to fit
+    in_loop = loop_fits(n_all, B + hs.npend);
   }
   return maps_check(ws, stream);
 }

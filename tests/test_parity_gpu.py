@@ -1034,6 +1034,22 @@ def test_stream_walk_list_sizes(M, ws, oracle, N, D, cap, B):
     check_stream(M, ws, oracle, N, D, 16384, cap, B, 300, 100000, 1000, w)
 
 
+@pytest.mark.parametrize("N,D,cap,B,Wn", [
+    # more batches than one launch of the one-block loop runs
+    (700, 4, 30000, 2, 50), (257, 3, 30000, 1, 20),
+    # the window at what the loop holds, and past it
+    (9000, 8, 262144, 512, 4096), (9000, 8, 262144, 512, 4097),
+    # queues past the ranked groups (512), and a system that outgrows the loop
+    # and comes back into it; batches and systems around 2,048 requests
+    (3000, 2, 40000, 100, 300), (9000, 2, 60000, 300, 500), (5000, 16, 262144, 2000, 500),
+    (5000, 16, 262144, 2048, 500), (5000, 64, 20000, 2049, 500),
+    # many completions in one batch: sorted by the network
+    (9000, 40, 262144, 900, 700)])
+def test_stream_one_block_loop_limits(M, ws, oracle, N, D, cap, B, Wn):
+    w = W.make_stream(n_requests=N)
+    check_stream(M, ws, oracle, N, D, 16384, cap, B, Wn, 100000, 1000, w)
+
+
 def test_stream_full_workload(M, ws, oracle):
     """All 1,000,000 requests of the streaming workload, bit for bit."""
     w = W.make_stream()
