@@ -211,6 +211,208 @@ stream_advance_kernel(int64_t hi, int D, int32_t cap, int acct, int per_step, co
 //     grows and nothing is freed since the head last failed), so the warp
 //     jumps to the next step with a completion or a preemption, or to s.
 //     Every iteration advances the step, so the loop ends.
+// A decoder's simulation between dispatch steps as one warp holds it.
+struct IntervalRun {
+  long long t, s;              // the current step, the dispatch step
+  long long qh, qe;            // the queue: its head and end in the order
+  long long seq, integ;        // next admission number; waiting steps summed
+  int n, ns, npre, nadm;       // running, preempted since the last dispatch step; counts
+};
+
+// The running set in registers, kS requests a lane in any slot, from t until s
+// or until an admission finds no free slot; then the set goes back to rbuf (and
+// g), where the general loop takes it up.  The tokens held are one running sum,
+// and the queue's head is kept, so an event reads no memory unless a request
+// moves: a lane's slots, one warp minimum and the uniform arithmetic (the steps
+// to a preemption are divided out only when one comes before the completion).
+template <int kS>
+__device__ void interval_registers(IntervalRun &v, int32_t cap, int acct, const int32_t *prompt,
+                                   const int32_t *true_len, const int32_t *U, int32_t *res_u, uint8_t *st,
+                                   int32_t *g, const int32_t *wid, const int32_t *wperm, long long *aseq,
+                                   int32_t *rbuf, int32_t *sbuf, int32_t *done_id, int32_t *done_rem,
+                                   long long s0, int *s_done) {
+  constexpr unsigned kAll = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  int id[kS], gi[kS], L[kS], pr[kS], ru[kS];  // id < 0: a free slot
+  long long as[kS];
+  long long tok = 0;
+#pragma unroll
+  for (int i = 0; i < kS; ++i) {
+    const int x = 32 * i + lane;
+    id[i] = x < v.n ? rbuf[x] : -1;
+  }
+#pragma unroll
+  for (int i = 0; i < kS; ++i) {
+    const bool ok = id[i] >= 0;
+    gi[i] = ok ? g[id[i]] : 0;
+    L[i] = ok ? true_len[id[i]] : 0;
+    pr[i] = ok ? prompt[id[i]] : 0;
+    ru[i] = ok ? res_u[id[i]] : 0;
+    as[i] = ok ? aseq[id[i]] : -1;
+    tok += static_cast<long long>(pr[i]) + gi[i];
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) tok += __shfl_xor_sync(kAll, tok, off);
+  // the stack's top, else the queue's head (hc < 0: nobody waits)
+  int hc = -1, hp = 0, hu = 0;
+  auto head = [&] {
+    hc = v.ns > 0 ? sbuf[v.ns - 1] : v.qh < v.qe ? wid[wperm[v.qh]] : -1;
+    hp = hc >= 0 ? prompt[hc] : 0;
+    hu = hc >= 0 ? U[hc] : 0;
+  };
+  head();
+  bool full = false;
+  while (v.t < v.s && !full) {
+    const int n = v.n;
+    long long je = LLONG_MAX;  // steps to the next completion or preemption
+    if (n > 0) {
+      uint32_t m = ~0u;
+#pragma unroll
+      for (int i = 0; i < kS; ++i) m = id[i] >= 0 ? min(m, static_cast<uint32_t>(L[i] - gi[i])) : m;
+      je = __reduce_min_sync(kAll, m);
+      if (n > 1 && tok + n * je > cap) je = tok + n > cap ? 1 : (cap - tok) / n + 1;
+    }
+    const long long te = je >= v.s - v.t ? v.s : v.t + je;
+    const int quiet = static_cast<int>(te - v.t - 1);  // steps of growth alone
+    if (quiet > 0) {
+#pragma unroll
+      for (int i = 0; i < kS; ++i) gi[i] += id[i] >= 0 ? quiet : 0;
+    }
+    v.integ += (v.ns + (v.qe - v.qh)) * (te - v.t - 1);
+    tok += n * (te - v.t - 1);
+    v.t = te;
+    // preempt the latest admitted while the next tokens do not fit
+    bool moved = false;
+    while (v.n > 1 && tok + v.n > cap) {
+      long long best = -1;
+      int bi = 0;
+#pragma unroll
+      for (int i = 0; i < kS; ++i)
+        if (id[i] >= 0 && as[i] > best) {
+          best = as[i];
+          bi = 32 * i + lane;
+        }
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) {
+        const long long ob = __shfl_xor_sync(kAll, best, off);
+        const int oi = __shfl_xor_sync(kAll, bi, off);
+        if (ob > best) {
+          best = ob;
+          bi = oi;
+        }
+      }
+      int held = 0;  // the victim's tokens, from its lane
+#pragma unroll
+      for (int i = 0; i < kS; ++i)
+        if (bi == 32 * i + lane) {
+          held = pr[i] + gi[i];
+          sbuf[v.ns] = id[i];
+          st[id[i]] = kWaiting;
+          g[id[i]] = 0;
+          id[i] = -1;
+        }
+      tok -= __shfl_sync(kAll, held, bi & 31);
+      v.n -= 1;
+      v.ns += 1;
+      v.npre += 1;
+      moved = true;
+      __syncwarp();
+    }
+    // one token each; completions free their slots
+    tok += v.n;
+    int gone = 0;
+    long long freed = 0;
+#pragma unroll
+    for (int i = 0; i < kS; ++i) {
+      const bool run = id[i] >= 0;
+      gi[i] += run ? 1 : 0;
+      const bool fin = run && gi[i] == L[i];
+      const unsigned fm = __ballot_sync(kAll, fin);
+      if (fm == 0) continue;
+      gone += __popc(fm);
+      if (fin) {
+        st[id[i]] = kDone;
+        const int o = atomicAdd(s_done, 1);
+        done_id[o] = id[i];
+        done_rem[o] = static_cast<int>(v.t - s0);
+        freed += static_cast<long long>(pr[i]) + gi[i];
+        id[i] = -1;
+      }
+    }
+    if (gone > 0) {
+      v.n -= gone;
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) freed += __shfl_xor_sync(kAll, freed, off);
+      tok -= freed;
+    }
+    if (v.t == v.s) break;
+    if (moved) head();
+    // admission in queue order (the stack first)
+    if (hc >= 0) {
+      long long used = tok;
+      if (acct != MAPS_STREAM_OCCUPANCY) {
+        used = 0;
+#pragma unroll
+        for (int i = 0; i < kS; ++i)
+          if (id[i] >= 0)
+            used += (acct == MAPS_STREAM_STAGED ? 1ll : 2ll) * pr[i] + max(ru[i], gi[i]);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) used += __shfl_xor_sync(kAll, used, off);
+      }
+      while (hc >= 0 && used + hp + hu <= cap) {
+        bool placed = false;
+#pragma unroll
+        for (int i = 0; i < kS; ++i) {
+          if (placed) continue;
+          const unsigned fl = __ballot_sync(kAll, id[i] < 0);
+          if (fl == 0) continue;
+          placed = true;
+          if (lane == __ffs(fl) - 1) {
+            id[i] = hc;
+            gi[i] = 0;
+            L[i] = true_len[hc];
+            pr[i] = hp;
+            ru[i] = hu;
+            as[i] = v.seq;
+            st[hc] = kRunning;
+            res_u[hc] = hu;
+            aseq[hc] = v.seq;
+          }
+        }
+        if (!placed) {
+          full = true;  // this admission is the general loop's
+          break;
+        }
+        if (v.ns > 0)
+          v.ns -= 1;
+        else
+          v.qh += 1;
+        v.n += 1;
+        v.seq += 1;
+        v.nadm += 1;
+        tok += hp;
+        used += acct == MAPS_STREAM_OCCUPANCY ? static_cast<long long>(hp)
+                : acct == MAPS_STREAM_STAGED  ? static_cast<long long>(hp) + hu
+                                              : 2ll * hp + hu;
+        head();
+      }
+    }
+    if (!full) v.integ += v.ns + (v.qe - v.qh);  // waiting through step t
+  }
+  // the running set and its tokens
+  int base = 0;
+#pragma unroll
+  for (int i = 0; i < kS; ++i) {
+    const unsigned rm = __ballot_sync(kAll, id[i] >= 0);
+    if (id[i] >= 0) {
+      g[id[i]] = gi[i];
+      rbuf[base + __popc(rm & ((1u << lane) - 1u))] = id[i];
+    }
+    base += __popc(rm);
+  }
+  __syncwarp();
+}
+
 __device__ void
 interval_block(int32_t *scratch, int64_t hi, int D, int32_t cap, int acct, const int64_t *arrival,
                const int32_t *prompt, const int32_t *true_len, const int32_t *U,
@@ -270,7 +472,17 @@ interval_block(int32_t *scratch, int64_t hi, int D, int32_t cap, int acct, const
     long long seq = dseq[k], integ = 0;
     int npre = 0, nadm = 0;
     long long t = s0;
+    bool admit_first = false;  // step t has been taken up to its admission
+    if (n <= 64 && s - s0 <= 0x7fffffff) {
+      IntervalRun v = {t, s, qh, qe, seq, 0, n, 0, 0, 0};
+      interval_registers<2>(v, cap, acct, prompt, true_len, U, res_u, st, g, wid, wperm, aseq, rbuf + base,
+                            sbuf + base, done_id, done_rem, s0, &s_done);
+      t = v.t, qh = v.qh, seq = v.seq, integ = v.integ;
+      n = v.n, ns = v.ns, npre = v.npre, nadm = v.nadm;
+      admit_first = t < s;
+    }
     while (t < s) {
+      if (!admit_first) {
       long long tok = 0;
       int jc = INT_MAX;
       for (int i = lane; i < n; i += 32) {
@@ -357,6 +569,8 @@ interval_block(int32_t *scratch, int64_t hi, int D, int32_t cap, int acct, const
       }
       n = kept;
       if (t == s) break;
+      }
+      admit_first = false;
       // admission in queue order (the stack first)
       long long used = 0;
       for (int i = lane; i < n; i += 32) {
@@ -1664,6 +1878,9 @@ __device__ uint32_t window_quantile(const int32_t *win_true, const int32_t *win_
   return lo;
 }
 
+// (kPerStep apart: the interval's code costs the other loop registers, 5% of a
+// batch that is mostly dispatch walk.)
+template <bool kPerStep>
 __global__ void __launch_bounds__(kSt, 1)
 stream_loop_kernel(const __grid_constant__ LoopArgs a) {
   pdl_prologue();
@@ -1706,13 +1923,13 @@ stream_loop_kernel(const __grid_constant__ LoopArgs a) {
       break;
     }
     __syncthreads();
-    if (c.per_step) {  // 1'.
+    if (kPerStep) {  // 1'.
       interval_block(scratch, hi, D, c.cap, c.accounting, a.arrival, a.prompt, a.true_len, w.U, w.res_u, w.st,
                      w.g, w.dec, act_in, w.wid, w.wperm, w.wseg, w.qhead, w.aseq, w.dseq, w.rbuf, w.sbuf,
                      w.done_id, w.done_rem, S, a.dst);
       __syncthreads();
     }
-    advance_block(hi, D, c.cap, c.accounting, c.per_step, a.arrival, a.prompt, a.true_len, w.res_u, w.st, w.g,
+    advance_block(hi, D, c.cap, c.accounting, kPerStep ? 1 : 0, a.arrival, a.prompt, a.true_len, w.res_u, w.st, w.g,
                   w.dec, act_in, act, w.done_id, w.done_rem, w.used, S, stats_b, a.dst);
     __syncthreads();
     int nact = S->nact;
@@ -1841,7 +2058,7 @@ stream_loop_kernel(const __grid_constant__ LoopArgs a) {
     }
     __syncthreads();
     const int64_t hi_next = b + 1 < a.nbatch ? min(hi + B, N) : hi;
-    admit_block(D, c.cap, c.accounting, c.per_step, nw, hi, hi_next, a.arrival, w.wseg, w.wperm, w.wid, a.prompt,
+    admit_block(D, c.cap, c.accounting, kPerStep ? 1 : 0, nw, hi, hi_next, a.arrival, w.wseg, w.wperm, w.wid, a.prompt,
                 w.U, w.used, w.st, w.g, w.res_u, w.aseq, w.dseq, w.qhead, S, stats_b, a.dst);  // 8.
     __syncthreads();
   }
@@ -1986,10 +2203,11 @@ int maps_stream_run(const maps_stream_cfg *cfg, const int64_t *arrival_ms, const
   long long total_done = 0;
   StreamState hs;
   // the one-block loop, where a batch fits it
+  void (*const loop)(LoopArgs) = per_step ? stream_loop_kernel<true> : stream_loop_kernel<false>;
   cudaFuncAttributes fa;
-  MAPS_TRY(cuda_ok(cudaFuncGetAttributes(&fa, stream_loop_kernel)));
+  MAPS_TRY(cuda_ok(cudaFuncGetAttributes(&fa, loop)));
   const size_t loop_smem = static_cast<size_t>(max_smem_optin()) - fa.sharedSizeBytes;
-  MAPS_TRY(cuda_ok(cudaFuncSetAttribute(stream_loop_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  MAPS_TRY(cuda_ok(cudaFuncSetAttribute(loop, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         static_cast<int>(loop_smem))));
   auto loop_fits = [&](int64_t system, int64_t cands) {  // requests in the system, candidates
     return c.window <= kLoopWindow && system + cands <= kLoopActive &&
@@ -2015,7 +2233,7 @@ int maps_stream_run(const maps_stream_cfg *cfg, const int64_t *arrival_ms, const
       la.nbatch = nbatch;
       la.b0 = b;
       la.total_done0 = total_done;
-      launch_pdl(stream_loop_kernel, 1, kSt, loop_smem, s, la);
+      launch_pdl(loop, 1, kSt, loop_smem, s, la);
       MAPS_TRY(launch_ok());
       MAPS_TRY(cuda_ok(cudaMemcpyAsync(&hs, w.S, sizeof(hs), cudaMemcpyDeviceToHost, s)));
       MAPS_TRY(cuda_ok(cudaStreamSynchronize(s)));
