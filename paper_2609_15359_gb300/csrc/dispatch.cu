@@ -1025,7 +1025,8 @@ dispatch_direct_kernel(int D, int H, const int32_t *__restrict__ K, const uint32
 constexpr int kSeqChunk = 128;
 constexpr int kRowWarps = 8;
 constexpr int kColWarps = 16;  // at most
-constexpr int kSeqD = 32 * ((kMaxD + 31) / 32);
+constexpr int kSeqWords = 9;    // per-decoder words beside the rows
+__host__ __device__ constexpr int seq_dw(int D) { return (D + 31) / 32 * 32; }
 
 struct SeqArgs {
   int D, H;
@@ -1073,10 +1074,11 @@ __device__ __forceinline__ void seq_bar(int warps) {
 __device__ __forceinline__ uint32_t max4(uint4 v) { return max(max(v.x, v.y), max(v.z, v.w)); }
 // the larger of m and the first n of v (n may be below 0 or above 4)
 __device__ __forceinline__ uint32_t max4_below(uint4 v, int n, uint32_t m) {
-  m = max(m, n > 0 ? v.x : 0u);
-  m = max(m, n > 1 ? v.y : 0u);
-  m = max(m, n > 2 ? v.z : 0u);
-  return max(m, n > 3 ? v.w : 0u);
+  if (n > 0) m = max(m, v.x);
+  if (n > 1) m = max(m, v.y);
+  if (n > 2) m = max(m, v.z);
+  if (n > 3) m = max(m, v.w);
+  return m;
 }
 
 // RD: decoders per lane of a pick, 0 for any number.
@@ -1085,10 +1087,6 @@ __global__ void __launch_bounds__(1024, 1)
 dispatch_sequential_kernel(const __grid_constant__ SeqArgs a) {
   constexpr unsigned kAll = 0xffffffffu;
   extern __shared__ __align__(16) uint32_t seq_smem[];
-  __shared__ int32_t s_cap[kMaxD], s_q[kMaxD];
-  __shared__ int32_t s_off[kMaxD];      // M + off is the infeasible key term
-  __shared__ uint2 s_col[2][kSeqD];     // (key, M) of each decoder for a candidate, by its parity
-  __shared__ int32_t s_colq[2][kMaxD];  // the queue length behind that key
   __shared__ int2 s_cand[64];           // (p, u) of candidate i at i mod 64; u = 0: none or invalid
   __shared__ __align__(16) uint32_t s_part[2][kRowWarps];  // the chosen row's maxima, per row warp
   __shared__ int4 s_crit[2];            // its (cap, Q, off)
@@ -1100,17 +1098,25 @@ dispatch_sequential_kernel(const __grid_constant__ SeqArgs a) {
   constexpr int nwarp = 32;
   const int64_t nb = (static_cast<int64_t>(H) + kSumBlock - 1) / kSumBlock;
   const int64_t nch = (static_cast<int64_t>(H) + kSeqChunk - 1) / kSeqChunk;
-  // offsets into shared memory, in words
+  // per-decoder words first (Dw, D in whole warps): (key, M) of each decoder for a
+  // candidate by its parity, the queue length behind that key, capacity, queue
+  // length, and off (M + off is the infeasible key term)
+  const int Dw = seq_dw(D);
+  uint2 *const s_col = reinterpret_cast<uint2 *>(seq_smem);  // [2][Dw]
+  int32_t *const words = reinterpret_cast<int32_t *>(seq_smem + 4 * Dw);
+  int32_t *const s_colq = words;                              // [2][Dw]
+  int32_t *const s_cap = words + 2 * Dw, *const s_q = words + 3 * Dw, *const s_off = words + 4 * Dw;
+  // then the rows; offsets in words
   const int ldF = P0 + 4, ld4 = P0 / 4 + 4, ld16 = P0 / 16 + 4, ldc = seq_ldc(P2);
   const int o4 = D * ldF, o16 = o4 + D * ld4, oc = o16 + D * ld16;
-  uint32_t *const F = seq_smem;
+  uint32_t *const F = seq_smem + kSeqWords * Dw;
   // --- capacities, the first candidates ---------------------------------------
   if (tid == 0) {
     s_q0 = 0x7fffffff;
     s_x0 = LLONG_MAX;
     s_umax = s_wide = 0;
   }
-  for (int k = D + tid; k < kSeqD; k += blockDim.x) s_col[0][k] = s_col[1][k] = make_uint2(~0u, 0u);
+  for (int k = D + tid; k < Dw; k += blockDim.x) s_col[k] = s_col[Dw + k] = make_uint2(~0u, 0u);
   __syncthreads();
   bool bad = false;
   for (int k = tid; k < D; k += blockDim.x) {
@@ -1197,42 +1203,56 @@ dispatch_sequential_kernel(const __grid_constant__ SeqArgs a) {
   const int low = part == 0 ? -1 : part == 1 ? 7 : 3;
   const int ldp = part == 0 ? ldc : part == 1 ? ld16 : part == 2 ? ld4 : ldF;
   const int op = part == 0 ? oc : part == 1 ? o16 : part == 2 ? o4 : 0;
-  auto score_col = [&](int64_t j, int k) {  // four lanes, decoder k
+  struct ColLane {  // what a lane keeps of its decoder
+    int k, kc;
+    int32_t cap, off;
+    const uint32_t *part;  // its part of the decoder's row
+  };
+  auto col_lane = [&](int k) {
+    ColLane c;
+    c.k = k, c.kc = min(k, D - 1);
+    c.cap = s_cap[c.kc], c.off = s_off[c.kc];
+    c.part = F + op + c.kc * ldp;
+    return c;
+  };
+  auto score_col = [&](int64_t j, const ColLane &cl) {  // four lanes a decoder
     const int2 cd = s_cand[j & 63];
-    const int u = cd.y, kc = min(k, D - 1);
+    const int u = cd.y;
     const bool in = u < P0;  // its chunk is resident (P0 is whole chunks)
     const int w = u >> sh;
     const int n = part == 0 ? min(w, P2) : in ? w & low : 0;
-    const uint32_t *b = F + op + kc * ldp + (in ? w & ~low : 0);
+    const uint32_t *b = cl.part + (in ? w & ~low : 0);
     const uint4 v0 = *reinterpret_cast<const uint4 *>(b), v1 = *reinterpret_cast<const uint4 *>(b + 4);
-    uint32_t m = max(max4_below(v0, n, 0u), max4_below(v1, n - 4, 0u));
+    uint32_t m = max4_below(v1, n - 4, max4_below(v0, n, 0u));
     if (n > 8)
       for (int i = 8; i < n; i += 4) m = max4_below(*reinterpret_cast<const uint4 *>(b + i), n - i, m);
-    if (!in && (u & (kSeqChunk - 1)) != 0) {  // the last chunk in global memory
-      const int c = u >> 7, n16 = (u >> 4) & 7, t0 = u & ~15;
-      const uint32_t *bg = a.km + kc * nb + c * 8;
-      const int32_t *row = a.K + static_cast<int64_t>(kc) * H + t0;
+    if (u >= P0) {
+      if ((u & (kSeqChunk - 1)) != 0) {  // the last chunk in global memory
+        const int c = u >> 7, n16 = (u >> 4) & 7, t0 = u & ~15;
+        const uint32_t *bg = a.km + cl.kc * nb + c * 8;
+        const int32_t *row = a.K + static_cast<int64_t>(cl.kc) * H + t0;
 #pragma unroll
-      for (int i = 0; i < 2; ++i)
-        if (part + 4 * i < n16) m = max(m, bg[part + 4 * i]);
+        for (int i = 0; i < 2; ++i)
+          if (part + 4 * i < n16) m = max(m, bg[part + 4 * i]);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int t = part + 4 * i;
-        if (t < (u & 15)) m = max(m, static_cast<uint32_t>(row[t]) + static_cast<uint32_t>(t0 + t));
+        for (int i = 0; i < 4; ++i) {
+          const int t = part + 4 * i;
+          if (t < (u & 15)) m = max(m, static_cast<uint32_t>(row[t]) + static_cast<uint32_t>(t0 + t));
+        }
       }
+      for (int c = P2 + part; c < (u >> 7); c += 4) m = max(m, a.cm[cl.kc * nch + c]);
     }
-    if ((u >> 7) > P2)
-      for (int c = P2 + part; c < (u >> 7); c += 4) m = max(m, a.cm[kc * nch + c]);
     m = max(m, __shfl_xor_sync(kAll, m, 1));
     m = max(m, __shfl_xor_sync(kAll, m, 2));
-    const int32_t q = s_q[kc];
-    const uint32_t key = key32(m, cd.x, s_cap[kc], q, s_off[kc], k);
-    if (part == 0 && k < D) {
-      s_col[j & 1][k] = make_uint2(key, m);
-      s_colq[j & 1][k] = q;
+    const int32_t q = s_q[cl.kc];
+    const uint32_t key = key32(m, cd.x, cl.cap, q, cl.off, cl.k);
+    if (part == 0 && cl.k < D) {
+      const int at = (j & 1) ? Dw + cl.k : cl.k;
+      s_col[at] = make_uint2(key, m);
+      s_colq[at] = q;
     }
   };
-  for (int k0 = warp * 8; k0 < D; k0 += nwarp * 8) score_col(0, k0 + (lane >> 2));
+  for (int k0 = warp * 8; k0 < D; k0 += nwarp * 8) score_col(0, col_lane(k0 + (lane >> 2)));
   __syncthreads();
 
   // The pick of candidate j (with p) at phase parity par: the decoder, and this
@@ -1247,7 +1267,7 @@ dispatch_sequential_kernel(const __grid_constant__ SeqArgs a) {
     key = ~0u;
     M = 0;
     auto take = [&](int k) {
-      uint2 e = s_col[par][k];
+      uint2 e = s_col[par * Dw + k];
       if (k == kprev) e = make_uint2(ckey, cM);
       M = e.x < key ? e.y : M;
       key = min(key, e.x);
@@ -1263,8 +1283,8 @@ dispatch_sequential_kernel(const __grid_constant__ SeqArgs a) {
     if ((best & 0x7fffffffu) < lim_key) return static_cast<int>(best & kmask);
     unsigned long long k64 = ~0ull;  // the wide keys
     for (int k = lane; k < D; k += 32) {
-      const uint32_t Mk = k == kprev ? cM : s_col[par][k].y;
-      const int32_t qk = k == kprev ? cr.y : s_colq[par][k];
+      const uint32_t Mk = k == kprev ? cM : s_col[par * Dw + k].y;
+      const int32_t qk = k == kprev ? cr.y : s_colq[par * Dw + k];
       const unsigned long long y =
           seq_key64(static_cast<long long>(s_cap[k]) - (static_cast<long long>(p) + 1 + Mk), qk, k, mc);
       if (y < k64) {
@@ -1371,9 +1391,21 @@ dispatch_sequential_kernel(const __grid_constant__ SeqArgs a) {
             if (lane == 0) set_cm(c, cx);
           }
         }
-        m1 = __reduce_max_sync(kAll, m1);
-        if (lane == 0) s_part[par][warp] = m1;
-        if (res0 && tb < u) fold(warp, bm0);
+        // publish, and fold the first chunk's maxima: one reduction, shuffle
+        // and store in flight with another's
+        if (res0 && tb < u) {
+          const uint32_t b1 = max(bm0, __shfl_xor_sync(kAll, bm0, 1));
+          m1 = __reduce_max_sync(kAll, m1);
+          const uint32_t cm0 = __reduce_max_sync(kAll, bm0);
+          const uint32_t b2 = max(b1, __shfl_xor_sync(kAll, b1, 2));
+          if (lane == 0) s_part[par][warp] = m1;
+          F[o4 + kk * ld4 + warp * 32 + lane] = bm0;
+          if ((lane & 3) == 0) F[o16 + kk * ld16 + warp * 8 + (lane >> 2)] = b2;
+          if (lane == 0) set_cm(warp, cm0);
+        } else {
+          m1 = __reduce_max_sync(kAll, m1);
+          if (lane == 0) s_part[par][warp] = m1;
+        }
       }
       kprev = kk;
       seq_bar(walkers);
@@ -1406,12 +1438,14 @@ dispatch_sequential_kernel(const __grid_constant__ SeqArgs a) {
     const int cw = warp - kRowWarps - 1;
     int2 cn = make_int2(0, 0);  // column warp 0: the 32 candidates of the next ring refill
     if (cw == 0) cn = load_cand(64 + lane);
+    const ColLane mine = col_lane(cw * 8 + (lane >> 2));  // every column warp has some decoder
     for (int64_t j = 0; j < a.J; ++j) {
       if (cw == 0 && (j & 31) == 0 && j > 0) {
         s_cand[(j + 32 + lane) & 63] = cn;
         cn = load_cand(j + 64 + lane);
       }
-      for (int k0 = cw * 8; k0 < D; k0 += 8 * a.ncol) score_col(j + 1, k0 + (lane >> 2));
+      score_col(j + 1, mine);
+      for (int k0 = (cw + a.ncol) * 8; k0 < D; k0 += 8 * a.ncol) score_col(j + 1, col_lane(k0 + (lane >> 2)));
       seq_bar(walkers);
     }
   }
@@ -2028,14 +2062,15 @@ int dispatch_sequential(int D, int H, int32_t *K, const int32_t *cap, int32_t *Q
   a.kb = 0;
   while ((1 << a.kb) < D) ++a.kb;
   a.ncol = std::min((D + 7) / 8, kColWarps);
-  // shared memory per row: a sixteenth for chunk maxima, the rest resident
-  // steps (1 + 1/4 + 1/16 words each); 44 KB are left to the static arrays
-  const int64_t words = ((max_smem_optin() - 45056) / 4 - kSeqPad) / D;
+  // shared memory per row: a thirty-second for chunk maxima, the rest resident
+  // steps (1 + 1/4 + 1/16 words each); 2 KB are left to the static arrays
+  const int64_t fixed = kSeqWords * seq_dw(D) + kSeqPad;
+  const int64_t words = ((max_smem_optin() - 2048) / 4 - fixed) / D;
   const int64_t chunks = (static_cast<int64_t>(H) + kSeqChunk - 1) / kSeqChunk;
-  a.P2 = static_cast<int>(std::min<int64_t>(chunks, words / 16));
+  a.P2 = static_cast<int>(std::min<int64_t>(chunks, words / 32));
   a.P0 = 0;
   while (a.P0 < chunks * kSeqChunk && seq_row_words(a.P0 + kSeqChunk, a.P2) <= words) a.P0 += kSeqChunk;
-  const size_t smem = 4 * (static_cast<size_t>(D) * seq_row_words(a.P0, a.P2) + kSeqPad);
+  const size_t smem = 4 * (static_cast<size_t>(D) * seq_row_words(a.P0, a.P2) + fixed);
   auto launch = [&](void (*kern)(SeqArgs)) {
     MAPS_TRY(cuda_ok(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           static_cast<int>(smem))));
