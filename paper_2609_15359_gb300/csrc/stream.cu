@@ -935,17 +935,19 @@ __device__ bool rebuild_tables(const int32_t *E, const int32_t *Bv, uint32_t *SS
 // step t = e - 1.  Reserving (u, p + 1) adds p + e to V where e <= u, and the
 // new pair's own V is P + p + u with P = K(u - 1) + u - 1, known from scoring
 // the candidate, so a reservation moves nothing.  M(u) is the larger of the V
-// with e < u and P: two warp reductions and a ballot.  A decision takes one
+// with e < u and P: two warp reductions.  A decision takes one
 // barrier: every warp picks from the keys published before it, the winner's
 // reserves, and all score the next candidate.  Keys as for maps_dispatch
 // SEQUENTIAL: a feasible decoder is min(Q - q0, lim) << 5 | k, an infeasible one
 // 1 << 31 | min(M - cap - x0, lim) << 5 | k; at lim the 64-bit keys decide.
 // Returns false when a list outgrows 32 kS pairs (nothing is kept then).
-// 32 warps issue every decision's instructions, so those are counted: 32
-// decoders at 16,000 tokens, 256 candidates: the dispatch kernel 160 -> 101 us
-// (0.33 us a candidate); before, two warps shared the walk on sorted lists in
-// shared memory.  (140 us with M and Q published beside every key and the
-// candidates clamped in every warp.)
+// The winner's chain (pick, reserve, score, publish: three warp reductions of
+// about 100 cycles among some 60 instructions) and 32 warps' instructions both
+// cost, so what can be kept is (a feasible key, the choices of 32 candidates).
+// 32 decoders at 16,000 tokens, a candidate: two warps sharing the walk over
+// sorted lists in shared memory 0.6 us, this form 0.38.  (Eight candidates
+// scored ahead by four lanes each, decoders reserved on meanwhile one by one:
+// fewer instructions, but the chain grew, 0.55 us.)
 struct WalkShared {
   uint32_t key[2][32];  // of each decoder for a candidate, by its parity
   uint32_t M[32];       // where the 64-bit keys decide: M and the queue length
@@ -957,7 +959,7 @@ template <int kS>
 __device__ bool walk_registers(int D, int nb, int mc, const int32_t *uE, const int32_t *uB,
                                const int32_t *s_base, const int32_t *s_n, int32_t *s_q,
                                const int32_t *s_cap, const int2 *cand, int32_t *choice,
-                               int64_t *headroom, WalkShared &w, bool &bad) {
+                               WalkShared &w, bool &bad) {
   constexpr unsigned kAll = 0xffffffffu;
   const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
   const bool has = k < D;
@@ -1030,37 +1032,46 @@ __device__ bool walk_registers(int D, int nb, int mc, const int32_t *uE, const i
   }
   if (lane >= D) w.key[0][lane] = w.key[1][lane] = ~0u;
   uint32_t P = 0, M = 0;
-  // candidate (p, u) scored into column `par`
-  const uint32_t kbit = static_cast<uint32_t>(k), kinf = kbit + 0x80000000u;
+  const uint32_t kinf = static_cast<uint32_t>(k) + 0x80000000u;
   const int32_t capf = mc ? 0 : cap;  // mc: no decoder is feasible
-  auto score = [&](int2 c, int par) {
-    const uint32_t u = static_cast<uint32_t>(c.y);
-    uint32_t sum = 0, cnt = 1, vm = 0;
+  // the key while feasible: it changes with the queue length alone
+  auto feasible_key = [&] {
+    return (min(static_cast<uint32_t>(q - q0), lim) << 5) + static_cast<uint32_t>(k);
+  };
+  uint32_t fkey = feasible_key();
+  // candidate (p, u) scored and its key published in `to`; ~0: invalid, or the end
+  auto score = [&](int2 c, uint32_t *to) {
+    const uint32_t u = static_cast<uint32_t>(c.y), t = u - 1;
+    uint32_t sum = 0, vm = 0;
 #pragma unroll
     for (int s = 0; s < kS; ++s) {
-      const bool live = e[s] >= u;  // at step u - 1
-      sum += live ? b[s] : 0u;
-      cnt += __popc(__ballot_sync(kAll, live));
+      const bool live = e[s] >= u;  // at step t: holds b + t tokens
+      sum += live ? b[s] + t : 0u;
       vm = max(vm, live ? 0u : V[s]);
     }
     sum = __reduce_add_sync(kAll, sum);
     vm = __reduce_max_sync(kAll, vm);
-    P = sum + (u - 1) * cnt;
+    P = sum + t;
     M = max(vm, P);
     // p + 1 + M <= cap: M < cap - p
-    const bool feas = M < static_cast<uint32_t>(max(capf - c.x, 0));
-    const uint32_t term = min(feas ? static_cast<uint32_t>(q - q0) : M + off, lim);
-    if (lane == 0) w.key[par][k] = (term << 5) + (feas ? kbit : kinf);
+    const bool feas = static_cast<int32_t>(M) < capf - c.x && static_cast<int32_t>(M) >= 0;
+    const uint32_t ikey = (min(M + off, lim) << 5) + kinf;
+    if (lane == 0) to[k] = u == 0 ? ~0u : feas ? fkey : ikey;
   };
-  int2 c = cand[0];
-  score(c, 0);
+  uint32_t *now = w.key[0], *next = w.key[1];
+  score(cand[0], now);
   named_bar(1, 32 * D);
+  const int2 *cp = cand;
+  int kept = 0;
   for (int j = 0; j < nb; ++j) {
-    const int2 c1 = cand[j + 1];  // there is one past the end
-    if (c.y > 0) {
-      const uint32_t best = __reduce_min_sync(kAll, w.key[j & 1][lane]);
-      int kk = static_cast<int>(best & 31u);
-      if ((best & 0x7fffffffu) >= lim_key) {  // in every warp alike
+    const int2 c1 = *++cp;  // there is one past the end
+    const uint32_t best = __reduce_min_sync(kAll, now[lane]);
+    int kk = static_cast<int>(best & 31u);
+    if ((best & 0x7fffffffu) >= lim_key) {  // in every warp alike
+      if (best == ~0u) {
+        kk = -1;
+        bad = true;
+      } else {  // the 64-bit keys
         if (lane == 0) {
           w.M[k] = M;
           w.q[k] = q;
@@ -1069,7 +1080,7 @@ __device__ bool walk_registers(int D, int nb, int mc, const int32_t *uE, const i
         unsigned long long k64 = ~0ull;
         if (lane < D)
           k64 = dispatch_key(static_cast<long long>(s_cap[lane]) -
-                                 (static_cast<long long>(c.x) + 1 + w.M[lane]),
+                                 (static_cast<long long>(cp[-1].x) + 1 + w.M[lane]),
                              w.q[lane], lane, mc);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
@@ -1079,36 +1090,38 @@ __device__ bool walk_registers(int D, int nb, int mc, const int32_t *uE, const i
         kk = static_cast<int>(k64 & 1023u);
         named_bar(1, 32 * D);  // M and q have been read
       }
-      if (kk == k) {
-        const uint32_t p = static_cast<uint32_t>(c.x), u = static_cast<uint32_t>(c.y);
-        if (lane == 0) {
-          choice[j] = kk;
-          if (headroom) headroom[j] = static_cast<long long>(cap) - (static_cast<long long>(p) + 1 + M);
-          if (n == 32 * kS) w.over = 1;
-        }
-#pragma unroll
-        for (int s = 0; s < kS; ++s) {
-          if (e[s] - 1u < u) V[s] += p + e[s];
-          if (n == 32 * s + lane) {
-            e[s] = u;
-            b[s] = p + 1u;
-            V[s] = P + p + u;
-          }
-        }
-        n += 1;
-        // the largest new cell, K + p + t + 1, is M + p + 1
-        bad |= q == 0x7fffffff || static_cast<long long>(p) + 1 + M > 0x7fffffffLL;
-        q += q == 0x7fffffff ? 0 : 1;
-      }
-    } else if (threadIdx.x == 0) {
-      bad = true;
-      choice[j] = -1;
-      if (headroom) headroom[j] = 0;
     }
-    score(c1, (j + 1) & 1);
-    c = c1;
+    if (kk == k) {
+      const int2 c = cp[-1];
+      const uint32_t p = static_cast<uint32_t>(c.x), u = static_cast<uint32_t>(c.y);
+#pragma unroll
+      for (int s = 0; s < kS; ++s) {
+        if (e[s] - 1u < u) V[s] += p + e[s];
+        if (n == 32 * s + lane) {
+          e[s] = u;
+          b[s] = p + 1u;
+          V[s] = P + p + u;
+        }
+      }
+      n += 1;  // past 32 kS: a list that did not fit
+      // the largest new cell, K + p + t + 1, is M + p + 1
+      bad |= q == 0x7fffffff || M + p > 0x7ffffffeu || M + p < M;
+      q += q == 0x7fffffff ? 0 : 1;
+      fkey = feasible_key();
+    }
+    score(c1, next);
+    if (k == 0) {  // every warp knows the choices: the first one keeps and writes them
+      kept = lane == (j & 31) ? kk : kept;
+      if ((j & 31) == 31 || j == nb - 1) {
+        if ((j & ~31) + lane <= j) choice[(j & ~31) + lane] = kept;
+      }
+    }
+    uint32_t *const t = now;
+    now = next;
+    next = t;
     named_bar(1, 32 * D);
   }
+  if (n > 32 * kS) w.over = 1;
   __syncthreads();
   const bool ok = w.over == 0;
   if (ok && lane == 0) s_q[k] = q;
@@ -1296,11 +1309,11 @@ dispatch_block(unsigned char *sdm, int D, int H, int nb, int mc, const int64_t *
   }
   __syncthreads();
 
-  // At most 32 decoders: a warp each, with the lists in registers; a list that
+  // At most 32 decoders and no headroom output: a warp each, with the lists in registers; a list that
   // outgrows a variant moves on to the next, the last one below.
   __shared__ WalkShared walk;
   bool walked = s_fast != 0;
-  if (!walked && D <= 32) {
+  if (!walked && D <= 32 && headroom == nullptr) {
     int nmax = 0;
     for (int k = 0; k < D; ++k) nmax = max(nmax, s_n[k]);
     const int about = nmax + 2 * nb / D;
@@ -1314,7 +1327,7 @@ dispatch_block(unsigned char *sdm, int D, int H, int nb, int mc, const int64_t *
     bool wbad = false;
     auto go = [&](auto walk_fn) {
       wbad = false;
-      walked = walk_fn(D, nb, mc, uE, uB, s_base, s_n, s_q, s_cap, cand, choice, headroom, walk, wbad);
+      walked = walk_fn(D, nb, mc, uE, uB, s_base, s_n, s_q, s_cap, cand, choice, walk, wbad);
       __syncthreads();
     };
     if (about <= 32) go(walk_registers<1>);
