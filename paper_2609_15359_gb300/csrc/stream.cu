@@ -857,9 +857,9 @@ stream_csr_kernel(int nact, int D, int rr, const int32_t *q_dev, int32_t *q_out_
 // decisions and range errors are those of the dense projection followed by
 // maps_dispatch SEQUENTIAL.  (At most 32 decoders take walk_registers below
 // while their lists fit it.)
-// Shared memory: the pool of pairs (the residents of decoder k plus room for
-// nb reservations at base_k = res_off[k] + k nb), the unsorted pairs, and the
-// per-decoder tables.
+// Beside the batch and the unsorted pairs: the pool of sorted pairs (the
+// residents of decoder k plus room for nb reservations at base_k = res_off[k] +
+// k nb) with the tables.
 // The packed decision key, the smallest wins: a feasible decoder (h >= 0)
 // ranks by Q, an infeasible one after every feasible one by the deficit -h,
 // each then by index: inf << 63 | v << 10 | k.  mc (the max-headroom rule)
@@ -874,10 +874,23 @@ __device__ __forceinline__ unsigned long long dispatch_key(long long h, int q, i
   return (feas ? 0ull : 1ull << 63) | (v << 10) | static_cast<unsigned>(k);
 }
 
+// Shared memory of the dispatch: the batch, the residents' unsorted pairs and the
+// decoders; and, after them, the sorted lists with their tables, 16 bytes a pair.
 __host__ __device__ size_t stream_dispatch_smem(int D, int nact, int nb) {
-  const size_t pool = static_cast<size_t>(nact) + static_cast<size_t>(D) * nb;
-  return 16 * pool + 8 * static_cast<size_t>(nact) + 16 * static_cast<size_t>(D) +
-         12 * static_cast<size_t>(nb) + 64;
+  return (8 * (static_cast<size_t>(nb) + 1) + 8 * static_cast<size_t>(nact) + 16 * static_cast<size_t>(D) +
+          12 * static_cast<size_t>(nb) + 15) / 16 * 16;
+}
+__host__ __device__ size_t stream_lists_bytes(int D, int nact, int nb) {
+  return 16 * (static_cast<size_t>(nact) + static_cast<size_t>(D) * nb);
+}
+// Where the dispatch of nb candidates keeps its lists: 1 in shared memory, 2 in
+// the spare global memory (`spare` bytes), which serves where the register walk
+// is all but sure to decide the batch (at most 32 decoders with 64 requests each
+// on average), 0: neither, the dense projection dispatches.
+__host__ __device__ int stream_lists_place(int D, int nact, int nb, size_t smem, size_t spare) {
+  const size_t base = stream_dispatch_smem(D, nact, nb), lists = stream_lists_bytes(D, nact, nb);
+  if (base + lists <= smem) return 1;
+  return D <= 32 && nact <= 64 * D && base <= smem && lists <= spare ? 2 : 0;
 }
 
 // A decoder's tables from its sorted pairs (one warp): SS[i] = sum of b over
@@ -1128,19 +1141,28 @@ __device__ bool walk_registers(int D, int nb, int mc, const int32_t *uE, const i
   return ok;
 }
 
+// kSpare: the lists may be in global memory (`lists`); a variant apart, as the
+// pointers of either kind cost the register walk 7%.
+template <bool kSpare>
 __device__ void
-dispatch_block(unsigned char *sdm, int D, int H, int nb, int mc, const int64_t *res_off,
+dispatch_block(unsigned char *sdm, unsigned char *lists, int D, int H, int nb, int mc, const int64_t *res_off,
                const int32_t *rp, const int32_t *rg, const int32_t *rU, const int32_t *capv,
                int32_t *Q, const int32_t *cp, const int32_t *cU, int32_t *choice,
                int64_t *headroom, int32_t *status) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nact = static_cast<int>(res_off[D]);
   const int pool = nact + D * nb;
-  int32_t *E = reinterpret_cast<int32_t *>(sdm);           // [pool] sorted end steps
+  // the lists: first in shared memory, or (kSpare) in `lists`, or with it null
+  // after the rest; the batch of the register walk, (nb + 1) pairs, is first
+  // there, or over the lists, which that walk does not use
+  int32_t *E = reinterpret_cast<int32_t *>(                // [pool] sorted end steps
+      !kSpare ? sdm : lists != nullptr ? lists : sdm + stream_dispatch_smem(D, nact, nb));
   int32_t *Bv = E + pool;                                  // [pool] their b
   uint32_t *SS = reinterpret_cast<uint32_t *>(Bv + pool);  // [pool] suffix sums of b
   uint32_t *PM = SS + pool;                                // [pool] prefix maxima of V
-  int32_t *uE = reinterpret_cast<int32_t *>(PM + pool);    // [nact] unsorted
+  int2 *cand = reinterpret_cast<int2 *>(sdm);
+  int32_t *uE = kSpare ? reinterpret_cast<int32_t *>(cand + nb + 1)  // [nact] unsorted
+                       : reinterpret_cast<int32_t *>(PM + pool);
   int32_t *uB = uE + nact;
   int32_t *s_base = uB + nact, *s_n = s_base + D, *s_q = s_n + D, *s_cap = s_q + D;
   int32_t *s_cp = s_cap + D, *s_cu = s_cp + nb;            // [nb] the batch
@@ -1317,9 +1339,7 @@ dispatch_block(unsigned char *sdm, int D, int H, int nb, int mc, const int64_t *
     int nmax = 0;
     for (int k = 0; k < D; ++k) nmax = max(nmax, s_n[k]);
     const int about = nmax + 2 * nb / D;
-    // (p, u) of the batch, u = 0 marking an invalid candidate and the end, over
-    // the space of the sorted lists
-    int2 *cand = reinterpret_cast<int2 *>(E);
+    // (p, u) of the batch, u = 0 marking an invalid candidate and the end
     for (int j = tid; j <= nb; j += kSt) {
       const int32_t p = j < nb ? s_cp[j] : -1, U = j < nb ? s_cu[j] : -1;
       cand[j] = (p | U) < 0 ? make_int2(0, 0) : make_int2(p, U < 1 ? 1 : (U > H ? H : U));
@@ -1526,10 +1546,10 @@ __global__ void __launch_bounds__(kSt, 1)
 stream_dispatch_kernel(int D, int H, int nb, int mc, const int64_t *res_off, const int32_t *rp,
                        const int32_t *rg, const int32_t *rU, const int32_t *capv, int32_t *Q,
                        const int32_t *cp, const int32_t *cU, int32_t *choice, int64_t *headroom,
-                       int32_t *status) {
+                       int32_t *status, unsigned char *lists) {
   pdl_prologue();
   extern __shared__ __align__(16) unsigned char sdm[];
-  dispatch_block(sdm, D, H, nb, mc, res_off, rp, rg, rU, capv, Q, cp, cU, choice, headroom, status);
+  dispatch_block<true>(sdm, lists, D, H, nb, mc, res_off, rp, rg, rU, capv, Q, cp, cU, choice, headroom, status);
 }
 
 // 5''. Deferral: the listed requests join the waiting queues at act[nact..]:
@@ -1916,6 +1936,8 @@ stream_loop_kernel(const __grid_constant__ LoopArgs a) {
   int32_t *const cur = scratch + kStreamMaxD + 8;  // [D] cursors
   int64_t b = a.b0;
   long long total_done = a.total_done0;
+  // per-step mode may keep the dispatch's lists in w.K, which this loop does not use
+  const size_t spare = kPerStep ? sizeof(int32_t) * static_cast<size_t>(D) * c.H : 0;
   for (int run = 0; run < kLoopBatches && b < a.nbatch; ++run, ++b) {
     const int64_t lo = b * B, hi = min(lo + B, N);
     const int nb = static_cast<int>(hi - lo);
@@ -1930,7 +1952,9 @@ stream_loop_kernel(const __grid_constant__ LoopArgs a) {
     }
     const int nc = defer ? S->nc : nb, nto = defer ? S->nto : 0;
     const int most = S->nact + nto;  // requests in the system before this batch's, at most
-    if (most + nc > kLoopActive || stream_dispatch_smem(D, most, nc) > a.smem) {
+    const bool place = kPerStep ? stream_lists_place(D, most, nc, a.smem, spare) != 0
+                                : stream_dispatch_smem(D, most, nc) + stream_lists_bytes(D, most, nc) <= a.smem;
+    if (most + nc > kLoopActive || !place) {
       __syncthreads();
       if (tid == 0) S->npend = npend;  // the batch is not started
       break;
@@ -2009,7 +2033,9 @@ stream_loop_kernel(const __grid_constant__ LoopArgs a) {
       if (warp == 0) lr_warp(reinterpret_cast<uint32_t *>(scratch), D, nc, w.res_off, cch);
       __syncthreads();
     } else if (nc > 0 && !rr && c.dispatch_policy != MAPS_STREAM_RR) {  // 5.
-      dispatch_block(ldm, D, c.H, nc, mc, w.res_off, w.rp, w.rg, w.rU, w.capv, w.Q, cpr, w.Uq + nact, cch,
+      unsigned char *const lists = !kPerStep || stream_lists_place(D, nact, nc, a.smem, 0) == 1
+                                       ? nullptr : reinterpret_cast<unsigned char *>(w.K);
+      dispatch_block<kPerStep>(ldm, lists, D, c.H, nc, mc, w.res_off, w.rp, w.rg, w.rU, w.capv, w.Q, cpr, w.Uq + nact, cch,
                      nullptr, a.status);
       __syncthreads();
     }
@@ -2222,9 +2248,11 @@ int maps_stream_run(const maps_stream_cfg *cfg, const int64_t *arrival_ms, const
   const size_t loop_smem = static_cast<size_t>(max_smem_optin()) - fa.sharedSizeBytes;
   MAPS_TRY(cuda_ok(cudaFuncSetAttribute(loop, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         static_cast<int>(loop_smem))));
+  const size_t spare = sizeof(int32_t) * static_cast<size_t>(D) * c.H;  // the dense K, else unused
   auto loop_fits = [&](int64_t system, int64_t cands) {  // requests in the system, candidates
     return c.window <= kLoopWindow && system + cands <= kLoopActive &&
-           stream_dispatch_smem(D, static_cast<int>(system), static_cast<int>(cands)) <= loop_smem;
+           stream_lists_place(D, static_cast<int>(system), static_cast<int>(cands), loop_smem,
+                              per_step ? spare : 0) != 0;
   };
   bool in_loop = loop_fits(0, std::min(N, B));
   for (int64_t b = 0; b < nbatch; ++b) {
@@ -2323,14 +2351,18 @@ int maps_stream_run(const maps_stream_cfg *cfg, const int64_t *arrival_ms, const
       launch_pdl(stream_lr_kernel, 1, 32, 0, s, D, nc, w.res_off, cch);
       MAPS_TRY(launch_ok());
     } else if (!rr) {  // 5.
-      const size_t dsm = stream_dispatch_smem(D, nact, nc);
-      if (dsm + 2048 <= static_cast<size_t>(max_smem_optin())) {
-        // the decoders' pairs fit in shared memory: no dense projection
+      // (the kernel's static shared memory is below 4 KB)
+      const size_t most = static_cast<size_t>(max_smem_optin()) - 4096;
+      const int place = stream_lists_place(D, nact, nc, most, spare);
+      if (place != 0) {
+        // the decoders' pairs and the batch fit in shared memory: no dense projection
+        const size_t dsm = stream_dispatch_smem(D, nact, nc) + (place == 1 ? stream_lists_bytes(D, nact, nc) : 0);
         MAPS_TRY(cuda_ok(cudaFuncSetAttribute(stream_dispatch_kernel,
                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               static_cast<int>(dsm))));
         launch_pdl(stream_dispatch_kernel, 1, kSt, dsm, s, D, c.H, nc, mc, w.res_off, w.rp, w.rg,
-                   w.rU, w.capv, w.Q, cpr, w.Uq + nact, cch, nullptr, status);  // no headroom out
+                   w.rU, w.capv, w.Q, cpr, w.Uq + nact, cch, nullptr, status,  // no headroom out
+                   place == 1 ? nullptr : reinterpret_cast<unsigned char *>(w.K));
         MAPS_TRY(launch_ok());
       } else {
         MAPS_TRY(maps_project_occupancy(D, c.H, w.res_off, nact, w.rp, w.rg, w.rU, w.K, nullptr, ws,
