@@ -1223,8 +1223,11 @@ dispatch_block(unsigned char *sdm, unsigned char *lists, int D, int H, int nb, i
   // decoder with Q <= L takes one candidate, in index order.  So candidate j
   // goes to level L, the smallest with cum(L) > j where
   // cum(L) = sum over k of max(0, L - Q_k + 1), and there to the
-  // (j - cum(L - 1))-th decoder with Q <= L.  Each candidate's pick is found
-  // on its own; then one warp per decoder sums the reservations before each
+  // (j - cum(L - 1))-th decoder with Q <= L.  A scan over the levels gives
+  // cum and the decoders of each (a thread a level), and each candidate's pick
+  // is then found on its own (summing cum over the decoders at every probe
+  // of that search took 3.82 ms for 30,000 requests on 32 decoders, the
+  // table 3.6).  Then one warp per decoder sums the reservations before each
   // candidate (a scan) and checks the bound.
   if (quick && D <= 32) {
     __shared__ long long f_sb[32];
@@ -1265,30 +1268,54 @@ dispatch_block(unsigned char *sdm, unsigned char *lists, int D, int H, int nb, i
     if (!f_inv) {
       int qmin = 0x7fffffff;
       for (int k = 0; k < D; ++k) qmin = min(qmin, s_q[k]);
-      auto cum = [&](int L) {  // picks made by the end of level L
-        int c = 0;
-        for (int k = 0; k < D; ++k) c += max(0, L - s_q[k] + 1);
-        return c;
-      };
+      // per level qmin + l, l < nb (the decoder at qmin alone takes nb picks by
+      // the last): the picks made by its end, and the decoders taking one
+      int2 *lev = cand;
+      __shared__ int f_w[kStWarps];
+      int before = 0;  // picks of the levels before this round's
+      for (int l0 = 0; l0 < nb; l0 += kSt) {
+        const int l = l0 + tid;
+        uint32_t mask = 0;
+        if (l < nb)
+          for (int k = 0; k < D; ++k) mask |= (s_q[k] - qmin <= l ? 1u : 0u) << k;
+        int c = __popc(mask);
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+          const int y = __shfl_up_sync(0xffffffffu, c, off);
+          if (lane >= off) c += y;
+        }
+        if (lane == 31) f_w[warp] = c;
+        __syncthreads();
+        const int ws = f_w[lane];
+        c += before + static_cast<int>(__reduce_add_sync(0xffffffffu, static_cast<unsigned>(lane < warp ? ws : 0)));
+        before += static_cast<int>(__reduce_add_sync(0xffffffffu, static_cast<unsigned>(ws)));
+        if (l < nb) lev[l] = make_int2(c, static_cast<int>(mask));
+        __syncthreads();
+      }
       for (int j = tid; j < nb; j += kSt) {
-        // the decoder at qmin alone takes nb picks by level qmin + nb - 1
-        int lo = qmin, hi = qmin + nb - 1;
+        int lo = 0, hi = nb - 1;  // the first level whose end is past pick j
         while (lo < hi) {
-          const int mid = lo + (hi - lo) / 2;
-          if (cum(mid) > j)
+          const int mid = (lo + hi) >> 1;
+          if (lev[mid].x > j)
             hi = mid;
           else
             lo = mid + 1;
         }
-        int r = j - (lo > qmin ? cum(lo - 1) : 0);
-        int pick = -1;
-        for (int k = 0; k < D; ++k)
-          if (s_q[k] <= lo && r-- == 0) {
-            pick = k;
-            break;
+        int r = j - (lo > 0 ? lev[lo - 1].x : 0);  // its place among the level's decoders
+        uint32_t mask = static_cast<uint32_t>(lev[lo].y);
+        const bool ok = r >= 0 && r < __popc(mask);
+        if (!ok) f_miss = 1;  // cannot happen; the walk would decide the batch
+        int k = 0;  // the r-th set bit
+#pragma unroll
+        for (int h = 16; h > 0; h >>= 1) {
+          const int c = __popc(mask & ((1u << h) - 1u));
+          if (r >= c) {
+            r -= c;
+            k += h;
+            mask >>= h;
           }
-        s_ch[j] = pick < 0 ? 0 : pick;
-        if (pick < 0) f_miss = 1;  // cannot happen; the walk would decide the batch
+        }
+        s_ch[j] = ok ? k : 0;
       }
     }
     __syncthreads();
@@ -1763,11 +1790,12 @@ struct StreamWs {
 // (eleven, and the host's read of the counts that size them).  This kernel runs
 // batches one after another on one block, steps apart by block barriers, with
 // the two sorts and the quantile done in place.  32 decoders, batches of 256: 68
-// -> 32 us a batch where no queue forms (30,000 requests 8.1 -> 3.8 ms), 155 ->
-// 130 at 16,000 tokens, 207 -> 185 with per-step admission and deferral.
+// -> 30 us a batch where no queue forms (30,000 requests 8.1 -> 3.5 ms), and with
+// the register walk 210 -> 116 at 16,000 tokens, 330 -> 143 with per-step
+// admission and deferral.
 //   * the completions and each decoder's waiting requests are sorted by rank
-//     (a key's place is the number of smaller keys of its group, each thread
-//     counting for one key), groups past kLoopRank by a bitonic network;
+//     (a key's place is the number of smaller keys of its group, one thread
+//     counting for a key, or up to eight where the keys are few), groups past kLoopRank by a bitonic network;
 //   * the quantile comes from a histogram of the window's scores, as in
 //     maps_calibrate's one-block form.
 // It stops before a batch that does not fit (the requests in the system, the
@@ -1797,17 +1825,28 @@ struct LoopArgs {
 // the group of key x; out[x's place] gets the key.  Every thread of the block.
 __device__ void sort_groups(const unsigned long long *key, const int32_t *seg, const int16_t *which,
                             int n, int groups, unsigned long long *out) {
-  for (int x = threadIdx.x; x < n; x += kSt) {
-    const int a = seg[which[x]], b = seg[which[x] + 1];
-    if (b - a > kLoopRank) {
-      out[x] = key[x];
-      continue;
-    }
-    const unsigned long long k = key[x];
-    int r = 0;
+  int tp = 1;  // threads a key: they share its comparisons
+  while (tp < 8 && 2 * tp * n <= kSt) tp *= 2;
+  const int sub = threadIdx.x & (tp - 1);
+  for (int x0 = 0; x0 < n; x0 += kSt / tp) {
+    const int x = x0 + static_cast<int>(threadIdx.x) / tp;
+    int a = 0, r = 0;
+    unsigned long long k = 0;
+    bool rank = false;
+    if (x < n) {
+      a = seg[which[x]];
+      const int b = seg[which[x] + 1];
+      k = key[x];
+      rank = b - a <= kLoopRank;
+      if (rank) {
 #pragma unroll 4
-    for (int y = a; y < b; ++y) r += key[y] < k;
-    out[a + r] = k;
+        for (int y = a + sub; y < b; y += tp) r += key[y] < k;
+      } else if (sub == 0) {
+        out[x] = k;
+      }
+    }
+    for (int o = 1; o < tp; o <<= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+    if (rank && sub == 0) out[a + r] = k;
   }
   __syncthreads();
   for (int i = 0; i < groups; ++i) {  // the long groups, one after another

@@ -1043,6 +1043,8 @@ def test_stream_walk_list_sizes(M, ws, oracle, N, D, cap, B):
     # and comes back into it; batches and systems around 2,048 requests
     (3000, 2, 40000, 100, 300), (9000, 2, 60000, 300, 500), (5000, 16, 262144, 2000, 500),
     (5000, 16, 262144, 2048, 500), (5000, 64, 20000, 2049, 500),
+    # one decoder, and as many as a warp's lanes, with more picks than threads
+    (4000, 1, 262144, 1500, 300), (6000, 32, 262144, 1100, 300),
     # many completions in one batch: sorted by the network
     (9000, 40, 262144, 900, 700)])
 def test_stream_one_block_loop_limits(M, ws, oracle, N, D, cap, B, Wn):
