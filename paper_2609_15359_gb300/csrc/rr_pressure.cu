@@ -28,12 +28,17 @@
 // round is ~0: the next completion is one 32-bit warp minimum, a completion clears
 // its slots and an admission fills the first free one.  The head of the queue
 // is held in every lane, the next 64 requests one per lane; the waiting
-// statistics are gathered at the admissions.  64 draws x 6 utilisations of
-// 10,000 requests on 4 decoders (1,536 streams): 4.10 -> 1.91 ms; before, the set
-// sat in shared memory and was compacted at every completion, with 64-bit
-// shuffle reductions and a 64-bit division an event, and the waiting statistics
-// took a second pass with a binary search a request.  (Four slots a lane for
-// every stream, 64-bit positions: 2.16 ms.)
+// statistics are gathered at the admissions.  Every load is a window ahead of
+// its use, the round boundary comes from a multiplication by the reciprocal of
+// a round and a remainder, tokens and loop counts are 32-bit.  64 draws x 6
+// utilisations of 10,000 requests on 4 decoders (1,536 streams): 4.10 -> 1.70
+// ms (1.91 with a division an event, waits for the windows' loads and 64-bit
+// counts); before, the set sat in shared memory and was compacted at every
+// completion, with 64-bit shuffle reductions and a 64-bit division an event, and
+// the waiting statistics took a second pass with a binary search a request.
+// (Four slots a lane for every stream, 64-bit positions: 2.16 ms.  The free
+// lanes kept as a mask, the next head shuffled ahead of its use, or a lone
+// completion's footprint by shuffle instead of the sum: 0 to 5% slower each.)
 // A stream that comes to run more than 64 (then 256) requests at once starts
 // over on the next variant, the last one with its running set in shared memory.
 #include "maps_internal.cuh"
@@ -100,6 +105,7 @@ struct RRSim {
 template <int kSlots>
 __device__ bool RRSim::run_registers() {
   constexpr unsigned kAll = 0xffffffffu;
+  constexpr int64_t kNever = INT64_MAX;
   const int lane = threadIdx.x & 31;
   uint32_t fin[kSlots];
   int32_t m[kSlots], pos[kSlots];
@@ -108,40 +114,53 @@ __device__ bool RRSim::run_registers() {
     fin[i] = ~0u;
     m[i] = pos[i] = 0;
   }
-  // lane l: requests wb + l and wb + 32 + l (the second in flight)
+  // lane l: requests wb + l and wb + 32 + l (the second in flight); past the
+  // last one the arrival is kNever, so it is neither admitted nor waited for
   const int n = static_cast<int>(n_d);
-  int64_t wa = 0, na = 0;
-  int32_t wm = 0, wo = 0, nm = 0, no = 0;
-  auto load = [&](int s, int64_t &a, int32_t &fm, int32_t &o) {
+  const int32_t tok_us = static_cast<int32_t>(tok), stride = 8 * N;
+  const uint32_t cap = static_cast<uint32_t>(C), hp = static_cast<uint32_t>(K_hp);
+  const int64_t *const Ad = A + d;
+  int64_t wa = kNever, na = kNever;
+  int32_t wp = 0, wo = 0, np = 0, no = 0;
+  auto load = [&](int s, int64_t &a, int32_t &p, int32_t &o) {
+    a = kNever;
     if (s < n) {
-      const int64_t i = d + static_cast<int64_t>(s) * N;
-      a = A[i];
-      o = O[i];
-      fm = P[i] + o;
+      const int64_t i = static_cast<int64_t>(s) * N;
+      a = Ad[i];
+      o = O[d + i];
+      p = P[d + i];
     }
   };
   int wi = 0;  // the head's lane
-  load(lane, wa, wm, wo);
-  load(32 + lane, na, nm, no);
+  load(lane, wa, wp, wo);
+  load(32 + lane, na, np, no);
   // arrivals counted for the longest queue: those before index ab all arrived
-  // before the last admission; lane l holds arrival ab + l
+  // before the last admission; lane l holds arrivals ab + l and ab + 32 + l
+  auto arrival = [&](int s) { return s < n ? Ad[static_cast<int64_t>(s) * N] : kNever; };
   int ab = 0;
-  int64_t aa = lane < n ? A[d + static_cast<int64_t>(lane) * N] : INT64_MAX;
-  int64_t t = n > 0 ? A[d] : 0, K = 0, t_s = 0;
-  int64_t *adm_h = adm + d;  // the head's admission time
-  uint32_t R = 0;
+  int64_t aa = arrival(lane), ab2 = arrival(32 + lane);
+  int64_t t = n > 0 ? Ad[0] : 0, t_s = 0;
+  char *adm_h = reinterpret_cast<char *>(adm + d);  // the head's admission time
+  char *const dn_d = reinterpret_cast<char *>(dn + d);
+  uint32_t R = 0, K = 0;
+  uint32_t f = ~0u;  // the smallest finishing round
   int qh = 0, n_run = 0, qm = 0;
   bool in_hp = false;
   int64_t ha = __shfl_sync(kAll, wa, 0);
-  int32_t hm = __shfl_sync(kAll, wm, 0), ho = __shfl_sync(kAll, wo, 0);
+  int32_t ho = __shfl_sync(kAll, wo, 0);
+  uint32_t hm = static_cast<uint32_t>(__shfl_sync(kAll, wp, 0) + ho);
+  // 1 / (lane + 1) steps of one token, for running sets up to 32
+  const float inv = 1.0f / (static_cast<float>(lane + 1) * static_cast<float>(tok_us));
   // every iteration admits, completes, or reaches an arrival's round boundary
-  for (int64_t left = 4 * n_d + 16; left > 0; --left) {
-    // admissions at t: the FIFO head while it has arrived and fits
-    while (ha <= t && K + hm <= C && qh < n) {
+  for (uint32_t left = 4u * static_cast<uint32_t>(n) + 16u; left > 0; --left) {
+    // admissions at t: the FIFO head while it has arrived and fits (K and a
+    // footprint are at most C < 2^31)
+    while (ha <= t && K + hm <= cap) {
       if (R > 0x7fffffffu - static_cast<uint32_t>(ho)) {
         fail = true;
         return true;
       }
+      const uint32_t fh = R + static_cast<uint32_t>(ho);
       bool placed = false;
 #pragma unroll
       for (int i = 0; i < kSlots; ++i) {
@@ -150,19 +169,21 @@ __device__ bool RRSim::run_registers() {
         if (free_lanes == 0) continue;
         placed = true;
         const bool me = lane == __ffs(free_lanes) - 1;
-        fin[i] = me ? R + static_cast<uint32_t>(ho) : fin[i];
-        m[i] = me ? hm : m[i];
+        fin[i] = me ? fh : fin[i];
+        m[i] = me ? static_cast<int32_t>(hm) : m[i];
         pos[i] = me ? qh : pos[i];
       }
       if (!placed) return false;
-      if (lane == 0) *adm_h = t;
-      adm_h += N;
+      f = min(f, fh);
+      if (lane == 0) *reinterpret_cast<int64_t *>(adm_h) = t;
+      adm_h += stride;
       // the requests that arrived before t and are not admitted before this one
       wait += t - ha;
       unsigned before;
       while ((before = __ballot_sync(kAll, aa < t)) == kAll) {
         ab += 32;
-        aa = ab + lane < n ? A[d + static_cast<int64_t>(ab + lane) * N] : INT64_MAX;
+        aa = ab2;
+        ab2 = arrival(ab + 32 + lane);
       }
       qm = max(qm, ab + __popc(before) - qh);
       ++n_run;
@@ -170,32 +191,41 @@ __device__ bool RRSim::run_registers() {
       ++qh;
       if (++wi == 32) {
         wi = 0;
-        wa = na, wm = nm, wo = no;
-        load(qh + 32 + lane, na, nm, no);
+        wa = na, wp = np, wo = no;
+        load(qh + 32 + lane, na, np, no);
       }
       ha = __shfl_sync(kAll, wa, wi);
-      hm = __shfl_sync(kAll, wm, wi);
       ho = __shfl_sync(kAll, wo, wi);
+      hm = static_cast<uint32_t>(__shfl_sync(kAll, wp, wi) + ho);
     }
-    if ((K >= K_hp) != in_hp) pressure(!in_hp, t, in_hp, t_s);
+    if ((K >= hp) != in_hp) pressure(!in_hp, t, in_hp, t_s);
     if (n_run == 0) {
       if (qh >= n) break;
       t = ha;  // idle until the head arrives (it fits an empty decoder)
       continue;
     }
     // next event: the first completion, or the boundary where the head arrives
-    uint32_t f = fin[0];
-#pragma unroll
-    for (int i = 1; i < kSlots; ++i) f = min(f, fin[i]);
-    f = __reduce_min_sync(kAll, f);
-    const int64_t step = static_cast<int64_t>(n_run) * tok;
+    const int64_t step = static_cast<int64_t>(n_run) * tok_us;
     const int64_t tc = static_cast<int64_t>(f - R) * step, gap = ha - t;
-    if (gap > 0 && gap < tc && qh < n) {
+    if (gap > 0 && gap < tc) {
       // rounds to the boundary, ceil(gap / step), at most f - R
-      const uint32_t k = ((gap | step) >> 31) == 0
-                             ? (static_cast<uint32_t>(gap) + static_cast<uint32_t>(step) - 1u) /
-                                   static_cast<uint32_t>(step)
-                             : static_cast<uint32_t>((gap + step - 1) / step);
+      uint32_t k;
+      if (((gap | step) >> 31) == 0) {
+        const uint32_t g = static_cast<uint32_t>(gap), st = static_cast<uint32_t>(step);
+        const float e = static_cast<float>(g) * __shfl_sync(kAll, inv, n_run - 1);
+        if (n_run <= 32 && e < 1e6f) {
+          // within one of the quotient: the factors' relative errors add up to
+          // less than 2^-21
+          k = static_cast<uint32_t>(e);
+          const int32_t rest = static_cast<int32_t>(g - k * st);
+          k += (rest > 0 ? 1 : 0) + (rest > static_cast<int32_t>(st) ? 1 : 0) -
+               (rest <= -static_cast<int32_t>(st) ? 1 : 0);
+        } else {
+          k = (g + st - 1u) / st;
+        }
+      } else {
+        k = static_cast<uint32_t>((gap + step - 1) / step);
+      }
       t += k * step;
       R += k;
     } else {
@@ -204,15 +234,18 @@ __device__ bool RRSim::run_registers() {
     }
     if (R == f) {  // completions
       uint32_t freed = 0, gone = 0;
+      f = ~0u;
 #pragma unroll
       for (int i = 0; i < kSlots; ++i) {
         const bool now = fin[i] == R;
-        if (now) dn[d + static_cast<int64_t>(pos[i]) * N] = t;
+        if (now) *reinterpret_cast<int64_t *>(dn_d + static_cast<int64_t>(pos[i]) * stride) = t;
         freed += now ? static_cast<uint32_t>(m[i]) : 0u;
         gone += now ? 1u : 0u;
         fin[i] = now ? ~0u : fin[i];
+        f = min(f, fin[i]);
       }
-      K -= __reduce_add_sync(kAll, freed);  // at most K <= C < 2^31
+      f = __reduce_min_sync(kAll, f);
+      K -= __reduce_add_sync(kAll, freed);
       n_run -= static_cast<int>(__reduce_add_sync(kAll, gone));
       t_last = t;
     }
@@ -409,7 +442,7 @@ rr_stream_kernel(int64_t n_real, int64_t n, int N, int64_t C, int64_t tok, uint3
   // the variant by the footprints a capacity holds on average, with room for
   // the spread; a set that turns out larger moves on to the next
   const int64_t about = C * n_d / (foot > 0 ? foot : 1);
-  const bool small = n_d <= 0x3fffffff;
+  const bool small = n_d <= 0x3ffffff0 && N < (1 << 28);  // what their 32-bit counts hold
   bool ran = small && about <= 44 && sim.run_registers<2>();
   if (!ran && small && about <= 200) {
     clear();

@@ -74,6 +74,19 @@ def test_rr_random(M, oracle, N, C, n, theta, tie):
     check(M, oracle, N, C, 1000, theta, arr, prompt, out)
 
 
+@pytest.mark.parametrize("tok", [1, 3, 33333, 1 << 20, (1 << 31) - 1])
+@pytest.mark.parametrize("most", [1, 31, 32, 33])
+def test_rr_round_boundaries(M, oracle, tok, most):
+    """Arrivals on a round boundary and one microsecond to either side of it,
+    near and thousands of rounds away (the quotient that finds the boundary)."""
+    rng = np.random.default_rng(tok % 1009 + most)
+    n = 12 * most + 40
+    out = rng.integers(1, 200_000, (2, n))
+    rounds = rng.choice([0, 1, 2, 7, 1000, 70_000], (2, n))
+    gaps = np.maximum(0, rounds * rng.integers(1, most + 1, (2, n)) * tok + rng.integers(-1, 2, (2, n)))
+    check(M, oracle, 1, 300_000 * most, tok, 850000, np.cumsum(gaps, axis=1), 300_000 - out, out)
+
+
 @pytest.mark.parametrize("most", [31, 32, 33, 63, 64, 65, 255, 256, 257, 400])
 def test_rr_running_set_sizes(M, oracle, most):
     """At most `most` requests run at once on a decoder (equal footprints):
