@@ -126,8 +126,9 @@ constexpr uint32_t kMergesUnsorted = 4200;
 static_assert(kSegMax % kMergeTile == 0, "merge tiles align with runs");
 
 // A long queue of at most kPairRuns chunks is ranked pairwise instead: for
-// every ordered pair of its sorted runs (A, B) one block counts, for each key
-// of A, the keys of B below it (the keys are unique); after one grid barrier
+// every two of its sorted runs (A, B) one block counts, for each key of A, the
+// keys of B below it, and for each of B those of A (the keys are unique), an
+// ordered pair each; after one grid barrier
 // a key's place in the queue is its place in A plus those counts.  The counts
 // are 16-bit, [pair][position in A]; the pairs a call may use are capped by
 // pair_budget(N), and a queue past the cap or past kPairRuns is merged.
@@ -188,6 +189,14 @@ __device__ __forceinline__ void warp_count(uint32_t *hist, int b, bool valid) {
 }
 
 __device__ __forceinline__ int bit_width(uint32_t x) { return x ? 32 - __clz(x) : 0; }
+
+// The sort items of fewer decoders than the plan has threads (one round of
+// them) are listed large ones first, those of more than kSegMax / 2 entries: the
+// sorting blocks take them in turn, so what runs last is small.  1,048,576
+// entries on 256 ragged queues, sort kernel: 35.4 -> 28 us cold (in decoder
+// order the busiest multiprocessor did 1.5 times the mean's work, now 1.2).
+// The two counts ride in one scan; sixteen classes with counters in shared
+// memory took the plan 2 us.
 
 // Segmented form, step 1 (one block, run by the last prep block): decoder
 // segment offsets, the sort items (a queue of at most kSegMax entries is one
@@ -1518,16 +1527,26 @@ __device__ void merge_level(int level, int ntiles, const int64_t *mt_off, const 
 // There may be hundreds of such queues (ragged queues just past kSegMax), so
 // their records are read into shared memory once, a pair finds its queue with
 // one look by every thread, and the keys of all of them are placed as one range
-// in which a key finds its queue by a binary search.  1,000,000 entries on 200
-// decoders (400 pairs), whole call: 294 -> 84 us; walking the records from
-// global memory, and one queue after another by blocks from 0 on, made up most
-// of it.  (In the pairs, consecutive keys a thread, each galloping on from the
-// one before: 42 against 36 us on 256 ragged queues, a serial chain instead of
-// independent searches.)
+// in which a key finds its queue by a binary search.  A block takes two runs
+// and merges them, each thread up to 18 outputs from its place on the merge
+// path on: a step decides one key and gives that key's count, where the run it
+// came from is kept as a bit, and the counts replace the keys in shared memory
+// once all are decided.  1,048,576 entries on 256 ragged queues (202 pairs of
+// runs), this kernel 28.4 -> 22 us cold; before, every key of either run took a
+// binary search of the other of its own, 13 probes instead of one.
+// 1,000,000 on 200 decoders (200 pairs), whole call: 294 us with the records
+// walked from global memory and one queue placed after another, 84 with the
+// searches, 67 now.
 constexpr int kPairQueues = 1024 / 2 + 1;
+union PairSmem {
+  unsigned long long key[2 * (kSegMax + 1)];  // run A, then run B from kSegMax + 1 on
+  uint4 cnt[2 * kSegMax / 8];                 // 16-bit counts of A's keys, then of B's
+};
+static_assert(kSegMax % 8 == 0, "counts are copied 16 bytes at a time");
+static_assert(2 * kSegIPT <= 32, "a thread's outputs are the bits of a word");
 __device__ void pair_rank_all(int64_t N, const OrderCounts *counts, const PairQueues &pq,
                               const unsigned long long *keys, int32_t *perm,
-                              unsigned long long *sB, GridBar *bar, int32_t *status) {
+                              PairSmem &sm, GridBar *bar, int32_t *status) {
   __shared__ int64_t s_off[kPairQueues];
   __shared__ int32_t s_n[kPairQueues], s_pair0[kPairQueues];
   __shared__ int32_t s_before[kPairQueues];  // entries of the queues before this one
@@ -1556,49 +1575,68 @@ __device__ void pair_rank_all(int64_t N, const OrderCounts *counts, const PairQu
     }
   }
   __syncthreads();
-  // (1) pair p = (queue q, runs A != B): for each key of A, the keys of B below it
-  for (int64_t p = blockIdx.x; p < npairs; p += gridDim.x) {
+  // (1) runs A < B of queue q, merged: for each key the other run's keys below it
+  for (int64_t u = blockIdx.x; u < npairs / 2; u += gridDim.x) {  // (reservations are even)
     if (threadIdx.x == 0) s_q = -1;
     __syncthreads();
-    for (int i = threadIdx.x; i < nq; i += blockDim.x) {  // the queue holding pair p
-      const int C = (s_n[i] + kSegMax - 1) / kSegMax;
-      if (p >= s_pair0[i] && p < s_pair0[i] + static_cast<int64_t>(C) * (C - 1)) s_q = i;
+    for (int i = threadIdx.x; i < nq; i += blockDim.x) {  // the queue holding pair u
+      const int C = (s_n[i] + kSegMax - 1) / kSegMax, u0 = s_pair0[i] / 2;
+      if (u >= u0 && u < u0 + C * (C - 1) / 2) s_q = i;
     }
     __syncthreads();
     const int q = s_q;
     if (q >= 0) {  // else a reservation no queue kept (uniform per block)
       const int64_t off = s_off[q];
       const int n = s_n[q], C = (n + kSegMax - 1) / kSegMax;
-      const int l = static_cast<int>(p - s_pair0[q]);
-      const int A = l / (C - 1), b = l % (C - 1), B = b < A ? b : b + 1;
+      int A = 0, l = static_cast<int>(u) - s_pair0[q] / 2;
+      while (l >= C - 1 - A) l -= C - 1 - A++;
+      const int B = A + 1 + l;
       const int nA = min(kSegMax, n - A * kSegMax), nB = min(kSegMax, n - B * kSegMax);
       const unsigned long long *rA = keys + off + static_cast<int64_t>(A) * kSegMax;
       const unsigned long long *rB = keys + off + static_cast<int64_t>(B) * kSegMax;
-      // a thread's keys are searched side by side (loads in flight together,
-      // the halving the same for all); ~0 past the run's end, never stored
-      unsigned long long key[kSegIPT];
-      int lo[kSegIPT];
 #pragma unroll
       for (int i = 0; i < kSegIPT; ++i) {
         const int x = i * kSegThreads + static_cast<int>(threadIdx.x);
-        if (x < nB) sB[x] = rB[x];
-        key[i] = x < nA ? rA[x] : ~0ull;
-        lo[i] = 0;
+        if (x < nA) sm.key[x] = rA[x];
+        if (x < nB) sm.key[kSegMax + 1 + x] = rB[x];
+      }
+      if (threadIdx.x == 0) sm.key[nA] = sm.key[kSegMax + 1 + nB] = ~0ull;  // above every key
+      __syncthreads();
+      const int per = (nA + nB + kSegThreads - 1) / kSegThreads;
+      const int d = static_cast<int>(threadIdx.x) * per, m = min(per, nA + nB - d);
+      // outputs [d, d + m) of the merge: bit i set where output i is A's
+      int ia0 = 0;
+      uint32_t of_a = 0;
+      if (m > 0) {
+        ia0 = merge_path(sm.key, nA, sm.key + kSegMax + 1, nB, d);
+        int ia = ia0, ib = d - ia0;
+        unsigned long long ka = sm.key[ia], kb = sm.key[kSegMax + 1 + ib];
+        for (int i = 0; i < m; ++i) {
+          const bool first = ka < kb;
+          of_a |= (first ? 1u : 0u) << i;
+          ia += first ? 1 : 0;
+          ib += first ? 0 : 1;
+          const unsigned long long next = sm.key[first ? ia : kSegMax + 1 + ib];
+          ka = first ? next : ka;
+          kb = first ? kb : next;
+        }
+      }
+      __syncthreads();  // the counts take the keys' place
+      uint16_t *const c16 = reinterpret_cast<uint16_t *>(sm.cnt);
+      for (int i = 0, ia = ia0, ib = d - ia0; i < m; ++i) {
+        const bool first = (of_a >> i) & 1u;
+        c16[first ? ia : kSegMax + ib] = static_cast<uint16_t>(first ? ib : ia);
+        ia += first ? 1 : 0;
+        ib += first ? 0 : 1;
       }
       __syncthreads();
-      for (int len = nB; len > 1; len -= len / 2) {  // keys of B below each key
-#pragma unroll
-        for (int i = 0; i < kSegIPT; ++i)
-          if (sB[lo[i] + len / 2 - 1] < key[i]) lo[i] += len / 2;
-      }
-      uint16_t *out = pq.cnt + p * kSegMax;
-#pragma unroll
-      for (int i = 0; i < kSegIPT; ++i) {
-        const int x = i * kSegThreads + static_cast<int>(threadIdx.x);
-        if (x < nA) out[x] = static_cast<uint16_t>(lo[i] + (sB[lo[i]] < key[i] ? 1 : 0));
-      }
+      // whole words: what lies past a run's end stays in its row and is not read
+      uint4 *const outA = reinterpret_cast<uint4 *>(pq.cnt + (s_pair0[q] + A * (C - 1) + B - 1) * static_cast<int64_t>(kSegMax));
+      uint4 *const outB = reinterpret_cast<uint4 *>(pq.cnt + (s_pair0[q] + B * (C - 1) + A) * static_cast<int64_t>(kSegMax));
+      for (int x = threadIdx.x; x < (nA + 7) / 8; x += kSegThreads) outA[x] = sm.cnt[x];
+      for (int x = threadIdx.x; x < (nB + 7) / 8; x += kSegThreads) outB[x] = sm.cnt[kSegMax / 8 + x];
     }
-    __syncthreads();  // sB and s_q serve the next pair
+    __syncthreads();  // the shared memory serves the next pair
   }
   if (!grid_barrier(bar, status, g_lookback_spins)) return;
   // (2) each key's place: its place in its run plus its counts in the others
@@ -1833,7 +1871,7 @@ order_finish_kernel(int n_hi, int64_t N, int D, int dbits, const OrderCounts *co
   if (*reinterpret_cast<const volatile uint32_t *>(&counts->segmented)) {
     if (counts->npairq > 0) {
       extern __shared__ __align__(16) unsigned char pair_raw[];
-      pair_rank_all(N, counts, pq, keyA, perm, reinterpret_cast<unsigned long long *>(pair_raw), bar, status);
+      pair_rank_all(N, counts, pq, keyA, perm, *reinterpret_cast<PairSmem *>(pair_raw), bar, status);
     }
     if (counts->nmtiles > 0) merge_all(N, counts, mt_off, mt_n, mt_t, keyA, keyB, perm, bar, status);
     return;
@@ -1884,8 +1922,7 @@ order_finish_kernel(int n_hi, int64_t N, int D, int dbits, const OrderCounts *co
 }
 
 static_assert(kPassThreads == kSegThreads, "a pair's keys are kSegIPT a thread");
-static_assert(sizeof(PassSmem) >= kSegMax * sizeof(unsigned long long),
-              "one sorted run fits the finishing kernel's shared memory");
+constexpr size_t kFinishSmem = sizeof(PassSmem) > sizeof(PairSmem) ? sizeof(PassSmem) : sizeof(PairSmem);
 
 // Blocks of the finishing kernel that can be resident at once (its grid limit
 // as a cooperative launch).
@@ -2066,7 +2103,7 @@ int maps_order_local(int64_t N, int32_t D, const int32_t *dec, const int32_t *bo
                                              2LL * sms);
   launch_pdl(order_segsort_kernel, static_cast<unsigned>(seg_grid), kSegThreads, seg_smem, s, N,
              w.counts, w.item_off, w.item_n, w.hi_orig, perm_out, w.keyA, bv);
-  const size_t smem = sizeof(PassSmem);
+  const size_t smem = kFinishSmem;
   MAPS_TRY(cuda_ok(cudaFuncSetAttribute(order_finish_kernel,
                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         static_cast<int>(smem))));

@@ -775,6 +775,30 @@ def test_order_shuffled_arrival_forms(M, ws, oracle, N, D, ubits, abits, skew):
     assert np.array_equal(seg, so)
 
 
+@pytest.mark.parametrize("sizes,D", [
+    # runs of 4,608 ranked pairwise: one entry past a run, whole runs, the most
+    # runs (16), and a queue past them merged by levels beside ranked ones
+    ([4609], 1), ([9216], 1), ([9217, 0, 4608, 1, 13823], 5), ([73728], 2), ([73729, 5000, 9000], 4),
+    # the last run within, and at, one and two outputs a thread
+    ([4608 + 511, 4608 + 512, 4608 + 513, 4608 * 2 + 256], 9)])
+@pytest.mark.parametrize("ordered", [True, False])
+def test_order_queue_sizes(M, ws, oracle, sizes, D, ordered):
+    """Queues of given lengths, keys with ties in every field."""
+    rng = np.random.default_rng(sum(sizes) + D)
+    dec = rng.permutation(np.repeat(np.arange(len(sizes)) * D // len(sizes), sizes)).astype(np.int32)
+    N = len(dec)
+    U = rng.integers(0, 300, N).astype(np.int32)
+    wait = rng.integers(0, 1200, N).astype(np.int32)
+    arr = rng.integers(0, 4000, N).astype(np.int32)
+    if ordered:
+        arr.sort()
+    sto, po, so = oracle.order_local(D, dec, U, wait, arr, 1000)
+    st, perm, seg = gpu_order(M, ws, D, dec, U, wait, arr, 1000)
+    assert st == sto == 0
+    assert np.array_equal(perm, po)
+    assert np.array_equal(seg, so)
+
+
 def test_order_degenerate_keys(M, ws, oracle):
     # every key identical: all digit passes trivial -> identity order
     N = 9000
