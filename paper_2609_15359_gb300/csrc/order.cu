@@ -192,7 +192,7 @@ __device__ __forceinline__ int bit_width(uint32_t x) { return x ? 32 - __clz(x) 
 
 // The sort items of fewer decoders than the plan has threads (one round of
 // them) are listed large ones first, those of more than kSegMax / 2 entries: the
-// sorting blocks take them in turn, so what runs last is small.  1,048,576
+// sorting blocks take them in turn, so what runs last is small.  1,114,112
 // entries on 256 ragged queues, sort kernel: 35.4 -> 28 us cold (in decoder
 // order the busiest multiprocessor did 1.5 times the mean's work, now 1.2).
 // The two counts ride in one scan; sixteen classes with counters in shared
@@ -213,6 +213,7 @@ __device__ void seg_plan_block(int64_t N, bool bucketed, int D, OrderCounts *cou
   __shared__ long long s_carry;
   __shared__ int s_bcarry;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5, nt = blockDim.x;
+  const bool by_size = D < nt;
   if (t == 0) {
     s_carry = 0;
     s_bcarry = 0;
@@ -222,11 +223,14 @@ __device__ void seg_plan_block(int64_t N, bool bucketed, int D, OrderCounts *cou
     const int k = base + t;
     const long long c = k < D ? __ldcg(dec_count + k) : 0;
     const int big = c > kSegMax ? 1 : 0;
+    const int full = big ? static_cast<int>(static_cast<uint32_t>(c) / kSegMax) : 0;  // chunks of kSegMax
+    const int rem = static_cast<int>(c) - full * kSegMax;  // the last item, if any
     // sort items of decoder k: its queue, or its chunks; item indices follow
     // from a scan, in decoder order
-    const int nch = big ? static_cast<int>((c + kSegMax - 1) / kSegMax) : 0;
-    const int nit = c > 0 ? (big ? nch : 1) : 0;
-    long long incl = c;
+    const int nit = full + (rem > 0 ? 1 : 0), nch = big ? nit : 0;
+    const int nl = by_size ? full + (rem > kSegMax / 2 ? 1 : 0) : 0;  // large items
+    const long long mine = c | (static_cast<long long>(nl) << 32);    // (entries are below 2^31)
+    long long incl = mine;
     int bincl = nit;
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
@@ -242,26 +246,36 @@ __device__ void seg_plan_block(int64_t N, bool bucketed, int D, OrderCounts *cou
       s_bw[warp] = bincl;
     }
     __syncthreads();
-    long long wb = 0;
+    long long wb = 0, all = 0;
     int bwb = 0;
-    for (int w = 0; w < warp; ++w) {
-      wb += s_w[w];
-      bwb += s_bw[w];
+    for (int w = 0; w < nt / 32; ++w) {
+      const long long v = s_w[w];
+      all += v;
+      wb += w < warp ? v : 0;
+      bwb += w < warp ? s_bw[w] : 0;
     }
     const long long carry = s_carry;
     const int bcarry = s_bcarry;
-    const long long start = carry + wb + incl - c;
+    const long long excl = wb + incl - mine;
+    const long long start = carry + (excl & 0xffffffffll);
     if (k <= D) seg_off[k] = start;
-    const uint32_t it = static_cast<uint32_t>(bcarry + bwb + bincl - nit);
-    if (k < D && c > 0 && !big) {
-      item_off[it] = start;
-      item_n[it] = static_cast<int32_t>(c);
-      item_dec[it] = k;
-    } else if (k < D && big) {
-      for (int j = 0; j < nch; ++j) {
+    uint32_t it = static_cast<uint32_t>(bcarry + bwb + bincl - nit);  // the first full chunk's item
+    uint32_t ir = it + static_cast<uint32_t>(full);                   // the last item's
+    if (by_size) {
+      const uint32_t l = static_cast<uint32_t>(excl >> 32);
+      ir = rem > kSegMax / 2 ? l + static_cast<uint32_t>(full) : static_cast<uint32_t>(all >> 32) + it - l;
+      it = l;
+    }
+    if (k < D && rem > 0) {
+      item_off[ir] = start + static_cast<int64_t>(full) * kSegMax;
+      item_n[ir] = big ? -rem : rem;
+      item_dec[ir] = k;
+    }
+    if (k < D && big) {
+      for (int j = 0; j < full; ++j) {
         item_dec[it + j] = k;
         item_off[it + j] = start + static_cast<int64_t>(j) * kSegMax;
-        item_n[it + j] = -static_cast<int32_t>(min(static_cast<long long>(kSegMax), c - static_cast<long long>(j) * kSegMax));
+        item_n[it + j] = -kSegMax;
       }
       bool paired = false;
       if (nch <= kPairRuns) {  // rank the runs pairwise when the budget allows
@@ -288,7 +302,7 @@ __device__ void seg_plan_block(int64_t N, bool bucketed, int D, OrderCounts *cou
     }
     __syncthreads();
     if (t == nt - 1) {
-      s_carry = carry + wb + incl;
+      s_carry = carry + ((wb + incl) & 0xffffffffll);
       s_bcarry = bcarry + bwb + bincl;
     }
     __syncthreads();
@@ -1531,7 +1545,7 @@ __device__ void merge_level(int level, int ntiles, const int64_t *mt_off, const 
 // and merges them, each thread up to 18 outputs from its place on the merge
 // path on: a step decides one key and gives that key's count, where the run it
 // came from is kept as a bit, and the counts replace the keys in shared memory
-// once all are decided.  1,048,576 entries on 256 ragged queues (202 pairs of
+// once all are decided.  1,114,112 entries on 256 ragged queues (202 pairs of
 // runs), this kernel 28.4 -> 22 us cold; before, every key of either run took a
 // binary search of the other of its own, 13 probes instead of one.
 // 1,000,000 on 200 decoders (200 pairs), whole call: 294 us with the records

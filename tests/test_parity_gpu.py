@@ -780,7 +780,9 @@ def test_order_shuffled_arrival_forms(M, ws, oracle, N, D, ubits, abits, skew):
     # runs (16), and a queue past them merged by levels beside ranked ones
     ([4609], 1), ([9216], 1), ([9217, 0, 4608, 1, 13823], 5), ([73728], 2), ([73729, 5000, 9000], 4),
     # the last run within, and at, one and two outputs a thread
-    ([4608 + 511, 4608 + 512, 4608 + 513, 4608 * 2 + 256], 9)])
+    ([4608 + 511, 4608 + 512, 4608 + 513, 4608 * 2 + 256], 9),
+    # listed by size (at most 511 decoders) and not; items around half a run
+    ([5000, 2304, 2305, 1, 4608, 6912, 6913, 0, 12000] * 3, 511), ([5000, 2304, 2305, 9, 7000], 512)])
 @pytest.mark.parametrize("ordered", [True, False])
 def test_order_queue_sizes(M, ws, oracle, sizes, D, ordered):
     """Queues of given lengths, keys with ties in every field."""
