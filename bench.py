@@ -794,7 +794,7 @@ def bench_stream(device, cpu_sample: int = 0) -> dict:
            "coverage": coverage,
            "value": N / secs, "unit": "decisions/s", "seconds": secs,
            "ms_per_batch": secs / nb * 1e3, "dispatch_mode": "SEQUENTIAL",
-           "timing": "host wall clock of one maps_stream_run call (it synchronises per batch)"}
+           "timing": "host wall clock of one maps_stream_run call (it synchronises after every launch of up to 256 batches)"}
     # the policy variants on the same arrivals: loop throughput and outcome
     # (waiting-queue integral in request-steps, over-capacity events,
     # admissions), at the workload's capacity (where no queue forms) and at a

@@ -1014,7 +1014,7 @@ dispatch_direct_kernel(int D, int H, const int32_t *__restrict__ K, const uint32
 // the pick is made on 64-bit keys.
 //
 // Measured, occupancy and walk: 16 decoders, H 16,384, 1,024 candidates 3.51 ->
-// 0.64 ms; 64 decoders, H 32,763, 2,003 candidates 8.1 -> 1.31 ms.  Before, one
+// 0.60 ms; 64 decoders, H 32,763, 2,003 candidates 8.1 -> 1.22 ms.  Before, one
 // block scored every decoder from global memory with four barriers a decision
 // (3.4 and 4.0 us each).  Forms in between: two warps a decoder, each scoring
 // and reserving in lockstep, 1.58 and 4.44 ms (issue bound: every warp ran the

@@ -18,8 +18,9 @@
 //      histogram whose reverse scan, plus the carry, gives every cell's live
 //      count and b-sum.  Cells are written through shared staging rows as
 //      whole 128-byte lines.
-// For horizons of more than kMaxTiles tiles a single-kernel form is used
-// instead, in which every tile CTA streams all of its decoder's residents.
+// For horizons of more than kMaxTiles tiles, and for few residents
+// (kDirectReads), a single-kernel form is used instead, in which every tile CTA
+// streams all of its decoder's residents.
 // Optionally every group of 16 steps also yields kmax[k][t/16] =
 // max (K[k][t] + t), a summary the dispatch uses for the prefix maxima of
 // earlier horizon tiles.

@@ -78,11 +78,11 @@ struct OrderCounts {
   uint32_t next_item;  // sort items taken beyond each block's first
 };
 
-// Segmented form: when arrival is non-decreasing along the index (so arrival
-// order is index order) and every decoder's queue fits in shared memory, the
-// entries are scattered to their decoder's segment in any order and each
-// segment is sorted by one block on the key (not promoted, primary, index),
-// which is unique, so no pass has to be stable across blocks.
+// Segmented form: the entries are scattered to their decoder's segment in any
+// order and each segment (or chunk of one) is sorted by one block on the key (not
+// promoted, primary, index), with the arrival before the index where arrival
+// order is not index order: the key is unique, so no pass has to be stable
+// across blocks.
 // With at most kStableD decoders the scatter keeps index order within each
 // decoder (stable): the prep and key passes split the entries into the same
 // contiguous block ranges, the prep pass counts each block's entries per
@@ -202,8 +202,7 @@ __device__ __forceinline__ int bit_width(uint32_t x) { return x ? 32 - __clz(x) 
 // segment offsets, the sort items (a queue of at most kSegMax entries is one
 // item whose sort writes the order; a longer one gives one item per chunk,
 // marked by a negative count, whose sort writes keys for the merges) and the
-// merge tiles of the long queues; the form applies when arrival is already
-// in index order.
+// merge tiles of the long queues, and whether the form applies.
 __device__ void seg_plan_block(int64_t N, bool bucketed, int D, OrderCounts *counts, const uint32_t *dec_count,
                                int64_t *seg_off, int64_t *item_off, int32_t *item_n,
                                int32_t *item_dec, int64_t *mt_off, int32_t *mt_n, int32_t *mt_t,

@@ -1795,7 +1795,8 @@ struct StreamWs {
 // admission and deferral.
 //   * the completions and each decoder's waiting requests are sorted by rank
 //     (a key's place is the number of smaller keys of its group, one thread
-//     counting for a key, or up to eight where the keys are few), groups past kLoopRank by a bitonic network;
+//     counting for a key, or up to eight where the keys are few), groups past
+//     kLoopRank by a bitonic network;
 //   * the quantile comes from a histogram of the window's scores, as in
 //     maps_calibrate's one-block form.
 // It stops before a batch that does not fit (the requests in the system, the
