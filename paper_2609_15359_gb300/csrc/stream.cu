@@ -1807,6 +1807,7 @@ constexpr int kLoopActive = 2048;  // requests in the system and the batch, at m
 constexpr int kLoopWindow = 4096;
 constexpr int kLoopRank = 512;     // keys of a group ranked by counting
 constexpr int kLoopBatches = 256;  // batches of one launch
+constexpr int kLoopUsual = 1024;   // requests in the system its shared memory is first sized for
 
 struct LoopArgs {
   maps_stream_cfg c;
@@ -2289,6 +2290,21 @@ int maps_stream_run(const maps_stream_cfg *cfg, const int64_t *arrival_ms, const
   MAPS_TRY(cuda_ok(cudaFuncSetAttribute(loop, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         static_cast<int>(loop_smem))));
   const size_t spare = sizeof(int32_t) * static_cast<size_t>(D) * c.H;  // the dense K, else unused
+  // What the loop leaves of the multiprocessor's memory is its L1 cache, which
+  // the requests' state then hits: it starts with what kLoopUsual requests in the
+  // system need, and takes all of it where a batch does not fit that.  Per step
+  // the dispatch's lists stay in K where the register walk (128 pairs a decoder)
+  // is all but sure to do without them: 64 requests a decoder at most (as the
+  // place has it) and 16 candidates.  32 decoders, batches of 256, 20,000 to
+  // 30,000 requests: 3.53 -> 3.34 ms where no queue forms, 9.14 -> 9.00 at 16,000
+  // tokens, 11.33 -> 11.13 per step.
+  const int nb0 = static_cast<int>(std::min(B, static_cast<int64_t>(kLoopActive)));
+  size_t usual = std::max<size_t>(18 * kLoopActive, sizeof(uint32_t) << kStepBits);  // the sorts, the quantile
+  usual = std::max(usual, per_step && D <= 32 && nb0 <= 16 * D
+                              ? stream_dispatch_smem(D, kLoopActive, nb0)
+                              : stream_dispatch_smem(D, kLoopUsual, nb0) + stream_lists_bytes(D, kLoopUsual, nb0));
+  usual = std::min(usual, loop_smem);
+  size_t give = usual;
   auto loop_fits = [&](int64_t system, int64_t cands) {  // requests in the system, candidates
     return c.window <= kLoopWindow && system + cands <= kLoopActive &&
            stream_lists_place(D, static_cast<int>(system), static_cast<int>(cands), loop_smem,
@@ -2310,19 +2326,20 @@ int maps_stream_run(const maps_stream_cfg *cfg, const int64_t *arrival_ms, const
       la.stats = stats_out;
       la.dst = dec_stats_out;
       la.status = status;
-      la.smem = loop_smem;
+      la.smem = give;
       la.nbatch = nbatch;
       la.b0 = b;
       la.total_done0 = total_done;
-      launch_pdl(loop, 1, kSt, loop_smem, s, la);
+      launch_pdl(loop, 1, kSt, give, s, la);
       MAPS_TRY(launch_ok());
       MAPS_TRY(cuda_ok(cudaMemcpyAsync(&hs, w.S, sizeof(hs), cudaMemcpyDeviceToHost, s)));
       MAPS_TRY(cuda_ok(cudaStreamSynchronize(s)));
       const bool stopped = hs.next_b < nbatch && hs.next_b < b + kLoopBatches;
       b = hs.next_b;
       total_done = hs.total_done;
-      if (!stopped) {
-        --b;  // all done, or a launch's worth
+      if (!stopped || give < loop_smem) {
+        --b;  // all done, or a launch's worth, or on with all of the memory
+        give = stopped ? loop_smem : usual;
         continue;
       }
       in_loop = false;  // batch b does not fit: it runs here
