@@ -112,18 +112,21 @@ constexpr int kSegThreads = 512;
 constexpr int kSegIPT = 9;
 constexpr int kSegMax = kSegThreads * kSegIPT;  // entries one block sorts
 // A longer queue is sorted as chunks of kSegMax entries, whose sorted runs are
-// then merged pairwise, level by level, in tiles of kMergeTile outputs
-// (kMergeTile divides kSegMax, so no tile straddles two runs).
+// then merged pairwise, level by level, in tiles of kMergeTile outputs or three or
+// nine times as many (which divide kSegMax, so no tile straddles two runs).
+// A level's time is a tile's chain (two searches, the load, the merge) and a grid
+// barrier, so the tile grows with N where a level would take the grid
+// several tiles a block.  One queue, arrival out of order, whole call, 1, 3 and 9
+// outputs a thread: 100,000 entries 74, 75 us; 150,000 98, 85, 99; 300,000 142
+// (512 outputs a tile and nothing else), 95, 107; 400,000 (two queues) -, 111,
+// 120; 600,000 (three) 9: 123.
 constexpr int kMergeTile = 512;
 constexpr int kMergeThreads = 512;  // the finishing kernel's block
-// With arrival out of index order, the most merge tiles times levels of the
-// segmented form.  Measured, whole call, segmented against global form: 200,003
-// entries on 64 decoders (no merges) 44 against 149 us; 1,000,000 on 200 (none)
-// 184 against 248; 1,000,000 on 32 (about 2,200 tile levels) 171 against 239;
-// 300,000 on one (4,100) 142 against 152; 1,000,000 on 4 (11,700) 240 against
-// 228; 1,000,000 on one (15,600) 318 against 227.
-constexpr uint32_t kMergesUnsorted = 4200;
-static_assert(kSegMax % kMergeTile == 0, "merge tiles align with runs");
+__host__ __device__ __forceinline__ int merge_per(int64_t N) {  // outputs a thread
+  const int64_t sweep = kPrepBlocks * static_cast<int64_t>(kMergeTile);
+  return N <= sweep / 2 ? 1 : N <= 3 * sweep ? 3 : 9;
+}
+static_assert(kSegMax % (9 * kMergeTile) == 0 && kMergeTile == kMergeThreads, "merge tiles align with runs");
 
 // A long queue of at most kPairRuns chunks is ranked pairwise instead: for
 // every two of its sorted runs (A, B) one block counts, for each key of A, the
@@ -290,7 +293,7 @@ __device__ void seg_plan_block(int64_t N, bool bucketed, int D, OrderCounts *cou
       }
       if (!paired) {  // pairwise merges, level by level
         atomicMax(&counts->max_levels, static_cast<uint32_t>(merge_levels(c)));
-        const int ntl = static_cast<int>((c + kMergeTile - 1) / kMergeTile);
+        const int tile = kMergeTile * merge_per(N), ntl = (static_cast<int>(c) + tile - 1) / tile;
         const uint32_t mt = atomicAdd(&counts->nmtiles, static_cast<uint32_t>(ntl));
         for (int j = 0; j < ntl; ++j) {
           mt_off[mt + j] = start;
@@ -307,13 +310,14 @@ __device__ void seg_plan_block(int64_t N, bool bucketed, int D, OrderCounts *cou
     __syncthreads();
   }
   // arrival out of index order: the bucketed form's keys then hold the arrival
-  // too, when (not promoted, primary, arrival, index) fits 63 bits
+  // too, when (not promoted, primary, arrival, index) fits 63 bits.  Segmented
+  // against global form, whole call: 200,003 entries on 64 decoders 44 against 149
+  // us; one queue of 300,000 95 against 152, of 1,000,000 150 against 227 (four
+  // queues: 129 against 228), of 4,000,000 446 against 625, of 8,000,000 985
+  // against 1,182.
   const int key_bits = 1 + bit_width(__ldcg(&counts->max_bound)) + bit_width(__ldcg(&counts->max_arrival)) +
                        index_bits(N);
-  // and little is left to merge levels (in tiles times levels)
-  const bool segmented = __ldcg(&counts->unsorted) == 0 ||
-                         (bucketed && key_bits <= 63 &&
-                          __ldcg(&counts->nmtiles) * __ldcg(&counts->max_levels) <= kMergesUnsorted);
+  const bool segmented = __ldcg(&counts->unsorted) == 0 || (bucketed && key_bits <= 63);
   const bool stable = segmented && D <= kStableD;
   if (t == 0) {
     counts->segmented = segmented ? 1u : 0u;
@@ -1440,10 +1444,13 @@ order_segsort_kernel(int64_t N, OrderCounts *counts, const int64_t *item_off,
 // L = kSegMax << level sorted keys are merged pairwise from buf[level & 1]
 // into buf[(level + 1) & 1], except at a queue's last level, which writes its
 // indices to the order; a queue needing fewer levels is left alone.
-// One block writes one tile of kMergeTile outputs: a merge-path search splits
+// One block writes one tile of kPer outputs a thread: a merge-path search splits
 // the two runs at the tile's ends, the tile's inputs are staged in shared
-// memory, and each thread merges kMergeTile / kMergeThreads outputs after a
-// second search.  Keys are unique, so there are no ties.
+// memory, and each thread merges its outputs after a second search, a probe
+// each, and hands them over in shared memory for whole-line stores.  Keys are
+// unique, so there are no ties.  1,000,000 entries in one queue (eight levels),
+// whole call: 263 -> 115 us with nine outputs a thread instead of one, arrival
+// in order; 4,000,000 1,149 -> 351.
 __device__ __forceinline__ int merge_path(const unsigned long long *A, int la,
                                           const unsigned long long *B, int lb, int d) {
   int lo = d > lb ? d - lb : 0, hi = d < la ? d : la;
@@ -1482,53 +1489,85 @@ __device__ __forceinline__ int merge_path_warp(const unsigned long long *A, int 
   return lo + __popc(__ballot_sync(0xffffffffu, take_a));
 }
 
+template <int kPer>
 __device__ void merge_level(int level, int ntiles, const int64_t *mt_off, const int32_t *mt_n,
-                            const int32_t *mt_t, unsigned long long *bufA,
-                            unsigned long long *bufB, int32_t *perm, unsigned long long imask) {
-  __shared__ unsigned long long s_a[kMergeTile], s_b[kMergeTile];
+                            const int32_t *mt_t, unsigned long long *bufA, unsigned long long *bufB,
+                            int32_t *perm, unsigned long long imask, unsigned long long *sk) {
+  constexpr int kOut = kPer * kMergeThreads;
   __shared__ int s_split[2];
   const unsigned long long *src = (level & 1) ? bufB : bufA;
   unsigned long long *dst = (level & 1) ? bufA : bufB;
   const int64_t L = static_cast<int64_t>(kSegMax) << level;
+  const int tid = threadIdx.x;
   for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int n = mt_n[tile];
     if (level >= merge_levels(n)) continue;  // this queue is complete (uniform per block)
     const int64_t off = mt_off[tile];
-    const int w0 = mt_t[tile] * kMergeTile, w1 = min(w0 + kMergeTile, n);
+    const int w0 = mt_t[tile] * kOut, w1 = min(w0 + kOut, n);
     const int64_t pstart = (w0 / (2 * L)) * (2 * L);
     const int64_t rest = n - pstart;  // entries from this pair's start to the queue's end
     const int la = static_cast<int>(rest < L ? rest : L);
     const int lb = static_cast<int>(rest > L ? (rest < 2 * L ? rest : 2 * L) - L : 0);
     const unsigned long long *A = src + off + pstart, *B = A + la;
     const int d0 = static_cast<int>(w0 - pstart), d1 = static_cast<int>(w1 - pstart);
-    if (threadIdx.x < 64) {  // warp 0 splits at d0, warp 1 at d1
-      const int r = merge_path_warp(A, la, B, lb, threadIdx.x < 32 ? d0 : d1);
-      if ((threadIdx.x & 31) == 0) s_split[threadIdx.x >> 5] = r;
+    if (tid < 64) {  // warp 0 splits at d0, warp 1 at d1
+      const int r = merge_path_warp(A, la, B, lb, tid < 32 ? d0 : d1);
+      if ((tid & 31) == 0) s_split[tid >> 5] = r;
     }
     __syncthreads();
     const int i0 = s_split[0], i1 = s_split[1];
-    const int j0 = d0 - i0, j1 = d1 - i1;
-    const int na = i1 - i0, nbb = j1 - j0;
-    for (int x = threadIdx.x; x < na; x += kMergeThreads) s_a[x] = A[i0 + x];
-    for (int x = threadIdx.x; x < nbb; x += kMergeThreads) s_b[x] = B[j0 + x];
+    const int na = i1 - i0, m = d1 - d0, nb = m - na;
+    unsigned long long *const sB = sk + na + 1;
+    // A's part, a key above all (the keys have at most 63 bits), B's part, another
+    unsigned long long key[kPer];
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+      const int x = q * kMergeThreads + tid;
+      key[q] = x < na ? A[i0 + x] : x < m ? B[d0 - i0 + (x - na)] : 0ull;
+    }
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+      const int x = q * kMergeThreads + tid;
+      if (x < m) sk[x < na ? x : x + 1] = key[q];
+    }
+    if (tid == 0) sk[na] = sB[nb] = ~0ull;
     __syncthreads();
-    constexpr int kPer = kMergeTile / kMergeThreads;
-    const int dt = threadIdx.x * kPer;
-    if (dt < na + nbb) {
-      int ia = merge_path(s_a, na, s_b, nbb, dt), ib = dt - ia;
-      // the queue's last level writes its order, the others the next runs
-      const bool last = level == merge_levels(n) - 1;
-      unsigned long long *out = dst + off + pstart + d0;
-      int32_t *pout = perm + off + pstart + d0;
+    const int dt = tid * kPer;
+    if (dt < m) {
+      int ia = merge_path(sk, na, sB, nb, dt), ib = dt - ia;
+      unsigned long long ka = sk[ia], kb = sB[ib];
 #pragma unroll
       for (int q = 0; q < kPer; ++q) {
-        if (dt + q >= na + nbb) break;
-        const bool takeA = ib >= nbb || (ia < na && s_a[ia] < s_b[ib]);
-        const unsigned long long k = takeA ? s_a[ia++] : s_b[ib++];
+        if (dt + q < m) {
+          const bool first = ka < kb;
+          key[q] = first ? ka : kb;
+          ia += first ? 1 : 0;
+          ib += first ? 0 : 1;
+          const unsigned long long next = first ? sk[ia] : sB[ib];
+          ka = first ? next : ka;
+          kb = first ? kb : next;
+        }
+      }
+    }
+    __syncthreads();
+    if (kPer > 1) {  // through shared memory, so that consecutive threads write consecutive outputs
+#pragma unroll
+      for (int q = 0; q < kPer; ++q)
+        if (dt + q < m) sk[dt + q] = key[q];
+      __syncthreads();
+    }
+    // the queue's last level writes its order, the others the next runs
+    const bool last = level == merge_levels(n) - 1;
+    const int64_t o0 = off + pstart + d0;
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+      const int x = q * kMergeThreads + tid;
+      if (x < m) {
+        const unsigned long long k = kPer > 1 ? sk[x] : key[0];
         if (last)
-          pout[dt + q] = static_cast<int32_t>(k & imask);
+          perm[o0 + x] = static_cast<int32_t>(k & imask);
         else
-          out[dt + q] = k;
+          dst[o0 + x] = k;
       }
     }
     __syncthreads();  // the next tile reuses shared memory
@@ -1675,13 +1714,18 @@ __device__ void pair_rank_all(int64_t N, const OrderCounts *counts, const PairQu
 
 __device__ void merge_all(int64_t N, const OrderCounts *counts, const int64_t *mt_off,
                           const int32_t *mt_n, const int32_t *mt_t, unsigned long long *bufA,
-                          unsigned long long *bufB, int32_t *perm, GridBar *bar,
-                          int32_t *status) {
+                          unsigned long long *bufB, int32_t *perm, unsigned long long *sk,
+                          GridBar *bar, int32_t *status) {
   const int ntiles = static_cast<int>(counts->nmtiles);
-  const int levels = static_cast<int>(counts->max_levels);
+  const int levels = static_cast<int>(counts->max_levels), per = merge_per(N);
   const unsigned long long imask = (1ull << index_bits(N)) - 1;
   for (int level = 0; level < levels; ++level) {
-    merge_level(level, ntiles, mt_off, mt_n, mt_t, bufA, bufB, perm, imask);
+    if (per == 1)
+      merge_level<1>(level, ntiles, mt_off, mt_n, mt_t, bufA, bufB, perm, imask, sk);
+    else if (per == 3)
+      merge_level<3>(level, ntiles, mt_off, mt_n, mt_t, bufA, bufB, perm, imask, sk);
+    else
+      merge_level<9>(level, ntiles, mt_off, mt_n, mt_t, bufA, bufB, perm, imask, sk);
     if (level + 1 < levels && !grid_barrier(bar, status, g_lookback_spins)) return;
   }
 }
@@ -1882,11 +1926,12 @@ order_finish_kernel(int n_hi, int64_t N, int D, int dbits, const OrderCounts *co
   // every block takes the same branches, so no block waits at a barrier alone;
   // a barrier that ran out (MAPS_E_TIMEOUT) ends the block at once
   if (*reinterpret_cast<const volatile uint32_t *>(&counts->segmented)) {
+    extern __shared__ __align__(16) unsigned char pair_raw[];
     if (counts->npairq > 0) {
-      extern __shared__ __align__(16) unsigned char pair_raw[];
       pair_rank_all(N, counts, pq, keyA, perm, *reinterpret_cast<PairSmem *>(pair_raw), bar, status);
     }
-    if (counts->nmtiles > 0) merge_all(N, counts, mt_off, mt_n, mt_t, keyA, keyB, perm, bar, status);
+    if (counts->nmtiles > 0) merge_all(N, counts, mt_off, mt_n, mt_t, keyA, keyB, perm,
+                                        reinterpret_cast<unsigned long long *>(pair_raw), bar, status);
     return;
   }
   if (blockIdx.x == 0) plan_block(N, D, dbits, counts, plan, dec_count, seg_off);

@@ -756,7 +756,7 @@ def test_order_long_queues(M, ws, oracle, N, D, blo, bhi, skew):
     (300000, 60, 14, 22, 0.0), (50000, 1024, 14, 20, 0.0),
     # one entry past a bucketing round, and ranges of several rounds
     (4097, 9, 10, 10, 0.0), (1300000, 300, 14, 25, 0.0),
-    # too many merges: sorted globally
+    # seven merge levels
     (400000, 1, 14, 22, 0.0)])
 def test_order_shuffled_arrival_forms(M, ws, oracle, N, D, ubits, abits, skew):
     rng = np.random.default_rng(N + D + ubits)
@@ -779,6 +779,8 @@ def test_order_shuffled_arrival_forms(M, ws, oracle, N, D, ubits, abits, skew):
     # runs of 4,608 ranked pairwise: one entry past a run, whole runs, the most
     # runs (16), and a queue past them merged by levels beside ranked ones
     ([4609], 1), ([9216], 1), ([9217, 0, 4608, 1, 13823], 5), ([73728], 2), ([73729, 5000, 9000], 4),
+    # merges at the most entries of one and of three outputs a thread, and past them
+    ([77824], 1), ([77825], 1), ([390000, 76944], 2), ([390000, 76945], 2),
     # the last run within, and at, one and two outputs a thread
     ([4608 + 511, 4608 + 512, 4608 + 513, 4608 * 2 + 256], 9),
     # listed by size (at most 511 decoders) and not; items around half a run
