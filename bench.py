@@ -65,15 +65,15 @@ L2_FLUSH_BYTES = 256 << 20
 TRAFFIC = {
     "dispatch_feasible": {"bytes": 0, "source": "dispatch.cu", "source_sha256": ""},
     "calibrate": {"bytes": 12529152, "source": "calibrate.cu", "source_sha256":
-        "276186c42f8478d5e6974baf53e2af9bb81b825d1d070bb4995dfe8d2de38920"},
-    "occupancy": {"bytes": 31169536, "source": "occupancy.cu", "source_sha256":
-        "fd537e3019c8991f53d529abba17e1a23b2664a7f4477b0936c6a78e22aa0746"},
-    "dispatch": {"bytes": 26562560, "source": "dispatch.cu", "source_sha256":
-        "bc228a45bdc7bb49327bd4b8871778b2d0a6aa7e4c877112d9afa425f6628241"},
-    "dispatch_scoring": {"bytes": 21107968, "source": "dispatch.cu", "source_sha256":
-        "bc228a45bdc7bb49327bd4b8871778b2d0a6aa7e4c877112d9afa425f6628241"},
-    "order": {"bytes": 28039168, "source": "order.cu", "source_sha256":
-        "9f99bc2e2751e755a279d07397d1df4fce876f9be2cfdee980f5c3fa25798411"},
+        "bee3446c753caa47a9a5219998f23f1032c3422bea5e6f2b1b5a0c3388db1333"},
+    "occupancy": {"bytes": 31214592, "source": "occupancy.cu", "source_sha256":
+        "eea478ebad90bd74e26218086061cb3ed62c3daef9b01ff7f4249e1868cf17a7"},
+    "dispatch": {"bytes": 26560256, "source": "dispatch.cu", "source_sha256":
+        "b759e8825262f3d3f45b9c2ae974c2cf85052998c0590251ae60ce864551d683"},
+    "dispatch_scoring": {"bytes": 21105408, "source": "dispatch.cu", "source_sha256":
+        "b759e8825262f3d3f45b9c2ae974c2cf85052998c0590251ae60ce864551d683"},
+    "order": {"bytes": 28051200, "source": "order.cu", "source_sha256":
+        "95adfa960a0cc3f9e622afc9180da0373bde740a1bf203f0cdeb8a7cc7326f7b"},
 }
 KERNELS = {
     "calibrate": "calibrate_fused_kernel (maps_calibrate: select passes and bounds in one "
