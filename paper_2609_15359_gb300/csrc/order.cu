@@ -102,6 +102,8 @@ __host__ __device__ __forceinline__ int64_t prep_chunk(int64_t N) {
 // The bucketed form (order_bucket_kernel): entries per thread per round, and
 // its blocks' ranges (whole rounds, at most kPrepBlocks blocks).
 constexpr int kBucketU = 8;
+constexpr int kBucketFew = 2;
+constexpr int kFewBlocks = 100;  // the most blocks of kBucketFew entries a thread
 constexpr int kBucketRound = 512 * kBucketU;
 __host__ __device__ __forceinline__ int64_t bucket_chunk(int64_t N) {
   const int64_t per = (N + kPrepBlocks - 1) / kPrepBlocks;
@@ -429,6 +431,8 @@ order_prep_kernel(int64_t N, int D, int64_t chunk, const int32_t *__restrict__ d
 //      arrival is non-decreasing along the index, as the prep pass does.
 // The last block to finish plans the segments (seg_plan_block).  The segment
 // sort then gathers decoder d's entries block by block, which is index order.
+// kU entries a thread and round: kBucketU, or kBucketFew where the call is small.
+template <int kU>
 __global__ void __launch_bounds__(512, 2)
 order_bucket_kernel(int64_t N, int D, int64_t chunk, int Dp, const int32_t *__restrict__ dec,
                     const int32_t *__restrict__ bound, const int32_t *__restrict__ wait,
@@ -444,13 +448,13 @@ order_bucket_kernel(int64_t N, int D, int64_t chunk, int Dp, const int32_t *__re
   __shared__ uint32_t s_w[kPassWarps];
   __shared__ bool s_last;
   __shared__ uint32_t s_umax, s_amax;  // largest non-promoted bound, largest arrival
-  constexpr int kU = kBucketU;
+  constexpr int kRound = 512 * kU;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t r_begin = static_cast<int64_t>(blockIdx.x) * chunk;
   const int64_t r_end = r_begin + chunk < N ? r_begin + chunk : N;
   // a range of one round keeps its loads in registers from the count to the
   // scatter (all of them issued together); longer ranges load twice
-  const bool one = r_end - r_begin <= kBucketRound;
+  const bool one = r_end - r_begin <= kRound;
   // per entry only its decoder and raw key stay live: validation, the largest
   // bound and the arrival check are taken as the loads land
   int32_t d[kU];
@@ -544,7 +548,7 @@ order_bucket_kernel(int64_t N, int D, int64_t chunk, int Dp, const int32_t *__re
   } else {
     for (int k = tid; k < Dp; k += blockDim.x) run[k] = 0;
     __syncthreads();
-    for (int64_t i0 = r_begin; i0 < r_end; i0 += kBucketRound) {
+    for (int64_t i0 = r_begin; i0 < r_end; i0 += kRound) {
       load(i0, false);
 #pragma unroll
       for (int q = 0; q < kU; ++q) {
@@ -598,7 +602,7 @@ order_bucket_kernel(int64_t N, int D, int64_t chunk, int Dp, const int32_t *__re
             (static_cast<unsigned long long>(kp[q]) << 32) | static_cast<unsigned long long>(i & 0xffffffff);
     }
   }
-  for (int64_t i0 = one ? r_end : r_begin; i0 < r_end; i0 += kBucketRound) {
+  for (int64_t i0 = one ? r_end : r_begin; i0 < r_end; i0 += kRound) {
     for (int k = tid; k < kPassWarps * Dp; k += blockDim.x) hw[k] = 0;
     load(i0, true);
     __syncthreads();  // counts zeroed
@@ -2007,6 +2011,7 @@ struct OrderWs {
   int32_t *item_dec;
   int64_t *mt_off;    // merge tiles of the long queues
   int32_t *mt_n, *mt_t;
+  bool few;  // the bucketing pass takes kBucketFew entries a thread
   int64_t nitems_max, ntiles_max;
   PairQueues pq;      // pairwise-ranked long queues
   unsigned long long *hi_orig, *keyA, *keyB;
@@ -2057,6 +2062,24 @@ OrderWs carve_order(Carve &c, int64_t N, int D) {
   w.valB = c.take<uint32_t>(n);
   w.blk = c.take<uint32_t>(D <= kStableD ? static_cast<size_t>(w.blocks) * w.Dp : 1);
   w.bst = c.take<uint32_t>(D <= kStableD ? static_cast<size_t>(w.blocks) * w.Dp : 1);
+  // Small calls: the bucketing pass takes ranges of one short round (more blocks,
+  // shorter chains; the segment sort gathers more and smaller buckets), where
+  // its larger counts fit keyB, which nothing uses before the finishing kernel.
+  // Two entries a thread against eight, whole call: 10,000 entries on 16 decoders
+  // 22.6 against 26.3 us, 20,500 on 120 23.1 against 29.2, 60,000 on 30 25.5
+  // against 29.3, 80,344 on 160 (arrival out of order) 34.2 against 39.6, 139,264 on
+  // 64 31.6 against 31.5, 200,003 on 64 35.6 against 33.1 (out of order 58 against
+  // 47).
+  w.few = false;
+  constexpr int64_t few = 512 * kBucketFew;
+  const int64_t fb = (N + few - 1) / few;
+  if (D <= kStableD && fb <= kFewBlocks && fb * w.Dp <= N) {
+    w.few = true;
+    w.chunk = few;
+    w.blocks = static_cast<int>(std::max<int64_t>(1, fb));
+    w.blk = reinterpret_cast<uint32_t *>(w.keyB);
+    w.bst = w.blk + fb * w.Dp;
+  }
   return w;
 }
 
@@ -2107,10 +2130,10 @@ int maps_order_local(int64_t N, int32_t D, const int32_t *dec, const int32_t *bo
   BucketView bv = {};
   if (bucketed) {
     const size_t bsmem = sizeof(uint32_t) * static_cast<size_t>(kPassWarps + 1) * w.Dp;
-    MAPS_TRY(cuda_ok(cudaFuncSetAttribute(order_bucket_kernel,
-                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
+    const auto bucket = w.few ? order_bucket_kernel<kBucketFew> : order_bucket_kernel<kBucketU>;
+    MAPS_TRY(cuda_ok(cudaFuncSetAttribute(bucket, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           static_cast<int>(bsmem))));
-    launch_pdl(order_bucket_kernel, w.blocks, 512, bsmem, s, N, D, w.chunk, w.Dp, dec, bound, wait,
+    launch_pdl(bucket, w.blocks, 512, bsmem, s, N, D, w.chunk, w.Dp, dec, bound, wait,
                arrival, max_wait, w.counts, w.dec_count, status, seg_off_out, w.item_off, w.item_n,
                w.item_dec, w.mt_off, w.mt_n, w.mt_t, w.pq, w.blk, w.bst, w.hi_orig);
     bv.on = 1;

@@ -655,6 +655,12 @@ def test_dispatch_errors(M, ws, oracle):
                                                 # the bucketing pass at its decoder limit, and
                                                 # with a count not a multiple of four
                                                 (200000, 1024, True), (200000, 1023, False),
+                                                # bucketing by two entries a thread: its last
+                                                # range full and of one entry, the most of them
+                                                # and one more, and counts past their room
+                                                (5120, 6, True), (5121, 900, False),
+                                                (102400, 333, False), (102401, 333, True),
+                                                (50001, 1023, True),
                                                 # past 304 x 4,096 entries the bucketing blocks
                                                 # take several rounds (loads issued twice);
                                                 # arrival out of order: the global key pass
