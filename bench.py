@@ -72,8 +72,8 @@ TRAFFIC = {
         "b759e8825262f3d3f45b9c2ae974c2cf85052998c0590251ae60ce864551d683"},
     "dispatch_scoring": {"bytes": 21105408, "source": "dispatch.cu", "source_sha256":
         "b759e8825262f3d3f45b9c2ae974c2cf85052998c0590251ae60ce864551d683"},
-    "order": {"bytes": 28051200, "source": "order.cu", "source_sha256":
-        "95adfa960a0cc3f9e622afc9180da0373bde740a1bf203f0cdeb8a7cc7326f7b"},
+    "order": {"bytes": 28051968, "source": "order.cu", "source_sha256":
+        "fb539521c56dde0a33e6d7cc639e55412aeecb48df1925cd54246196181efc3f"},
 }
 KERNELS = {
     "calibrate": "calibrate_fused_kernel (maps_calibrate: select passes and bounds in one "
