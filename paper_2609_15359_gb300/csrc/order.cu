@@ -498,7 +498,7 @@ order_bucket_kernel(int64_t N, int D, int64_t chunk, int Dp, const int32_t *__re
       atomicMax(&s_amax, amax);
     }
   };
-  if (tid == 0) s_umax = s_amax = 0;
+  if (tid == 0) s_umax = s_amax = 0;  // either form below has a barrier before the first load(., true)
   // base << 16 | leader lane << 8 | rank in the group, the base in the leader's
   // lane alone: this warp's matches and per-warp counts, in item order, so ranks
   // follow the index; the base is the entries of the decoder before the group
@@ -526,9 +526,9 @@ order_bucket_kernel(int64_t N, int D, int64_t chunk, int Dp, const int32_t *__re
   uint32_t v0 = 0, v1 = 0;
   const int k0 = 2 * tid;
   if (one) {
-    load(r_begin, true);
     for (int k = tid; k < kPassWarps * Dp; k += blockDim.x) hw[k] = 0;
-    __syncthreads();
+    __syncthreads();  // the counts, and the maxima that load adds to, are zeroed
+    load(r_begin, true);
     rank_round();
     __syncthreads();
     if (k0 < Dp) {  // Dp is a multiple of four

@@ -724,6 +724,35 @@ def test_order_bucketing_rounds_range_error(M, ws, oracle):
     assert perm.min() >= -1 and perm.max() < N
 
 
+# blocks of 1,024 entries (64 a warp) and of 4,096 (256 a warp), one round each
+@pytest.mark.parametrize("N,D,per_warp", [(20500, 8, 64), (200003, 60, 256)])
+@pytest.mark.parametrize("ordered", [True, False])
+def test_order_bucketing_largest_in_each_warp(M, ws, oracle, N, D, per_warp, ordered):
+    """The widths of the key's fields come from the largest bound and the
+    largest arrival of all entries: each in turn held by one entry of one warp
+    of a block, far above the rest (a width too small runs the fields into
+    each other)."""
+    rng = np.random.default_rng(N)
+    dec = rng.integers(0, D, N).astype(np.int32)
+    wait = rng.integers(0, 5, N).astype(np.int32)
+    for warp in range(16):
+        U = rng.integers(0, 200, N).astype(np.int32)
+        arr = np.sort(rng.integers(0, 500, N)).astype(np.int32)
+        if not ordered:
+            arr = rng.permutation(arr)
+        block = int(rng.integers(0, N // (16 * per_warp)))
+        at = (block * 16 + warp) * per_warp
+        U[at + int(rng.integers(0, per_warp))] = 2**20 + 7
+        if ordered:
+            arr[at:] += 2**18  # non-decreasing still
+        else:
+            arr[at + int(rng.integers(0, per_warp))] = 2**18 + 3
+        sto, po, so = oracle.order_local(D, dec, U, wait, arr, 5)
+        st, perm, seg = gpu_order(M, ws, D, dec, U, wait, arr, 5)
+        assert st == sto == 0
+        assert np.array_equal(perm, po) and np.array_equal(seg, so), warp
+
+
 @pytest.mark.parametrize("N,D,blo,bhi,skew", [
     # one queue far past a block (16 chunks), bounds of 17 bits
     (70000, 256, 0, 70000, 0.95),
