@@ -56,6 +56,14 @@ int maps_test_absent_block(int32_t block);
  * finished before the settings change.  Returns MAPS_OK or MAPS_E_CUDA. */
 int maps_test_calibrate_absent_block(int32_t block, uint32_t spin_limit);
 
+/* The merge tiles of maps_order_local, in host arithmetic alone (no device is
+ * used): *tiles of them for a queue of n of the call's N entries (1 <= n <= N),
+ * and the outputs [*begin, *end) of tile number `tile`, counted from 0.  Queues
+ * of up to INT32_MAX entries are allowed, which no test can hold.  Returns
+ * MAPS_OK or MAPS_E_INVALID. */
+int maps_test_merge_tiles(int64_t N, int64_t n, int64_t tile, int64_t *tiles, int64_t *begin,
+                          int64_t *end);
+
 #ifdef __cplusplus
 }
 #endif

@@ -129,6 +129,12 @@ __host__ __device__ __forceinline__ int merge_per(int64_t N) {  // outputs a thr
   return N <= sweep / 2 ? 1 : N <= 3 * sweep ? 3 : 9;
 }
 static_assert(kSegMax % (9 * kMergeTile) == 0 && kMergeTile == kMergeThreads, "merge tiles align with runs");
+// Tiles of `tile` outputs that a queue of n entries takes, and where the one
+// beginning at w0 ends: in 64 bits, as n may be INT32_MAX and n + tile is not.
+__host__ __device__ __forceinline__ int64_t merge_tiles(int64_t n, int64_t tile) { return (n + tile - 1) / tile; }
+__host__ __device__ __forceinline__ int64_t merge_tile_end(int64_t w0, int64_t tile, int64_t n) {
+  return w0 + tile < n ? w0 + tile : n;
+}
 
 // A long queue of at most kPairRuns chunks is ranked pairwise instead: for
 // every two of its sorted runs (A, B) one block counts, for each key of A, the
@@ -295,7 +301,7 @@ __device__ void seg_plan_block(int64_t N, bool bucketed, int D, OrderCounts *cou
       }
       if (!paired) {  // pairwise merges, level by level
         atomicMax(&counts->max_levels, static_cast<uint32_t>(merge_levels(c)));
-        const int tile = kMergeTile * merge_per(N), ntl = (static_cast<int>(c) + tile - 1) / tile;
+        const int ntl = static_cast<int>(merge_tiles(c, kMergeTile * merge_per(N)));
         const uint32_t mt = atomicAdd(&counts->nmtiles, static_cast<uint32_t>(ntl));
         for (int j = 0; j < ntl; ++j) {
           mt_off[mt + j] = start;
@@ -1507,7 +1513,7 @@ __device__ void merge_level(int level, int ntiles, const int64_t *mt_off, const 
     const int n = mt_n[tile];
     if (level >= merge_levels(n)) continue;  // this queue is complete (uniform per block)
     const int64_t off = mt_off[tile];
-    const int w0 = mt_t[tile] * kOut, w1 = min(w0 + kOut, n);
+    const int64_t w0 = static_cast<int64_t>(mt_t[tile]) * kOut, w1 = merge_tile_end(w0, kOut, n);
     const int64_t pstart = (w0 / (2 * L)) * (2 * L);
     const int64_t rest = n - pstart;  // entries from this pair's start to the queue's end
     const int la = static_cast<int>(rest < L ? rest : L);
@@ -2262,6 +2268,18 @@ extern "C" int maps_order_local_static(int64_t N, int32_t D, const int32_t *dec,
 extern "C" int maps_test_absent_block(int32_t block) {
   using namespace maps;
   MAPS_TRY(cuda_ok(cudaMemcpyToSymbol(g_absent_block, &block, sizeof(block))));
+  return MAPS_OK;
+}
+
+extern "C" int maps_test_merge_tiles(int64_t N, int64_t n, int64_t tile, int64_t *tiles, int64_t *begin,
+                                     int64_t *end) {
+  using namespace maps;
+  if (N < 1 || n < 1 || n > N || tile < 0 || tiles == nullptr || begin == nullptr || end == nullptr)
+    return MAPS_E_INVALID;
+  const int64_t out = static_cast<int64_t>(kMergeTile) * merge_per(N);
+  *tiles = static_cast<int>(merge_tiles(n, out));
+  *begin = tile * out;
+  *end = merge_tile_end(*begin, out, n);
   return MAPS_OK;
 }
 

@@ -58,3 +58,24 @@ def test_static_order_array_holds_its_largest_calls(libmaps):
         assert M.lib.maps_order_local_workspace_size(65536, D) <= 5 << 20
     small = M.lib.maps_order_local_workspace_size(65536, 1)
     assert small > 15 * 14 * 4608 * 2  # 210 run pairs of 16-bit counts
+
+
+@pytest.mark.parametrize("N", [4609, 77824, 77825, 466944, 466945, 2**31 - 4609, 2**31 - 1])
+def test_order_merge_tiles_cover_their_queue(libmaps, N):
+    """The tiles of a long queue's merges are consecutive and cover it, up to
+    queues of INT32_MAX entries (whose sizes plus a tile are past 32 bits) and at
+    the sizes where the tile grows."""
+    from paper_2609_15359_gb300 import maps as M
+
+    def tile_of(n, i):
+        out = [ctypes.c_int64() for _ in range(3)]
+        assert M.lib.maps_test_merge_tiles(N, n, i, *map(ctypes.byref, out)) == 0
+        return [x.value for x in out]
+
+    for n in {max(4609, N - x) for x in (0, 1, 511, 512, 4607, 4608)}:
+        tiles, begin, size = tile_of(n, 0)  # the first of several tiles is a whole one
+        assert begin == 0 and size in (512, 1536, 4608) and tiles == -(-n // size)
+        for i in (1, tiles // 2, tiles - 2, tiles - 1):
+            _, begin, end = tile_of(n, i)
+            assert begin == i * size and end == min(n, begin + size)
+        assert tile_of(n, tiles - 1)[2] == n
