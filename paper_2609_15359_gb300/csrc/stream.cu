@@ -2048,6 +2048,7 @@ stream_loop_kernel(const __grid_constant__ LoopArgs a) {
     }
     if (tid == 0) *w.q_dev = q;
     if (nto > 0) {  // timed out: round robin with the horizon as bound
+      __syncthreads();  // every thread has read S->nact, which the enqueue sets
       enqueue_list(nto, nact, D, c.H, hi, a.arrival, w.tout, nullptr, w.Uq, a.choice, w.st, w.dec, w.disp, w.g,
                    w.U, act, S, a.status);
       nact += nto;

@@ -108,6 +108,21 @@ def test_shapes(M, ws, oracle, N, D, H, cap, B, Wn, a, mw):
               acc=1, loc=1)
 
 
+@pytest.mark.parametrize("per_step", [0, 1])
+@pytest.mark.parametrize("beta,every", [(0, 1), (0, 3), (40, 1)])
+def test_timed_out_batches_without_completions(M, ws, oracle, per_step, beta, every):
+    """Batches that only time out (no prediction in, no completion yet, so no
+    bound either), alone or among others whose predictions are in: the requests
+    in the system are counted once."""
+    N = 1900
+    w = W.make_stream(n_requests=N)
+    w["true"] = np.full(N, 1 << 20, np.int32)
+    delay = np.where(np.arange(N) % every == 0, 1 << 24, 0).astype(np.int32)
+    so, _ = on_stream(M, ws, oracle, w, N, 8, 16384, 262144, 50, 500, 100000, 1000,
+                      per_step=per_step, beta=beta, delay=delay)
+    assert so[:, 0].sum() == 0
+
+
 def test_full_workload(M, ws, oracle):
     """All 1,000,000 requests: per-step admission at the workload's capacity
     with prediction delays and beta = 1 s, and at a capacity of 16,000 where
