@@ -1893,15 +1893,14 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
 }
 
 constexpr int kMaxH = 1 << 28;
+constexpr size_t kStaticSmem = 2048;  // left to the kernels' static arrays (1 KB at most)
 
 // Events recorded around the scoring kernel (maps_set_dispatch_events).
 thread_local cudaEvent_t g_score_ev[2] = {nullptr, nullptr};
 
 template <int W2>
 int run_snapshot(int64_t grid, size_t smem, cudaStream_t s, const CUtensorMap &tmap, const SnapArgs &a) {
-  MAPS_TRY(cuda_ok(cudaFuncSetAttribute(dispatch_snapshot_kernel<W2>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        static_cast<int>(smem))));
+  MAPS_TRY(allow_smem(dispatch_snapshot_kernel<W2>, smem_beside(kStaticSmem)));
   if (g_score_ev[0]) MAPS_TRY(cuda_ok(cudaEventRecord(g_score_ev[0], s)));
   launch_pdl(dispatch_snapshot_kernel<W2>, static_cast<unsigned>(grid), kMainThreads, smem, s, tmap, a);
   MAPS_TRY(launch_ok());
@@ -2063,17 +2062,17 @@ int dispatch_sequential(int D, int H, int32_t *K, const int32_t *cap, int32_t *Q
   while ((1 << a.kb) < D) ++a.kb;
   a.ncol = std::min((D + 7) / 8, kColWarps);
   // shared memory per row: a thirty-second for chunk maxima, the rest resident
-  // steps (1 + 1/4 + 1/16 words each); 2 KB are left to the static arrays
+  // steps (1 + 1/4 + 1/16 words each)
   const int64_t fixed = kSeqWords * seq_dw(D) + kSeqPad;
-  const int64_t words = ((max_smem_optin() - 2048) / 4 - fixed) / D;
+  const size_t limit = smem_beside(kStaticSmem);
+  const int64_t words = (static_cast<int64_t>(limit) / 4 - fixed) / D;
   const int64_t chunks = (static_cast<int64_t>(H) + kSeqChunk - 1) / kSeqChunk;
   a.P2 = static_cast<int>(std::min<int64_t>(chunks, words / 32));
   a.P0 = 0;
   while (a.P0 < chunks * kSeqChunk && seq_row_words(a.P0 + kSeqChunk, a.P2) <= words) a.P0 += kSeqChunk;
   const size_t smem = 4 * (static_cast<size_t>(D) * seq_row_words(a.P0, a.P2) + fixed);
   auto launch = [&](void (*kern)(SeqArgs)) {
-    MAPS_TRY(cuda_ok(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          static_cast<int>(smem))));
+    MAPS_TRY(allow_smem(kern, limit));
     launch_pdl(kern, 1, 1024, smem, s, a);
     return launch_ok();
   };

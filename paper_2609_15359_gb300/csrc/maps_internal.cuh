@@ -225,6 +225,18 @@ int dispatch_sequential(int D, int H, int32_t *K, const int32_t *cap, int32_t *Q
 int sm_count();           // multiprocessors of the current device
 int max_smem_optin();     // opt-in shared memory per block, bytes
 
+// The dynamic shared memory a kernel may be launched with is kept with the kernel
+// on the device, for every thread of the process: it is set to one limit that
+// does not depend on the call (a size set for each call could be lowered by
+// another thread's smaller call before the launch, which then fails).
+template <typename... KArgs>
+inline int allow_smem(void (*kernel)(KArgs...), size_t limit) {
+  return cuda_ok(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      static_cast<int>(limit)));
+}
+// The limit that leaves `fixed` bytes to a kernel's static arrays.
+inline size_t smem_beside(size_t fixed) { return static_cast<size_t>(max_smem_optin()) - fixed; }
+
 #define MAPS_TRY(expr)            \
   do {                            \
     int maps_try_rc_ = (expr);    \

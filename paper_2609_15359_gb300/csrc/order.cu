@@ -2137,8 +2137,7 @@ int maps_order_local(int64_t N, int32_t D, const int32_t *dec, const int32_t *bo
   if (bucketed) {
     const size_t bsmem = sizeof(uint32_t) * static_cast<size_t>(kPassWarps + 1) * w.Dp;
     const auto bucket = w.few ? order_bucket_kernel<kBucketFew> : order_bucket_kernel<kBucketU>;
-    MAPS_TRY(cuda_ok(cudaFuncSetAttribute(bucket, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          static_cast<int>(bsmem))));
+    MAPS_TRY(allow_smem(bucket, sizeof(uint32_t) * (kPassWarps + 1) * static_cast<size_t>(kStableD)));
     launch_pdl(bucket, w.blocks, 512, bsmem, s, N, D, w.chunk, w.Dp, dec, bound, wait,
                arrival, max_wait, w.counts, w.dec_count, status, seg_off_out, w.item_off, w.item_n,
                w.item_dec, w.mt_off, w.mt_n, w.mt_t, w.pq, w.blk, w.bst, w.hi_orig);

@@ -2287,9 +2287,8 @@ int maps_stream_run(const maps_stream_cfg *cfg, const int64_t *arrival_ms, const
   void (*const loop)(LoopArgs) = per_step ? stream_loop_kernel<true> : stream_loop_kernel<false>;
   cudaFuncAttributes fa;
   MAPS_TRY(cuda_ok(cudaFuncGetAttributes(&fa, loop)));
-  const size_t loop_smem = static_cast<size_t>(max_smem_optin()) - fa.sharedSizeBytes;
-  MAPS_TRY(cuda_ok(cudaFuncSetAttribute(loop, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        static_cast<int>(loop_smem))));
+  const size_t loop_smem = smem_beside(fa.sharedSizeBytes);
+  MAPS_TRY(allow_smem(loop, loop_smem));
   const size_t spare = sizeof(int32_t) * static_cast<size_t>(D) * c.H;  // the dense K, else unused
   // What the loop leaves of the multiprocessor's memory is its L1 cache, which
   // the requests' state then hits: it starts with what kLoopUsual requests in the
@@ -2409,15 +2408,12 @@ int maps_stream_run(const maps_stream_cfg *cfg, const int64_t *arrival_ms, const
       launch_pdl(stream_lr_kernel, 1, 32, 0, s, D, nc, w.res_off, cch);
       MAPS_TRY(launch_ok());
     } else if (!rr) {  // 5.
-      // (the kernel's static shared memory is below 4 KB)
-      const size_t most = static_cast<size_t>(max_smem_optin()) - 4096;
+      const size_t most = smem_beside(4096);  // (the kernel's static arrays take 1.2 KB)
       const int place = stream_lists_place(D, nact, nc, most, spare);
       if (place != 0) {
         // the decoders' pairs and the batch fit in shared memory: no dense projection
         const size_t dsm = stream_dispatch_smem(D, nact, nc) + (place == 1 ? stream_lists_bytes(D, nact, nc) : 0);
-        MAPS_TRY(cuda_ok(cudaFuncSetAttribute(stream_dispatch_kernel,
-                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              static_cast<int>(dsm))));
+        MAPS_TRY(allow_smem(stream_dispatch_kernel, most));
         launch_pdl(stream_dispatch_kernel, 1, kSt, dsm, s, D, c.H, nc, mc, w.res_off, w.rp, w.rg,
                    w.rU, w.capv, w.Q, cpr, w.Uq + nact, cch, nullptr, status,  // no headroom out
                    place == 1 ? nullptr : reinterpret_cast<unsigned char *>(w.K));
