@@ -383,14 +383,16 @@ select_small_kernel(const int32_t *__restrict__ L, const int32_t *__restrict__ P
     w = s_w;
     k = s_k;
   }
-  if (lo > 0x7fffffffu) {
-    if (tid == 0) flag_error(status, MAPS_E_RANGE);
-    return;
-  }
-  const int32_t q = static_cast<int32_t>(lo);
+  // (a quantile above INT32_MAX: flagged, and 0 stands for it, as in the
+  // cooperative kernel, not what an earlier call left in the workspace)
+  const bool q_ok = lo <= 0x7fffffffu;
+  const int32_t q = q_ok ? static_cast<int32_t>(lo) : 0;
   if (tid == 0) {
     st->q = q;
-    if (q_dev_out) *q_dev_out = q;
+    if (!q_ok)
+      flag_error(status, MAPS_E_RANGE);
+    else if (q_dev_out)
+      *q_dev_out = q;
   }
   bool bad = false;
 #pragma unroll

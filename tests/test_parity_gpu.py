@@ -264,6 +264,29 @@ def test_calibrate_fused_register_limits(M, ws, oracle, n, m, shift):
     assert np.array_equal(host(Ub)[:-1], oracle.bound(big[:-1], oracle.calibrate(L, P, 100000)[1])[1])
 
 
+@pytest.mark.parametrize("n", [3, 16384, 16385])
+@pytest.mark.parametrize("m", [5, 16384, 16385])
+def test_calibrate_range_error_keeps_no_earlier_quantile(M, oracle, n, m):
+    """A quantile above INT32_MAX, in every form: the range error, and what is
+    written beside it (the host's quantile, the bounds) does not depend on the
+    call that used the workspace before."""
+    query = np.arange(m, dtype=np.int32)
+    U = torch.empty(m, dtype=torch.int32, device="cuda")
+    L, P = dev(np.full(n, I32_MAX, np.int32)), dev(np.full(n, -5, np.int32))
+    seen = []
+    for earlier in (77, 123456):
+        ws = M.Workspace()
+        st, q = M.maps_calibrate(dev(np.full(9, earlier, np.int32)), dev(np.zeros(9, np.int32)),
+                                 500000, q_host=True, ws=ws)
+        assert st == 0 and q == earlier
+        U.fill_(-9)
+        st, q = M.maps_calibrate(L, P, 500000, dev(query), U, q_host=True, ws=ws)
+        assert st == M.MAPS_E_RANGE
+        seen.append((q, host(U).tolist()))
+    assert seen[0] == seen[1]
+    assert seen[0] == (0, query.tolist())
+
+
 @pytest.mark.parametrize("name", ["tiny", "d16", "d64", "large"])
 def test_calibrate_workloads(M, ws, oracle, name):
     w = W.make(name)
