@@ -836,21 +836,27 @@ dispatch_snapshot_kernel(const __grid_constant__ CUtensorMap tmap, SnapArgs a) {
 constexpr int kDirectWarps = 8;
 constexpr int kDirectRows = 8;
 
-// At most this many (candidate, decoder) scores, half as many of them times the
-// 2,048-step spans of the horizon, and cells of K, and a horizon that a warp
-// reads in time even if every candidate lives through all of it.  Measured,
-// one launch against four (candidates of a few hundred steps; all through the
-// horizon): 4 decoders, H 4,096, 32 candidates 4.7 against 13.1 us (5.2; 12.9);
-// 16, 16,381, 1,021: 7.2 against 20.6 (11.2; 18.6); 100, 8,192, 600: 12.1
-// against 16.4 (19.2; 16.5); 64, 4,096, 2,048: 16.2 against 18.6; past the
-// line 16, 2,048, 16,384: 25.9 against 20.7; 256, 2,048, 1,024: 22.6 against
-// 18.4; 12, 50,000, 100: 7.8 against 16.4, but 63 against 14.5.
+// At most this many candidates, (candidate, decoder) scores, twice as many of
+// those times the 2,048-step spans of the horizon, cells of K, and a horizon.
+// Candidates of a few hundred steps decide where the lines lie; in brackets the
+// same with all of them through the horizon, which no size tells the host.
+// Measured, one launch against four: 4 decoders, H 4,096, 32 candidates 4.7
+// against 13.1 us (5.2; 12.9); 16, 16,381, 1,021: 7.2 against 20.6 (11.2; 18.6);
+// 100, 8,192, 600: 12.1 against 16.4 (19.2; 16.5); 64, 4,096, 2,048: 16.2 against
+// 18.6; 1, 30,000, 8,192: 10.7 against 20.5 (25.9; 17.5).  Past the lines: 16,
+// 2,048, 16,384: 25.9 against 20.7; 256, 2,048, 1,024: 22.6 against 18.4; 2, 100,
+// 24,000: 19.9 against 17.5; 2, 256, 65,536: 40.9 against 19.1; 12, 50,000, 100: 7.8
+// against 16.4, but 63 against 14.5.  Where the summary's rows are no whole
+// 16-byte words (330 decoders, H 2,760, 256 candidates: 10.9 against 24.6) a lane has
+// four words in flight as well; with one, that took 28.5.
+constexpr int64_t kDirectCands = 1 << 14;
 constexpr int64_t kDirectScores = 1 << 17;
 constexpr int64_t kDirectCells = 1 << 20;
 constexpr int kDirectH = 32768;
 bool direct_fits(int D, int H, int64_t J) {
-  return J * D <= kDirectScores && J * D * std::max(1, H / 2048) <= 2 * kDirectScores &&
-         H <= kDirectH && static_cast<int64_t>(D) * H <= kDirectCells;
+  return J <= kDirectCands && J * D <= kDirectScores &&
+         J * D * std::max(1, H / 2048) <= 2 * kDirectScores && H <= kDirectH &&
+         static_cast<int64_t>(D) * H <= kDirectCells;
 }
 
 template <bool VEC>
@@ -908,12 +914,17 @@ dispatch_direct_kernel(int D, int H, const int32_t *__restrict__ K, const uint32
               }
             }
           } else {
-            for (int b = lane; b < nfull; b += 32) {
-              uint32_t v[kDirectRows];
+            for (int b = lane; b < nfull; b += 128) {  // one by one: four in flight a lane, too
+              uint32_t v[4][kDirectRows];
 #pragma unroll
-              for (int i = 0; i < kDirectRows; ++i) v[i] = __ldg(km + (i < rows ? i : rows) * nb + b);
+              for (int q = 0; q < 4; ++q)
 #pragma unroll
-              for (int i = 0; i < kDirectRows; ++i) m[i] = max(m[i], v[i]);
+                for (int i = 0; i < kDirectRows; ++i)
+                  v[q][i] = b + 32 * q < nfull ? __ldg(km + (i < rows ? i : rows) * nb + b + 32 * q) : 0u;
+#pragma unroll
+              for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int i = 0; i < kDirectRows; ++i) m[i] = max(m[i], v[q][i]);
             }
           }
 #pragma unroll
