@@ -18,9 +18,9 @@
 //      histogram whose reverse scan, plus the carry, gives every cell's live
 //      count and b-sum.  Cells are written through shared staging rows as
 //      whole 128-byte lines.
-// For horizons of more than kMaxTiles tiles, and for few residents
-// (kDirectReads), a single-kernel form is used instead, in which every tile CTA
-// streams all of its decoder's residents.
+// For horizons of more than kMaxTiles tiles or of few, and for small grids
+// (kDirectT, kDirectTiles), a single-kernel form is used instead, in which every
+// tile CTA streams all of its decoder's residents.
 // Optionally every group of 16 steps also yields kmax[k][t/16] =
 // max (K[k][t] + t), a summary the dispatch uses for the prefix maxima of
 // earlier horizon tiles.
@@ -43,13 +43,22 @@ constexpr int kPerThread = 4;  // entries a thread loads per round
 constexpr int kRound = kPerThread * kOccThreads;
 constexpr int kBucketRound = kPerThread * kBucketThreads;
 constexpr int kMaxTiles = 128;  // tiles per decoder of the bucketed form
-// Residents read over all tiles up to which every tile CTA streams its
-// decoder's residents itself: one launch instead of two.  Measured, one launch
-// against two: 4 decoders of 64 residents, H 4,096 2.7 against 5.3 us; 16 of
-// 509, 16,381 4.6 against 7.9; 8 of 9,000, 4,096 7.2 against 17.8; 64 of 2,048,
-// 32,768 (1,048,576 reads) 7.0 against 8.9; 256 of 4,096, 65,536 (16 times as
-// many) 29 for the two.
-constexpr int64_t kDirectReads = 1 << 20;
+// Where every tile CTA streams its decoder's residents itself, one launch instead
+// of two: horizons of up to kDirectT tiles, and grids of up to kDirectTiles tile
+// CTAs.  The residents are then read once a tile, but a bucket kernel has one CTA a
+// decoder, which a long horizon's many tiles pay for and a few do not.  Measured,
+// one launch against two (residents a decoder 4; 512; 2,048; 8,192):
+//   640 tiles (40 decoders of 16 tiles)  6.8; 7.1; 9.0; 18.0  against  7.2; 7.8; 9.4; 24.3
+//   768 (48 of 16)                       7.4; 7.8; 10.3; 20.6          7.7; 8.1; 9.9; 26.7
+//   1,024 (128 of 8)                     8.6; 9.0; 12.0; 24.6          8.4; 9.3; 10.9; 29.7
+//   2,560 (512 of 5)                     18.7; 19.6; 24.8; 54.3        15.8; 18.5; 21.8; 58.2
+//   6,144 (2,048 of 3)                   42.6; 46.3; 62.3; -           44.2; 54.9; 68.4; -
+//   8,192 (2,048 of 4)                   56.0; 60.2; 79.7; -           49.8; 60.0; 74.0; -
+// and one decoder of 1,048,576 on one tile 506 against 1,328 us.  A line on the
+// residents read (2^20 over all tiles) took 1,024 decoders of 128 on 8 tiles to
+// the one launch (56.8 us) that the two do in 39.6.
+constexpr int kDirectT = 3;
+constexpr int64_t kDirectTiles = 640;
 constexpr int kBHold = 8;       // residents a bucket thread keeps in registers
 // A tile holding at most this many end steps skips the histogram: its pairs
 // are kept as a list that every thread scans for its own cells.
@@ -569,7 +578,7 @@ occ_tile_kernel(int H, int D, int T, const int64_t *__restrict__ res_off, int64_
 }
 
 // ---------------------------------------------------------------------------
-// Long horizons: every tile CTA streams all of its decoder's residents.
+// One launch: every tile CTA streams all of its decoder's residents.
 // ---------------------------------------------------------------------------
 template <int CPT, bool VEC>
 __global__ void __launch_bounds__(kOccThreads, 4)
@@ -647,12 +656,13 @@ struct OccPlan {
   bool bucketed;
 };
 
-OccPlan plan_occ(int32_t H, int64_t R) {
+OccPlan plan_occ(int32_t D, int32_t H, int64_t R) {
   OccPlan p;
   p.cpt = H <= 1024 ? 4 : (H <= 2048 ? 8 : 16);
   p.log2W = 8 + (p.cpt == 4 ? 2 : (p.cpt == 8 ? 3 : 4));  // W = 256 threads x CPT
   p.T = static_cast<int>((static_cast<int64_t>(H) + (1 << p.log2W) - 1) >> p.log2W);
-  p.bucketed = p.T <= kMaxTiles && R <= 0x7fffffffLL && R * p.T > kDirectReads;
+  p.bucketed = p.T <= kMaxTiles && R <= 0x7fffffffLL && p.T > kDirectT &&
+               static_cast<int64_t>(D) * p.T > kDirectTiles;
   return p;
 }
 
@@ -705,7 +715,7 @@ size_t maps_project_occupancy_workspace_size(int32_t D, int32_t H, int64_t R) {
   int2 *bucket = nullptr;
   int32_t *tile_off = nullptr;
   uint2 *tile_carry = nullptr;
-  return carve_occ(c, D, R, plan_occ(H, R), &bucket, &tile_off, &tile_carry);
+  return carve_occ(c, D, R, plan_occ(D, H, R), &bucket, &tile_off, &tile_carry);
 }
 
 int maps_project_occupancy(int32_t D, int32_t H, const int64_t *res_off, int64_t R,
@@ -719,7 +729,7 @@ int maps_project_occupancy(int32_t D, int32_t H, const int64_t *res_off, int64_t
   MAPS_TRY(check_ws(ws, ws_bytes, maps_project_occupancy_workspace_size(D, H, R)));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   int32_t *status = status_word(ws);
-  const OccPlan p = plan_occ(H, R);
+  const OccPlan p = plan_occ(D, H, R);
   const int64_t blocks = static_cast<int64_t>(D) * p.T;
   if (blocks > 0x7fffffffLL) return MAPS_E_INVALID;
   Carve c(ws);

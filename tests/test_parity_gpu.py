@@ -314,9 +314,11 @@ def random_residents(rng, D, H, per_max, with_empty=True):
 
 @pytest.mark.parametrize("D,H", [(1, 1), (3, 3), (2, 8), (5, 511), (4, 512), (3, 513), (7, 4095),
                                  (2, 4097), (9, 4100), (3, 12289), (2, 65536),
-                                 # 64 horizon tiles (the most the bucketed form takes), then
-                                 # more, which stream every resident per tile instead
-                                 (2, 524288), (2, 524292), (1, 600001)])
+                                 # 128 horizon tiles (the most the bucketed form takes), then
+                                 # more, which stream every resident per tile instead; grids
+                                 # past 640 tiles at those, and with few steps a tile
+                                 (2, 524288), (2, 524292), (1, 600001), (6, 524288), (6, 524292),
+                                 (170, 16384), (700, 1000)])
 def test_occupancy_random(M, ws, oracle, D, H):
     rng = np.random.default_rng(D * 100003 + H)
     off, p, g, U = random_residents(rng, D, H, 700)
@@ -341,10 +343,12 @@ def test_occupancy_workloads(M, ws, oracle, name):
 
 
 @pytest.mark.parametrize("D,H,per", [(2, 20000, 9000), (3, 3000, 4097),
-                                     # 1,048,576 reads over all tiles exactly, and past
-                                     # them, bucketed
                                      (16, 65536, 4096), (16, 65536, 4097), (2, 60001, 40000),
-                                     (3, 400000, 4097)])
+                                     (3, 400000, 4097),
+                                     # 640 tiles, and past them and three a decoder, bucketed;
+                                     # 768 tiles of three a decoder, one launch
+                                     (40, 65536, 2049), (41, 65535, 4097), (129, 20001, 2500),
+                                     (7, 400000, 9000), (161, 12289, 1500), (256, 12288, 700)])
 def test_occupancy_many_residents_per_decoder(M, ws, oracle, D, H, per):
     """More residents on one decoder than a block stages at once."""
     rng = np.random.default_rng(H + per)
