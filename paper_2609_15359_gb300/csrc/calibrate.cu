@@ -291,20 +291,24 @@ bound_kernel(const int32_t *__restrict__ pred, int64_t m, const SelectState *st,
 }
 
 // Small calibration sets (n <= kSmallN): the same select in one block, scores
-// in registers, then the bounds of up to kSmallM queries: one
+// in registers (kItems a thread), then the bounds of up to kSmallM queries: one
 // launch without a memset or a grid barrier.  A chain of latencies: loads, the
 // block's histogram, its scan (the bins' totals by warp shuffles, the warps' by
-// one reduction), the bounds.  Replayed calls: 1,000 scores and 288 bounds 4.7 us
-// (sorted by a bitonic network: 10.1), 2,000 and 1,000 5.0 (17.2), 8,000 and
-// 8,000 6.5 (three fixed digits: 6.8); 10,007 and 9,165 6.9 (the cooperative
-// kernel: 10.0), 16,384 and 16,384 8.3 (9.6).
-constexpr int kSmallItems = 16;  // scores a thread keeps
+// one reduction), the bounds; with 16 scores a thread for every n its loads and
+// predicates alone were 1.5 us of a small call's.  At most kCountN scores are ranked
+// by counting instead.  Replayed calls, no queries, lengths (in brackets scores over
+// all 32 bits, three passes instead of two): 16 scores 2.4 us (2.3), 128 2.9 (2.9),
+// 1,000 3.0 (4.1), 4,000 4.0 (5.5), 8,000 5.1 (7.1), 12,000 6.5 (8.9), 16,384 7.1
+// (10.1).  A bitonic network up to 2,048: 3.0, 4.8, 10.0; three fixed digits to
+// 8,192: 4.9 (4.8), 5.8 (5.5); the cooperative kernel 10.1 (19).
 constexpr int kSmallHold = 8;    // predictions loaded before the select
 constexpr int kSmallThreads = 1024;
-constexpr int kSmallN = kSmallItems * kSmallThreads;
-constexpr int kSmallM = kSmallItems * kSmallThreads;
+constexpr int kCountN = 128;     // up to this many scores are ranked by counting
+constexpr int kSmallN = 16 * kSmallThreads;
+constexpr int kSmallM = 16 * kSmallThreads;
 static_assert(kBins == 4 * kSmallThreads, "four bins a thread");
 
+template <int kItems>
 __global__ void __launch_bounds__(kSmallThreads)
 select_small_kernel(const int32_t *__restrict__ L, const int32_t *__restrict__ P, int n,
                     uint32_t k, const int32_t *__restrict__ pred, int m_inblock,
@@ -316,10 +320,10 @@ select_small_kernel(const int32_t *__restrict__ L, const int32_t *__restrict__ P
   __shared__ uint32_t s_lo, s_k;
   __shared__ int s_w;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  uint32_t sv[kSmallItems];
+  uint32_t sv[kItems];
   int32_t pv[kSmallHold];
 #pragma unroll
-  for (int i = 0; i < kSmallItems; ++i) {
+  for (int i = 0; i < kItems; ++i) {
     const int x = i * kSmallThreads + tid;
     sv[i] = x < n ? score(__ldg(L + x), __ldg(P + x)) : 0u;
   }
@@ -330,12 +334,29 @@ select_small_kernel(const int32_t *__restrict__ L, const int32_t *__restrict__ P
   }
   uint32_t lo = 0;
   int w = 32;
+  if (n <= kCountN) {  // few scores: the one with its rank among all of them
+    if (tid < kCountN) hist[tid] = tid < n ? sv[0] : 0xffffffffu;
+    __syncthreads();
+    if (tid < n) {
+      uint32_t below = 0, upto = 0;
+#pragma unroll 8
+      for (int i = 0; 4 * i < n; ++i) {
+        const uint4 c = reinterpret_cast<const uint4 *>(hist)[i];
+        below += (c.x < sv[0]) + (c.y < sv[0]) + (c.z < sv[0]) + (c.w < sv[0]);
+        upto += (c.x <= sv[0]) + (c.y <= sv[0]) + (c.z <= sv[0]) + (c.w <= sv[0]);
+      }
+      if (below < k && k <= upto) s_lo = sv[0];  // (equal scores all write the same)
+    }
+    __syncthreads();
+    lo = s_lo;
+    w = 0;
+  }
   for (int pass = 0; pass < kPasses && w > 0; ++pass) {
     const int shift = w > kStepBits ? w - kStepBits : 0;
     reinterpret_cast<uint4 *>(hist)[tid] = make_uint4(0, 0, 0, 0);
     __syncthreads();
 #pragma unroll
-    for (int i = 0; i < kSmallItems; ++i) {
+    for (int i = 0; i < kItems; ++i) {
       if (i * kSmallThreads >= n) break;
       const bool valid = i * kSmallThreads + tid < n;
       if (pass == 0) {  // zero scores by one ballot a warp, the others alone
@@ -343,11 +364,9 @@ select_small_kernel(const int32_t *__restrict__ L, const int32_t *__restrict__ P
         const unsigned zeros = __ballot_sync(0xffffffffu, valid && d == 0);
         if (zeros && lane == __ffs(zeros) - 1) atomicAdd(&hist[0], static_cast<uint32_t>(__popc(zeros)));
         if (valid && d > 0) atomicAdd(&hist[d], 1u);
-      } else {  // the scores inside the range, w <= 24 here; equal bins together
+      } else {  // the scores inside the range, w <= 24 here: few but for ties
         const uint32_t r = sv[i] - lo;
-        const int d = valid && sv[i] >= lo && r < (1u << w) ? static_cast<int>(r >> shift) : -1;
-        const unsigned peers = __match_any_sync(0xffffffffu, d);
-        if (d >= 0 && lane == __ffs(peers) - 1) atomicAdd(&hist[d], static_cast<uint32_t>(__popc(peers)));
+        if (valid && sv[i] >= lo && r < (1u << w)) atomicAdd(&hist[r >> shift], 1u);
       }
     }
     __syncthreads();
@@ -396,7 +415,7 @@ select_small_kernel(const int32_t *__restrict__ L, const int32_t *__restrict__ P
   }
   bool bad = false;
 #pragma unroll
-  for (int i = 0; i < kSmallItems; ++i) {
+  for (int i = 0; i < kSmallM / kSmallThreads; ++i) {
     const int x = i * kSmallThreads + tid;
     if (x < m_inblock) {
       const long long u = static_cast<long long>(i < kSmallHold ? pv[i % kSmallHold] : __ldg(pred + x)) + q;
@@ -456,7 +475,11 @@ int maps_calibrate(const int32_t *true_len, const int32_t *pred_len, int64_t n,
   const unsigned long long kk = static_cast<unsigned long long>(k);
   if (n <= kSmallN) {
     const int mi = m <= kSmallM ? static_cast<int>(m) : 0;  // bounds in the same block
-    launch_pdl(select_small_kernel, 1, kSmallThreads, 0, s, true_len, pred_len, static_cast<int>(n),
+    const auto kern = n <= kSmallThreads       ? select_small_kernel<1>
+                      : n <= 4 * kSmallThreads ? select_small_kernel<4>
+                      : n <= 8 * kSmallThreads ? select_small_kernel<8>
+                                               : select_small_kernel<16>;
+    launch_pdl(kern, 1, kSmallThreads, 0, s, true_len, pred_len, static_cast<int>(n),
                static_cast<uint32_t>(k), query_pred, mi, bound_out, st, q_dev_out, status);
     MAPS_TRY(launch_ok());
     if (m <= kSmallM) m = 0;

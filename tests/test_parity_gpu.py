@@ -145,9 +145,10 @@ def test_golden_worked_example(M, ws, golden):
 # calibration
 # ---------------------------------------------------------------------------
 
-# one-block sizes: a bitonic sort up to 2,048 scores, a radix select up to
-# 8,192; then the cooperative kernel
-@pytest.mark.parametrize("n", [1, 2, 3, 9, 10, 1000, 1024, 1025, 2048, 2049, 4097, 65537, 1000003])
+# one-block sizes: ranked by counting up to 128 scores, then the histogram select
+# with 1, 4, 8 and 16 scores a thread; past 16,384 the cooperative kernel
+@pytest.mark.parametrize("n", [1, 2, 3, 9, 10, 127, 128, 129, 1000, 1024, 1025, 2048, 2049, 4096, 4097,
+                               8192, 8193, 16384, 16385, 65537, 1000003])
 def test_calibrate_random(M, ws, oracle, n):
     rng = np.random.default_rng(n)
     L = rng.integers(-(2**31), 2**31, n, dtype=np.int64).astype(np.int32) if n % 2 else \
@@ -191,10 +192,11 @@ def test_calibrate_unaligned_and_ranges(M, ws, oracle):
     assert M.maps_calibrate(Ld, Pd, 0, ws=ws)[0] == M.MAPS_E_INVALID
 
 
-@pytest.mark.parametrize("seed", [0, 1, 2])
-def test_calibrate_grid_bucket_edges(M, ws, oracle, seed):
-    """Grid form (n above the one-block limit): scores on the first pass's bin
-    edges (the last exact bin, each leading-bit boundary, each 7-bit step) and
+@pytest.mark.parametrize("seed,n", [(0, 20011), (1, 20011), (2, 20011), (0, 16384), (1, 9001), (2, 5003),
+                                    (0, 4096), (1, 1024), (2, 1000), (0, 128)])
+def test_calibrate_grid_bucket_edges(M, ws, oracle, seed, n):
+    """Grid form (n above the one-block limit) and the one-block forms: scores
+    on the first pass's bin edges (the last exact bin, each leading-bit boundary, each 7-bit step) and
     up to 2^32 - 1, so that quantiles resolve after one, two or three passes and
     some lie above INT32_MAX (range error)."""
     rng = np.random.default_rng(seed)
@@ -203,7 +205,6 @@ def test_calibrate_grid_bucket_edges(M, ws, oracle, seed):
         step = 1 << (e - 7)
         edges |= {(1 << e) - 1, 1 << e, (1 << e) + 1, (1 << e) + step - 1, (1 << e) + step}
     edges = np.array(sorted(edges), dtype=np.int64)
-    n = 20011
     s = rng.choice(edges, n)
     s[: n // 3] = rng.integers(0, 2**32, n // 3, dtype=np.int64)  # full range
     P = np.full(n, -(2**31), dtype=np.int64)
@@ -227,8 +228,8 @@ def test_calibrate_grid_bucket_edges(M, ws, oracle, seed):
     (1300007, 4099, 0),
     # more predictions than the grid keeps in registers, at an unaligned address
     (20011, 1300003, 1),
-    # just past the one-block limit, no queries; then a ragged, unaligned few
-    (8193, 0, 0), (10001, 777, 1),
+    # no queries; then a ragged, unaligned few
+    (8193, 0, 0), (10001, 777, 1), (4096, 16384, 0),
     # the one-block form at 16,384 residuals and queries, and past each limit;
     # a thread's last items, and queries past those loaded before the select
     (16384, 16384, 0), (16384, 16385, 1), (16385, 0, 0), (16385, 777, 1), (1024, 8193, 1),
@@ -1106,10 +1107,10 @@ def test_stream_golden(M, ws, stream_golden):
     (3000, 200, 2048, 60000, 256, 300, 100000, 1000),
     # 48 decoders: the shared-memory walk past one warp's decoders, with queues
     (4000, 48, 4096, 30000, 64, 200, 100000, 1000),
-    # a window of 10,000 completions: once it holds more than 8,192 the quantile is
-    # taken by the cooperative calibration kernel inside the loop
+    # a window of 10,000 completions, more than the one-block loop holds: batch by
+    # batch from the host, the quantile by the one-block calibration
     (30000, 8, 16384, 262144, 512, 10000, 100000, 1000),
-    # and one of 17,000, past the one-block calibration
+    # and one of 17,000, past that: by the cooperative kernel
     (40000, 8, 16384, 262144, 512, 17000, 100000, 1000),
 ])
 def test_stream_prefix(M, ws, oracle, N, D, H, cap, B, Wn, a, mw):

@@ -1,6 +1,6 @@
 """A bounded device wait that runs out is reported, and the device stays usable.
 
-The calibration's cooperative kernel (calibration sets above 8,192 residuals)
+The calibration's cooperative kernel (calibration sets above 16,384 residuals)
 waits at a bounded grid barrier after each select pass; the test aid
 maps_test_calibrate_absent_block makes one of its blocks return at once, so
 the others' wait runs out.
