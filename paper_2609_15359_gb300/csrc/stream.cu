@@ -27,9 +27,10 @@
 // step-by-step simulation of each decoder (stream_interval); deferral splits
 // the arrived requests at each dispatch step into those with a bound, those
 // timed out to round robin and those that keep waiting (stream_select).
-// The host issues the launches; it reads 40 bytes of loop state once per
-// batch (the request, completion and waiting counts, and the deferral's list
-// lengths, that size the calls).
+// Batches that fit one block run inside one kernel, up to 256 a launch
+// (stream_loop_kernel).  The others are launched step by step by the host, which
+// reads the 56 bytes of loop state once a batch (the request, completion and waiting
+// counts, and the deferral's list lengths, that size the calls).
 #include <algorithm>
 #include <climits>
 
@@ -52,7 +53,7 @@ struct StreamState {
   int32_t nc;        // deferral: requests for the dispatch policy at this step
   int32_t nto;       // deferral: requests timed out to round robin at this step
   int32_t adm_i;     // per-step mode: admissions between the dispatch steps
-  int32_t pad;
+  int32_t lists;     // the last dispatch: 1 walked sorted lists of up to 32 decoders, 2 left that to the host
   long long next_b;      // the one-block loop: the batch it stopped before
   long long total_done;  // completions by then
 };
@@ -102,6 +103,7 @@ __global__ void stream_init_kernel(int64_t first_hi, int D, int32_t cap, const i
     S->nc = 0;
     S->nto = 0;
     S->adm_i = 0;
+    S->lists = 0;
     S->next_b = 0;
     S->total_done = 0;
   }
@@ -853,10 +855,13 @@ stream_csr_kernel(int nact, int D, int rr, const int32_t *q_dev, int32_t *q_out_
 // score is a binary search for the pairs with e <= u and two reads.  One warp
 // walks the batch: a lane scores a decoder, the warp picks (feasible with the
 // smallest Q, else the largest headroom, ties to the lowest index), inserts
-// (u, p + 1) into the chosen decoder's list and rebuilds its tables.  The
-// decisions and range errors are those of the dense projection followed by
-// maps_dispatch SEQUENTIAL.  (At most 32 decoders take walk_registers below
-// while their lists fit it.)
+// (u, p + 1) into the chosen decoder's list and rebuilds its tables.  At most 32
+// decoders take walk_registers below while their lists fit it, and where this
+// kernel is launched by itself two warps share the walk over longer ones, one
+// picking while the other updates the list chosen before: 511 candidates on 6
+// decoders of some 650 pairs 1.76 against 2.56 ms by one warp.  The decisions and
+// range errors are those of the dense projection followed by maps_dispatch
+// SEQUENTIAL.
 // Beside the batch and the unsorted pairs: the pool of sorted pairs (the
 // residents of decoder k plus room for nb reservations at base_k = res_off[k] +
 // k nb) with the tables.
@@ -893,16 +898,26 @@ __host__ __device__ int stream_lists_place(int D, int nact, int nb, size_t smem,
   return D <= 32 && nact <= 64 * D && base <= smem && lists <= spare ? 2 : 0;
 }
 
-// A decoder's tables from its sorted pairs (one warp): SS[i] = sum of b over
-// pairs i.. n-1, and PM[i] = the largest V over pairs 0..i, with
-// V_i = SS[i] + (E[i] - 1)(n - i + 1) (K + t at t = E[i] - 1).  Returns
-// whether some K(t) exceeds INT32_MAX (the projection's range error); below
-// that every SS, V and PM fits 32 bits.
+// Whether two warps' walk of up to 32 decoders' lists is worth leaving the one-block
+// loop for, batch after batch: it saves about 4 ns a candidate and pair of its
+// decoder's list, and costs 50 us.  Whole runs, every such batch left against none:
+// batches of 334 on 5 decoders of some 100 pairs 1.73 against 2.01 ms, of 348 on 5
+// 5.7 against 7.1, of 458 on 5 3.5 against 4.6; but of 81 on 4 of 200 4.8 against
+// 2.9, of 38 on 4 4.1 against 3.0.
+__host__ __device__ inline bool stream_lists_long(int D, int nact, int nb) {
+  return static_cast<int64_t>(nb) * (nact + nb / 2) > static_cast<int64_t>(12000) * D;
+}
+
 // Barrier `id` over the first `count` threads (whole warps) of the block.
 __device__ __forceinline__ void named_bar(int id, int count) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
 }
 
+// A decoder's tables from its sorted pairs (one warp): SS[i] = sum of b over
+// pairs i.. n-1, and PM[i] = the largest V over pairs 0..i, with
+// V_i = SS[i] + (E[i] - 1)(n - i + 1) (K + t at t = E[i] - 1).  Returns
+// whether some K(t) exceeds INT32_MAX (the projection's range error); below
+// that every SS, V and PM fits 32 bits.
 __device__ bool rebuild_tables(const int32_t *E, const int32_t *Bv, uint32_t *SS, uint32_t *PM,
                                int n) {
   const int lane = threadIdx.x & 31;
@@ -1141,32 +1156,32 @@ __device__ bool walk_registers(int D, int nb, int mc, const int32_t *uE, const i
   return ok;
 }
 
-// kSpare: the lists may be in global memory (`lists`); a variant apart, as the
-// pointers of either kind cost the register walk 7%.
-template <bool kSpare>
+// The sorted lists are in shared memory behind the rest, or (kGlobal) in `lists`.
+// kTwo: up to 32 decoders' sorted lists are walked by two warps.  In the one-block
+// loop, whose registers that code would take from the register walk (2 to 4% of its
+// batches), one warp walks them, where they fit its `smem` bytes and are not long
+// (stream_lists_long); else nothing is decided and the host launches the dispatch.
+// *walked_lists: 0 no sorted lists (or more decoders), 1 walked here, 2 left.
+template <bool kGlobal, bool kTwo>
 __device__ void
 dispatch_block(unsigned char *sdm, unsigned char *lists, int D, int H, int nb, int mc, const int64_t *res_off,
                const int32_t *rp, const int32_t *rg, const int32_t *rU, const int32_t *capv,
                int32_t *Q, const int32_t *cp, const int32_t *cU, int32_t *choice,
-               int64_t *headroom, int32_t *status) {
+               int64_t *headroom, int32_t *status, int32_t *walked_lists, size_t smem) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nact = static_cast<int>(res_off[D]);
   const int pool = nact + D * nb;
-  // the lists: first in shared memory, or (kSpare) in `lists`, or with it null
-  // after the rest; the batch of the register walk, (nb + 1) pairs, is first
-  // there, or over the lists, which that walk does not use
-  int32_t *E = reinterpret_cast<int32_t *>(                // [pool] sorted end steps
-      !kSpare ? sdm : lists != nullptr ? lists : sdm + stream_dispatch_smem(D, nact, nb));
-  int32_t *Bv = E + pool;                                  // [pool] their b
-  uint32_t *SS = reinterpret_cast<uint32_t *>(Bv + pool);  // [pool] suffix sums of b
-  uint32_t *PM = SS + pool;                                // [pool] prefix maxima of V
-  int2 *cand = reinterpret_cast<int2 *>(sdm);
-  int32_t *uE = kSpare ? reinterpret_cast<int32_t *>(cand + nb + 1)  // [nact] unsorted
-                       : reinterpret_cast<int32_t *>(PM + pool);
+  int2 *cand = reinterpret_cast<int2 *>(sdm);                        // [nb + 1] the register walk's batch
+  int32_t *uE = reinterpret_cast<int32_t *>(cand + nb + 1);          // [nact] unsorted
   int32_t *uB = uE + nact;
   int32_t *s_base = uB + nact, *s_n = s_base + D, *s_q = s_n + D, *s_cap = s_q + D;
   int32_t *s_cp = s_cap + D, *s_cu = s_cp + nb;            // [nb] the batch
   int32_t *s_ch = s_cu + nb;                               // [nb] choices (fast path)
+  int32_t *E = reinterpret_cast<int32_t *>(                // [pool] sorted end steps
+      kGlobal ? lists : sdm + stream_dispatch_smem(D, nact, nb));
+  int32_t *Bv = E + pool;                                  // [pool] their b
+  uint32_t *SS = reinterpret_cast<uint32_t *>(Bv + pool);  // [pool] suffix sums of b
+  uint32_t *PM = SS + pool;                                // [pool] prefix maxima of V
   __shared__ int s_bad, s_fast;
   if (tid == 0) {
     s_bad = 0;
@@ -1384,6 +1399,12 @@ dispatch_block(unsigned char *sdm, unsigned char *lists, int D, int H, int nb, i
     __syncthreads();
   }
 
+  if (!kTwo && !walked && D <= 32 &&
+      (stream_lists_long(D, nact, nb) ||
+       stream_dispatch_smem(D, nact, nb) + stream_lists_bytes(D, nact, nb) > smem)) {
+    if (tid == 0) *walked_lists = 2;
+    return;
+  }
   if (!walked) {
     // sort each decoder's pairs by e (rank among the decoder's pairs, ties by
     // position), and check sum b <= INT32_MAX (K at step 0)
@@ -1416,7 +1437,230 @@ dispatch_block(unsigned char *sdm, unsigned char *lists, int D, int H, int nb, i
   // e <= u), then M = max(PM[c - 1], SS[c] + (u - 1)(n - c + 1)); a packed key
   // picks (feasible first, then Q or the largest headroom, then the lowest
   // index); the warp inserts the footprint and rebuilds that decoder's tables.
-  if (!walked && warp == 0) {
+  if (walked) {
+    // decided above
+  } else if (kTwo && D <= 32) {
+    // Two warps, one decoder per lane.  Warp 0 holds each decoder's list
+    // length, base, Q and capacity in registers, scores the candidates, picks
+    // and books each decision and hands it to warp 1 through shared memory
+    // (named barrier 1); warp 1 inserts the reservation into the chosen
+    // decoder's list and scores that decoder again for the next candidate
+    // (named barrier 2).  Meanwhile warp 0 scores the next candidate on the
+    // lists as they stand: a reservation only raises the chosen decoder's Q
+    // and occupancy, so every other decoder's key is already final and the
+    // chosen one's is replaced by warp 1's.  Keys: inf << 63 | v << 10 | k,
+    // the smallest wins.
+    __shared__ int h_bk, h_pos, h_n, h_base, h_q, h_cap, h_c;
+    __shared__ long long h_M;
+    __shared__ unsigned long long h_key;
+    auto clampu = [&](int32_t U) { return U < 1 ? 1 : (U > H ? H : U); };
+    // c = the pairs with e <= u of a sorted list (8-ary search: eight
+    // independent probes per level, one level for up to 8 pairs)
+    auto count_le = [&](const int32_t *Ek, int n, int u) {
+      int lo = 0, hi = n;
+      while (lo < hi) {
+        const int len = hi - lo;
+        int nlo = lo, nhi = hi;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {  // probes cover every position when len <= 8
+          const int pi = lo + (len * i) / 8;
+          if (Ek[pi] <= u)
+            nlo = max(nlo, pi + 1);
+          else
+            nhi = min(nhi, pi);
+        }
+        lo = nlo;
+        hi = nhi;
+      }
+      return lo;
+    };
+    auto key_of = [mc](int k, int q, int cap, int32_t p, long long M) {
+      const long long h = static_cast<long long>(cap) - (static_cast<long long>(p) + 1 + M);
+      return dispatch_key(h, q, k, mc);
+    };
+    if (warp == 0) {
+      const int k = lane;
+      const bool has = k < D;
+      int n_r = has ? s_n[k] : 0, q_r = has ? s_q[k] : 0;
+      const int base_r = has ? s_base[k] : 0, cap_r = has ? s_cap[k] : 0;
+      bool bad = false, have = false;  // have: key, c and M are the current candidate's
+      unsigned long long key = ~0ull;
+      long long M = 0;
+      int c = 0;
+      auto score = [&](int32_t pp, int uu) {
+        key = ~0ull;
+        if (!has) return;
+        if (quick && n_r > 0) {
+          const long long mub = max(static_cast<long long>(PM[base_r + n_r - 1]),
+                                    static_cast<long long>(SS[base_r]) +
+                                        static_cast<long long>(uu - 1) * (n_r + 1));
+          if (static_cast<long long>(pp) + 1 + mub <= cap_r) {
+            key = (static_cast<unsigned long long>(q_r) << 10) | static_cast<unsigned>(k);
+            c = -1;   // found at insertion
+            M = mub;  // bounds every new cell: no range error (cap <= INT32_MAX)
+            return;
+          }
+        }
+        c = count_le(E + base_r, n_r, uu);
+        const long long full = c > 0 ? static_cast<long long>(PM[base_r + c - 1]) : LLONG_MIN;
+        const long long part = static_cast<long long>(c < n_r ? SS[base_r + c] : 0u) +
+                               static_cast<long long>(uu - 1) * (n_r - c + 1);
+        M = max(full, part);
+        key = key_of(k, q_r, cap_r, pp, M);
+      };
+      for (int j = 0; j < nb; ++j) {
+        const int32_t p = s_cp[j], U = s_cu[j];
+        int bk = -1;
+        if ((p | U) >= 0) {
+          if (!have) score(p, clampu(U));
+          // the warp's smallest key: one 32-bit reduction when every value
+          // fits 21 bits (inf << 31 | v << 10 | k, the same order), else a ladder
+          const unsigned long long kv = (key >> 10) & ((1ull << 53) - 1);
+          const bool none = key == ~0ull;
+          if (__all_sync(0xffffffffu, none || kv < (1ull << 21))) {
+            const uint32_t k32 = none ? 0xffffffffu
+                                      : (static_cast<uint32_t>(key >> 63) << 31) |
+                                            (static_cast<uint32_t>(kv) << 10) | static_cast<uint32_t>(key & 1023u);
+            bk = static_cast<int>(__reduce_min_sync(0xffffffffu, k32) & 1023u);
+          } else {
+            unsigned long long kk = key;
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) {
+              const unsigned long long o = __shfl_xor_sync(0xffffffffu, kk, off);
+              kk = o < kk ? o : kk;
+            }
+            bk = static_cast<int>(kk & 1023u);
+          }
+          if (lane == bk) {  // the chosen decoder's lane books the decision
+            choice[j] = bk;
+            bad |= q_r == 0x7fffffff;
+            q_r += q_r == 0x7fffffff ? 0 : 1;
+            // every new cell K + p + t + 1 (t < u) is at most M + p + 1
+            bad |= static_cast<long long>(p) + 1 + M > 0x7fffffffLL;
+            h_bk = bk;
+            h_pos = c;
+            h_n = n_r;
+            h_base = base_r;
+            h_q = q_r;
+            h_cap = cap_r;
+            n_r += 1;
+          }
+        } else if (lane == 0) {
+          bad = true;
+          choice[j] = -1;
+          h_bk = -1;
+        }
+        named_bar(1, 64);  // the decision goes to warp 1
+        const bool nxt = j + 1 < nb;
+        const int32_t p1 = nxt ? s_cp[j + 1] : 0, U1 = nxt ? s_cu[j + 1] : 0;
+        const bool ok1 = nxt && (p1 | U1) >= 0;
+        if (ok1) score(p1, clampu(U1));  // the chosen decoder's key is replaced below
+        named_bar(2, 64);  // warp 1 has updated the list and scored it again
+        if (ok1 && lane == bk) {
+          key = h_key;
+          c = h_c;
+          M = h_M;
+        }
+        have = ok1;
+      }
+      if (__any_sync(0xffffffffu, bad) && lane == 0) flag_error(status, MAPS_E_RANGE);
+      if (has) {
+        s_n[k] = n_r;
+        s_q[k] = q_r;
+      }
+    } else if (warp == 1) {
+      for (int j = 0; j < nb; ++j) {
+        named_bar(1, 64);
+        const int bk = h_bk;
+        if (bk >= 0) {
+          const int n = h_n, base = h_base, m = n + 1;
+          const int32_t p = s_cp[j];
+          const int u = clampu(s_cu[j]);
+          int pos = h_pos;  // -1: the scoring took the bound, count the pairs with e <= u here
+          if (pos < 0) {
+            if (n < 32)
+              pos = __popc(__ballot_sync(0xffffffffu, lane < n && E[base + lane] <= u));
+            else
+              pos = count_le(E + base, n, u);
+          }
+          const bool nxt = j + 1 < nb;
+          const int32_t p1 = nxt ? s_cp[j + 1] : 0, U1 = nxt ? s_cu[j + 1] : 0;
+          const bool ok1 = nxt && (p1 | U1) >= 0;
+          const int u1 = clampu(U1);
+          int c1 = 0;
+          long long M1 = 0;
+          if (m <= 32) {
+            // one round: lane i takes pair i of the new list; the suffix sums
+            // follow from the old ones (b more before the new pair, the same
+            // after it) and one shuffle scan gives the prefix maxima of V, in
+            // 32 bits (the booking's check keeps every K + t within INT32_MAX)
+            const int src = lane <= pos ? lane : lane - 1;
+            const bool old_ok = src < n;
+            const int eo = old_ok ? E[base + src] : 0, bo = old_ok ? Bv[base + src] : 0;
+            const uint32_t so = old_ok ? SS[base + src] : 0u;
+            const uint32_t bnew = static_cast<uint32_t>(p) + 1u;
+            const int e2 = lane == pos ? u : eo;
+            const int b2 = lane == pos ? static_cast<int>(bnew) : bo;
+            const uint32_t suf = lane <= pos ? so + bnew : so;
+            uint32_t V = lane < m ? suf + static_cast<uint32_t>(e2 - 1) * static_cast<uint32_t>(m - lane + 1) : 0u;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+              const uint32_t y = __shfl_up_sync(0xffffffffu, V, off);
+              if (lane >= off) V = max(V, y);
+            }
+            __syncwarp();  // every lane has read the old list
+            if (lane < m) {
+              E[base + lane] = e2;
+              Bv[base + lane] = b2;
+              SS[base + lane] = suf;
+              PM[base + lane] = V;
+            }
+            // the new list's count and table values at the next candidate's u
+            c1 = __popc(__ballot_sync(0xffffffffu, lane < m && e2 <= u1));
+            const uint32_t pmb = __shfl_sync(0xffffffffu, V, c1 > 0 ? c1 - 1 : 0);
+            const uint32_t ssb = __shfl_sync(0xffffffffu, suf, c1 < m ? c1 : 0);
+            const long long full = c1 > 0 ? static_cast<long long>(pmb) : LLONG_MIN;
+            const long long part = static_cast<long long>(c1 < m ? ssb : 0u) +
+                                   static_cast<long long>(u1 - 1) * (m - c1 + 1);
+            M1 = max(full, part);
+          } else {
+            // a list past 32 pairs: shift [pos, n) up by one (last round
+            // first), place the new pair, rebuild the tables
+            for (int r = (n - 1) >> 5; r >= 0; --r) {
+              const int i = r * 32 + lane;
+              const bool mv = i < n && i >= pos;
+              const int e = mv ? E[base + i] : 0, b = mv ? Bv[base + i] : 0;
+              __syncwarp();
+              if (mv) {
+                E[base + i + 1] = e;
+                Bv[base + i + 1] = b;
+              }
+              __syncwarp();
+            }
+            if (lane == 0) {
+              E[base + pos] = u;
+              Bv[base + pos] = p + 1;
+            }
+            __syncwarp();
+            rebuild_tables(E + base, Bv + base, SS + base, PM + base, m);
+            if (ok1) {
+              c1 = count_le(E + base, m, u1);
+              const long long full = c1 > 0 ? static_cast<long long>(PM[base + c1 - 1]) : LLONG_MIN;
+              const long long part = static_cast<long long>(c1 < m ? SS[base + c1] : 0u) +
+                                     static_cast<long long>(u1 - 1) * (m - c1 + 1);
+              M1 = max(full, part);
+            }
+          }
+          if (ok1 && lane == 0) {
+            h_key = key_of(bk, h_q, h_cap, p1, M1);
+            h_c = c1;
+            h_M = M1;
+          }
+        }
+        named_bar(2, 64);
+      }
+    }
+  } else if (warp == 0) {
     for (int j = 0; j < nb; ++j) {
       const int32_t p = s_cp[j], U = s_cu[j];
       if ((p | U) < 0) {
@@ -1569,14 +1813,16 @@ dispatch_block(unsigned char *sdm, unsigned char *lists, int D, int H, int nb, i
   __syncthreads();
   for (int k = tid; k < D; k += kSt) Q[k] = s_q[k];
 }
+template <bool kGlobal>
 __global__ void __launch_bounds__(kSt, 1)
 stream_dispatch_kernel(int D, int H, int nb, int mc, const int64_t *res_off, const int32_t *rp,
                        const int32_t *rg, const int32_t *rU, const int32_t *capv, int32_t *Q,
                        const int32_t *cp, const int32_t *cU, int32_t *choice, int64_t *headroom,
-                       int32_t *status, unsigned char *lists) {
+                       int32_t *status, unsigned char *lists, StreamState *S) {
   pdl_prologue();
   extern __shared__ __align__(16) unsigned char sdm[];
-  dispatch_block<true>(sdm, lists, D, H, nb, mc, res_off, rp, rg, rU, capv, Q, cp, cU, choice, headroom, status);
+  dispatch_block<kGlobal, true>(sdm, lists, D, H, nb, mc, res_off, rp, rg, rU, capv, Q, cp, cU, choice, headroom,
+                               status, &S->lists, 0);
 }
 
 // 5''. Deferral: the listed requests join the waiting queues at act[nact..]:
@@ -1800,14 +2046,23 @@ struct StreamWs {
 //   * the quantile comes from a histogram of the window's scores, as in
 //     maps_calibrate's one-block form.
 // It stops before a batch that does not fit (the requests in the system, the
-// window, the dispatch's shared memory); the host then runs that batch by the
-// launches below and comes back when the system is smaller.
+// window, the dispatch's shared memory), or at the dispatch of one whose sorted
+// lists two warps should walk; the host then runs that batch, or the rest of it, by
+// the launches below and comes back when the next one fits.
 // ---------------------------------------------------------------------------
-constexpr int kLoopActive = 2048;  // requests in the system and the batch, at most
-constexpr int kLoopWindow = 4096;
-constexpr int kLoopRank = 512;     // keys of a group ranked by counting
+// Requests in the system and the batch, at most (their sort keys take 18 bytes each
+// of shared memory).  1,024 and 4,096 instead: 20,000 requests on 20 decoders at
+// 40,000 tokens, batches of 512, 8.3 and 6.8 against 6.8 ms; batches of 1,024 on 32
+// with room 2.8 and 1.7 against 2.6; batches of 256 with room 3.3 all three.
+constexpr int kLoopActive = 2048;
+constexpr int kLoopWindow = 4096;  // four scores a thread
+// Keys of a group ranked by counting, n^2 comparisons by all threads against the
+// network's log^2 n barriers.  128, 256 and 1,024 instead: 30,000 requests with room
+// 3.65, 3.47 and 3.29 against 3.30 ms (some 250 completions a batch).
+constexpr int kLoopRank = 512;
 constexpr int kLoopBatches = 256;  // batches of one launch
 constexpr int kLoopUsual = 1024;   // requests in the system its shared memory is first sized for
+constexpr int kListsD = 16;        // with room for sorted lists below this many decoders
 
 struct LoopArgs {
   maps_stream_cfg c;
@@ -1822,6 +2077,14 @@ struct LoopArgs {
   int64_t b0;             // the first batch to run
   long long total_done0;  // completions before it
 };
+
+// Shared memory the loop's dispatch cannot do without: none for the policies that
+// walk nothing; of up to 32 decoders not the sorted lists, whose walk the host can
+// launch.
+__host__ __device__ inline size_t loop_dispatch_smem(const maps_stream_cfg &c, int nact, int nb) {
+  if (c.dispatch_policy != MAPS_STREAM_MAPS && c.dispatch_policy != MAPS_STREAM_MC) return 0;
+  return stream_dispatch_smem(c.D, nact, nb) + (c.D <= 32 ? 0 : stream_lists_bytes(c.D, nact, nb));
+}
 
 // Sorts groups of unique keys: group i is key[seg[i], seg[i + 1]), with which[x]
 // the group of key x; out[x's place] gets the key.  Every thread of the block.
@@ -1977,8 +2240,8 @@ stream_loop_kernel(const __grid_constant__ LoopArgs a) {
   int32_t *const cur = scratch + kStreamMaxD + 8;  // [D] cursors
   int64_t b = a.b0;
   long long total_done = a.total_done0;
-  // per-step mode may keep the dispatch's lists in w.K, which this loop does not use
-  const size_t spare = kPerStep ? sizeof(int32_t) * static_cast<size_t>(D) * c.H : 0;
+  __shared__ int32_t s_lists;
+  if (tid == 0) s_lists = 0;  // (2 at the end: batch b stopped at its dispatch in this launch)
   for (int run = 0; run < kLoopBatches && b < a.nbatch; ++run, ++b) {
     const int64_t lo = b * B, hi = min(lo + B, N);
     const int nb = static_cast<int>(hi - lo);
@@ -1993,9 +2256,7 @@ stream_loop_kernel(const __grid_constant__ LoopArgs a) {
     }
     const int nc = defer ? S->nc : nb, nto = defer ? S->nto : 0;
     const int most = S->nact + nto;  // requests in the system before this batch's, at most
-    const bool place = kPerStep ? stream_lists_place(D, most, nc, a.smem, spare) != 0
-                                : stream_dispatch_smem(D, most, nc) + stream_lists_bytes(D, most, nc) <= a.smem;
-    if (most + nc > kLoopActive || !place) {
+    if (most + nc > kLoopActive || loop_dispatch_smem(c, most, nc) > a.smem) {
       __syncthreads();
       if (tid == 0) S->npend = npend;  // the batch is not started
       break;
@@ -2075,11 +2336,10 @@ stream_loop_kernel(const __grid_constant__ LoopArgs a) {
       if (warp == 0) lr_warp(reinterpret_cast<uint32_t *>(scratch), D, nc, w.res_off, cch);
       __syncthreads();
     } else if (nc > 0 && !rr && c.dispatch_policy != MAPS_STREAM_RR) {  // 5.
-      unsigned char *const lists = !kPerStep || stream_lists_place(D, nact, nc, a.smem, 0) == 1
-                                       ? nullptr : reinterpret_cast<unsigned char *>(w.K);
-      dispatch_block<kPerStep>(ldm, lists, D, c.H, nc, mc, w.res_off, w.rp, w.rg, w.rU, w.capv, w.Q, cpr, w.Uq + nact, cch,
-                     nullptr, a.status);
+      dispatch_block<false, false>(ldm, nullptr, D, c.H, nc, mc, w.res_off, w.rp, w.rg, w.rU, w.capv, w.Q, cpr,
+                                   w.Uq + nact, cch, nullptr, a.status, &s_lists, a.smem);
       __syncthreads();
+      if (s_lists == 2) break;  // the host takes the batch up from here
     }
     if (!defer)  // 6.
       enqueue_batch(lo, nb, nact, hi, D, a.arrival, a.choice, w.Uq, w.st, w.dec, w.disp, w.g, w.U, act, S,
@@ -2147,6 +2407,7 @@ stream_loop_kernel(const __grid_constant__ LoopArgs a) {
   if (tid == 0) {
     S->next_b = b;
     S->total_done = total_done;
+    S->lists = s_lists;
   }
 }
 
@@ -2291,27 +2552,30 @@ int maps_stream_run(const maps_stream_cfg *cfg, const int64_t *arrival_ms, const
   MAPS_TRY(allow_smem(loop, loop_smem));
   const size_t spare = sizeof(int32_t) * static_cast<size_t>(D) * c.H;  // the dense K, else unused
   // What the loop leaves of the multiprocessor's memory is its L1 cache, which
-  // the requests' state then hits: it starts with what kLoopUsual requests in the
-  // system need, and takes all of it where a batch does not fit that.  Per step
-  // the dispatch's lists stay in K where the register walk (128 pairs a decoder)
-  // is all but sure to do without them: 64 requests a decoder at most (as the
-  // place has it) and 16 candidates.  32 decoders, batches of 256, 20,000 to
-  // 30,000 requests: 3.53 -> 3.34 ms where no queue forms, 9.14 -> 9.00 at 16,000
-  // tokens, 11.33 -> 11.13 per step.
+  // the requests' state then hits: it starts with what the usual batch needs, and
+  // takes all of it where a batch does not fit that.  The usual batch has kLoopUsual
+  // requests in the system, and sorted lists below kListsD decoders (above, lists
+  // past the register walk's 128 pairs are rare in a system of 2,048).
   const int nb0 = static_cast<int>(std::min(B, static_cast<int64_t>(kLoopActive)));
-  size_t usual = std::max<size_t>(18 * kLoopActive, sizeof(uint32_t) << kStepBits);  // the sorts, the quantile
-  usual = std::max(usual, per_step && D <= 32 && nb0 <= 16 * D
-                              ? stream_dispatch_smem(D, kLoopActive, nb0)
-                              : stream_dispatch_smem(D, kLoopUsual, nb0) + stream_lists_bytes(D, kLoopUsual, nb0));
+  size_t usual = loop_dispatch_smem(c, D >= kListsD && D <= 32 ? kLoopActive : kLoopUsual, nb0);
+  if (usual > 0 && D < kListsD) usual += stream_lists_bytes(D, kLoopUsual, nb0);
+  usual = std::max<size_t>({usual, 18 * kLoopActive, sizeof(uint32_t) << kStepBits});  // the sorts, the quantile
   usual = std::min(usual, loop_smem);
   size_t give = usual;
   auto loop_fits = [&](int64_t system, int64_t cands) {  // requests in the system, candidates
     return c.window <= kLoopWindow && system + cands <= kLoopActive &&
-           stream_lists_place(D, static_cast<int>(system), static_cast<int>(cands), loop_smem,
-                              per_step ? spare : 0) != 0;
+           loop_dispatch_smem(c, static_cast<int>(system), static_cast<int>(cands)) <= loop_smem;
+  };
+  // whether the loop, with all of the memory, walks that batch's lists itself
+  auto walks_here = [&](int64_t system, int64_t cands) {
+    const int n = static_cast<int>(system), nc = static_cast<int>(cands);
+    return !stream_lists_long(D, n, nc) &&
+           stream_dispatch_smem(D, n, nc) + stream_lists_bytes(D, n, nc) <= loop_smem;
   };
   bool in_loop = loop_fits(0, std::min(N, B));
+  int64_t left = -1;  // the batch the loop last left at its dispatch
   for (int64_t b = 0; b < nbatch; ++b) {
+    bool resume = false;  // the loop has taken batch b up to its dispatch
     if (in_loop) {
       LoopArgs la;
       la.c = c;
@@ -2337,30 +2601,34 @@ int maps_stream_run(const maps_stream_cfg *cfg, const int64_t *arrival_ms, const
       const bool stopped = hs.next_b < nbatch && hs.next_b < b + kLoopBatches;
       b = hs.next_b;
       total_done = hs.total_done;
-      if (!stopped || give < loop_smem) {
+      resume = hs.lists == 2;
+      if (resume && walks_here(hs.nact, defer ? hs.nc : std::min(B, N - b * B))) give = loop_smem;
+      if (!resume && (!stopped || give < loop_smem)) {
         --b;  // all done, or a launch's worth, or on with all of the memory
         give = stopped ? loop_smem : usual;
         continue;
       }
-      in_loop = false;  // batch b does not fit: it runs here
+      in_loop = false;  // batch b does not fit, or its lists are long: it runs here
     }
     const int64_t lo = b * B, hi = std::min(lo + B, N);
     const int nb = static_cast<int>(hi - lo);
     int32_t *act_in = w.act[b & 1], *act = w.act[(b & 1) ^ 1];
     int64_t *stats_b = stats_out + 4 * b;
-    if (defer)  // 4 (first half): who is dispatched at this step
-      launch_pdl(stream_select_kernel, 1, kSt, 0, s, lo, nb, hi, c.beta, b + 1 == nbatch ? 1 : 0,
-                 arrival_ms, pred_delay, w.pend[b & 1], w.pend[(b & 1) ^ 1], w.cid, w.tout, w.S);
-    if (per_step)  // 1'.
-      launch_pdl(stream_interval_kernel, 1, kSt, 0, s, hi, D, c.cap, c.accounting, arrival_ms,
-                 prompt, true_len, w.U, w.res_u, w.st, w.g, w.dec, act_in, w.wid, w.wperm, w.wseg,
-                 w.qhead, w.aseq, w.dseq, w.rbuf, w.sbuf, w.done_id, w.done_rem, w.S, dec_stats_out);
-    launch_pdl(stream_advance_kernel, 1, kSt, 0, s, hi, D, c.cap, c.accounting, per_step, arrival_ms,
-               prompt, true_len, w.res_u, w.st, w.g, w.dec, act_in, act, w.done_id, w.done_rem,
-               w.used, w.S, stats_b, dec_stats_out);
-    MAPS_TRY(launch_ok());
-    MAPS_TRY(cuda_ok(cudaMemcpyAsync(&hs, w.S, sizeof(hs), cudaMemcpyDeviceToHost, s)));
-    MAPS_TRY(cuda_ok(cudaStreamSynchronize(s)));
+    if (!resume) {
+      if (defer)  // 4 (first half): who is dispatched at this step
+        launch_pdl(stream_select_kernel, 1, kSt, 0, s, lo, nb, hi, c.beta, b + 1 == nbatch ? 1 : 0,
+                   arrival_ms, pred_delay, w.pend[b & 1], w.pend[(b & 1) ^ 1], w.cid, w.tout, w.S);
+      if (per_step)  // 1'.
+        launch_pdl(stream_interval_kernel, 1, kSt, 0, s, hi, D, c.cap, c.accounting, arrival_ms,
+                   prompt, true_len, w.U, w.res_u, w.st, w.g, w.dec, act_in, w.wid, w.wperm, w.wseg,
+                   w.qhead, w.aseq, w.dseq, w.rbuf, w.sbuf, w.done_id, w.done_rem, w.S, dec_stats_out);
+      launch_pdl(stream_advance_kernel, 1, kSt, 0, s, hi, D, c.cap, c.accounting, per_step, arrival_ms,
+                 prompt, true_len, w.res_u, w.st, w.g, w.dec, act_in, act, w.done_id, w.done_rem,
+                 w.used, w.S, stats_b, dec_stats_out);
+      MAPS_TRY(launch_ok());
+      MAPS_TRY(cuda_ok(cudaMemcpyAsync(&hs, w.S, sizeof(hs), cudaMemcpyDeviceToHost, s)));
+      MAPS_TRY(cuda_ok(cudaStreamSynchronize(s)));
+    }
     int nact = hs.nact;
     const int ndone = hs.ndone, nwait = hs.nwait;
     // the policy's candidates: the batch, or (deferral) the listed ids
@@ -2369,35 +2637,38 @@ int maps_stream_run(const maps_stream_cfg *cfg, const int64_t *arrival_ms, const
     const int32_t *cpr = defer ? w.cp : prompt + lo;
     int32_t *cch = defer ? w.cch : choice_out + lo;
 
-    if (ndone > 0) {  // 2.
-      MAPS_TRY(maps_order_local(ndone, 1, w.zeros, w.done_rem, w.zeros, w.done_id, 0, w.done_perm,
-                                w.done_seg, ws, w.sub_bytes, stream));
-      launch_pdl(stream_window_kernel, grid_for(ndone), 256, 0, s, ndone, total_done, c.window,
-                                                           w.done_perm, w.done_id, true_len, pred,
-                                                           w.win_true, w.win_pred);
-      total_done += ndone;
-    }
-    const int64_t win_len = std::min<long long>(total_done, c.window);
-    if (nto > 0) {  // 4 (second half): timed out, round robin with the horizon as bound
-      launch_pdl(stream_enqueue_list_kernel, grid_for(nto), 256, 0, s, nto, nact, D, c.H, hi,
-                 arrival_ms, w.tout, nullptr, w.Uq, choice_out, w.st, w.dec, w.disp, w.g, w.U, act,
-                 w.S, status);
-      nact += nto;
-    }
+    bool rr = false;  // (a batch taken up has a bound)
+    if (!resume) {
+      if (ndone > 0) {  // 2.
+        MAPS_TRY(maps_order_local(ndone, 1, w.zeros, w.done_rem, w.zeros, w.done_id, 0, w.done_perm,
+                                  w.done_seg, ws, w.sub_bytes, stream));
+        launch_pdl(stream_window_kernel, grid_for(ndone), 256, 0, s, ndone, total_done, c.window,
+                                                             w.done_perm, w.done_id, true_len, pred,
+                                                             w.win_true, w.win_pred);
+        total_done += ndone;
+      }
+      const int64_t win_len = std::min<long long>(total_done, c.window);
+      if (nto > 0) {  // 4 (second half): timed out, round robin with the horizon as bound
+        launch_pdl(stream_enqueue_list_kernel, grid_for(nto), 256, 0, s, nto, nact, D, c.H, hi,
+                   arrival_ms, w.tout, nullptr, w.Uq, choice_out, w.st, w.dec, w.disp, w.g, w.U, act,
+                   w.S, status);
+        nact += nto;
+      }
 
-    launch_pdl(stream_gather_kernel, grid_for(nact + nc), 256, 0, s, nact, nc, lo, act, cids, pred,
-               prompt, w.qpred, w.cp);
-    const int cs = maps_calibrate(w.win_true, w.win_pred, win_len, c.alpha_ppm, w.qpred, nact + nc,
-                                  w.Uq, w.q_dev, nullptr, ws, w.sub_bytes, stream);  // 3.
-    const bool rr = cs == MAPS_E_UNBOUNDED;
-    if (cs != MAPS_OK && !rr) return cs;
-    if (rr)
-      launch_pdl(stream_rr_kernel, grid_for(nact + nc), 256, 0, s, nact + nc, nc, lo, D, 1, w.qpred,
-                 w.Uq, cids, cch);
-    launch_pdl(stream_csr_kernel, 1, kSt, 0, s, nact, D, rr ? 1 : 0, w.q_dev, q_out + b, act, w.st, w.g,
-               w.dec, prompt, w.Uq, w.U, w.res_off, w.rp, w.rg, w.rU, w.Q, arrival_ms, pdl, hi,
-               c.H);  // 4.
-    MAPS_TRY(launch_ok());
+      launch_pdl(stream_gather_kernel, grid_for(nact + nc), 256, 0, s, nact, nc, lo, act, cids, pred,
+                 prompt, w.qpred, w.cp);
+      const int cs = maps_calibrate(w.win_true, w.win_pred, win_len, c.alpha_ppm, w.qpred, nact + nc,
+                                    w.Uq, w.q_dev, nullptr, ws, w.sub_bytes, stream);  // 3.
+      rr = cs == MAPS_E_UNBOUNDED;
+      if (cs != MAPS_OK && !rr) return cs;
+      if (rr)
+        launch_pdl(stream_rr_kernel, grid_for(nact + nc), 256, 0, s, nact + nc, nc, lo, D, 1, w.qpred,
+                   w.Uq, cids, cch);
+      launch_pdl(stream_csr_kernel, 1, kSt, 0, s, nact, D, rr ? 1 : 0, w.q_dev, q_out + b, act, w.st, w.g,
+                 w.dec, prompt, w.Uq, w.U, w.res_off, w.rp, w.rg, w.rU, w.Q, arrival_ms, pdl, hi,
+                 c.H);  // 4.
+      MAPS_TRY(launch_ok());
+    }
     const int mc = c.dispatch_policy == MAPS_STREAM_MC ? 1 : 0;
     if (nc == 0) {
       // nobody to dispatch at this step
@@ -2413,10 +2684,11 @@ int maps_stream_run(const maps_stream_cfg *cfg, const int64_t *arrival_ms, const
       if (place != 0) {
         // the decoders' pairs and the batch fit in shared memory: no dense projection
         const size_t dsm = stream_dispatch_smem(D, nact, nc) + (place == 1 ? stream_lists_bytes(D, nact, nc) : 0);
-        MAPS_TRY(allow_smem(stream_dispatch_kernel, most));
-        launch_pdl(stream_dispatch_kernel, 1, kSt, dsm, s, D, c.H, nc, mc, w.res_off, w.rp, w.rg,
-                   w.rU, w.capv, w.Q, cpr, w.Uq + nact, cch, nullptr, status,  // no headroom out
-                   place == 1 ? nullptr : reinterpret_cast<unsigned char *>(w.K));
+        const auto kern = place == 1 ? stream_dispatch_kernel<false> : stream_dispatch_kernel<true>;
+        MAPS_TRY(allow_smem(kern, most));
+        launch_pdl(kern, 1, kSt, dsm, s, D, c.H, nc, mc, w.res_off, w.rp, w.rg, w.rU, w.capv, w.Q, cpr,
+                   w.Uq + nact, cch, nullptr, status,  // no headroom out
+                   place == 1 ? nullptr : reinterpret_cast<unsigned char *>(w.K), w.S);
         MAPS_TRY(launch_ok());
       } else {
         MAPS_TRY(maps_project_occupancy(D, c.H, w.res_off, nact, w.rp, w.rg, w.rU, w.K, nullptr, ws,
@@ -2447,8 +2719,12 @@ int maps_stream_run(const maps_stream_cfg *cfg, const int64_t *arrival_ms, const
                arrival_ms, w.wseg, w.wperm, w.wid, prompt, w.U, w.used, w.st, w.g, w.res_u, w.aseq,
                w.dseq, w.qhead, w.S, stats_b, dec_stats_out);  // 8.
     MAPS_TRY(launch_ok());
-    // back to the one block once the next batch is sure to fit
-    in_loop = loop_fits(n_all, B + hs.npend);
+    // back to the one block once the next batch is sure to fit; but not while lists
+    // that it leaves to the host are walked (as of the batch before), or right after
+    // two such batches in a row
+    const bool again = walks_here(nact, nc) || (resume ? left != b - 1 : hs.lists == 0);
+    if (resume) left = b;
+    in_loop = again && loop_fits(n_all, B + hs.npend);
   }
   return maps_check(ws, stream);
 }

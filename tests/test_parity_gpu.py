@@ -1141,7 +1141,13 @@ def test_stream_walk_list_sizes(M, ws, oracle, N, D, cap, B):
     # one decoder, and as many as a warp's lanes, with more picks than threads
     (4000, 1, 262144, 1500, 300), (6000, 32, 262144, 1100, 300),
     # many completions in one batch: sorted by the network
-    (9000, 40, 262144, 900, 700)])
+    (9000, 40, 262144, 900, 700),
+    # sorted lists past 128 pairs a decoder: walked in the loop (short), left to the
+    # host at the dispatch (long), both in turn, on one decoder and on as many as a
+    # warp's lanes; no room for them with 16 decoders and more
+    (3000, 4, 229000, 40, 300), (2453, 5, 87144, 458, 980), (4501, 5, 97355, 348, 262),
+    (1983, 1, 57103, 47, 50), (3000, 15, 30000, 300, 200), (3000, 16, 30000, 300, 200),
+    (6000, 32, 15000, 400, 300), (3000, 33, 20000, 300, 200)])
 def test_stream_one_block_loop_limits(M, ws, oracle, N, D, cap, B, Wn):
     w = W.make_stream(n_requests=N)
     check_stream(M, ws, oracle, N, D, 16384, cap, B, Wn, 100000, 1000, w)

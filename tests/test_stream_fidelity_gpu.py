@@ -108,6 +108,18 @@ def test_shapes(M, ws, oracle, N, D, H, cap, B, Wn, a, mw):
               acc=1, loc=1)
 
 
+@pytest.mark.parametrize("seed,N,D,H,cap,B,Wn,per_step,pol", [
+    # the one-block loop left at a dispatch and taken up again right after, where the
+    # next batch may not fit it either (deferred requests pile up), or dispatches nobody
+    (14, 20392, 12, 16384, 125195, 488, 1550, 0, 0), (40, 15899, 6, 10007, 76442, 242, 1423, 1, 0),
+    (96, 4485, 6, 16384, 222783, 112, 516, 1, 0), (224, 6682, 4, 16384, 229637, 81, 319, 0, 0),
+    (1, 9000, 5, 4096, 60000, 300, 400, 0, 1), (2, 9000, 5, 4096, 60000, 300, 400, 1, 1)])
+def test_deferral_with_long_lists(M, ws, oracle, seed, N, D, H, cap, B, Wn, per_step, pol):
+    w = W.make_stream(seed=seed, n_requests=N)
+    on_stream(M, ws, oracle, w, N, D, H, cap, B, Wn, 100000, 1000, per_step=per_step, beta=1000,
+              delay=w["pred_delay_ms"], pol=pol)
+
+
 @pytest.mark.parametrize("per_step", [0, 1])
 @pytest.mark.parametrize("beta,every", [(0, 1), (0, 3), (40, 1)])
 def test_timed_out_batches_without_completions(M, ws, oracle, per_step, beta, every):
