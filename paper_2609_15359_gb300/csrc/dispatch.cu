@@ -124,6 +124,41 @@ kmax_from_K_kernel(int D, int H, const int32_t *__restrict__ K, uint32_t *__rest
   if (neg) flag_error(status, MAPS_E_RANGE);
 }
 
+// The same summary for the SEQUENTIAL walk, with the maxima of its 128-step chunks
+// (eight blocks, eight lanes' maxima).
+constexpr int kSeqChunk = 128;
+__global__ void __launch_bounds__(256)
+seq_summary_kernel(int D, int H, const int32_t *__restrict__ K, uint32_t *__restrict__ km,
+                   uint32_t *__restrict__ cm, int32_t *status) {
+  pdl_prologue();
+  const int64_t nb = (static_cast<int64_t>(H) + kSumBlock - 1) / kSumBlock;
+  const int64_t nch = (static_cast<int64_t>(H) + kSeqChunk - 1) / kSeqChunk;
+  const int64_t total = 8 * nch * D;  // lanes: whole chunks
+  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+  const int lane = threadIdx.x & 31;
+  bool neg = false;
+  for (int64_t i0 = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x - lane; i0 < total; i0 += stride) {
+    const int64_t i = i0 + lane, ch = i >> 3, k = ch / nch, b = (ch - k * nch) * 8 + (i & 7);
+    uint32_t m = 0;
+    if (i < total && b < nb) {
+      const int32_t *row = K + k * H;
+#pragma unroll
+      for (int c = 0; c < kSumBlock; ++c) {
+        const int64_t t = b * kSumBlock + c;
+        const int32_t v = t < H ? __ldg(row + t) : 0;
+        if (v < 0) neg = true;
+        if (t < H) m = max(m, static_cast<uint32_t>(v) + static_cast<uint32_t>(t));
+      }
+      km[k * nb + b] = m;
+    }
+    m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
+    m = max(m, __shfl_xor_sync(0xffffffffu, m, 2));
+    m = max(m, __shfl_xor_sync(0xffffffffu, m, 4));
+    if (i < total && (lane & 7) == 0) cm[ch] = m;
+  }
+  if (neg) flag_error(status, MAPS_E_RANGE);
+}
+
 // A caller's summary is compared with K at four blocks of every row (the
 // first, the last, the middle and one that varies with the decoder); a
 // mismatch there is reported, any other gives unspecified results.
@@ -1016,7 +1051,12 @@ dispatch_direct_kernel(int D, int H, const int32_t *__restrict__ K, const uint32
 // steps, 3 of 4 and 3 cells: one kind to each of the four lanes.  The first P0
 // steps of each row with these maxima live in shared memory, the steps past
 // them in L2 (with maxima of 16 steps), where a candidate costs some L2 round
-// trips.
+// trips; a warp of the chosen row has two of its chunks there in flight, four
+// consecutive steps a lane.  (One chunk, with lanes on consecutive steps: 64 decoders,
+// H 32,763, candidates of up to 6,000 steps 2.84 against 2.08 us a decision.)  Rows
+// are loaded as far as a candidate reaches, and the chunks' maxima come from the
+// summary's kernel: a single candidate through the horizon of 200 decoders, H 32,768,
+// 37 us against 122 with them made here (and 42 by the walk in global memory alone).
 //
 // The 32-bit pick keys, the smallest wins: a feasible decoder is
 // min(Q - q0, lim) << kb | k, an infeasible one 1 << 31 |
@@ -1025,7 +1065,7 @@ dispatch_direct_kernel(int D, int H, const int32_t *__restrict__ K, const uint32
 // the pick is made on 64-bit keys.
 //
 // Measured, occupancy and walk: 16 decoders, H 16,384, 1,024 candidates 3.51 ->
-// 0.60 ms; 64 decoders, H 32,763, 2,003 candidates 8.1 -> 1.22 ms.  Before, one
+// 0.58 ms; 64 decoders, H 32,763, 2,003 candidates 8.1 -> 1.18 ms.  Before, one
 // block scored every decoder from global memory with four barriers a decision
 // (3.4 and 4.0 us each).  Forms in between: two warps a decoder, each scoring
 // and reserving in lockstep, 1.58 and 4.44 ms (issue bound: every warp ran the
@@ -1033,7 +1073,6 @@ dispatch_direct_kernel(int D, int H, const int32_t *__restrict__ K, const uint32
 // decoder in the columns and the pick and its bookkeeping in every row warp,
 // 0.93 and 1.68 ms.
 // ---------------------------------------------------------------------------
-constexpr int kSeqChunk = 128;
 constexpr int kRowWarps = 8;
 constexpr int kColWarps = 16;  // at most
 constexpr int kSeqWords = 9;    // per-decoder words beside the rows
@@ -1047,7 +1086,7 @@ struct SeqArgs {
   int kb, mc;
   int32_t *K;
   uint32_t *km;        // [D][ceil(H/16)]  max of F per 16 steps
-  uint32_t *cm;        // [D][ceil(H/128)]  max of F per chunk, from chunk P2 on
+  uint32_t *cm;        // [D][ceil(H/128)]  max of F per chunk; kept up to date from chunk P2 on
   const int32_t *cap;
   int32_t *Q;
   int64_t J;
@@ -1155,38 +1194,42 @@ dispatch_sequential_kernel(const __grid_constant__ SeqArgs a) {
   umax = __reduce_max_sync(kAll, umax);
   if (lane == 0) atomicMax(&s_umax, umax);
   if (tid < 64) s_cand[tid] = load_cand(tid);
-  // --- the resident rows --------------------------------------------------------
+  __syncthreads();
+  // --- the resident rows, as far as a candidate reaches, two chunks in flight ----
   const int rch = P0 / kSeqChunk;  // resident chunks of a row
-  for (int e = warp; e < D * rch; e += nwarp) {
-    const int k = e / rch, t0 = (e - k * rch) * kSeqChunk;
-    const int32_t *row = a.K + static_cast<int64_t>(k) * H + t0;
-    uint32_t *const f = F + k * ldF + t0;
-    uint32_t x[4];
+  const int lch = min(rch, (s_umax + kSeqChunk - 1) / kSeqChunk);
+  for (int e0 = warp; e0 < D * lch; e0 += 2 * nwarp) {
+    uint32_t x[2][4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int t = 32 * i + lane;
-      x[i] = t0 + t < H ? static_cast<uint32_t>(row[t]) + static_cast<uint32_t>(t0 + t) : 0u;
+    for (int h = 0; h < 2; ++h) {
+      const int e = min(e0 + h * nwarp, D * lch - 1), k = e / lch, t0 = (e - k * lch) * kSeqChunk;
+      const int32_t *row = a.K + static_cast<int64_t>(k) * H + t0;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int t = 32 * i + lane;
+        x[h][i] = t0 + t < H ? static_cast<uint32_t>(row[t]) + static_cast<uint32_t>(t0 + t) : 0u;
+      }
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) f[32 * i + lane] = x[i];
-    __syncwarp();
-    uint32_t m = max4(reinterpret_cast<const uint4 *>(f)[lane]);
-    F[o4 + k * ld4 + t0 / 4 + lane] = m;
-    m = max(m, __shfl_xor_sync(kAll, m, 1));
-    m = max(m, __shfl_xor_sync(kAll, m, 2));
-    if ((lane & 3) == 0) F[o16 + k * ld16 + t0 / 16 + (lane >> 2)] = m;
+    for (int h = 0; h < 2; ++h) {
+      const int e = e0 + h * nwarp, k = e / lch, t0 = (e - k * lch) * kSeqChunk;
+      if (e >= D * lch) break;
+      uint32_t *const f = F + k * ldF + t0;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) f[32 * i + lane] = x[h][i];
+      __syncwarp();
+      uint32_t m = max4(reinterpret_cast<const uint4 *>(f)[lane]);
+      F[o4 + k * ld4 + t0 / 4 + lane] = m;
+      m = max(m, __shfl_xor_sync(kAll, m, 1));
+      m = max(m, __shfl_xor_sync(kAll, m, 2));
+      if ((lane & 3) == 0) F[o16 + k * ld16 + t0 / 16 + (lane >> 2)] = m;
+    }
   }
-  __syncthreads();
-  const int cmax = s_umax >> 7;  // scores read the chunk maxima below this one
+  const int cmax = min(s_umax >> 7, P2);  // scores read the chunk maxima below this one
+#pragma unroll 4
   for (int e = tid; e < cmax * D; e += blockDim.x) {
     const int k = e / cmax, c = e - k * cmax;
-    uint32_t m = 0;
-    for (int i = 0; i < 8; ++i)
-      if ((c * 8 + i) * kSumBlock < H) m = max(m, __ldcg(a.km + k * nb + c * 8 + i));
-    if (c < P2)
-      F[oc + k * ldc + c] = m;
-    else
-      a.cm[k * nch + c] = m;
+    F[oc + k * ldc + c] = __ldcg(a.cm + k * nch + c);
   }
   const long long x0 = s_x0;
   for (int k = tid; k < D; k += blockDim.x) {
@@ -1319,6 +1362,9 @@ dispatch_sequential_kernel(const __grid_constant__ SeqArgs a) {
     int2 c1 = s_cand[0];
     const bool res0 = warp < rch;           // this warp's first chunk is resident
     const int tb = warp * kSeqChunk, tl = tb + 4 * lane;
+    const int later = res0 ? tb + kRowWarps * kSeqChunk : tb;  // where its other chunks begin
+    // its first chunk in global memory
+    const int cg = (rch > warp ? (rch - warp + kRowWarps - 1) / kRowWarps * kRowWarps : 0) + warp;
     for (int64_t j = 0; j < a.J; ++j) {
       const int2 cd = c1;
       c1 = s_cand[(j + 1) & 63];
@@ -1359,10 +1405,10 @@ dispatch_sequential_kernel(const __grid_constant__ SeqArgs a) {
           bm0 = max4(v);  // folded once the score is published
           if (tb < u) *reinterpret_cast<uint4 *>(fr + tb) = v;
         }
-        // the later chunks of a long horizon
-        for (int c = res0 ? warp + kRowWarps : warp; c * kSeqChunk < ue; c += kRowWarps) {
-          const int t0 = c * kSeqChunk;
-          if (c < rch) {
+        // the later chunks of a long horizon: one branch on the chain of the others
+        if (__builtin_expect(later < ue, 0)) {
+          for (int c = warp + kRowWarps; c < rch && c * kSeqChunk < ue; c += kRowWarps) {
+            const int t0 = c * kSeqChunk;
             uint4 v = *reinterpret_cast<const uint4 *>(fr + t0);
             add_to(v, t0 + 4 * lane);
             m1 = max4_below(v, u1 - (t0 + 4 * lane), m1);
@@ -1370,36 +1416,49 @@ dispatch_sequential_kernel(const __grid_constant__ SeqArgs a) {
               *reinterpret_cast<uint4 *>(fr + t0) = v;
               fold(c, max4(v));
             }
-            continue;
           }
-          int32_t *const row = a.K + static_cast<int64_t>(kk) * H;
-          uint32_t x[4], cx = 0;
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int t = t0 + 32 * i + lane;
-            x[i] = t < H ? static_cast<uint32_t>(row[t]) : 0u;
-          }
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int t = t0 + 32 * i + lane;
-            const uint32_t te = static_cast<uint32_t>(t);
-            if (t < u) {
-              x[i] += static_cast<uint32_t>(p) + 1u + te;
-              row[t] = static_cast<int32_t>(x[i]);
+          // those in global memory, two in flight, four consecutive steps a lane
+          for (int c0 = cg; c0 * kSeqChunk < ue; c0 += 2 * kRowWarps) {
+            int32_t *const row = a.K + static_cast<int64_t>(kk) * H;
+            uint4 v[2];
+  #pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const int t0 = (c0 + h * kRowWarps) * kSeqChunk, t = t0 + 4 * lane;
+              v[h] = make_uint4(0, 0, 0, 0);
+              if (t0 >= ue) continue;
+              if (t < H) v[h].x = static_cast<uint32_t>(row[t]);
+              if (t + 1 < H) v[h].y = static_cast<uint32_t>(row[t + 1]);
+              if (t + 2 < H) v[h].z = static_cast<uint32_t>(row[t + 2]);
+              if (t + 3 < H) v[h].w = static_cast<uint32_t>(row[t + 3]);
             }
-            uint32_t f = t < H ? x[i] + te : 0u;
-            if (t < u1) m1 = max(m1, f);
-            if (t0 < u) {
-              cx = max(cx, f);
-#pragma unroll
-              for (int off = 8; off > 0; off >>= 1) f = max(f, __shfl_xor_sync(kAll, f, off));
-              const int b = (t0 >> 4) + 2 * i + (lane >> 4);
-              if ((lane & 15) == 0 && b * kSumBlock < H) a.km[kk * nb + b] = f;
+  #pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const int c = c0 + h * kRowWarps, t0 = c * kSeqChunk, t = t0 + 4 * lane;
+              if (t0 >= ue) break;
+              add_to(v[h], t);
+              if (t0 < u) {
+                if (t < u) row[t] = static_cast<int32_t>(v[h].x);
+                if (t + 1 < u) row[t + 1] = static_cast<int32_t>(v[h].y);
+                if (t + 2 < u) row[t + 2] = static_cast<int32_t>(v[h].z);
+                if (t + 3 < u) row[t + 3] = static_cast<int32_t>(v[h].w);
+              }
+              // F = K + t on the steps within the horizon
+              const uint32_t te = static_cast<uint32_t>(t);
+              v[h].x += t < H ? te : 0u;
+              v[h].y += t + 1 < H ? te + 1u : 0u;
+              v[h].z += t + 2 < H ? te + 2u : 0u;
+              v[h].w += t + 3 < H ? te + 3u : 0u;
+              m1 = max4_below(v[h], u1 - t, m1);
+              if (t0 < u) {
+                uint32_t f = max4(v[h]);
+                f = max(f, __shfl_xor_sync(kAll, f, 1));
+                f = max(f, __shfl_xor_sync(kAll, f, 2));
+                const int b = (t0 >> 4) + (lane >> 2);
+                if ((lane & 3) == 0 && b * kSumBlock < H) a.km[kk * nb + b] = f;
+                f = __reduce_max_sync(kAll, f);
+                if (lane == 0) set_cm(c, f);
+              }
             }
-          }
-          if (t0 < u) {
-            cx = __reduce_max_sync(kAll, cx);
-            if (lane == 0) set_cm(c, cx);
           }
         }
         // publish, and fold the first chunk's maxima: one reduction, shuffle
@@ -1466,7 +1525,7 @@ dispatch_sequential_kernel(const __grid_constant__ SeqArgs a) {
   for (int k = warp; k < D; k += nwarp) {
     int32_t *row = a.K + static_cast<int64_t>(k) * H;
 #pragma unroll 8
-    for (int t = lane; t < P0 && t < H; t += 32)
+    for (int t = lane; t < lch * kSeqChunk && t < H; t += 32)
       row[t] = static_cast<int32_t>(F[k * ldF + t] - static_cast<uint32_t>(t));
   }
 }
@@ -2051,9 +2110,9 @@ int dispatch_sequential(int D, int H, int32_t *K, const int32_t *cap, int32_t *Q
   int32_t *status = status_word(ws);
   Carve cv(ws);
   const SeqWs w = carve_seq(cv, D, H);
-  const int64_t nb = (static_cast<int64_t>(H) + kSumBlock - 1) / kSumBlock;
-  const int gk = static_cast<int>(std::min<int64_t>((nb * D + 255) / 256, 8LL * sm_count()));
-  launch_pdl(kmax_from_K_kernel, gk, 256, 0, s, D, H, K, w.km, status);
+  const int64_t chunks = (static_cast<int64_t>(H) + kSeqChunk - 1) / kSeqChunk;
+  const int gk = static_cast<int>(std::min<int64_t>((8 * chunks * D + 255) / 256, 8LL * sm_count()));
+  launch_pdl(seq_summary_kernel, gk, 256, 0, s, D, H, K, w.km, w.cm, status);
   SeqArgs a;
   a.D = D;
   a.H = H;
@@ -2077,10 +2136,13 @@ int dispatch_sequential(int D, int H, int32_t *K, const int32_t *cap, int32_t *Q
   const int64_t fixed = kSeqWords * seq_dw(D) + kSeqPad;
   const size_t limit = smem_beside(kStaticSmem);
   const int64_t words = (static_cast<int64_t>(limit) / 4 - fixed) / D;
-  const int64_t chunks = (static_cast<int64_t>(H) + kSeqChunk - 1) / kSeqChunk;
-  a.P2 = static_cast<int>(std::min<int64_t>(chunks, words / 32));
+  // One or two candidates are not worth the rows' way to shared memory and back.  24
+  // decoders, H 4,800, candidates of a few hundred steps, without it and with: one
+  // 7.9 against 10.7 us, two 8.8 against 12.8; of three it pays.
+  const bool few = J <= 2;
+  a.P2 = few ? 0 : static_cast<int>(std::min<int64_t>(chunks, words / 32));
   a.P0 = 0;
-  while (a.P0 < chunks * kSeqChunk && seq_row_words(a.P0 + kSeqChunk, a.P2) <= words) a.P0 += kSeqChunk;
+  while (!few && a.P0 < chunks * kSeqChunk && seq_row_words(a.P0 + kSeqChunk, a.P2) <= words) a.P0 += kSeqChunk;
   const size_t smem = 4 * (static_cast<size_t>(D) * seq_row_words(a.P0, a.P2) + fixed);
   auto launch = [&](void (*kern)(SeqArgs)) {
     MAPS_TRY(allow_smem(kern, limit));

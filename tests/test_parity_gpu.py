@@ -556,12 +556,16 @@ def test_dispatch_sequential_workloads(M, ws, oracle, name):
 
 
 @pytest.mark.parametrize("D,H,J,spread", [
-    # four, two and one warps a decoder, and several decoders a warp, at the
-    # edges; horizons around a 128-cell chunk and a 16-step block; rows past
-    # what shared memory holds; a last chunk of candidates that is not full
+    # one column warp and many, and several decoders a lane; horizons around a
+    # 128-step chunk and a 16-step block; rows past what shared memory holds; a
+    # last refill of candidates that is not full
     (1, 127, 33, 3000), (8, 129, 65, 3000), (9, 1000, 64, 3000), (16, 16384, 200, 6000),
     (17, 2049, 100, 3000), (32, 4111, 150, 3000), (33, 4096, 100, 3000), (64, 9001, 130, 6000),
     (100, 5000, 60, 3000), (300, 700, 50, 3000), (1, 300000, 40, 100000),
+    # one and two candidates (no row in shared memory), and three; candidates that end
+    # in either of the two global chunks in flight
+    (1, 5, 1, 3000), (3, 130, 2, 3000), (24, 16509, 2, 6000), (8, 32768, 3, 6000), (200, 4801, 1, 3000),
+    (64, 9001, 4, 6000), (1, 300001, 2, 100000), (40, 20003, 30, 6000), (12, 30004, 25, 6000),
     # headrooms further apart than the 32-bit keys hold
     (5, 600, 60, 2**30), (40, 600, 60, 2**30)])
 def test_dispatch_sequential_edges(M, ws, oracle, D, H, J, spread):
@@ -572,7 +576,7 @@ def test_dispatch_sequential_edges(M, ws, oracle, D, H, J, spread):
     Q = rng.integers(0, 3, D).astype(np.int32)
     cp = rng.integers(0, 500, J).astype(np.int32)
     cb = np.where(rng.random(J) < 0.5, rng.integers(0, H + 5, J), rng.integers(0, 40, J)).astype(np.int32)
-    cb[: min(J, 4)] = [0, 16, 128, H][: min(J, 4)]
+    cb[: min(J, 4)] = ([H] if J < 3 else [0, 16, 128, H])[: min(J, 4)] * (2 if J == 2 else 1)
     check_dispatch(M, ws, oracle, 1, D, H, K, cap, Q, cp, cb)
     cp[J // 2] = -1  # skipped and reported
     check_dispatch(M, ws, oracle, 1, D, H, K, cap, Q, cp, cb)
