@@ -871,8 +871,9 @@ dispatch_snapshot_kernel(const __grid_constant__ CUtensorMap tmap, SnapArgs a) {
 constexpr int kDirectWarps = 8;
 constexpr int kDirectRows = 8;
 
-// At most this many candidates, (candidate, decoder) scores, twice as many of
-// those times the 2,048-step spans of the horizon, cells of K, and a horizon.
+// At most this many (candidate, decoder) scores, decoders counted as whole groups of
+// kDirectRows a warp, twice as many (without that) times the 2,048-step spans of the
+// horizon, cells of K, and a horizon.
 // Candidates of a few hundred steps decide where the lines lie; in brackets the
 // same with all of them through the horizon, which no size tells the host.
 // Measured, one launch against four: 4 decoders, H 4,096, 32 candidates 4.7
@@ -880,16 +881,22 @@ constexpr int kDirectRows = 8;
 // 100, 8,192, 600: 12.1 against 16.4 (19.2; 16.5); 64, 4,096, 2,048: 16.2 against
 // 18.6; 1, 30,000, 8,192: 10.7 against 20.5 (25.9; 17.5).  Past the lines: 16,
 // 2,048, 16,384: 25.9 against 20.7; 256, 2,048, 1,024: 22.6 against 18.4; 2, 100,
-// 24,000: 19.9 against 17.5; 2, 256, 65,536: 40.9 against 19.1; 12, 50,000, 100: 7.8
-// against 16.4, but 63 against 14.5.  Where the summary's rows are no whole
-// 16-byte words (330 decoders, H 2,760, 256 candidates: 10.9 against 24.6) a lane has
-// four words in flight as well; with one, that took 28.5.
-constexpr int64_t kDirectCands = 1 << 14;
+// 24,000: 19.9 against 17.5; 2, 256, 65,536: 40.9 against 19.1; 18, 104, 6,271: 24.6
+// against 19.7; 12, 50,000, 100: 7.8 against 16.4, but 63 against 14.5.  Where the
+// summary's rows are no whole 16-byte words (330 decoders, H 2,760, 256 candidates:
+// 10.9 against 24.6) a lane has four words in flight as well; with one, 28.5.
 constexpr int64_t kDirectScores = 1 << 17;
 constexpr int64_t kDirectCells = 1 << 20;
 constexpr int kDirectH = 32768;
+// warps a candidate: as many as have kDirectRows rows each
+int direct_share(int D) {
+  int share = 1;
+  while (share < kDirectWarps && share * kDirectRows < D) share *= 2;
+  return share;
+}
 bool direct_fits(int D, int H, int64_t J) {
-  return J <= kDirectCands && J * D <= kDirectScores &&
+  const int step = direct_share(D) * kDirectRows;
+  return J * ((D + step - 1) / step * step) <= kDirectScores &&
          J * D * std::max(1, H / 2048) <= 2 * kDirectScores && H <= kDirectH &&
          static_cast<int64_t>(D) * H <= kDirectCells;
 }
@@ -2001,9 +2008,7 @@ int launch_snapshot(int D, int H, const int32_t *K, const uint32_t *kmax, const 
     kmax = w.kmax;
   }
   if (direct) {
-    // warps to a candidate: as many as have kDirectRows rows each
-    int share = 1;
-    while (share < kDirectWarps && share * kDirectRows < D) share *= 2;
+    const int share = direct_share(D);
     const int64_t blocks = (J * share + kDirectWarps - 1) / kDirectWarps;
     // the reading of K takes blocks of its own where the candidates have few
     const int64_t reading = static_cast<int64_t>(D) * H / (32 * kDirectWarps * 16);

@@ -445,9 +445,9 @@ def test_dispatch_snapshot_random(M, ws, oracle, D, H, J):
     # not; 32-decoder groups at their edges; one candidate
     (31, 640, 100, True), (33, 1000, 1, False), (64, 64, 65, False), (1024, 100, 9, True),
     # rows read word by word, around 128 blocks of the summary and past twice as many;
-    # the most candidates of the one-launch form
+    # the most candidates of the one-launch form, of few decoders and of 18 in four groups
     (330, 2047, 20, False), (330, 2081, 20, False), (9, 4400, 70, True), (3, 30001, 33, False),
-    (2, 300, 16384, False), (2, 300, 16385, False),
+    (2, 300, 16384, False), (2, 300, 16385, False), (18, 104, 4096, False), (18, 104, 4097, False),
     # wide tiles of the bucketed form (few decoders, many candidates)
     (5, 4099, 60000, False), (40, 4096, 9000, True)])
 def test_dispatch_snapshot_forms(M, ws, oracle, D, H, J, unaligned):
@@ -475,7 +475,8 @@ def test_dispatch_snapshot_forms(M, ws, oracle, D, H, J, unaligned):
         assert np.array_equal(host(ch), co) and np.array_equal(host(hr), ho)
     # a negative cell is reported: without a summary, and with one too in the
     # one-launch form (the bucketed form reads only the candidates' tiles then)
-    one_launch = (J <= 2**14 and J * D <= 2**17 and J * D * max(1, H // 2048) <= 2**18
+    rows = next(8 * s for s in (1, 2, 4, 8) if 8 * s >= D or s == 8)  # whole groups of 8 a warp
+    one_launch = (J * (-(-D // rows) * rows) <= 2**17 and J * D * max(1, H // 2048) <= 2**18
                   and H <= 32768 and D * H <= 2**20)
     Kd[D - 1, H // 2] = -5
     for summary in (kd, None) if one_launch else (None,):
