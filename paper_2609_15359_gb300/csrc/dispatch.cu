@@ -1877,10 +1877,12 @@ alg1_sequential_kernel(int D, int S, const long long *B_eff, const int32_t *cap,
 }
 
 // Few candidates on many decoders: a thread a decoder, the block's choice by a vote, a
-// maximum and the lowest index that has it.  The warp above first takes 16 or 32
-// decoders a lane into registers, which a decision or three do not repay: 518 decoders,
-// one candidate, whole call 10.5 us against 16.6; 977, three 20.6 against 24.4.
-constexpr int kFewCands = 3;
+// maximum and the lowest index that has it, 0.6 to 1 us a decision.  The warp above
+// first takes 16 or 32 decoders a lane into registers, which a few decisions do not
+// repay: replayed calls of 4 and 8 candidates, this form against the warp, 257
+// decoders 5.3 and 7.3 us against 7.2 and 8.9; 1,024 8.3 and 12.1 against 19.0 and
+// 18.6 (with the block's shared memory and Q in global memory 15.6 and 28.2).
+constexpr int kFewCands = 8;
 constexpr int kFewD = 256;
 __global__ void __launch_bounds__(kMaxD)
 alg1_few_kernel(int D, int S, const long long *B_eff, const int32_t *cap, int32_t *Q, int64_t J,

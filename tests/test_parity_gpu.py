@@ -618,9 +618,9 @@ def test_dispatch_alg1_workloads(M, ws, oracle, name, S):
     (1, 33, 1, 2000), (31, 65, 16, 3000), (32, 1, 16, 3000), (33, 700, 1, 3000),
     (64, 1000, 16, 5000), (65, 500, 32, 5000), (200, 500, 16, 5000), (257, 300, 1, 4000),
     (600, 400, 16, 4000), (1024, 300, 16, 4000),
-    # up to three candidates on more than 256 decoders, a thread a decoder; and beside it
-    (257, 1, 16, 4000), (512, 2, 1, 4000), (1024, 3, 16, 4000), (1000, 3, 1, 2**24), (256, 3, 16, 4000),
-    (257, 4, 16, 4000),
+    # up to eight candidates on more than 256 decoders, a thread a decoder; and beside it
+    (257, 1, 16, 4000), (512, 2, 1, 4000), (1024, 8, 16, 4000), (1000, 7, 1, 2**24), (256, 8, 16, 4000),
+    (257, 9, 16, 4000),
     # budgets further apart than a 32-bit key holds (the wide comparison), from
     # the start and after some reservations
     (5, 400, 1, 2**30), (1000, 300, 1, 2**24), (2, 3000, 1, 2**29)])
