@@ -1167,7 +1167,7 @@ __device__ void
 dispatch_block(unsigned char *sdm, unsigned char *lists, int D, int H, int nb, int mc, const int64_t *res_off,
                const int32_t *rp, const int32_t *rg, const int32_t *rU, const int32_t *capv,
                int32_t *Q, const int32_t *cp, const int32_t *cU, int32_t *choice,
-               int64_t *headroom, int32_t *status, int32_t *walked_lists, size_t smem) {
+               int32_t *status, int32_t *walked_lists, size_t smem) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nact = static_cast<int>(res_off[D]);
   const int pool = nact + D * nb;
@@ -1216,10 +1216,10 @@ dispatch_block(unsigned char *sdm, unsigned char *lists, int D, int H, int nb, i
     uB[x] = b;
   }
   __syncthreads();
-  // Without a headroom output and with the Q-first rule, a decoder whose peak
-  // is provably within its capacity is decided by (Q, index) alone.
-  const bool quick = headroom == nullptr && mc == 0;
-  // Fast path (at most 32 decoders, no headroom output, Q-first rule): the
+  // With the Q-first rule, a decoder whose peak is provably within its capacity is
+  // decided by (Q, index) alone.
+  const bool quick = mc == 0;
+  // Fast path (at most 32 decoders, Q-first rule): the
   // choices by (Q, index) alone, taken when every decoder is shown feasible at
   // every step, before any list is sorted.  For t < u,
   // K(t) + t = S(t) + t (C(t) + 1) with S <= the decoder's b-sum and C <= n
@@ -1373,11 +1373,11 @@ dispatch_block(unsigned char *sdm, unsigned char *lists, int D, int H, int nb, i
   }
   __syncthreads();
 
-  // At most 32 decoders and no headroom output: a warp each, with the lists in registers; a list that
+  // At most 32 decoders: a warp each, with the lists in registers; a list that
   // outgrows a variant moves on to the next, the last one below.
   __shared__ WalkShared walk;
   bool walked = s_fast != 0;
-  if (!walked && D <= 32 && headroom == nullptr) {
+  if (!walked && D <= 32) {
     int nmax = 0;
     for (int k = 0; k < D; ++k) nmax = max(nmax, s_n[k]);
     const int about = nmax + 2 * nb / D;
@@ -1667,7 +1667,6 @@ dispatch_block(unsigned char *sdm, unsigned char *lists, int D, int H, int nb, i
         if (lane == 0) {
           flag_error(status, MAPS_E_RANGE);
           choice[j] = -1;
-          if (headroom) headroom[j] = 0;
         }
         continue;
       }
@@ -1749,7 +1748,6 @@ dispatch_block(unsigned char *sdm, unsigned char *lists, int D, int H, int nb, i
       }
       if (lane == 0) {
         choice[j] = bk;
-        if (headroom) headroom[j] = static_cast<long long>(s_cap[bk]) - (static_cast<long long>(p) + 1 + Mb);
         if (s_q[bk] == 0x7fffffff)
           flag_error(status, MAPS_E_RANGE);
         else
@@ -1817,12 +1815,12 @@ template <bool kGlobal>
 __global__ void __launch_bounds__(kSt, 1)
 stream_dispatch_kernel(int D, int H, int nb, int mc, const int64_t *res_off, const int32_t *rp,
                        const int32_t *rg, const int32_t *rU, const int32_t *capv, int32_t *Q,
-                       const int32_t *cp, const int32_t *cU, int32_t *choice, int64_t *headroom,
-                       int32_t *status, unsigned char *lists, StreamState *S) {
+                       const int32_t *cp, const int32_t *cU, int32_t *choice, int32_t *status,
+                       unsigned char *lists, StreamState *S) {
   pdl_prologue();
   extern __shared__ __align__(16) unsigned char sdm[];
-  dispatch_block<kGlobal, true>(sdm, lists, D, H, nb, mc, res_off, rp, rg, rU, capv, Q, cp, cU, choice, headroom,
-                               status, &S->lists, 0);
+  dispatch_block<kGlobal, true>(sdm, lists, D, H, nb, mc, res_off, rp, rg, rU, capv, Q, cp, cU, choice, status,
+                               &S->lists, 0);
 }
 
 // 5''. Deferral: the listed requests join the waiting queues at act[nact..]:
@@ -2337,7 +2335,7 @@ stream_loop_kernel(const __grid_constant__ LoopArgs a) {
       __syncthreads();
     } else if (nc > 0 && !rr && c.dispatch_policy != MAPS_STREAM_RR) {  // 5.
       dispatch_block<false, false>(ldm, nullptr, D, c.H, nc, mc, w.res_off, w.rp, w.rg, w.rU, w.capv, w.Q, cpr,
-                                   w.Uq + nact, cch, nullptr, a.status, &s_lists, a.smem);
+                                   w.Uq + nact, cch, a.status, &s_lists, a.smem);
       __syncthreads();
       if (s_lists == 2) break;  // the host takes the batch up from here
     }
@@ -2687,7 +2685,7 @@ int maps_stream_run(const maps_stream_cfg *cfg, const int64_t *arrival_ms, const
         const auto kern = place == 1 ? stream_dispatch_kernel<false> : stream_dispatch_kernel<true>;
         MAPS_TRY(allow_smem(kern, most));
         launch_pdl(kern, 1, kSt, dsm, s, D, c.H, nc, mc, w.res_off, w.rp, w.rg, w.rU, w.capv, w.Q, cpr,
-                   w.Uq + nact, cch, nullptr, status,  // no headroom out
+                   w.Uq + nact, cch, status,
                    place == 1 ? nullptr : reinterpret_cast<unsigned char *>(w.K), w.S);
         MAPS_TRY(launch_ok());
       } else {
