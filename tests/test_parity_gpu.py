@@ -1161,6 +1161,25 @@ def test_stream_one_block_loop_limits(M, ws, oracle, N, D, cap, B, Wn):
     check_stream(M, ws, oracle, N, D, 16384, cap, B, Wn, 100000, 1000, w)
 
 
+@pytest.mark.parametrize("seed,a", [(0, 100000), (1, 300000), (2, 20000), (3, 700000)])
+def test_stream_quantile_bin_edges(M, ws, oracle, seed, a):
+    """The loop's own quantile, of a window of scores on the bin edges of its
+    passes (each batch completes the one before, whose true lengths are those
+    scores over predictions of zero)."""
+    rng = np.random.default_rng(seed)
+    edges = {1, 1022, 1023, 1024, 1025, 2**30 + 2**24}
+    for e in range(10, 31):
+        step = 1 << (e - 7)
+        edges |= {(1 << e) - 1, 1 << e, (1 << e) + 1, (1 << e) + step - 1, (1 << e) + step}
+    N, B = 1200, 15
+    spread = rng.choice(np.array(sorted(edges)), N)
+    true = np.where(np.arange(N) // 300 % 2 == 0, spread, rng.integers(1, 2**30, N))
+    zeros = np.zeros(N, np.int32)
+    w = dict(arrival_ms=np.arange(N) // B * 2**32, prompt=zeros, pred=zeros, true=true.astype(np.int32))
+    qo, so = check_stream(M, ws, oracle, N, 8, 64, I32_MAX, B, 250, a, 1000, w)
+    assert (so[1:, 0] == B).all() and (qo[-60:] > 0).all() and len(set(qo.tolist())) >= 10
+
+
 def test_stream_full_workload(M, ws, oracle):
     """All 1,000,000 requests of the streaming workload, bit for bit."""
     w = W.make_stream()
