@@ -22,9 +22,10 @@ extern "C" {
 int maps_set_dispatch_events(void *before, void *after);
 
 /* Exercises the bounded waits of maps_order_local's global form (the form
- * taken when arrival is not non-decreasing along the index and the call is
- * larger than one block): on the current device, later calls let tile `tile`
- * of every radix pass publish nothing to the decoupled look-back, and every
+ * taken, past one block, when arrival is not non-decreasing along the index and
+ * there are more than 1,024 decoders or the key of promotion, bound, arrival and
+ * index needs more than 63 bits): on the current device, later calls let tile
+ * `tile` of every radix pass publish nothing to the decoupled look-back, and every
  * look-back wait gives up after `spin_limit` polls (0: the library default).
  * The tile after the withheld one then waits until the limit, records
  * MAPS_E_TIMEOUT (read with maps_check) and carries on; the order of that

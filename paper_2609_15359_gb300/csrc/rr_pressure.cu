@@ -440,7 +440,15 @@ rr_stream_kernel(int64_t n_real, int64_t n, int N, int64_t C, int64_t tok, uint3
   };
   clear();
   // the variant by the footprints a capacity holds on average, with room for
-  // the spread; a set that turns out larger moves on to the next
+  // the spread; a set that turns out larger moves on to the next.  192
+  // realisations of 10,000 requests, two a lane against eight a lane against shared
+  // memory: at the usual loads, capacities of 24 footprints 1.51, 1.71 and 3.81 ms,
+  // of 64 1.55, 1.76 and 3.93, of 90 (two a lane starts over) 3.19, 1.77 and 3.96,
+  // of 200 3.23, 1.81 and 4.04.  Overloaded, when the set fills the capacity: 43
+  // 1.00, 1.17 and 2.54, 56 1.01, 1.18 and 2.70, 64 (starting over) 1.24, 1.19 and
+  // 2.70, 220 eight a lane 1.31 against 3.15, 250 (starting over) 3.09 against 3.22.
+  // So the sets of this workload stay within a variant's room to some 0.9 of it;
+  // the lines leave a third and a fifth for footprints that spread more.
   const int64_t about = C * n_d / (foot > 0 ? foot : 1);
   const bool small = n_d <= 0x3ffffff0 && N < (1 << 28);  // what their 32-bit counts hold
   bool ran = small && about <= 44 && sim.run_registers<2>();

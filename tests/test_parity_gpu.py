@@ -196,9 +196,9 @@ def test_calibrate_unaligned_and_ranges(M, ws, oracle):
                                     (0, 4096), (1, 1024), (2, 1000), (0, 128)])
 def test_calibrate_grid_bucket_edges(M, ws, oracle, seed, n):
     """Grid form (n above the one-block limit) and the one-block forms: scores
-    on the first pass's bin edges (the last exact bin, each leading-bit boundary, each 7-bit step) and
-    up to 2^32 - 1, so that quantiles resolve after one, two or three passes and
-    some lie above INT32_MAX (range error)."""
+    on the first pass's bin edges (the last exact bin, each leading-bit boundary,
+    each 7-bit step) and up to 2^32 - 1, so that quantiles resolve after one, two
+    or three passes and some lie above INT32_MAX (range error)."""
     rng = np.random.default_rng(seed)
     edges = {0, 1, 1022, 1023, 1024, 1025, 2**32 - 1}
     for e in range(10, 32):
@@ -235,10 +235,10 @@ def test_calibrate_grid_bucket_edges(M, ws, oracle, seed, n):
     (16384, 16384, 0), (16384, 16385, 1), (16385, 0, 0), (16385, 777, 1), (1024, 8193, 1),
     (1025, 1, 0), (15361, 9000, 0)])
 def test_calibrate_fused_register_limits(M, ws, oracle, n, m, shift):
-    """Calibration sets above the one-block limit take one cooperative kernel;
-    its scores and predictions live in registers up to eight per thread, else
-    they are read from memory: q, the bounds and the status match the oracle
-    either way."""
+    """Calibration sets above 16,384 scores take one cooperative kernel; its
+    scores and predictions live in registers up to eight per thread, else they
+    are read from memory, as the one-block form's queries past its eight are: q,
+    the bounds and the status match the oracle either way."""
     rng = np.random.default_rng(n + m)
     L = rng.integers(0, 40000, n).astype(np.int32)
     P = rng.integers(0, 40000, n).astype(np.int32)

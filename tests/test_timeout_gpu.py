@@ -5,13 +5,14 @@ waits at a bounded grid barrier after each select pass; the test aid
 maps_test_calibrate_absent_block makes one of its blocks return at once, so
 the others' wait runs out.
 
-The local order's global form (arrival not in index order) sorts with
-decoupled look-back between tiles: each tile waits, bounded, for its
-predecessors' published counts.  The test aid maps_test_withhold_lookback
-makes one tile publish nothing, so the next tile's wait runs out after a short
-limit.  The call must then report MAPS_E_TIMEOUT through maps_check, write
-only inside its outputs, and the next call on a fresh workspace must give the
-oracle's order exactly.  Nothing faults, traps or hangs.
+The local order's global form (arrival not in index order, and a key past 63
+bits) sorts with decoupled look-back between tiles: each tile waits, bounded,
+for its predecessors' published counts.  The test aid
+maps_test_withhold_lookback makes one tile publish nothing, so the next tile's
+wait runs out after a short limit.  The call must then report MAPS_E_TIMEOUT
+through maps_check, write only inside its outputs, and the next call on a
+fresh workspace must give the oracle's order exactly.  Nothing faults, traps or
+hangs.
 """
 import numpy as np
 import pytest
