@@ -64,16 +64,16 @@ L2_FLUSH_BYTES = 256 << 20
 # valid only for the kernel source it was taken on.
 TRAFFIC = {
     "dispatch_feasible": {"bytes": 0, "source": "dispatch.cu", "source_sha256": ""},
-    "calibrate": {"bytes": 12529152, "source": "calibrate.cu", "source_sha256":
-        "bee3446c753caa47a9a5219998f23f1032c3422bea5e6f2b1b5a0c3388db1333"},
-    "occupancy": {"bytes": 31214592, "source": "occupancy.cu", "source_sha256":
-        "eea478ebad90bd74e26218086061cb3ed62c3daef9b01ff7f4249e1868cf17a7"},
-    "dispatch": {"bytes": 26560256, "source": "dispatch.cu", "source_sha256":
-        "b759e8825262f3d3f45b9c2ae974c2cf85052998c0590251ae60ce864551d683"},
-    "dispatch_scoring": {"bytes": 21105408, "source": "dispatch.cu", "source_sha256":
-        "b759e8825262f3d3f45b9c2ae974c2cf85052998c0590251ae60ce864551d683"},
-    "order": {"bytes": 28051968, "source": "order.cu", "source_sha256":
-        "fb539521c56dde0a33e6d7cc639e55412aeecb48df1925cd54246196181efc3f"},
+    "calibrate": {"bytes": 12528896, "source": "calibrate.cu", "source_sha256":
+        "2f83dd02ef548a1ccd5f242dcc4e1acbc042d27ed766c09a9fee8254258a9f08"},
+    "occupancy": {"bytes": 31162112, "source": "occupancy.cu", "source_sha256":
+        "95fe750b69fea13a50b9de4e10b594bd6205d337663abdff186ad19f26cdc64c"},
+    "dispatch": {"bytes": 26569728, "source": "dispatch.cu", "source_sha256":
+        "788a080e0f93cd3224dde11564cf2454c6346cf5204b8a668de901d09b4b0aa7"},
+    "dispatch_scoring": {"bytes": 21115904, "source": "dispatch.cu", "source_sha256":
+        "788a080e0f93cd3224dde11564cf2454c6346cf5204b8a668de901d09b4b0aa7"},
+    "order": {"bytes": 28059136, "source": "order.cu", "source_sha256":
+        "87e262bc4decc273368b898d6494fe57330bb886e0904bea27c7cb185493aae3"},
 }
 KERNELS = {
     "calibrate": "calibrate_fused_kernel (maps_calibrate: select passes and bounds in one "
